@@ -1,26 +1,31 @@
-// First-layer ("stem") convolution on the tensor cores: C_in <= 4 (the RGB input), kernel up to
-// 7x7, stride 1 or 2, up to 64 output channels, bias + activation.
+// First-layer ("stem") convolution on the tensor cores: C_in <= 4 (the RGB input), kernel up to 11x11, stride 1, 2 or 4,
+// up to 64 output channels, bias + activation.
 //
-// With three input channels a tap is only 6 bytes wide, far below what TMA can address (16-byte
-// strides) or a UMMA K step can use, so the implicit-GEMM operand is built in shared memory by the
-// CTA's own threads: for output pixel m and kernel row r the kw * C_in input values are contiguous
-// in NHWC memory; they go (zero outside the image) into K positions r*KR .. r*KR+kw*C_in-1 of row m
-// of a 128-byte-swizzled A tile (KR = kw*C_in rounded up to 8, K = kh*KR rounded up to 64).  The
-// input patch under a tile of output pixels is a few KB, the A tile built from it 10x that, so the
-// patch is first staged in shared memory (one pass of 2-byte loads, prefetched a tile ahead into
-// registers) and the A rows are then cut out of it with 4-byte shared loads, a 16-bit funnel shift
-// where a row starts on an odd half, and 16-byte swizzled stores.  The positions between kw*C_in
-// and KR receive the next pixels of the patch (finite values) and meet zero weights.
-// The weights are laid out the same way once per CTA.  One thread then issues the UMMAs
-// (M = 128 pixels, N = C_out, K) into one of two TMEM accumulators while the same eight warps
-// build the next tile and drain the previous one (bias, activation, fp16 rounding, staging tile,
-// TMA store).  Eq. 1 counts kh*kw*C_in*C_out MACs per output pixel; the padded K positions hold
-// zeros on both operands.
+// With three input channels a tap is only 6 bytes wide, far below what TMA can address (16-byte strides), so the CTA's own
+// threads stage the input patch in shared memory - but nothing more than the patch: no im2col rows are built.  A pixel is
+// padded to four channels (8 bytes), two pixels make a 16-byte unit, and the units of a patch row are laid out so that
+// neighbouring OUTPUT pixels are neighbouring units.  That is exactly a K-major operand without swizzle: eight pixels of
+// the tile's row are one 8 x 16-byte core matrix (128 contiguous bytes), the next row of the tile is `stride` patch rows
+// further (the descriptor's stride offset), and the next two kernel columns are another window of the same units, a fixed
+// distance away (its leading offset).  Every K = 16 step therefore reads the patch in place; overlapping windows cost
+// nothing but the tensor core's own operand reads.
+//   stride 1: unit u = pixels u, u + 1 (each pixel stored twice); kernel columns 4i .. 4i+3 = units x + 4i, x + 4i + 2
+//   stride 2: unit u = pixels 2u, 2u + 1;                         kernel columns 4i .. 4i+3 = units x + 2i, x + 2i + 1
+//   stride 4: even and odd pairs in two planes;                   kernel columns 4i .. 4i+3 = unit x + i of either plane
+// Kernel columns past k_w, the fourth channel and output channels past C_out meet zero weights.
+//
+// Work item = 1 .. 4 tiles of 8 x 16 output pixels (M = 128) side by side that share one patch.  Eight warps build
+// patches (two buffers), two warps issue the UMMAs of alternate tiles (N = C_out), four groups of four warps each own one
+// accumulator and drain every fourth tile (bias, activation, fp16 rounding, staging tile, TMA store).
+// Bound by the patch builders' and epilogue warps' instruction streams (an instruction per warp every eleven cycles, 0.6
+// per scheduler and cycle; the output's HBM writes come to a third to a half of the time).  Against the first version,
+// which cut im2col rows of K = kh * kw * C_in out of the patch with eight warps that also drained the tiles: 7x7/2 3 -> 64
+// at 224x224, batch 32 50.2 -> 27.1 us; 3x3/2 3 -> 32, batch 64 66.0 -> 32.2 us; 3x3 3 -> 64, batch 8 33.3 -> 17.5 us; one
+// image of the 7x7/2 layer 9.4 -> 7.3 us; 11x11/4 3 -> 64 (which ran on the CUDA cores) at batch 32 590 -> 23.6 us.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -29,380 +34,423 @@ namespace dlf {
 
 namespace {
 
-constexpr int kWorkWarps = 8;                 // warps 0..7 build A tiles and run the epilogue
-constexpr int kMmaWarp = kWorkWarps;          // warp 8 issues the UMMAs and owns the TMEM allocation
-constexpr int kThreads = 32 * (kWorkWarps + 1);
-constexpr int kPlane = 128 * 128;             // one 64-wide K chunk of the A tile
-constexpr int kMaxKChunks = 4;
-constexpr int kMaxDynSmem = 232448 - 1024;   // the 227 KB per CTA less the kernel's static shared memory
+constexpr int kGroups = 4;                     // epilogue groups of four warps (one per TMEM lane quarter); group g owns accumulator g
+constexpr int kEpiWarps = 4 * kGroups;         // warps 0..15
+constexpr int kPatchWarp0 = kEpiWarps;         // warps 16..23 build patches
+constexpr int kPatchWarps = 8;
+constexpr int kMmaWarp0 = kPatchWarp0 + kPatchWarps;
+constexpr int kMmaWarps = 2;                   // issuers, alternate tiles: a lone warp's instruction stream would be the bound
+constexpr int kThreads = 32 * (kMmaWarp0 + kMmaWarps);
+constexpr int kTileW = 8, kTileH = 16;         // output pixels of one UMMA tile
+constexpr int kMaxTiles = 4;                   // tiles side by side in a work item
+constexpr int kStage = 128 * 128;              // staging tile: 128 pixels x 64 channels
+constexpr int kUnroll = 4;                     // units a patch thread has in flight
+constexpr int kMaxDynSmem = 232448 - 1024;     // the 227 KB per CTA less the kernel's static shared memory
 
 struct StemParams {
     const __half* x;
     const __half* w;
     const float* bias;
     int* status;
-    int N, H, W, Cin, Ho, Wo, Cout;
+    int H, W, Ho, Wo, Cout;
     int kh, kw, stride, pad, act;
-    int KR, kchunks, BN;
-    int TW, TH, TN, tiles_w, tiles_h, tiles_n, n_work;
-    int lw, lh;                 // log2 of TW, TH (tile extents are powers of two)
-    int rows_img, pitch_w;      // patch rows per image of the tile, 32-bit words per patch row
-    int patch_words, patch_off; // words of one patch buffer; byte offset of the two patch buffers
+    int BN, steps;                  // steps: K = 16 UMMAs per kernel row
+    int tiles, tiles_w, tiles_h, n_work;   // tiles per work item; work items per row and column of an image
+    int units, n_units;             // units per patch row (both planes), units of the patch
+    int lp;                         // log2 of the number of planes
+    int pitch, plane_bytes, patch_bytes;
+    int px_unit;                    // input pixels from one unit to the next
+    int a_lbo, a_step, b_lbo, b_step;   // bytes: second half of a K step, next K step
+    uint32_t units_magic, kw_magic, per_co_magic;   // quotients by multiplication (see magic())
+    int last_word, tail;            // last 32-bit word of the input; 1: only its lower half belongs to the tensor
+    int stage_off, patch_off;
 };
 
-constexpr int kPatchRegs = 8;                 // prefetched patch words per thread
-constexpr int kMaxPatchWords = kPatchRegs * 32 * kWorkWarps;
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes, `lbo` bytes between the two core matrices of a
+// K = 16 step, `sbo` bytes between groups of eight rows.
+__device__ __forceinline__ uint64_t umma_desc_plain(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(lbo >> 4) << 16) | (static_cast<uint64_t>(sbo >> 4) << 32) |
+           (static_cast<uint64_t>(1) << 46);
+}
 
-__device__ __forceinline__ void work_bar_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kWorkWarps) : "memory"); }
+__device__ __forceinline__ int quotient(int i, uint32_t magic) { return magic ? static_cast<int>(__umulhi(static_cast<uint32_t>(i), magic)) : i; }
 
-// CIN > 0: the channel count is a compile-time constant (the tap / channel index arithmetic of the
-// gather folds away); CIN == 0: any channel count up to 4.
+struct ItemOrigin { int wo0, ho0, n; };
+__device__ __forceinline__ ItemOrigin decode_item(const StemParams& p, int t) {
+    ItemOrigin o;
+    o.wo0 = (t % p.tiles_w) * p.tiles * kTileW;
+    t /= p.tiles_w;
+    o.ho0 = (t % p.tiles_h) * kTileH;
+    o.n = t / p.tiles_h;
+    return o;
+}
+// tiles of an item that hold any output pixel
+__device__ __forceinline__ int item_tiles(const StemParams& p, const ItemOrigin& o) {
+    return min(p.tiles, (p.Wo - o.wo0 + kTileW - 1) / kTileW);
+}
+
+// The K = 16 steps of one tile: kernel rows are patch rows, the steps of a row are further windows of the same units.  Sizes
+// known at compile time unroll into straight-line issue code (a loop costs its warp about 100 cycles per UMMA).
+template <int KH, int STEPS>
+__device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t a_row16, uint32_t a_step16, uint32_t b_step16, uint32_t idesc) {
+#pragma unroll
+    for (int r = 0; r < KH; r++, ad += a_row16) {
+#pragma unroll
+        for (int i = 0; i < STEPS; i++, bd += b_step16) umma_f16(d_tmem, ad + static_cast<uint32_t>(i) * a_step16, bd, idesc, (r | i) != 0);
+    }
+}
+
 template <int CIN>
 __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_constant__ CUtensorMap tmy, const StemParams p) {
-    const int cin = CIN > 0 ? CIN : p.Cin;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t a_full_bar[2], t_full_bar[2];
+    __shared__ uint64_t wfull_bar, pfull_bar[2], pempty_bar[2], tfull_bar[kGroups], tempty_bar[kGroups];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    __shared__ float bias_s[64];
+    __shared__ __align__(16) float bias_s[64];
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* sbase = smem_raw + (base - smem_u32(smem_raw));
-    // layout: A[2][kchunks][128 x 128 B] | B[kchunks][64 x 128 B] | staging [2][128 x 128 B] | patch [2]
-    const int a_bytes = p.kchunks * kPlane;
-    uint8_t* bsm = sbase + 2 * a_bytes;
-    uint8_t* stage_out = bsm + p.kchunks * 8192;
-    uint32_t* patch = reinterpret_cast<uint32_t*>(sbase + p.patch_off);   // [2][patch_words]
+    // layout: weights [kh * steps][2][BN][16 B] (padded: see b_step) | staging tiles | two patches
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort_flag = &abort_s;
 
     if (threadIdx.x == 0) {
         abort_s = 0;
+        mbar_init(&wfull_bar, kEpiWarps);
         for (int i = 0; i < 2; i++) {
-            mbar_init(&a_full_bar[i], kWorkWarps);
-            mbar_init(&t_full_bar[i], 1);
+            mbar_init(&pfull_bar[i], kPatchWarps);
+            mbar_init(&pempty_bar[i], kMmaWarps);
+        }
+        for (int i = 0; i < kGroups; i++) {
+            mbar_init(&tfull_bar[i], 1);
+            mbar_init(&tempty_bar[i], 4);
         }
         fence_barrier_init();
         tma_prefetch_desc(&tmy);
     }
-    if (warp == kMmaWarp) {
-        tmem_alloc(&tmem_base_s, 128);
+    if (warp == kMmaWarp0) {
+        tmem_alloc(&tmem_base_s, 64 * kGroups);
         tmem_relinquish();
     }
-    if (threadIdx.x < 64) bias_s[threadIdx.x] = threadIdx.x < p.Cout ? __ldg(p.bias + threadIdx.x) : 0.0f;
-    // zero both A buffers (their K padding is never written again) and lay out the weights
-    for (int i = threadIdx.x; i < (2 * a_bytes + p.kchunks * 8192) / 16; i += kThreads)
-        reinterpret_cast<uint4*>(sbase)[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = threadIdx.x; i < 2 * p.patch_words; i += kThreads) patch[i] = 0u;
-    __syncthreads();
-    {
-        const int per_co = p.kh * p.kw * cin;
-        for (int i = threadIdx.x; i < p.Cout * per_co; i += kThreads) {
-            const int co = i / per_co, rem = i - co * per_co;
-            const int r = rem / (p.kw * cin), sc = rem - r * (p.kw * cin);
-            const int k = r * p.KR + sc;
-            *reinterpret_cast<__half*>(bsm + (k >> 6) * 8192 + co * 128 + ((((k & 63) >> 3) ^ (co & 7)) << 4) + (k & 7) * 2) = p.w[i];
-        }
-    }
-    fence_proxy_async_smem();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     pdl_launch_dependents();
-    pdl_wait();  // weights are constants; the input may come from the previous kernel
     const uint32_t tmem_base = tmem_base_s;
 
-    if (warp == kMmaWarp) {
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_f16(p.BN);
-            uint32_t j = 0;
-            for (int t = blockIdx.x; t < p.n_work; t += gridDim.x, j++) {
-                const uint32_t b = j & 1u;
-                if (!mbar_wait(&a_full_bar[b], (j >> 1) & 1u, abort_flag, p.status, 0x900 | (blockIdx.x << 12))) break;
+    if (warp >= kMmaWarp0) {
+        // ---- UMMA issuers: warp-uniform loops, one elected lane issues; issuer w takes every other tile ----
+        const uint32_t w = warp - kMmaWarp0;
+        const uint32_t idesc = umma_idesc_f16(p.BN);
+        const uint64_t a_desc = umma_desc_plain(base + p.patch_off, p.a_lbo, p.stride * p.pitch);
+        const uint64_t b_desc = umma_desc_plain(base, p.b_lbo, 128);
+        const uint32_t a_row16 = static_cast<uint32_t>(p.pitch) >> 4, a_step16 = static_cast<uint32_t>(p.a_step) >> 4, b_step16 = static_cast<uint32_t>(p.b_step) >> 4;
+        const int shape = p.kh == p.kw ? p.kh : 0;
+        uint32_t j = 0, seq = 0, ph = 0;   // ph: phase of this issuer's accumulators (two each, taken in turn)
+        bool ok = mbar_wait_warp(&wfull_bar, 0u, abort_flag, p.status, 0x800 | (blockIdx.x << 12));
+        for (int t = blockIdx.x; t < p.n_work && ok; t += gridDim.x, j++) {
+            const int nt = item_tiles(p, decode_item(p, t));
+            const uint32_t b = j & 1u;
+            ok = mbar_wait_warp(&pfull_bar[b], (j >> 1) & 1u, abort_flag, p.status, 0x900 | (blockIdx.x << 12));
+            if (!ok) break;
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int k = 0; k < nt; k++, seq++) {
+                if ((seq & 1u) != w) continue;
+                const uint32_t acc = seq & (kGroups - 1);
+                ok = mbar_wait_warp(&tempty_bar[acc], ph ^ 1u, abort_flag, p.status, 0xB00 | (blockIdx.x << 12));
+                if (!ok) break;
+                if (acc == w + 2) ph ^= 1u;
                 tc_fence_after_sync();
-                const uint32_t d_tmem = tmem_base + b * 64u;
-                for (int kc = 0; kc < p.kchunks; kc++) {
-                    const uint32_t a_lo = umma_desc_lo(base + b * a_bytes + kc * kPlane);
-                    const uint32_t b_lo = umma_desc_lo(base + 2 * a_bytes + kc * 8192);
-#pragma unroll
-                    for (int ks = 0; ks < 4; ks++)
-                        umma_f16_lo(d_tmem, a_lo + 2 * ks, kDescHiSw128, b_lo + 2 * ks, idesc, (kc | ks) != 0);
+                const uint32_t d_tmem = tmem_base + acc * 64u;
+                const uint64_t ad = a_desc + ((b * static_cast<uint32_t>(p.patch_bytes) + k * 128u) >> 4);
+                if (elect_one()) {
+                    if (shape == 3) issue_tile<3, 1>(d_tmem, ad, b_desc, a_row16, a_step16, b_step16, idesc);
+                    else if (shape == 5) issue_tile<5, 2>(d_tmem, ad, b_desc, a_row16, a_step16, b_step16, idesc);
+                    else if (shape == 7) issue_tile<7, 2>(d_tmem, ad, b_desc, a_row16, a_step16, b_step16, idesc);
+                    else if (shape == 11) issue_tile<11, 3>(d_tmem, ad, b_desc, a_row16, a_step16, b_step16, idesc);
+                    else {
+                        uint64_t arow = ad, bd = b_desc;
+#pragma unroll 1
+                        for (int r = 0; r < p.kh; r++, arow += a_row16)
+#pragma unroll 1
+                            for (int i = 0; i < p.steps; i++, bd += b_step16) umma_f16(d_tmem, arow + static_cast<uint32_t>(i) * a_step16, bd, idesc, (r | i) != 0);
+                    }
+                    umma_commit(&tfull_bar[acc]);
                 }
-                umma_commit(&t_full_bar[b]);
+                __syncwarp();
             }
+            if (ok && elect_one()) umma_commit(&pempty_bar[b]);   // the patch is free once this issuer's UMMAs have read it
+            __syncwarp();
+        }
+    } else if (warp >= kPatchWarp0) {
+        // ---- patch builders ----
+        pdl_wait();   // the input may come from the previous kernel
+        const uint32_t* x32 = reinterpret_cast<const uint32_t*>(p.x);
+        // (a tensor with an odd number of elements ends in half a word)
+        const uint32_t tail_word = p.tail ? static_cast<uint32_t>(__half_as_ushort(p.x[2 * static_cast<long long>(p.last_word)])) : 0u;
+        const int tid = threadIdx.x - 32 * kPatchWarp0;
+        constexpr int kWords = CIN <= 2 ? 2 : 4;   // aligned words that cover a unit's pixels
+        uint32_t j = 0;
+        for (int t = blockIdx.x; t < p.n_work; t += gridDim.x, j++) {
+            const ItemOrigin o = decode_item(p, t);
+            const int hi0 = o.ho0 * p.stride - p.pad, wi0 = o.wo0 * p.stride - p.pad;
+            const int g0 = ((o.n * p.H + hi0) * p.W + wi0) * CIN, row_halves = p.W * CIN;
+            const uint32_t b = j & 1u;
+            if (!mbar_wait(&pempty_bar[b], ((j >> 1) & 1u) ^ 1u, abort_flag, p.status, 0xC00 | (blockIdx.x << 12))) break;
+            uint8_t* patch = sbase + p.patch_off + b * p.patch_bytes;
+#pragma unroll 1
+            for (int i0 = tid; i0 < p.n_units; i0 += 32 * kPatchWarps * kUnroll) {
+                // a unit = two neighbouring pixels: up to 8 consecutive halves of the tensor, which start on any half; the
+                // aligned words that cover them are loaded (all units of the pass in flight together), shifted into place and
+                // spread to four channels per pixel
+                uint32_t w[kUnroll][4];
+                int gw[kUnroll], dst[kUnroll];
+                uint32_t flags = 0u;   // per unit: first pixel inside, second pixel inside, odd start
+                bool edge = false;     // some of the words lie outside the tensor
+#pragma unroll
+                for (int u = 0; u < kUnroll; u++) {
+                    const int i = i0 + u * 32 * kPatchWarps;
+                    const int row = quotient(i, p.units_magic), v = i - row * p.units;
+                    const int wi = wi0 + v * p.px_unit;
+                    const bool row_ok = static_cast<unsigned>(hi0 + row) < static_cast<unsigned>(p.H) && i < p.n_units;
+                    const bool ok0 = row_ok && static_cast<unsigned>(wi) < static_cast<unsigned>(p.W), ok1 = row_ok && static_cast<unsigned>(wi + 1) < static_cast<unsigned>(p.W);
+                    const int g = ok0 || ok1 ? g0 + row * row_halves + v * p.px_unit * CIN : 0;   // a unit with no pixel inside reads the tensor's start
+                    flags |= ((ok0 ? 1u : 0u) | (ok1 ? 2u : 0u) | ((g & 1) ? 4u : 0u)) << (4 * u);
+                    gw[u] = g >> 1;
+                    edge = edge || gw[u] < 0 || gw[u] + kWords - 1 > p.last_word - p.tail;
+                    dst[u] = i < p.n_units ? (v & ((1 << p.lp) - 1)) * p.plane_bytes + row * p.pitch + (v >> p.lp) * 16 : -1;
+                }
+                if (!edge) {
+#pragma unroll
+                    for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+                        for (int e = 0; e < kWords; e++) w[u][e] = __ldg(x32 + gw[u] + e);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < kUnroll; u++)
+#pragma unroll
+                        for (int e = 0; e < kWords; e++) {
+                            const int k = max(min(gw[u] + e, p.last_word), 0);
+                            const uint32_t full = __ldg(x32 + min(k, p.last_word - p.tail));
+                            w[u][e] = k > p.last_word - p.tail ? tail_word : full;
+                        }
+                }
+#pragma unroll
+                for (int u = 0; u < kUnroll; u++) {
+                    const uint32_t f = flags >> (4 * u), sh = (f & 4u) << 2;
+                    uint4 q;
+                    if (CIN == 1) {
+                        const uint32_t a0 = __funnelshift_r(w[u][0], w[u][1], sh);
+                        q = make_uint4(a0 & 0xFFFFu, 0u, a0 >> 16, 0u);
+                    } else if (CIN == 2) {
+                        q = make_uint4(w[u][0], 0u, w[u][1], 0u);
+                    } else if (CIN == 3) {
+                        const uint32_t a0 = __funnelshift_r(w[u][0], w[u][1], sh), a1 = __funnelshift_r(w[u][1], w[u][2], sh), a2 = __funnelshift_r(w[u][2], w[u][3], sh);
+                        q = make_uint4(a0, a1 & 0xFFFFu, __funnelshift_r(a1, a2, 16), a2 >> 16);
+                    } else {
+                        q = make_uint4(w[u][0], w[u][1], w[u][2], w[u][3]);
+                    }
+                    if ((f & 3u) != 3u) {
+                        if (!(f & 1u)) q.x = q.y = 0u;
+                        if (!(f & 2u)) q.z = q.w = 0u;
+                    }
+                    if (dst[u] >= 0) *reinterpret_cast<uint4*>(patch + dst[u]) = q;
+                }
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pfull_bar[b]);
         }
     } else {
-        const int q = warp & 3, half = warp >> 2;
-        const uint32_t* x32 = reinterpret_cast<const uint32_t*>(p.x);
-        const int row_halves = p.W * cin;
-        // Patch word `widx` of a tile sits at (image nl, patch row y, word wI); that split does not
-        // depend on the tile, so each thread keeps it, and the row's offset in the tensor, for its
-        // kPatchRegs words.
-        uint32_t meta[kPatchRegs];
-        int rel[kPatchRegs];
+        // ---- the weights, laid out once as the B operand (constants: ahead of the wait for the previous kernel) ----
+        const int grp = warp >> 2;
+        auto epi_sync = [&]() { asm volatile("bar.sync 5, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
+        for (int i = threadIdx.x; i < p.kh * p.steps * p.b_step / 16; i += 32 * kEpiWarps) reinterpret_cast<uint4*>(sbase)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (threadIdx.x < 64) bias_s[threadIdx.x] = threadIdx.x < p.Cout ? __ldg(p.bias + threadIdx.x) : 0.0f;
+        {
+            const int per_co = p.kh * p.kw * CIN, vecs = p.Cout * per_co / 8;   // (C_out is a multiple of 8)
+            constexpr int kVecs = 4;
+            bool cleared = false;
+            for (int v0 = threadIdx.x; v0 < vecs || !cleared; v0 += 32 * kEpiWarps * kVecs) {
+                uint4 wv[kVecs];
 #pragma unroll
-        for (int i = 0; i < kPatchRegs; i++) {
-            const int widx = min(static_cast<int>(threadIdx.x) + i * 32 * kWorkWarps, p.patch_words - 1);
-            const int prow = widx / p.pitch_w, wI = widx - prow * p.pitch_w;
-            const int nl = prow / p.rows_img, y = prow - nl * p.rows_img;
-            meta[i] = static_cast<uint32_t>(wI) | (static_cast<uint32_t>(y) << 12) | (static_cast<uint32_t>(nl) << 22);
-            rel[i] = (nl * p.H + y) * row_halves;
-        }
-        // A patch row is kept as the aligned 32-bit words of the tensor that cover it, so a row whose
-        // first element sits on an odd half starts one half into its buffer row.  One unconditional
-        // clamped load per word, all in flight together; `okm` keeps which halves lie inside the
-        // image and the batch (the others become zero when the words are stored).
-        // first output pixel of a tile; decoded once per tile (three divisions) and handed from the patch fetch to the
-        // build to the drain
-        struct TileOrigin { int wo0, ho0, n0; };
-        auto decode = [&](int t) {
-            TileOrigin o;
-            int mt = t;
-            o.wo0 = (mt % p.tiles_w) * p.TW;
-            mt /= p.tiles_w;
-            o.ho0 = (mt % p.tiles_h) * p.TH;
-            o.n0 = (mt / p.tiles_h) * p.TN;
-            return o;
-        };
-        auto load_patch = [&](const TileOrigin& to, uint32_t (&pw)[kPatchRegs], uint32_t& okm) {
-            const int wo0 = to.wo0, ho0 = to.ho0, n0 = to.n0;
-            const int wi0 = wo0 * p.stride - p.pad, hi0 = ho0 * p.stride - p.pad;
-            const int tile_base = ((n0 * p.H + hi0) * p.W + wi0) * cin;
-            const int h_lo = max(0, -wi0) * cin, h_hi = (p.W - wi0) * cin;   // halves of a patch row inside the image
-            okm = 0u;
+                for (int u = 0; u < kVecs; u++) wv[u] = __ldg(reinterpret_cast<const uint4*>(p.w) + min(v0 + u * 32 * kEpiWarps, vecs - 1));
+                if (!cleared) { epi_sync(); cleared = true; }   // the zeros are all written
+#pragma unroll 1
+                for (int u = 0; u < kVecs; u++) {
+                    const int v = v0 + u * 32 * kEpiWarps;
+                    if (v >= vecs) break;
+                    int co = quotient(v * 8, p.per_co_magic);
+                    const int rem = v * 8 - co * per_co, rs = rem / CIN;
+                    int c = rem - rs * CIN, r = quotient(rs, p.kw_magic), s = rs - r * p.kw;
+                    const uint4 cur = u == 0 ? wv[0] : (u == 1 ? wv[1] : (u == 2 ? wv[2] : wv[3]));
+                    const unsigned short* h = reinterpret_cast<const unsigned short*>(&cur);
 #pragma unroll
-            for (int i = 0; i < kPatchRegs; i++) {
-                if (i * 32 * kWorkWarps >= p.patch_words) break;   // (uniform) a small patch needs only the first few passes
-                const int wI = meta[i] & 0xFFF, y = (meta[i] >> 12) & 0x3FF, nl = meta[i] >> 22;
-                const int n = n0 + nl, hi_row = hi0 + y;
-                const bool row_ok = n < p.N && hi_row >= 0 && hi_row < p.H;
-                const int g_row = tile_base + rel[i];                // first half of the patch row in the tensor
-                const int h0 = 2 * wI - (g_row & 1);                 // this word's halves, counted from there
-                const bool ok0 = row_ok && h0 >= h_lo && h0 < h_hi, ok1 = row_ok && h0 + 1 >= h_lo && h0 + 1 < h_hi;
-                const int gw = ((g_row & ~1) >> 1) + wI;
-                pw[i] = __ldg(x32 + ((ok0 || ok1) ? gw : 0));
-                okm |= ((ok0 ? 1u : 0u) | (ok1 ? 2u : 0u)) << (2 * i);
-            }
-        };
-        auto store_patch = [&](uint32_t* dst, const uint32_t (&pw)[kPatchRegs], uint32_t okm) {
-#pragma unroll
-            for (int i = 0; i < kPatchRegs; i++) {
-                if (i * 32 * kWorkWarps >= p.patch_words) break;
-                const int widx = threadIdx.x + i * 32 * kWorkWarps;
-                const uint32_t m = ((okm >> (2 * i)) & 1u ? 0x0000FFFFu : 0u) | ((okm >> (2 * i)) & 2u ? 0xFFFF0000u : 0u);
-                if (widx < p.patch_words) dst[widx] = pw[i] & m;
-            }
-        };
-        // rows of the A tile from the staged patch, CH 16-byte chunks per kernel row
-        auto build_rows = [&](auto ch_tag, const TileOrigin& to, uint8_t* abuf, const uint32_t* pbuf) {
-            constexpr int CH = decltype(ch_tag)::value;
-            const int wo0 = to.wo0, ho0 = to.ho0, n0 = to.n0;
-            const int tile_base = ((n0 * p.H + ho0 * p.stride - p.pad) * p.W + wo0 * p.stride - p.pad) * cin;
-            const int sc = p.stride * cin;
-#pragma unroll 2
-            for (int item = threadIdx.x; item < 128 * p.kh; item += 32 * kWorkWarps) {
-                const int m = item & 127, r = item >> 7;
-                const int tx = m & (p.TW - 1), ty = (m >> p.lw) & (p.TH - 1), nl = m >> (p.lw + p.lh);
-                const int yrow = ty * p.stride + r;
-                const int off = ((tile_base + (nl * p.H + yrow) * row_halves) & 1) + tx * sc;   // first half of the K slice
-                const uint32_t* src = pbuf + (nl * p.rows_img + yrow) * p.pitch_w + (off >> 1);
-                const uint32_t sh = (off & 1) * 16;
-                uint32_t w[4 * CH + 1];
-#pragma unroll
-                for (int i = 0; i <= 4 * CH; i++) w[i] = src[i];
-#pragma unroll
-                for (int ck = 0; ck < CH; ck++) {
-                    uint4 o;
-                    o.x = __funnelshift_r(w[4 * ck], w[4 * ck + 1], sh);
-                    o.y = __funnelshift_r(w[4 * ck + 1], w[4 * ck + 2], sh);
-                    o.z = __funnelshift_r(w[4 * ck + 2], w[4 * ck + 3], sh);
-                    o.w = __funnelshift_r(w[4 * ck + 3], w[4 * ck + 4], sh);
-                    const int kchunk = r * CH + ck;  // 16-byte chunk index along K
-                    *reinterpret_cast<uint4*>(abuf + (kchunk >> 3) * kPlane + m * 128 + (((kchunk & 7) ^ (m & 7)) << 4)) = o;
-                }
-            }
-        };
-        uint32_t pw[kPatchRegs];
-        uint32_t pok = 0u;
-        TileOrigin cur = decode(blockIdx.x), next = cur, prev = cur;
-        if (static_cast<int>(blockIdx.x) < p.n_work) {
-            load_patch(cur, pw, pok);
-            store_patch(patch, pw, pok);
-        }
-        // the activation as a clamp: none (-inf, inf), ReLU [0, inf), ReLU6 [0, 6]
-        // (applied to the rounded pair: rounding is monotone and 0 and 6 are fp16 values, so clamping after the rounding gives
-        // the same bits as before it, at one instruction per two values)
-        const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
-        // this warp's 32 output channels per pass of the epilogue keep their bias in registers
-        float breg[32];
-#pragma unroll
-        for (int e = 0; e < 32; e++) breg[e] = bias_s[(half * 32 + e) & 63];
-        work_bar_sync();
-        DLF_TRACE_DECL(tacc, tmark);
-        uint32_t j = 0;
-        bool ok = true;
-        int prev_t = -1;
-        // software pipeline: fetch the patch of tile j+1, build tile j, then drain tile j-1 while the
-        // tensor core works on tile j
-        for (int t = blockIdx.x;; t += gridDim.x, j++) {
-            const bool have = t < p.n_work;
-            const bool have_next = have && t + static_cast<int>(gridDim.x) < p.n_work;
-            DLF_TRACE_ACC(tacc, 0, tmark);
-            if (have_next) {
-                next = decode(t + gridDim.x);
-                load_patch(next, pw, pok);
-            }
-            DLF_TRACE_ACC(tacc, 1, tmark);
-            if (have) {
-                uint8_t* abuf = sbase + (j & 1u) * a_bytes;
-                const uint32_t* pbuf = patch + (j & 1u) * p.patch_words;
-                switch (p.KR >> 3) {
-                    case 1: build_rows(std::integral_constant<int, 1>{}, cur, abuf, pbuf); break;
-                    case 2: build_rows(std::integral_constant<int, 2>{}, cur, abuf, pbuf); break;
-                    case 3: build_rows(std::integral_constant<int, 3>{}, cur, abuf, pbuf); break;
-                    default: build_rows(std::integral_constant<int, 4>{}, cur, abuf, pbuf); break;
-                }
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&a_full_bar[j & 1u]);
-                DLF_TRACE_ACC(tacc, 2, tmark);
-            }
-            if (prev_t >= 0) {
-                const uint32_t jb = j - 1, b = jb & 1u;
-                ok = mbar_wait(&t_full_bar[b], (jb >> 1) & 1u, abort_flag, p.status, 0xA00 | (blockIdx.x << 12));
-                DLF_TRACE_ACC(tacc, 3, tmark);
-                if (!ok) break;
-                tc_fence_after_sync();
-                const int wo0 = prev.wo0, ho0 = prev.ho0, n0 = prev.n0;
-                const int m = q * 32 + lane;
-                const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + b * 64u;
-                uint8_t* sout = stage_out + b * kPlane;   // its previous store was waited for before the last barrier
-                const int cc = half * 32;
-                if (cc < p.BN) {
-                    float v[32];
-                    const int nc = min(32, p.BN - cc);
-                    if (nc == 32) tmem_ld32(taddr + cc, v);
-                    else tmem_ld16(taddr + cc, v);
-#pragma unroll
-                    for (int g = 0; g < 4; g++) {
-                        if (g * 8 >= nc) break;
-                        uint4 o;
-                        uint32_t* ou = reinterpret_cast<uint32_t*>(&o);
-#pragma unroll
-                        for (int e = 0; e < 4; e++)
-                        {
-                            const __half2 hv = __hmin2(__hmax2(__floats2half2_rn(v[g * 8 + 2 * e] + breg[g * 8 + 2 * e], v[g * 8 + 2 * e + 1] + breg[g * 8 + 2 * e + 1]), act_lo), act_hi);
-                            ou[e] = *reinterpret_cast<const uint32_t*>(&hv);
-                        }
-                        const int g8 = (cc >> 3) + g;
-                        *reinterpret_cast<uint4*>(sout + m * 128 + (((g8 & 7) ^ (m & 7)) << 4)) = o;
+                    for (int e = 0; e < 8; e++) {
+                        *reinterpret_cast<unsigned short*>(sbase + (r * p.steps + (s >> 2)) * p.b_step + ((s >> 1) & 1) * p.b_lbo + co * 16 + (s & 1) * 8 + c * 2) = h[e];
+                        if (++c == CIN) { c = 0; if (++s == p.kw) { s = 0; if (++r == p.kh) { r = 0; co++; } } }
                     }
                 }
-                tc_fence_before_sync();
+            }
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&wfull_bar);
+        epi_sync();   // (the bias)
+        pdl_wait();   // the output's memory may still be in use
+
+        // ---- epilogue: group g drains every fourth tile ----
+        const int q = warp & 3;
+        const int m = q * 32 + lane;
+        const bool issuer = (threadIdx.x & 127) == 0;
+        const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
+        uint8_t* sout = sbase + p.stage_off + grp * kStage;
+        uint32_t seq = 0, ph = 0;
+        auto group_sync = [&]() {
+            if (grp == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+            else if (grp == 1) asm volatile("bar.sync 2, 128;" ::: "memory");
+            else if (grp == 2) asm volatile("bar.sync 3, 128;" ::: "memory");
+            else asm volatile("bar.sync 4, 128;" ::: "memory");
+        };
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + grp * 64u;
+        for (int t = blockIdx.x; t < p.n_work; t += gridDim.x) {
+            const ItemOrigin o = decode_item(p, t);
+            const int nt = item_tiles(p, o);
+#pragma unroll 1
+            for (int k = 0; k < nt; k++, seq++) {
+                if ((seq & (kGroups - 1)) != static_cast<uint32_t>(grp)) continue;
+                // (after a wait that gave up the warp goes on to the end without storing: the others of its group are at the
+                // group's barriers, and every later wait returns at once)
+                const bool ok = mbar_wait(&tfull_bar[grp], ph, abort_flag, p.status, 0xA00 | (blockIdx.x << 12));
+                ph ^= 1u;
+                __syncwarp();
+                tc_fence_after_sync();
+                uint32_t r[32];
+                tmem_ld32_issue(taddr, r);
+                if (issuer) tma_store_wait_read();
+                group_sync();   // the staging tile's last store has read it
+#pragma unroll 1
+                for (int cc = 0; cc < p.BN; cc += 32) {
+                    tmem_ld32_wait(r);
+                    if (cc + 32 >= p.BN) {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&tempty_bar[grp]);
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; g++) {
+                        const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g * 8), b1 = *reinterpret_cast<const float4*>(bias_s + cc + g * 8 + 4);
+                        uint4 out;
+                        // (the activation as a clamp of the rounded pair: rounding is monotone and the bounds are fp16 values)
+                        out.x = pack_half2_clamp(__uint_as_float(r[g * 8 + 0]) + b0.x, __uint_as_float(r[g * 8 + 1]) + b0.y, act_lo, act_hi);
+                        out.y = pack_half2_clamp(__uint_as_float(r[g * 8 + 2]) + b0.z, __uint_as_float(r[g * 8 + 3]) + b0.w, act_lo, act_hi);
+                        out.z = pack_half2_clamp(__uint_as_float(r[g * 8 + 4]) + b1.x, __uint_as_float(r[g * 8 + 5]) + b1.y, act_lo, act_hi);
+                        out.w = pack_half2_clamp(__uint_as_float(r[g * 8 + 6]) + b1.z, __uint_as_float(r[g * 8 + 7]) + b1.w, act_lo, act_hi);
+                        const int g8 = (cc >> 3) + g;
+                        *reinterpret_cast<uint4*>(sout + m * 128 + (((g8 & 7) ^ (m & 7)) << 4)) = out;
+                    }
+                    if (cc + 32 < p.BN) {
+                        __syncwarp();
+                        tmem_ld32_issue(taddr + cc + 32, r);
+                    }
+                }
                 fence_proxy_async_smem();
-                DLF_TRACE_ACC(tacc, 4, tmark);
-                work_bar_sync();
-                if (threadIdx.x == 0) {
-                    tma_store_4d(&tmy, sout, 0, wo0, ho0, n0);
+                group_sync();
+                if (issuer && ok) {
+                    tma_store_4d(&tmy, sout, 0, o.wo0 + k * kTileW, o.ho0, o.n);
                     tma_store_commit();
                 }
             }
-            if (!have) break;
-            prev_t = t;
-            prev = cur;
-            cur = next;
-            DLF_TRACE_ACC(tacc, 5, tmark);
-            if (have_next) store_patch(patch + ((j + 1) & 1u) * p.patch_words, pw, pok);
-            // the staging buffer the next drain writes was read by the store before the newest one
-            if (threadIdx.x == 0) tma_store_wait_read1();
-            work_bar_sync();
-            DLF_TRACE_ACC(tacc, 6, tmark);
         }
-        DLF_TRACE_FLUSH(p.status, tacc);
-        if (threadIdx.x == 0) tma_store_wait_read();
+        if (issuer) tma_store_wait_read();
     }
 
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == kMmaWarp) {
+    if (warp == kMmaWarp0) {
         if (abort_s) __nanosleep(20000);
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, 128);
+        tmem_dealloc(tmem_base, 64 * kGroups);
     }
 }
 
-struct Tile {
-    int tw, th, tn;
+// Multiplier for quotient(): i * ceil(2^32 / d) / 2^32 is exact while i < 2^32 / d (here i and d stay below 2^16); 0 for d = 1.
+uint32_t magic(int d) { return d <= 1 ? 0u : static_cast<uint32_t>(((1ull << 32) + d - 1) / d); }
+
+// Everything the geometry decides; tiles == 0 if the layer does not fit.
+struct Layout {
+    int BN, steps, b_lbo, b_step, tiles, rows, units, planes, pitch, plane_bytes, patch_bytes, weight_bytes;
+    size_t smem;
 };
 
-int k_row(const ConvArgs& a) { return (a.kw * a.Cin + 7) / 8 * 8; }
-int k_chunks(const ConvArgs& a) { return (a.kh * k_row(a) + 63) / 64; }
+Layout layout_for(const ConvArgs& a, int tiles) {
+    Layout l{};
+    l.BN = (a.Cout + 15) / 16 * 16;
+    l.steps = (a.kw + 3) / 4;
+    l.rows = (kTileH - 1) * a.stride + a.kh;
+    l.planes = a.stride == 4 ? 2 : 1;
+    // units per plane that the windows of the item's 8 * tiles output columns reach
+    const int cols = kTileW * tiles;
+    const int per_plane = a.stride == 1 ? cols + 4 * l.steps - 2 : (a.stride == 2 ? cols + 2 * l.steps - 1 : cols + l.steps - 1);
+    l.units = per_plane * l.planes;
+    l.pitch = per_plane * 16;
+    l.plane_bytes = (l.rows * l.pitch + 127) / 128 * 128;
+    l.patch_bytes = l.planes * l.plane_bytes;
+    // padded so that neighbouring taps of an output channel, which neighbouring threads scatter, fall into different banks
+    l.b_lbo = l.BN * 16 + 64;
+    l.b_step = 2 * l.b_lbo + 16;
+    l.weight_bytes = (a.kh * l.steps * l.b_step + 1023) / 1024 * 1024;
+    l.smem = static_cast<size_t>(l.weight_bytes) + kGroups * kStage + 2 * l.patch_bytes + 1024;
+    l.tiles = l.smem <= static_cast<size_t>(kMaxDynSmem) && l.rows * l.units < 65536 ? tiles : 0;
+    return l;
+}
 
-// 32-bit words of one input-patch row under a tile `tw` pixels wide: an odd first half, the last
-// pixel's K slice and the word the funnel shift looks ahead
-// The pitch is then padded (by up to 31 words) to the value for which the 32 lanes of a warp, which
-// read the same word of 32 consecutive output pixels' K slices, spread over the most banks.
-int patch_pitch_words(const ConvArgs& a, int tw, int th) {
-    const int need = (((tw - 1) * a.stride * a.Cin + k_row(a) + 4 + 7) / 8 * 8) / 2;
-    const int rows_img = (th - 1) * a.stride + a.kh;
-    int best = need, best_conf = 1 << 30;
-    for (int pitch = need; pitch < need + 32; pitch++) {
-        int worst = 0;
-        for (int q = 0; q < 4 && q * 32 < 128; q++)
-            for (int odd = 0; odd < 2; odd++) {
-                int cnt[32] = {0};
-                for (int lane = 0; lane < 32; lane++) {
-                    const int m = q * 32 + lane, tx = m % tw, ty = (m / tw) % th, nl = m / (tw * th);
-                    const int off = odd + tx * a.stride * a.Cin;
-                    cnt[((nl * rows_img + ty * a.stride) * pitch + (off >> 1)) & 31]++;
-                }
-                int mx = 0;
-                for (int b = 0; b < 32; b++) mx = std::max(mx, cnt[b]);
-                worst = std::max(worst, mx);
-            }
-        if (worst < best_conf) {
-            best_conf = worst;
-            best = pitch;
+// Tiles per work item: wider items share the halo of the patch, narrower ones spread a small map over more SMs and leave a
+// shorter last round.  Cost = rounds of the grid x the slower of an item's UMMAs (or its epilogue) and its patch, plus the
+// first patch, which nothing overlaps; in SM clocks.
+Layout pick_layout(const ConvArgs& a, int sm_count) {
+    Layout best{};
+    double best_cost = 0.0;
+    for (int tiles = 1; tiles <= kMaxTiles; tiles++) {
+        if (tiles > 1 && kTileW * (tiles - 1) >= a.Wo) break;
+        const Layout l = layout_for(a, tiles);
+        if (l.tiles == 0) continue;
+        const long long items = static_cast<long long>((a.Wo + kTileW * tiles - 1) / (kTileW * tiles)) * ((a.Ho + kTileH - 1) / kTileH) * a.N;
+        const long long rounds = (items + sm_count - 1) / sm_count;
+        const double tile = std::max(a.kh * l.steps * 48.0, l.BN <= 32 ? 180.0 : 300.0), patch = 900.0 + l.rows * l.units * 0.35;
+        const double cost = rounds * std::max(tiles * tile, patch) + patch;
+        if (best.tiles == 0 || cost < best_cost) {
+            best = l;
+            best_cost = cost;
         }
     }
     return best;
 }
-int patch_rows(const ConvArgs& a, int th) { return (th - 1) * a.stride + a.kh; }
 
-// Fewest tiles of 128 output pixels (tw x th x tn, powers of two) whose input patch fits the
-// prefetch registers; tw == 0 if none does.
-Tile pick_tile(const ConvArgs& a) {
-    const int N = a.N, Ho = a.Ho, Wo = a.Wo;
-    Tile best{0, 0, 0};
-    long long best_tiles = -1;
-    for (int tw = 128; tw >= 1; tw >>= 1)
-        for (int th = 128 / tw; th >= 1; th >>= 1) {
-            const int tn = 128 / (tw * th);
-            if (static_cast<long long>(tn) * patch_rows(a, th) * patch_pitch_words(a, tw, th) > kMaxPatchWords) continue;
-            const long long tiles = static_cast<long long>((Wo + tw - 1) / tw) * ((Ho + th - 1) / th) * ((N + tn - 1) / tn);
-            if (best_tiles < 0 || tiles < best_tiles) {
-                best_tiles = tiles;
-                best = Tile{tw, th, tn};
-            }
-        }
-    return best;
-}
-
-// The patch is fetched as aligned 32-bit words indexed with 32-bit arithmetic: an even number of
-// input elements (no word straddles the end of the tensor) below 2^31.
+// 32-bit indexing of the input, with room for the patch rows and columns outside the image.
 bool input_ok(const ConvArgs& a) {
-    const long long total = static_cast<long long>(a.N) * a.H * a.W * a.Cin;
-    return total % 2 == 0 && total + 2LL * 128 * a.H * a.W * a.Cin < 0x7fffffffLL;
+    const long long row = static_cast<long long>(a.W) * a.Cin;
+    const long long total = static_cast<long long>(a.N) * a.H * row;
+    return total >= 2 && total + 256 * (row + 256) < 0x7fffffffLL;
 }
-size_t fixed_bytes(const ConvArgs& a) { return static_cast<size_t>(k_chunks(a)) * (2 * kPlane + 8192) + 2 * kPlane; }
-size_t smem_bytes(const ConvArgs& a) { return fixed_bytes(a) + 2 * kMaxPatchWords * 4 + 1024; }
+
+typedef void (*KernelFn)(const CUtensorMap, const StemParams);
+KernelFn pick_kernel(int cin) {
+    switch (cin) {
+        case 1: return stem_tc_kernel<1>;
+        case 2: return stem_tc_kernel<2>;
+        case 3: return stem_tc_kernel<3>;
+        default: return stem_tc_kernel<4>;
+    }
+}
 
 }  // namespace
 
 bool stem_tc_supported(const ConvArgs& a) {
-    return a.groups == 1 && a.Cin >= 1 && a.Cin <= 4 && a.Cout % 8 == 0 && a.Cout >= 8 && a.Cout <= 64 && a.kh <= 7 &&
-           a.kw <= 7 && (a.stride == 1 || a.stride == 2) && a.pool == 0 && a.res == nullptr && k_chunks(a) <= kMaxKChunks &&
-           a.N >= 1 && a.Ho >= 1 && a.Wo >= 1 && smem_bytes(a) <= static_cast<size_t>(kMaxDynSmem) && input_ok(a) && pick_tile(a).tw > 0;
+    return a.groups == 1 && a.Cin >= 1 && a.Cin <= 4 && a.Cout % 8 == 0 && a.Cout >= 8 && a.Cout <= 64 && a.kh >= 1 && a.kh <= 11 &&
+           a.kw >= 1 && a.kw <= 11 && (a.stride == 1 || a.stride == 2 || a.stride == 4) && a.pool == 0 && a.res == nullptr && a.N >= 1 && a.Ho >= 1 &&
+           a.Wo >= 1 && input_ok(a) && layout_for(a, 1).tiles > 0;
 }
 
 int stem_tc_init() {
@@ -410,9 +458,10 @@ int stem_tc_init() {
     const int dev = current_device_slot();
     if (dev < 0) return DLF_E_UNSUPPORTED;
     if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(stem_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(stem_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
-        if (e != cudaSuccess) return cuda_fail(e);
+        for (int cin = 1; cin <= 4; cin++) {
+            cudaError_t e = cudaFuncSetAttribute(pick_kernel(cin), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+            if (e != cudaSuccess) return cuda_fail(e);
+        }
         attr_set[dev] = true;
     }
     return DLF_OK;
@@ -423,42 +472,44 @@ int launch_stem_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_
     if (reinterpret_cast<uintptr_t>(a.x) & 3u) return DLF_E_INVALID_ARG;
     int rc = stem_tc_init();
     if (rc) return rc;
+    const Layout l = pick_layout(a, sm_count);
     StemParams p{};
     p.x = static_cast<const __half*>(a.x); p.w = static_cast<const __half*>(a.w); p.bias = a.bias; p.status = status_dev;
-    p.N = a.N; p.H = a.H; p.W = a.W; p.Cin = a.Cin; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
+    p.H = a.H; p.W = a.W; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
     p.kh = a.kh; p.kw = a.kw; p.stride = a.stride; p.pad = a.pad; p.act = a.act;
-    p.KR = k_row(a);
-    p.kchunks = k_chunks(a);
-    p.BN = (a.Cout + 15) / 16 * 16;
-    const Tile tl = pick_tile(a);
-    p.TW = tl.tw; p.TH = tl.th; p.TN = tl.tn;
-    for (p.lw = 0; (1 << p.lw) < tl.tw; p.lw++) {}
-    for (p.lh = 0; (1 << p.lh) < tl.th; p.lh++) {}
-    p.rows_img = patch_rows(a, tl.th);
-    p.pitch_w = patch_pitch_words(a, tl.tw, tl.th);
-    p.patch_words = tl.tn * p.rows_img * p.pitch_w;
-    p.patch_off = static_cast<int>(fixed_bytes(a));
-    p.tiles_w = (a.Wo + tl.tw - 1) / tl.tw;
-    p.tiles_h = (a.Ho + tl.th - 1) / tl.th;
-    p.tiles_n = (a.N + tl.tn - 1) / tl.tn;
-    const long long n_work = static_cast<long long>(p.tiles_w) * p.tiles_h * p.tiles_n;
+    p.BN = l.BN; p.steps = l.steps; p.tiles = l.tiles;
+    p.tiles_w = (a.Wo + kTileW * l.tiles - 1) / (kTileW * l.tiles);
+    p.tiles_h = (a.Ho + kTileH - 1) / kTileH;
+    const long long n_work = static_cast<long long>(p.tiles_w) * p.tiles_h * a.N;
     if (n_work > 0x7fffffffLL) return DLF_E_UNSUPPORTED;
     p.n_work = static_cast<int>(n_work);
+    p.units = l.units; p.n_units = l.rows * l.units;
+    p.lp = l.planes == 2 ? 1 : 0;
+    p.pitch = l.pitch; p.plane_bytes = l.plane_bytes; p.patch_bytes = l.patch_bytes;
+    p.px_unit = a.stride == 1 ? 1 : 2;
+    p.a_lbo = a.stride == 1 ? 32 : (a.stride == 2 ? 16 : l.plane_bytes);
+    p.a_step = a.stride == 1 ? 64 : (a.stride == 2 ? 32 : 16);
+    p.b_lbo = l.b_lbo; p.b_step = l.b_step;
+    p.units_magic = magic(l.units); p.kw_magic = magic(a.kw); p.per_co_magic = magic(a.kh * a.kw * a.Cin);
+    const long long total = static_cast<long long>(a.N) * a.H * a.W * a.Cin;
+    p.last_word = static_cast<int>((total - 1) / 2);
+    p.tail = static_cast<int>(total & 1);
+    p.stage_off = l.weight_bytes;
+    p.patch_off = l.weight_bytes + kGroups * kStage;
     CUtensorMap tmy;
     {
         const uint64_t dims[4] = {static_cast<uint64_t>(a.Cout), static_cast<uint64_t>(a.Wo), static_cast<uint64_t>(a.Ho),
                                   static_cast<uint64_t>(a.N)};
         const uint64_t strides[3] = {static_cast<uint64_t>(a.Cout) * 2, static_cast<uint64_t>(a.Wo) * a.Cout * 2,
                                      static_cast<uint64_t>(a.Ho) * a.Wo * a.Cout * 2};
-        const uint32_t box[4] = {64, static_cast<uint32_t>(tl.tw), static_cast<uint32_t>(tl.th), static_cast<uint32_t>(tl.tn)};
+        const uint32_t box[4] = {64, kTileW, kTileH, 1};
         const uint32_t es[4] = {1, 1, 1, 1};
         rc = encode_tmap(&tmy, a.y, 4, dims, strides, box, es);
         if (rc) return rc;
     }
     const int grid = std::max(1, std::min(sm_count, p.n_work));
-    const size_t smem = std::max<size_t>(smem_bytes(a), 120 * 1024);
-    cudaError_t e = a.Cin == 3 ? launch_kernel(stem_tc_kernel<3>, grid, kThreads, smem, s, tmy, p)
-                               : launch_kernel(stem_tc_kernel<0>, grid, kThreads, smem, s, tmy, p);
+    const size_t smem = std::max<size_t>(l.smem, 120 * 1024);   // (one CTA of a persistent grid per SM)
+    cudaError_t e = launch_kernel(pick_kernel(a.Cin), grid, kThreads, smem, s, tmy, p);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
