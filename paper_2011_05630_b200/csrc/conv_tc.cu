@@ -1204,17 +1204,16 @@ int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
-int g_seq_cooperative = 0;
 bool conv_seq_layer_supported(const ConvArgs& a) { return conv_tc_supported(a); }
 int conv_seq_max_layers() { return kMaxSeq; }
 
-// Several dense convolutions as one persistent kernel on `sm_count` CTAs (a cooperative launch: every CTA must be resident,
-// they wait for one another between the layers).  `sync_dev`: two words of device memory that are zero between launches.
+// Several dense convolutions as one persistent kernel on `sm_count` CTAs (every CTA must be resident: they wait for
+// one another between the layers).  `sync_dev`: two words of device memory that are zero between launches.
 int launch_conv_seq(const ConvArgs* layers, int n_layers, int sm_count, int* status_dev, unsigned* sync_dev, cudaStream_t s) {
     if (n_layers < 1 || n_layers > kMaxSeq || !sync_dev) return DLF_E_PLAN;
     int rc = conv_tc_init();
     if (rc) return rc;
-    static SeqParams sp;   // (large: not on the stack; the launch copies it)
+    static thread_local SeqParams sp;   // (large: not on the stack; the launch copies it)
     std::memset(&sp, 0, sizeof(sp));
     size_t smem = 0;
     for (int l = 0; l < n_layers; l++) {
@@ -1234,17 +1233,8 @@ int launch_conv_seq(const ConvArgs* layers, int n_layers, int sm_count, int* sta
     sp.n_layers = n_layers;
     sp.sync = sync_dev;
     sp.status = status_dev;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(sm_count));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = g_seq_cooperative ? 1 : 0;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, conv_seq_kernel, sp);
+    // (not overlapped with the kernel before it: its CTAs wait for one another and must all find a free SM)
+    cudaError_t e = launch_kernel_opt(conv_seq_kernel, sm_count, kThreads, smem, s, false, sp);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 

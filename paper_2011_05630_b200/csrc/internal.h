@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/dlfusion.h"
@@ -86,12 +87,32 @@ int kernels_init();
 int conv_tc_init();
 int chain_tc_init();
 
+// While set (calling thread only), launch_kernel() gives this node of an instantiated graph the launch's parameters instead
+// of launching: a captured plan follows its caller's input and output buffers without being captured again.
+struct GraphNodeUpdate {
+    cudaGraphExec_t exec;
+    cudaGraphNode_t node;
+};
+extern thread_local const GraphNodeUpdate* g_node_update;
+
 // Launches a kernel, optionally with programmatic dependent launch (the kernel must then call
 // pdl_wait() before it touches anything its predecessor in the stream produces).
 extern int g_use_pdl;
 extern int g_conv_row_mode;  // conv_tc row mode: 0 never, 1 where it cuts the streamed bytes by a fifth, 2 wherever it applies
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args... args) {
+inline cudaError_t launch_kernel_opt(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args&&... args) {
+    if (g_node_update) {
+        std::tuple<KArgs...> vals(static_cast<KArgs>(args)...);
+        void* ptrs[sizeof...(KArgs)];
+        std::apply([&](auto&... v) { int i = 0; ((ptrs[i++] = const_cast<void*>(static_cast<const void*>(&v))), ...); }, vals);
+        cudaKernelNodeParams np = {};
+        np.func = reinterpret_cast<void*>(kernel);
+        np.gridDim = dim3(static_cast<unsigned>(grid));
+        np.blockDim = dim3(static_cast<unsigned>(block));
+        np.sharedMemBytes = static_cast<unsigned>(smem);
+        np.kernelParams = ptrs;
+        return cudaGraphExecKernelNodeSetParams(g_node_update->exec, g_node_update->node, &np);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(static_cast<unsigned>(block));
@@ -101,8 +122,12 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), int grid, int block, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = g_use_pdl ? 1 : 0;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, Args&&... args) {
+    return launch_kernel_opt(kernel, grid, block, smem, s, g_use_pdl != 0, args...);
 }
 
 // kernels_mem.cu

@@ -3,7 +3,8 @@
 // max / global-average pooling and the weight-streaming fully connected layer.  All use 128-bit
 // accesses along the channel dimension of the NHWC tensors, fp32 arithmetic and a single
 // round-to-nearest-even to fp16 per layer.  Grids are sized from the SM-count knob and loop over
-// the work with a grid stride.
+// the work with a grid stride.  Launched like the tensor-core kernels with programmatic dependent launch: a kernel's blocks
+// start while its predecessor drains, and wait before they read what it wrote.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -32,6 +33,8 @@ constexpr int kDirCi = 64;
 
 __global__ void __launch_bounds__(128) conv_direct_kernel(ConvArgs a, long long n_pix, int co_blocks) {
     __shared__ float wsm[kDirCi][kDirCo];
+    pdl_launch_dependents();
+    pdl_wait();
     const __half* x = static_cast<const __half*>(a.x);
     const __half* w = static_cast<const __half*>(a.w);
     const __half* res = static_cast<const __half*>(a.res);
@@ -122,6 +125,7 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
     const int c8n = a.Cout / 8;
     const long long tid = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     const long long nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
+    pdl_launch_dependents();
     if (tid >= total) return;
     const int c0 = static_cast<int>(tid % c8n) * 8;
     float w[9][8], b[8];
@@ -137,6 +141,7 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
             for (int t = 0; t < 9; t++) w[t][j] = __half2float(wv[j * 9 + t]);
         }
     }
+    pdl_wait();   // (the weights above are constants)
     const __half2 lo = __float2half2_rn(a.act >= 1 ? 0.0f : -INFINITY), hi = __float2half2_rn(a.act == 2 ? 6.0f : INFINITY);   // applied to rounded pairs
     const __half* x = static_cast<const __half*>(a.x);
     const __half* res = static_cast<const __half*>(a.res);
@@ -221,6 +226,8 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
 __global__ void __launch_bounds__(256) maxpool_kernel(const __half* x, __half* y, int N, int H, int W, int C, int k,
                                                       int stride, int pad, int Ho, int Wo, long long total) {
     const int c8n = C / 8;
+    pdl_launch_dependents();
+    pdl_wait();
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
         const int c8 = static_cast<int>(i % c8n);
@@ -257,6 +264,8 @@ __global__ void __launch_bounds__(256) maxpool_kernel(const __half* x, __half* y
 __global__ void __launch_bounds__(128) gavgpool_kernel(const __half* x, __half* y, int N, int HW, int C, long long total) {
     const int c8n = C / 8;
     const float inv = 1.0f / static_cast<float>(HW);
+    pdl_launch_dependents();
+    pdl_wait();
     for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
          i += static_cast<long long>(gridDim.x) * blockDim.x) {
         const int c8 = static_cast<int>(i % c8n);
@@ -290,6 +299,8 @@ __global__ void __launch_bounds__(256) fc_kernel(const __half* x, const __half* 
     __shared__ float red[8][kFcFo * kFcNb];
     const int k8n = K / 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_launch_dependents();
+    pdl_wait();
     for (int blk = blockIdx.x; blk < o_blocks * n_blocks; blk += gridDim.x) {
         const int o0 = (blk % o_blocks) * kFcFo, n0 = (blk / o_blocks) * kFcNb;
         float acc[kFcFo][kFcNb];
@@ -355,8 +366,7 @@ int launch_conv_direct(const ConvArgs& a, int sm_count, cudaStream_t s) {
     const int co_blocks = (a.Cout + kDirCo - 1) / kDirCo;
     const long long blocks = (n_pix + 127) / 128 * co_blocks;
     if (blocks == 0) return DLF_OK;
-    conv_direct_kernel<<<grid_for(blocks, sm_count), 128, 0, s>>>(a, n_pix, co_blocks);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(conv_direct_kernel, grid_for(blocks, sm_count), 128, 0, s, a, n_pix, co_blocks);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
@@ -383,9 +393,7 @@ int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
     }
     long long blocks = std::min<long long>((total + 127) / 128, static_cast<long long>(sm_count) * occ[v]);
     blocks = std::max<long long>(step, blocks / step * step);
-    if (a.stride == 1) dw3x3_kernel<1><<<static_cast<int>(blocks), 128, 0, s>>>(a, total, strips);
-    else dw3x3_kernel<2><<<static_cast<int>(blocks), 128, 0, s>>>(a, total, strips);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(a.stride == 1 ? dw3x3_kernel<1> : dw3x3_kernel<2>, static_cast<int>(blocks), 128, 0, s, a, total, strips);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
@@ -394,9 +402,8 @@ int launch_maxpool(const void* x, void* y, int N, int H, int W, int C, int k, in
     if (C % 8) return DLF_E_UNSUPPORTED;
     const long long total = static_cast<long long>(N) * Ho * Wo * (C / 8);
     if (total == 0) return DLF_OK;
-    maxpool_kernel<<<grid_for((total + 255) / 256, sm_count), 256, 0, s>>>(
-        static_cast<const __half*>(x), static_cast<__half*>(y), N, H, W, C, k, stride, pad, Ho, Wo, total);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(maxpool_kernel, grid_for((total + 255) / 256, sm_count), 256, 0, s, static_cast<const __half*>(x),
+                                  static_cast<__half*>(y), N, H, W, C, k, stride, pad, Ho, Wo, total);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
@@ -404,9 +411,8 @@ int launch_gavgpool(const void* x, void* y, int N, int H, int W, int C, int sm_c
     if (C % 8) return DLF_E_UNSUPPORTED;
     const long long total = static_cast<long long>(N) * (C / 8);
     if (total == 0) return DLF_OK;
-    gavgpool_kernel<<<grid_for((total + 127) / 128, sm_count), 128, 0, s>>>(
-        static_cast<const __half*>(x), static_cast<__half*>(y), N, H * W, C, total);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(gavgpool_kernel, grid_for((total + 127) / 128, sm_count), 128, 0, s, static_cast<const __half*>(x),
+                                  static_cast<__half*>(y), N, H * W, C, total);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
@@ -416,9 +422,8 @@ int launch_fc(const void* x, const void* w, const float* bias, void* y, int N, i
     if (N == 0) return DLF_OK;
     const int o_blocks = (M + kFcFo - 1) / kFcFo, n_blocks = (N + kFcNb - 1) / kFcNb;
     const int grid = grid_for(static_cast<long long>(o_blocks) * n_blocks, sm_count);
-    fc_kernel<<<grid, 256, 0, s>>>(static_cast<const __half*>(x), static_cast<const __half*>(w), bias,
-                                   static_cast<__half*>(y), N, K, M, act, o_blocks, n_blocks);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(fc_kernel, grid, 256, 0, s, static_cast<const __half*>(x), static_cast<const __half*>(w), bias,
+                                  static_cast<__half*>(y), N, K, M, act, o_blocks, n_blocks);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
