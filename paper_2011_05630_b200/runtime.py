@@ -6,6 +6,8 @@ inside libdlfusion.so.
 """
 from __future__ import annotations
 
+import threading
+
 import numpy as np
 import torch
 
@@ -40,6 +42,7 @@ class Session:
         self.out_shape = B.net_layer_info(self.net, len(layers) - 1)[2]
         self.out = torch.empty(self.out_shape, dtype=torch.float16, device=self.device)
         self.n_groups = 0
+        self._staging, self._staging_lock = None, threading.Lock()
 
     def close(self):
         if self.net is not None:
@@ -63,7 +66,17 @@ class Session:
 
     def upload(self, x: np.ndarray) -> torch.Tensor:
         assert x.dtype == np.float16 and tuple(x.shape) == self.shape
-        return _to_dev(np.ascontiguousarray(x), self.device)
+        # through a page-locked buffer of the session: the host copy into it runs on all cores and the transfer at the
+        # link's rate (2.4 MB: 157 us as a pageable copy); the caller's array is free and the tensor filled on return
+        src = torch.from_numpy(np.ascontiguousarray(x).view(np.int16)).view(torch.float16)
+        dst = torch.empty(self.shape, dtype=torch.float16, device=self.device)
+        with self._staging_lock:
+            if self._staging is None:
+                self._staging = torch.empty(self.shape, dtype=torch.float16, pin_memory=True)
+            self._staging.copy_(src)
+            dst.copy_(self._staging, non_blocking=True)
+            torch.cuda.current_stream(self.device).synchronize()
+        return dst
 
     def run(self, x_dev: torch.Tensor) -> torch.Tensor:
         stream = torch.cuda.current_stream().cuda_stream
