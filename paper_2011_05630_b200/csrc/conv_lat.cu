@@ -1,0 +1,498 @@
+// Implicit-GEMM convolution on tcgen05 for layers too small to fill the chip twice: one output tile per CTA, nothing
+// persistent.  What bounds these layers is not a rate but the chain set-up -> first copy -> UMMAs -> drain -> store of one
+// tile, so this kernel keeps that chain short: every warp has one job, the weights are on their way before the previous
+// kernel has finished, the tile leaves by plain 16-byte stores straight from the warps that finish it, and the CTA is small
+// enough (384 threads, at most 110 KB of shared memory, 64 columns of tensor memory) to be set up beside its predecessor.
+//
+// A long K (a 3x3 layer on 512 channels has 72 chunks of 64) is shared out over a cluster of SPLIT CTAs that work on the same
+// tile.  Their fp32 partial tiles meet in distributed shared memory: CTA d of the cluster adds up, in the order of the ranks,
+// and finishes every SPLIT-th run of rows; each warp writes the rows it drained straight into the shared memory of the CTA
+// they belong to, and the cluster's barrier says when all have.  No global scratch, no atomics, the same sum whatever the timing.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace dlf {
+
+namespace {
+
+constexpr int kEpiWarps = 8;                // warps 0..7: warp & 3 = TMEM lane quarter, warp >> 2 = even or odd 16-column groups
+constexpr int kProdWarp0 = kEpiWarps;       // warps 8..10 load: warp w takes ring stages w, w + 3, ...
+constexpr int kProdWarps = 3;
+constexpr int kMmaWarp0 = kProdWarp0 + kProdWarps;
+constexpr int kMmaWarps = 2;                // issuers: warp w takes chunks w, w + 2, ... into an accumulator of its own
+constexpr int kThreads = 32 * (kMmaWarp0 + kMmaWarps);
+constexpr int kMaxBN = 128;
+constexpr int kMaxStages = 12;
+constexpr int kItems = 4;                   // finished 8-channel vectors per epilogue thread
+constexpr int kMaxOut = kItems * 32 * kEpiWarps * 8;   // so that a CTA finishes at most 8192 values
+constexpr int kMaxDynSmem = 226 * 1024;     // 227 KB per CTA less the static part
+constexpr int kPairSmem = 110 * 1024;       // two CTAs fit an SM: this one is set up while its predecessor's still runs
+
+struct LatParams {
+    int N, Ho, Wo, Cout;
+    int kw, stride, pad;
+    int TW, TH, rows, tiles_w, tiles_h, n_tiles_n, BN;
+    int TN;
+    int kchunks, kchunks1, ksteps_last;     // 64-channel chunks per tap (both sources), of the first source; UMMAs of the last one
+    int total, share;                       // (tap, chunk) pairs of K, and how many a CTA of the cluster takes
+    int stride2, grouped;
+    int stages, a_bytes, stage_bytes, red_off;
+    int rows_per, act;
+    const float* bias;
+    const float* bias2;
+    const __half* res;
+    __half* out;
+    int* status;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// The address of the same shared-memory location in another CTA of the cluster.
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float a, float b, float c, float d) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+// Hardware barrier of the cluster: every thread arrives and waits once per phase.  (Bounded: what comes before a thread's
+// arrival is made of bounded waits.)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <int SPLIT>
+__global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kThreads, 2)
+conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx2,
+                const __grid_constant__ CUtensorMap tmw2, const __grid_constant__ LatParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tfull_bar;
+    __shared__ uint32_t tmem_base_s;
+    __shared__ int abort_s;
+    __shared__ __align__(16) float bias_s[kMaxBN];
+
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    uint8_t* sbase = smem_raw + (base - smem_u32(smem_raw));
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    volatile int* abort_flag = &abort_s;
+    const int rank = SPLIT > 1 ? static_cast<int>(cluster_rank()) : 0;
+    const int tile = SPLIT > 1 ? static_cast<int>(blockIdx.x) / SPLIT : static_cast<int>(blockIdx.x);
+    const int co0 = (tile % p.n_tiles_n) * p.BN;
+    int mt = tile / p.n_tiles_n;
+    const int wo0 = (mt % p.tiles_w) * p.TW;
+    mt /= p.tiles_w;
+    const int ho0 = (mt % p.tiles_h) * p.TH, n0 = (mt / p.tiles_h) * p.TN;
+    const int k_first = rank * p.share, k_count = min(p.share, p.total - k_first);
+
+    if (warp == kProdWarp0 && lane == 0) {
+        abort_s = 0;
+        for (int i = 0; i < p.stages; i++) {
+            mbar_init(&full_bar[i], 1);
+            mbar_init(&empty_bar[i], 1);
+        }
+        mbar_init(&tfull_bar, kMmaWarps);
+        fence_barrier_init();
+        tma_prefetch_desc(&tmw);
+        tma_prefetch_desc(&tmx);
+        if (p.kchunks1 < p.kchunks) { tma_prefetch_desc(&tmx2); tma_prefetch_desc(&tmw2); }
+    }
+    if (warp == kMmaWarp0) {
+        tmem_alloc(&tmem_base_s, kMaxBN * kMmaWarps);
+        tmem_relinquish();
+    }
+    if (threadIdx.x < kMaxBN) {
+        const int co = co0 + threadIdx.x;
+        bias_s[threadIdx.x] = co < p.Cout ? __ldg(p.bias + co) + (p.bias2 ? __ldg(p.bias2 + co) : 0.0f) : 0.0f;
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (SPLIT > 1) cluster_arrive();   // first phase: all CTAs of the cluster run (waited for before rows go to the others)
+    tc_fence_after_sync();
+    pdl_launch_dependents();
+    const uint32_t tmem_base = tmem_base_s;
+
+    if (warp >= kProdWarp0 && warp < kMmaWarp0) {
+        // ---- producers: warp w owns ring stages w, w + 3, ...; one elected lane issues; the weights of the first ring pass are
+        // on their way before the wait for the previous kernel ----
+        const int w = warp - kProdWarp0;
+        const uint32_t stage_tx = static_cast<uint32_t>(p.rows + p.BN) * 128u;
+        const int hi0 = ho0 * p.stride - p.pad, wi0 = wo0 * p.stride - p.pad;
+        const int tap0 = k_first / p.kchunks, r0 = tap0 / p.kw;
+        // position of a chunk in K, advanced one chunk at a time (a division costs a lone warp about a hundred cycles)
+        struct Pos { int tap, r, s, kc; };
+        const Pos start{tap0, r0, tap0 - r0 * p.kw, k_first - tap0 * p.kchunks};
+        auto advance = [&](Pos& c) {
+            if (++c.kc == p.kchunks) {
+                c.kc = 0;
+                c.tap++;
+                if (++c.s == p.kw) { c.s = 0; c.r++; }
+            }
+        };
+        auto load_b = [&](const Pos& c, int st) {
+            uint8_t* dst = sbase + st * p.stage_bytes + p.a_bytes;
+            if (c.kc >= p.kchunks1) tma_load_3d(dst, &tmw2, &full_bar[st], (c.kc - p.kchunks1) * 64, 0, co0);
+            else tma_load_3d(dst, &tmw, &full_bar[st], c.kc * 64, c.tap, co0);
+        };
+        auto load_a = [&](const Pos& c, int st) {
+            uint8_t* dst = sbase + st * p.stage_bytes;
+            if (c.kc >= p.kchunks1) tma_load_4d(dst, &tmx2, &full_bar[st], (c.kc - p.kchunks1) * 64, wo0 * p.stride2, ho0 * p.stride2, n0);
+            else tma_load_4d(dst, &tmx, &full_bar[st], c.kc * 64, wi0 + c.s, hi0 + c.r, n0);
+        };
+        const int first_pass = min(p.stages, k_count);
+        if (elect_one()) {
+            Pos c = start;
+            int turn = 0;
+#pragma unroll 1
+            for (int i = 0; i < first_pass; i++, advance(c)) {
+                if (turn == w) {
+                    mbar_expect_tx(&full_bar[i], stage_tx);
+                    load_b(c, i);
+                }
+                if (++turn == kProdWarps) turn = 0;
+            }
+        }
+        __syncwarp();
+        pdl_wait();
+        Pos c = start;
+        int turn = 0, st = 0;
+        uint32_t ph = 1;
+#pragma unroll 1
+        for (int i = 0; i < k_count; i++, advance(c)) {
+            if (turn == w) {
+                if (i >= first_pass && !mbar_wait_warp<true>(&empty_bar[st], ph, abort_flag, p.status, 0xE00 | (blockIdx.x << 12))) break;
+                if (elect_one()) {
+                    if (i >= first_pass) {
+                        mbar_expect_tx(&full_bar[st], stage_tx);
+                        load_b(c, st);
+                    }
+                    load_a(c, st);
+                }
+                __syncwarp();
+            }
+            if (++turn == kProdWarps) turn = 0;
+            if (++st == p.stages) { st = 0; turn = 0; ph ^= 1u; }
+        }
+    } else if (warp >= kMmaWarp0) {
+        // ---- issuers.  A run of UMMAs holds its warp until it has almost executed, and what the warp does between two runs
+        // (the wait, descriptors, the commit) takes as long again: two warps with an accumulator each hide one behind the other
+        // (540 -> 290 clocks per chunk of 64 channels); the epilogue adds the two sums ----
+        const int w = warp - kMmaWarp0;
+        const uint32_t idesc = umma_idesc_f16(p.BN), d_tmem = tmem_base + w * kMaxBN;
+        const uint64_t desc0 = umma_desc_sw128(0) + (base >> 4);
+        const uint32_t stage16 = static_cast<uint32_t>(p.stage_bytes) >> 4, b16 = static_cast<uint32_t>(p.a_bytes) >> 4;
+        const int last = k_count - 1 - ((k_count - 1 - w) & 1);   // this issuer's last chunk (negative: it has none)
+        int st = w % p.stages, kc = (k_first + w) % p.kchunks;
+        uint32_t ph = static_cast<uint32_t>(w / p.stages) & 1u;
+        uint64_t ad = desc0 + static_cast<uint32_t>(st) * stage16;
+#pragma unroll 1
+        for (int i = w; i < k_count; i += 2) {
+            if (!mbar_wait_warp<true>(&full_bar[st], ph, abort_flag, p.status, 0xE10 | (blockIdx.x << 12))) break;
+            tc_fence_after_sync();
+            const int ksteps = kc == p.kchunks - 1 ? p.ksteps_last : 4;
+            const uint64_t bd = ad + b16;
+            if (elect_one()) {
+                umma_f16(d_tmem, ad, bd, idesc, i != w);
+                if (ksteps > 1) umma_f16(d_tmem, ad + 2, bd + 2, idesc, 1);
+                if (ksteps > 2) umma_f16(d_tmem, ad + 4, bd + 4, idesc, 1);
+                if (ksteps > 3) umma_f16(d_tmem, ad + 6, bd + 6, idesc, 1);
+                if (i + p.stages < k_count) umma_commit(&empty_bar[st]);
+                if (i == last) umma_commit(&tfull_bar);
+            }
+            __syncwarp();
+            kc += 2;
+            if (kc >= p.kchunks) kc -= p.kchunks;
+            if (kc >= p.kchunks) kc -= p.kchunks;   // (one chunk per tap)
+            st += 2;
+            ad += 2 * stage16;
+            if (st >= p.stages) { st -= p.stages; ph ^= 1u; ad -= static_cast<uint32_t>(p.stages) * stage16; }
+        }
+        if (last < 0 && lane == 0) mbar_arrive(&tfull_bar);
+    } else {
+        // ---- epilogue ----
+        const int q = warp & 3, half = warp >> 2;
+        const int bn8 = p.BN >> 3;
+        const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
+        // the vectors this thread will finish: where they go, and their residual (its latency hides behind the UMMAs)
+        long long off[kItems];
+        uint32_t src[kItems];   // byte offset of the vector's first half in a rank's rows; its second half is 16 bytes beside it
+        int bias_at[kItems];
+        uint4 rv[kItems];
+        const int n_items = p.rows_per * bn8;
+        // a row's 16-byte vectors are stored in an order that depends on the row, so that the lanes of a warp (one row each)
+        // fall into different banks
+        const uint32_t swz = p.BN % 32 == 0 ? 7u : 3u;
+#pragma unroll
+        for (int it = 0; it < kItems; it++) {
+            const int i = static_cast<int>(threadIdx.x) + it * 32 * kEpiWarps;
+            off[it] = -1;
+            src[it] = 0u;
+            bias_at[it] = 0;
+            if (i >= n_items) continue;
+            const int r = i / bn8, g = i - r * bn8, m = rank * p.rows_per + r;
+            const int tw = m % p.TW, t2 = m / p.TW, th = t2 % p.TH, tn = t2 / p.TH;
+            const int n = n0 + tn, ho = ho0 + th, wo = wo0 + tw, co = co0 + g * 8;
+            src[it] = static_cast<uint32_t>(r * p.BN * 4) + ((static_cast<uint32_t>(2 * g) ^ (static_cast<uint32_t>(r) & swz)) << 4);
+            bias_at[it] = g * 8;
+            if (m < p.rows && n < p.N && ho < p.Ho && wo < p.Wo && co < p.Cout)
+                off[it] = ((static_cast<long long>(n) * p.Ho + ho) * p.Wo + wo) * p.Cout + co;
+        }
+        pdl_wait();
+        if (p.res) {
+#pragma unroll
+            for (int it = 0; it < kItems; it++) rv[it] = off[it] >= 0 ? __ldg(reinterpret_cast<const uint4*>(p.res + off[it])) : make_uint4(0u, 0u, 0u, 0u);
+        } else {
+#pragma unroll
+            for (int it = 0; it < kItems; it++) rv[it] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        const int m = q * 32 + lane, dest = m / p.rows_per, row = m - dest * p.rows_per;
+        const uint32_t slab = static_cast<uint32_t>(p.rows_per * p.BN * 4);   // one rank's partial rows
+        const uint32_t my = base + p.red_off + rank * slab + row * p.BN * 4;
+        const uint32_t dst = SPLIT > 1 ? mapa(my, min(dest, SPLIT - 1)) : my;
+        bool ok = mbar_wait<true>(&tfull_bar, 0u, abort_flag, p.status, 0xE20 | (blockIdx.x << 12));
+        __syncwarp();
+        tc_fence_after_sync();
+        if (SPLIT > 1) cluster_wait();
+#pragma unroll 1
+        for (int c0 = half * 16; c0 < p.BN; c0 += 32) {
+            float v[16];
+            const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + c0;
+            tmem_ld16(taddr, v);
+            if (k_count > 1) {
+                float v2[16];
+                tmem_ld16(taddr + kMaxBN, v2);
+#pragma unroll
+                for (int e = 0; e < 16; e++) v[e] += v2[e];
+            }
+            if (ok && m < p.rows) {
+#pragma unroll
+                for (int e = 0; e < 4; e++) {
+                    const uint32_t a = dst + ((static_cast<uint32_t>((c0 >> 2) + e) ^ (static_cast<uint32_t>(row) & swz)) << 4);
+                    if (SPLIT > 1) st_cluster_v4(a, v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                    else asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[4 * e]), "f"(v[4 * e + 1]), "f"(v[4 * e + 2]), "f"(v[4 * e + 3]) : "memory");
+                }
+            }
+            __syncwarp();
+        }
+        tc_fence_before_sync();
+        if (SPLIT > 1) {
+            __syncwarp();
+            cluster_arrive();   // second phase: every CTA's rows have arrived
+            cluster_wait();
+        } else {
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+        }
+        const uint8_t* red = sbase + p.red_off;
+#pragma unroll
+        for (int it = 0; it < kItems; it++) {
+            if (off[it] < 0 || !ok) continue;
+            float4 a = *reinterpret_cast<const float4*>(red + src[it]), b = *reinterpret_cast<const float4*>(red + (src[it] ^ 16u));
+#pragma unroll
+            for (int sp = 1; sp < SPLIT; sp++) {
+                const float4 a2 = *reinterpret_cast<const float4*>(red + sp * slab + src[it]), b2 = *reinterpret_cast<const float4*>(red + sp * slab + (src[it] ^ 16u));
+                a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w;
+                b.x += b2.x; b.y += b2.y; b.z += b2.z; b.w += b2.w;
+            }
+            const float4 c0 = *reinterpret_cast<const float4*>(bias_s + bias_at[it]), c1 = *reinterpret_cast<const float4*>(bias_s + bias_at[it] + 4);
+            a.x += c0.x; a.y += c0.y; a.z += c0.z; a.w += c0.w;
+            b.x += c1.x; b.y += c1.y; b.z += c1.z; b.w += c1.w;
+            const __half2* rh = reinterpret_cast<const __half2*>(&rv[it]);
+            const float2 f0 = __half22float2(rh[0]), f1 = __half22float2(rh[1]), f2 = __half22float2(rh[2]), f3 = __half22float2(rh[3]);
+            uint4 o;
+            o.x = pack_half2_clamp(a.x + f0.x, a.y + f0.y, act_lo, act_hi);
+            o.y = pack_half2_clamp(a.z + f1.x, a.w + f1.y, act_lo, act_hi);
+            o.z = pack_half2_clamp(b.x + f2.x, b.y + f2.y, act_lo, act_hi);
+            o.w = pack_half2_clamp(b.z + f3.x, b.w + f3.y, act_lo, act_hi);
+            *reinterpret_cast<uint4*>(p.out + off[it]) = o;
+        }
+    }
+    __syncwarp();
+    if (SPLIT > 1 && warp >= kEpiWarps) {
+        cluster_wait();
+        cluster_arrive();
+        cluster_wait();
+    }
+    __syncthreads();
+    if (warp == kMmaWarp0) {
+        if (abort_s) __nanosleep(20000);   // let copies in flight land before the CTA retires
+        tc_fence_after_sync();
+        tmem_dealloc(tmem_base, kMaxBN * kMmaWarps);
+    }
+}
+
+typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const LatParams);
+KernelFn pick_kernel(int split) {
+    switch (split) {
+        case 1: return conv_lat_kernel<1>;
+        case 2: return conv_lat_kernel<2>;
+        case 4: return conv_lat_kernel<4>;
+        default: return conv_lat_kernel<8>;
+    }
+}
+
+struct Tile { int tw, th, tn; };
+
+// Output tile of at most `cap` pixels: the fewest tiles, then the fewest rows.
+Tile pick_tile(int N, int Ho, int Wo, int cap) {
+    Tile best{1, 1, 1};
+    long long best_tiles = -1;
+    int best_rows = 0;
+    for (int tn = 1; tn <= std::min(N, cap); tn++)
+        for (int th = 1; th <= std::min(Ho, cap / tn); th++) {
+            const int tw_max = std::min(Wo, cap / (tn * th)), cols = (Wo + tw_max - 1) / tw_max, tw = (Wo + cols - 1) / cols;
+            const int rows = tn * th * tw;
+            const long long tiles = static_cast<long long>(cols) * ((Ho + th - 1) / th) * ((N + tn - 1) / tn);
+            if (best_tiles < 0 || tiles < best_tiles || (tiles == best_tiles && rows < best_rows)) {
+                best_tiles = tiles;
+                best_rows = rows;
+                best = Tile{tw, th, tn};
+            }
+        }
+    return best;
+}
+
+struct Choice {
+    Tile tile;
+    int BN, split, share, stages, rows_per;
+    double cost;   // SM clocks between set-up and the last store; negative: none
+};
+
+Choice choose(const ConvArgs& a, int total, int sm_count, const int (&max_clusters)[4]) {
+    Choice best{};
+    best.cost = -1.0;
+    const int cout16 = (a.Cout + 15) / 16 * 16;
+    for (int cap : {128, 96, 64, 32}) {
+        const Tile t = pick_tile(a.N, a.Ho, a.Wo, cap);
+        const int rows = t.tw * t.th * t.tn, a_bytes = (rows + 7) / 8 * 1024;
+        const long long m_tiles = static_cast<long long>((a.Wo + t.tw - 1) / t.tw) * ((a.Ho + t.th - 1) / t.th) * ((a.N + t.tn - 1) / t.tn);
+        for (int bn : {64, 128}) {
+            if (bn == 128 && cout16 <= 64) continue;
+            const int BN = std::min(cout16, bn), stage = a_bytes + BN * 128;
+            const long long tiles = m_tiles * ((cout16 + BN - 1) / BN);
+            for (int lg = 0; lg <= 3; lg++) {
+                const int split = 1 << lg, share = (total + split - 1) / split, rows_per = (rows + split - 1) / split;
+                if (tiles * split > sm_count) break;
+                if ((split > 1 && (split - 1) * share >= total) || rows_per * BN > kMaxOut) continue;
+                for (int smem : {kPairSmem, kMaxDynSmem}) {
+                    const int budget = smem - 1024 - split * rows_per * BN * 4 - (128 * 128 - a_bytes);
+                    int stages = std::min({kMaxStages, budget / stage, share});
+                    if (stages < share) stages &= ~1;   // the ring goes round: a stage belongs to one issuer
+                    if (stages < std::min(share, 2)) continue;
+                    if (tiles > (smem > kPairSmem ? max_clusters[lg] : 2 * max_clusters[lg])) continue;   // (a second wave of clusters)
+                    // Fitted to about 600 measured (layer, tile, split) times: a chunk costs what its copy or its two issuers
+                    // take, and with a ring that goes round its part of a round trip; sharing a tile costs the exchange of its
+                    // sums, and more when the clusters have to be packed (eight CTAs, more than half of the SMs).
+                    double chunk = std::max(stage / 52.0, 320.0 + 0.4 * BN);
+                    if (stages < share) chunk = std::max(chunk, 1700.0 / stages);
+                    const double cost = 2000.0 + share * chunk + rows * BN * (lg > 0 ? 0.3 : 0.11) + (lg > 0 ? 500.0 : 0.0) + (lg == 3 ? 1000.0 : 0.0) +
+                                        (lg > 0 && tiles * split > sm_count / 2 ? 900.0 : 0.0) + (smem > kPairSmem ? 1000.0 : 0.0);
+                    if (best.cost < 0 || cost < best.cost) best = Choice{t, BN, split, share, stages, rows_per, cost};
+                }
+            }
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
+// Clusters of 1, 2, 4, 8 CTAs that run at the same time on an otherwise empty device, one CTA per SM (conv_lat_init).
+static int g_max_clusters[kMaxDevices][4];
+
+int launch_conv_lat(const ConvArgs& a_in, int sm_count, int* status_dev, cudaStream_t s) {
+    const bool dual = a_in.x2 != nullptr;
+    if (a_in.pool || !conv_tc_supported(a_in) || (dual && !conv_tc_dual_supported(a_in))) return DLF_E_UNSUPPORTED;
+    ConvArgs a = a_in;
+    const long long flat_pixels = static_cast<long long>(a.N) * a.H * a.W;
+    if (a.kh == 1 && a.kw == 1 && a.stride == 1 && a.pad == 0 && !dual && flat_pixels < (1ll << 31)) {   // no spatial structure: one list of pixels
+        a.N = 1; a.H = 1; a.Ho = 1;
+        a.W = a.Wo = static_cast<int>(flat_pixels);
+    }
+    if (static_cast<long long>(a.N) * a.Ho * a.Wo > 128ll * sm_count) return DLF_E_UNSUPPORTED;
+    LatParams p{};
+    p.kchunks1 = (a.Cin + 63) / 64;
+    p.ksteps_last = ((a.Cin - (p.kchunks1 - 1) * 64) + 15) / 16;
+    p.kchunks = p.kchunks1 + (dual ? a.Cin2 / 64 : 0);
+    p.total = a.kh * a.kw * p.kchunks;
+    const int dev = current_device_slot();
+    if (dev < 0) return DLF_E_UNSUPPORTED;
+    const Choice c = choose(a, p.total, sm_count, g_max_clusters[dev]);
+    // the persistent kernel: 2.5 us in a network for a tile with one chunk, 0.16 us for every further one (3.4 us for 64 -> 64
+    // at one 56x56 image against 2.6 us here; 6.3 us for 128 -> 128 3x3 at eight 28x28 images against 7.1 us)
+    if (c.cost < 0 || c.cost > 4100.0 + 310.0 * p.total) return DLF_E_UNSUPPORTED;
+    p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
+    p.kw = a.kw; p.stride = a.stride; p.pad = a.pad; p.stride2 = dual ? a.stride2 : 1;
+    p.TW = c.tile.tw; p.TH = c.tile.th; p.TN = c.tile.tn;
+    p.rows = p.TW * p.TH * p.TN;
+    p.tiles_w = (a.Wo + p.TW - 1) / p.TW; p.tiles_h = (a.Ho + p.TH - 1) / p.TH;
+    const int tiles_n = (a.N + p.TN - 1) / p.TN;
+    p.BN = c.BN;
+    p.n_tiles_n = ((a.Cout + 15) / 16 * 16 + c.BN - 1) / c.BN;
+    p.share = c.share; p.stages = c.stages; p.rows_per = c.rows_per;
+    p.a_bytes = (p.rows + 7) / 8 * 1024;
+    p.stage_bytes = p.a_bytes + p.BN * 128;
+    // (the UMMA always reads 128 rows: behind a shorter last slab it reads on into memory that must still be this CTA's)
+    p.red_off = p.stages * p.stage_bytes + (128 * 128 - p.a_bytes);
+    p.act = a.act;
+    p.bias = a.bias; p.bias2 = dual ? a.bias2 : nullptr;
+    p.res = static_cast<const __half*>(a.res); p.out = static_cast<__half*>(a.y);
+    p.status = status_dev;
+    CUtensorMap tmx, tmw, tmx2, tmw2;
+    auto input_map = [&](CUtensorMap* m, const void* x, int W, int H, int C, int stride) {
+        const uint64_t dims[4] = {static_cast<uint64_t>(C), static_cast<uint64_t>(W), static_cast<uint64_t>(H), static_cast<uint64_t>(a.N)};
+        const uint64_t strides[3] = {static_cast<uint64_t>(C) * 2, static_cast<uint64_t>(W) * C * 2, static_cast<uint64_t>(H) * W * C * 2};
+        const uint32_t box[4] = {64, static_cast<uint32_t>(p.TW * stride), static_cast<uint32_t>(p.TH * stride), static_cast<uint32_t>(p.TN)};
+        const uint32_t es[4] = {1, static_cast<uint32_t>(stride), static_cast<uint32_t>(stride), 1};
+        return encode_tmap(m, x, 4, dims, strides, box, es);
+    };
+    auto weight_map = [&](CUtensorMap* m, const void* w, int C, int taps) {
+        const uint64_t dims[3] = {static_cast<uint64_t>(C), static_cast<uint64_t>(taps), static_cast<uint64_t>(a.Cout)};
+        const uint64_t strides[2] = {static_cast<uint64_t>(C) * 2, static_cast<uint64_t>(taps) * C * 2};
+        const uint32_t box[3] = {64, 1, static_cast<uint32_t>(p.BN)};
+        const uint32_t es[3] = {1, 1, 1};
+        return encode_tmap(m, w, 3, dims, strides, box, es);
+    };
+    int rc = input_map(&tmx, a.x, a.W, a.H, a.Cin, a.stride);
+    if (rc == DLF_OK) rc = weight_map(&tmw, a.w, a.Cin, a.kh * a.kw);
+    tmx2 = tmx;
+    tmw2 = tmw;
+    if (rc == DLF_OK && dual) rc = input_map(&tmx2, a.x2, a.W2, a.H2, a.Cin2, a.stride2);
+    if (rc == DLF_OK && dual) rc = weight_map(&tmw2, a.w2, a.Cin2, 1);
+    if (rc) return rc;
+    const int grid = p.tiles_w * p.tiles_h * tiles_n * p.n_tiles_n * c.split;
+    const size_t smem = static_cast<size_t>(p.red_off) + static_cast<size_t>(c.split) * p.rows_per * p.BN * 4 + 1024;
+    cudaError_t e = launch_kernel(pick_kernel(c.split), grid, kThreads, smem, s, tmx, tmw, tmx2, tmw2, p);
+    return e == cudaSuccess ? DLF_OK : cuda_fail(e);
+}
+
+int conv_lat_init() {
+    static bool attr_set[kMaxDevices] = {};
+    const int dev = current_device_slot();
+    if (dev < 0) return DLF_E_UNSUPPORTED;
+    if (!attr_set[dev]) {
+        for (int lg = 0; lg <= 3; lg++) {
+            cudaError_t e = cudaFuncSetAttribute(pick_kernel(1 << lg), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+            if (e != cudaSuccess) return cuda_fail(e);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(1u << lg);
+            cfg.blockDim = dim3(kThreads);
+            cfg.dynamicSmemBytes = kMaxDynSmem;
+            int n = 0;
+            e = cudaOccupancyMaxActiveClusters(&n, pick_kernel(1 << lg), &cfg);
+            if (e != cudaSuccess) return cuda_fail(e);
+            g_max_clusters[dev][lg] = n;
+        }
+        attr_set[dev] = true;
+    }
+    return DLF_OK;
+}
+
+}  // namespace dlf

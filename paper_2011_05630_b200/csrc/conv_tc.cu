@@ -1196,6 +1196,8 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
 int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s) {
     int rc = conv_tc_init();
     if (rc) return rc;
+    rc = launch_conv_lat(a, sm_count, status_dev, s);
+    if (rc != DLF_E_UNSUPPORTED) return rc;
     ConvTcLaunch L;
     rc = conv_tc_prepare(a, sm_count, status_dev, &L);
     if (rc) return rc;
@@ -1262,7 +1264,7 @@ int conv_tc_init() {
         }
         attr_set[dev] = true;
     }
-    return DLF_OK;
+    return conv_lat_init();
 }
 
 }  // namespace dlf
