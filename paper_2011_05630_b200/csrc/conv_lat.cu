@@ -389,11 +389,11 @@ Choice choose(const ConvArgs& a, int total, int sm_count, const int (&max_cluste
                     if (tiles > (smem > kPairSmem ? max_clusters[lg] : 2 * max_clusters[lg])) continue;   // (a second wave of clusters)
                     // Fitted to about 600 measured (layer, tile, split) times: a chunk costs what its copy or its two issuers
                     // take, and with a ring that goes round its part of a round trip; sharing a tile costs the exchange of its
-                    // sums, and more when the clusters have to be packed (eight CTAs, more than half of the SMs).
+                    // sums, and more when the clusters have to be packed (eight CTAs, more than half of the SMs); so do CTAs on nearly all SMs.
                     double chunk = std::max(stage / 52.0, 320.0 + 0.4 * BN);
                     if (stages < share) chunk = std::max(chunk, 1700.0 / stages);
                     const double cost = 2000.0 + share * chunk + rows * BN * (lg > 0 ? 0.3 : 0.11) + (lg > 0 ? 500.0 : 0.0) + (lg == 3 ? 1000.0 : 0.0) +
-                                        (lg > 0 && tiles * split > sm_count / 2 ? 900.0 : 0.0) + (smem > kPairSmem ? 1000.0 : 0.0);
+                                        (tiles * split > (lg > 0 ? sm_count / 2 : sm_count * 3 / 4) ? 1000.0 : 0.0) + (smem > kPairSmem ? 1000.0 : 0.0);
                     if (best.cost < 0 || cost < best.cost) best = Choice{t, BN, split, share, stages, rows_per, cost};
                 }
             }
@@ -426,8 +426,10 @@ int launch_conv_lat(const ConvArgs& a_in, int sm_count, int* status_dev, cudaStr
     if (dev < 0) return DLF_E_UNSUPPORTED;
     const Choice c = choose(a, p.total, sm_count, g_max_clusters[dev]);
     // the persistent kernel: 2.5 us in a network for a tile with one chunk, 0.16 us for every further one (3.4 us for 64 -> 64
-    // at one 56x56 image against 2.6 us here; 6.3 us for 128 -> 128 3x3 at eight 28x28 images against 7.1 us)
-    if (c.cost < 0 || c.cost > 4100.0 + 310.0 * p.total) return DLF_E_UNSUPPORTED;
+    // at one 56x56 image against 2.6 us here; 6.3 us for 128 -> 128 3x3 at eight 28x28 images against 7.1 us), 0.12 us where it
+    // loads a kernel row's window once (4.6 us for 64 -> 64 3x3 at five 27x29 images against 4.7 us)
+    const bool row = a.kh == 3 && a.kw == 3 && a.stride == 1 && a.Cin % 64 == 0 && g_conv_row_mode > 0;
+    if (c.cost < 0 || c.cost > 4100.0 + (row ? 240.0 : 310.0) * p.total) return DLF_E_UNSUPPORTED;
     p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
     p.kw = a.kw; p.stride = a.stride; p.pad = a.pad; p.stride2 = dual ? a.stride2 : 1;
     p.TW = c.tile.tw; p.TH = c.tile.th; p.TN = c.tile.tn;
