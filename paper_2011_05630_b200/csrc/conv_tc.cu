@@ -85,8 +85,10 @@ struct TileCoord {
     int tile, ks;  // split-K: the tile's number and which share of K this work item takes
 };
 
-template <bool SPLIT = false>
-__device__ __forceinline__ TileCoord decode_work(const ConvTcParams& p, int t) {
+// With PAIR, work item t is two neighbouring pixel tiles, one for either CTA of the pair (the last one may lie past the batch:
+// zeros are loaded for it and nothing is stored).
+template <bool SPLIT = false, bool PAIR = false>
+__device__ __forceinline__ TileCoord decode_work(const ConvTcParams& p, int t, int rank = 0) {
     TileCoord c;
     c.ks = 0;
     if (SPLIT) {   // the shares of one tile are neighbours in the work list: they run side by side
@@ -96,6 +98,7 @@ __device__ __forceinline__ TileCoord decode_work(const ConvTcParams& p, int t) {
     c.tile = t;
     const int nt = t % p.n_tiles_n;
     int mt = t / p.n_tiles_n;
+    if (PAIR) mt = 2 * mt + rank;
     c.co0 = nt * p.BN;
     c.wo0 = (mt % p.tiles_w) * p.TW;
     mt /= p.tiles_w;
@@ -151,14 +154,20 @@ struct ConvBars {
 
 // The warp roles of one layer: everything between the CTA's set-up (barriers initialised, tensor memory allocated) and
 // its wind-down.  Called once by the single-layer kernel and once per layer by the multi-layer kernel.
-template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT>
+template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT, bool PAIR>
 __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CUtensorMap* tmw_p, const CUtensorMap* tmy_p,
                                               const CUtensorMap* tmr_p, const CUtensorMap* tmx2_p, const CUtensorMap* tmw2_p,
                                               const ConvTcParams& p, const ConvBars& sm, uint32_t tmem_base,
                                               uint8_t* stage0, uint32_t base, const GridSync& gs) {
     float* bias_s = reinterpret_cast<float*>(stage0 + p.bias_off);
     constexpr int kTps = ROW ? 3 : 1;   // taps per ring stage: a whole kernel row in the row mode
-    const int stage_bytes = p.kg * (p.a_bytes + kTps * p.BN * 128);
+    // A CTA pair works on two pixel tiles and the same output channels: either CTA loads its own tile's pixels and half of the
+    // weight slab's rows, the UMMAs (M = 256) issued by the first one read both.
+    const int b_rows = PAIR ? p.BN >> 1 : p.BN;
+    const int stage_bytes = p.kg * (p.a_bytes + kTps * b_rows * 128);
+    const int rank = PAIR ? static_cast<int>(blockIdx.x) & 1 : 0;
+    const int w_first = PAIR ? static_cast<int>(blockIdx.x) >> 1 : static_cast<int>(blockIdx.x);
+    const int w_step = PAIR ? static_cast<int>(gridDim.x) >> 1 : static_cast<int>(gridDim.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort_flag = sm.abort_s;
     const int k_iters = p.tgroups * p.kgroups;
@@ -172,7 +181,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             uint8_t* stage_out = stage0 + p.stage_out_off;
             auto planes_of = [&](const TileCoord& c) { return (min(p.BN, ((p.Cout - c.co0) + 15) & ~15) + 63) >> 6; };
             auto fetch_residual = [&](int t, uint32_t b) {
-                const TileCoord c = decode_work(p, t);
+                const TileCoord c = decode_work<false, PAIR>(p, t, rank);
                 const int planes = planes_of(c);
                 if (lane == 0) mbar_expect_tx(&sm.sfree_bar[b], static_cast<uint32_t>(planes * p.rows) * 128u);
                 __syncwarp();
@@ -182,7 +191,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             if (RES)
 #pragma unroll 1
                 for (int jj = 0; jj < p.out_bufs; jj++)
-                    if (static_cast<int>(blockIdx.x) + jj * static_cast<int>(gridDim.x) < p.n_work) fetch_residual(blockIdx.x + jj * gridDim.x, jj);
+                    if (w_first + jj * w_step < p.n_work) fetch_residual(w_first + jj * w_step, jj);
             // Up to `store_depth` stores are in flight: a store takes about 1.5 us from its issue until it has read its
             // buffer whatever its size (measured), so a layer of short tiles (one or two loads each) that waited for
             // every store before the next was bound by that latency, not by any bandwidth.  Every lane commits a group
@@ -190,14 +199,14 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             const int depth = p.store_depth, bufs = p.out_bufs;
             int b = 0, fb = 0;                // staging buffer of tile j / of the oldest store in flight
             uint32_t ph = 0;                  // phase of sfull[b]
-            int t_free = blockIdx.x, j = 0;   // tile of the oldest store in flight
+            int t_free = w_first, j = 0;   // tile of the oldest store in flight
             DLF_TRACE_DECL(sacc, smark);  // cycles of CTA 0's store warp: 0 wait for a staged tile, 1 store and its read, 2 residual fetch
 #pragma unroll 1
-            for (int t = blockIdx.x; t < p.n_work; t += gridDim.x, j++) {
+            for (int t = w_first; t < p.n_work; t += w_step, j++) {
                 if (!mbar_wait_warp(&sm.sfull_bar[b], ph, abort_flag, p.status, 0x500 | (blockIdx.x << 12))) break;
                 DLF_TRACE_ACC(sacc, 0, smark);
-                const TileCoord c = decode_work(p, t);
-                if (lane < planes_of(c))
+                const TileCoord c = decode_work<false, PAIR>(p, t, rank);
+                if (lane < planes_of(c) && (!PAIR || c.n0 < p.N))
                     tma_store_4d(tmy_p, stage_out + b * p.out_buf_bytes + lane * kABytes, c.co0 + lane * 64, c.wo0, c.ho0, c.n0);
                 tma_store_commit();
                 if (++b == bufs) { b = 0; ph ^= 1u; }
@@ -205,14 +214,14 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                     tma_store_wait_read_n(depth - 1);  // the oldest store has read its buffer: it may take the next residual / tile
                     __syncwarp();
                     DLF_TRACE_ACC(sacc, 1, smark);
-                    const int t2 = t_free + bufs * static_cast<int>(gridDim.x);
+                    const int t2 = t_free + bufs * w_step;
                     if (RES) {
                         if (t2 < p.n_work) fetch_residual(t2, fb);
                     } else if (lane == 0) {
                         mbar_arrive(&sm.sfree_bar[fb]);
                     }
                     if (++fb == bufs) fb = 0;
-                    t_free += gridDim.x;
+                    t_free += w_step;
                     DLF_TRACE_ACC(sacc, 2, smark);
                 }
             }
@@ -231,14 +240,14 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             const bool is_b = role >= 2;
             // the first work item is decoded ahead of the wait for the previous kernel: the divisions (about a hundred
             // cycles each for a lone warp) then cost nothing on the path from that kernel's end to the first copy
-            const TileCoord c_first = decode_work<SPLIT>(p, blockIdx.x);
+            const TileCoord c_first = decode_work<SPLIT, PAIR>(p, w_first, rank);
             if (role == 0 && lane == 0 && gs.counter == nullptr) DLF_TRACE_POINT(p.status, 25);
             if (!is_b) {
                 pdl_wait();
                 if (!grid_wait(gs, lane, abort_flag, p.status)) return;   // the input may be a layer of this launch
             }
             const uint32_t parity = role & 1;
-            const uint32_t my_bytes = static_cast<uint32_t>(p.kg) * (is_b ? static_cast<uint32_t>(kTps * p.BN) : static_cast<uint32_t>(p.rows)) * 128u;
+            const uint32_t my_bytes = static_cast<uint32_t>(p.kg) * (is_b ? static_cast<uint32_t>(kTps * b_rows) : static_cast<uint32_t>(p.rows)) * 128u;
             uint32_t it = 0;
             bool ok = true;
             DLF_TRACE_DECL(pacc, pmark);  // cycles of CTA 0's producers: 0 wait for a free stage, 1 issue
@@ -258,12 +267,28 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 DLF_TRACE_ACC(pacc, 0, pmark);
                 if (it == 0 && role == 0 && lane == 0 && gs.counter == nullptr) DLF_TRACE_POINT(p.status, 26);
                 uint8_t* sa = stage0 + static_cast<size_t>(st) * stage_bytes;
-                if (lane == 0) mbar_expect_tx(&sm.full_bar[st], my_bytes);
+                // (a pair's loads all complete on the first CTA's barrier, which counts both CTAs' bytes)
+                if (lane == 0 && rank == 0) mbar_expect_tx(&sm.full_bar[st], PAIR ? 2 * my_bytes : my_bytes);
                 __syncwarp();
                 if (lane < p.kg) {   // a chunk past C_in / 64 lies outside the tensor map and arrives as zeros
                     const int kc = kq * p.kg + lane;
                     const bool second = kc >= p.kchunks1;   // (1x1 layers with whole 64-channel chunks only: see conv_tc_dual_supported)
-                    if (is_b) {
+                    if constexpr (PAIR) {
+                        const uint32_t bar = mapa(smem_u32(&sm.full_bar[st]), 0);
+                        if (is_b) {
+                            uint8_t* dst = sa + p.kg * p.a_bytes + lane * kTps * b_rows * 128;
+                            const int co = c.co0 + rank * b_rows;
+                            if (second) tma_load_4d_pair(dst, tmw2_p, bar, 0, co, 0, kc - p.kchunks1);
+                            else if (p.grouped) tma_load_4d_pair(dst, tmw_p, bar, 0, co, tap, kc);
+                            else tma_load_3d_pair(dst, tmw_p, bar, kc * 64, tap, co);
+                        } else {
+                            const int wi = c.wo0 * p.stride - p.pad + s, hi = c.ho0 * p.stride - p.pad + r;
+                            uint8_t* dst = sa + lane * p.a_bytes;
+                            if (second) tma_load_5d_pair(dst, tmx2_p, bar, 0, c.wo0 * p.stride2, c.ho0 * p.stride2, c.n0, kc - p.kchunks1);
+                            else if (p.grouped) tma_load_5d_pair(dst, tmx_p, bar, 0, wi, hi, c.n0, kc);
+                            else tma_load_4d_pair(dst, tmx_p, bar, kc * 64, wi, hi, c.n0);
+                        }
+                    } else if (is_b) {
                         uint8_t* dst = sa + p.kg * p.a_bytes + lane * kTps * p.BN * 128;
                         if (second) tma_load_4d(dst, tmw2_p, &sm.full_bar[st], 0, c.co0, 0, kc - p.kchunks1);
                         else if (p.grouped) tma_load_4d(dst, tmw_p, &sm.full_bar[st], 0, c.co0, tap, kc);
@@ -282,8 +307,8 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 return true;
             };
 #pragma unroll 1
-            for (int t = blockIdx.x; t < p.n_work && ok; t += gridDim.x) {
-                const TileCoord c = t == static_cast<int>(blockIdx.x) ? c_first : decode_work<SPLIT>(p, t);
+            for (int t = w_first; t < p.n_work && ok; t += w_step) {
+                const TileCoord c = t == w_first ? c_first : decode_work<SPLIT, PAIR>(p, t, rank);
                 if (SPLIT) {   // this item's share of the tile's (tap group, K-chunk group) list
                     const int l0 = c.ks * p.kgs, l1 = min(k_iters, l0 + p.kgs);
 #pragma unroll 1
@@ -306,16 +331,25 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
         }
     } else if (warp == kMmaWarp) {
         // ---- MMA issuer: the whole warp walks the loop (warp-uniform addresses), one elected lane issues ----
-        const uint32_t idesc = umma_idesc_f16(p.BN);
+        if (PAIR && rank != 0) return;   // the first CTA of the pair issues for both
+        const uint32_t idesc = PAIR ? umma_idesc_f16_pair(p.BN) : umma_idesc_f16(p.BN);
+        auto umma = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
+            if (PAIR) umma_f16_pair(d, a, b, idesc, accumulate);
+            else umma_f16(d, a, b, idesc, accumulate);
+        };
+        auto commit = [&](uint64_t* bar) {
+            if (PAIR) umma_commit_pair(bar);
+            else umma_commit(bar);
+        };
         const uint64_t desc0 = umma_desc_sw128(0);
-        const uint32_t b_chunk16 = static_cast<uint32_t>(p.BN) * 8u;  // one 64-channel weight slab, in 16-byte units
+        const uint32_t b_chunk16 = static_cast<uint32_t>(b_rows) * 8u;  // one 64-channel weight slab, in 16-byte units
         const uint32_t a_chunk16 = static_cast<uint32_t>(p.a_bytes) >> 4;  // one 64-channel slab of the tile's pixels (rows rounded up to 8)
         uint32_t it = 0, j = 0, ring_ph = 0;
         int ring_st = 0;   // ring position and phase as counters: no division in the issue loop
         bool ok = true;
         DLF_TRACE_DECL(macc, mmark);  // cycles of CTA 0's issuer: 0 accumulator wait, 1 stage wait, 2 issue
 #pragma unroll 1
-        for (int t = blockIdx.x; t < p.n_work && ok; t += gridDim.x, j++) {
+        for (int t = w_first; t < p.n_work && ok; t += w_step, j++) {
             const uint32_t acc = j & 1u;
             ok = mbar_wait_warp(&sm.tempty_bar[acc], ((j >> 1) & 1u) ^ 1u, abort_flag, p.status, 0x200 | (blockIdx.x << 12));
             if (!ok) break;
@@ -324,7 +358,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             const uint32_t d_tmem = tmem_base + acc * p.acc_stride;
             int kq = 0, k_end = k_iters;
             if (SPLIT) {   // this item's share of the (tap group, K-chunk group) list
-                const int l0 = decode_work<SPLIT>(p, t).ks * p.kgs;
+                const int l0 = decode_work<SPLIT, PAIR>(p, t, rank).ks * p.kgs;
                 k_end = min(k_iters - l0, p.kgs);
                 kq = l0 % p.kgroups;
             }
@@ -346,10 +380,10 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                         for (int g = 0; g < g_end; g++) {
                             const uint64_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g) * b_chunk16;
                             const int ksteps = (kq * p.kg + g == p.kchunks - 1) ? p.ksteps_last : 4;
-                            umma_f16(d_tmem, ad, bd, idesc, (ki | g) != 0);
-                            if (ksteps > 1) umma_f16(d_tmem, ad + 2, bd + 2, idesc, 1);
-                            if (ksteps > 2) umma_f16(d_tmem, ad + 4, bd + 4, idesc, 1);
-                            if (ksteps > 3) umma_f16(d_tmem, ad + 6, bd + 6, idesc, 1);
+                            umma(d_tmem, ad, bd, (ki | g) != 0);
+                            if (ksteps > 1) umma(d_tmem, ad + 2, bd + 2, 1);
+                            if (ksteps > 2) umma(d_tmem, ad + 4, bd + 4, 1);
+                            if (ksteps > 3) umma(d_tmem, ad + 6, bd + 6, 1);
                         }
                     } else {
                         // row mode (whole 64-channel chunks): the three taps of a kernel row read the same window, one
@@ -359,20 +393,20 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                             uint64_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g * 3) * b_chunk16;
 #pragma unroll
                             for (int sx = 0; sx < 3; sx++, ad += 8, bd += b_chunk16) {
-                                umma_f16(d_tmem, ad, bd, idesc, (ki | g | sx) != 0);
-                                umma_f16(d_tmem, ad + 2, bd + 2, idesc, 1);
-                                umma_f16(d_tmem, ad + 4, bd + 4, idesc, 1);
-                                umma_f16(d_tmem, ad + 6, bd + 6, idesc, 1);
+                                umma(d_tmem, ad, bd, (ki | g | sx) != 0);
+                                umma(d_tmem, ad + 2, bd + 2, 1);
+                                umma(d_tmem, ad + 4, bd + 4, 1);
+                                umma(d_tmem, ad + 6, bd + 6, 1);
                             }
                         }
                     }
-                    umma_commit(&sm.empty_bar[st]);  // frees the stage once these MMAs have read it
+                    commit(&sm.empty_bar[st]);  // frees the stage once these MMAs have read it
                 }
                 __syncwarp();
                 DLF_TRACE_ACC(macc, 2, mmark);
                 if (++kq == p.kgroups) kq = 0;
             }
-            if (ok && elect_one()) umma_commit(&sm.tfull_bar[acc]);
+            if (ok && elect_one()) commit(&sm.tfull_bar[acc]);
             __syncwarp();
             if (j == 0 && lane == 0) DLF_TRACE_POINT(p.status, 4);
         }
@@ -399,8 +433,8 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
         if (RES && POOL) ok = grid_wait(gs, lane, abort_flag, p.status);   // residual read with plain loads
         DLF_TRACE_DECL(eacc, emark);  // cycles of CTA 0's first epilogue thread: 0 staging-buffer wait, 1 accumulator wait, 2 drain
 #pragma unroll 1
-        for (int t = blockIdx.x; t < p.n_work && ok; t += gridDim.x, j++) {
-            const TileCoord c = decode_work<SPLIT>(p, t);
+        for (int t = w_first; t < p.n_work && ok; t += w_step, j++) {
+            const TileCoord c = decode_work<SPLIT, PAIR>(p, t, rank);
             const uint32_t acc = j & 1u;
             const int n = c.n0 + tn, ho = c.ho0 + th, wo = c.wo0 + tw;
             const bool valid = m < p.rows && n < p.N && ho < p.Ho && wo < p.Wo;
@@ -575,7 +609,10 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             }
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.tempty_bar[acc]);  // the accumulator is drained
+            if (lane == 0) {   // the accumulator is drained
+                if (PAIR) mbar_arrive_cluster(mapa(smem_u32(&sm.tempty_bar[acc]), 0));
+                else mbar_arrive(&sm.tempty_bar[acc]);
+            }
             if (!POOL) {
                 fence_proxy_async_smem();  // the staging tile is read by the TMA unit
                 __syncwarp();
@@ -590,7 +627,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
 }
 
 // Initialises the barriers for a ring of `stages` stages (thread 0; `again`: they hold valid objects already).
-__device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, int stages, bool again) {
+__device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, int stages, bool again, bool pair = false) {
     if (again) {
         for (int i = 0; i < 8; i++) { mbar_inval(&sm.full_bar[i]); mbar_inval(&sm.empty_bar[i]); }
         for (int i = 0; i < 2; i++) { mbar_inval(&sm.tfull_bar[i]); mbar_inval(&sm.tempty_bar[i]); }
@@ -602,7 +639,7 @@ __device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, int stages
     }
     for (int i = 0; i < 2; i++) {
         mbar_init(&sm.tfull_bar[i], 1);
-        mbar_init(&sm.tempty_bar[i], kEpiWarps);
+        mbar_init(&sm.tempty_bar[i], pair ? 2 * kEpiWarps : kEpiWarps);
     }
     for (int i = 0; i < kMaxOutBufs; i++) {
         mbar_init(&sm.sfull_bar[i], kEpiWarps);
@@ -611,11 +648,9 @@ __device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, int stages
     fence_barrier_init();
 }
 
-template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT>
-__global__ void __launch_bounds__(kThreads, 1)
-conv_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
-               const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmr,
-               const __grid_constant__ CUtensorMap tmx2, const __grid_constant__ CUtensorMap tmw2, const ConvTcParams p) {
+template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT, bool PAIR>
+__device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmx, const CUtensorMap& tmw, const CUtensorMap& tmy, const CUtensorMap& tmr,
+                                             const CUtensorMap& tmx2, const CUtensorMap& tmw2, const ConvTcParams& p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[8], empty_bar[8], tfull_bar[2], tempty_bar[2];
     __shared__ uint64_t sfull_bar[kMaxOutBufs], sfree_bar[kMaxOutBufs];  // staging buffer: filled by the epilogue / free again (residual landed)
@@ -630,7 +665,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
 
     if (threadIdx.x == 0) {
         abort_s = 0;
-        conv_tc_init_bars(sm, p.stages, false);
+        conv_tc_init_bars(sm, p.stages, false, PAIR);
         tma_prefetch_desc(&tmx);
         tma_prefetch_desc(&tmw);
         if (!POOL) tma_prefetch_desc(&tmy);
@@ -638,11 +673,20 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
         if (p.kchunks1 < p.kchunks) { tma_prefetch_desc(&tmx2); tma_prefetch_desc(&tmw2); }
     }
     if (warp == kMmaWarp) {
-        tmem_alloc(&tmem_base_s, p.tmem_cols);
-        tmem_relinquish();
+        if (PAIR) {
+            tmem_alloc_pair(&tmem_base_s, p.tmem_cols);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(&tmem_base_s, p.tmem_cols);
+            tmem_relinquish();
+        }
     }
     tc_fence_before_sync();
     __syncthreads();
+    if (PAIR) {   // both CTAs' barriers are initialised before either is signalled
+        cluster_arrive();
+        cluster_wait();
+    }
     tc_fence_after_sync();
     pdl_launch_dependents();
     // everything above overlapped the previous kernel; from here on its outputs are read - except by the
@@ -651,16 +695,36 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ 
     if (threadIdx.x == 0) DLF_TRACE_POINT(p.status, 1);
     const uint32_t tmem_base = tmem_base_s;
 
-    conv_tc_roles<ACT, POOL, RES, ROW, SPLIT>(&tmx, &tmw, &tmy, &tmr, &tmx2, &tmw2, p, sm, tmem_base, stage0, base, GridSync{nullptr, 0u});
+    conv_tc_roles<ACT, POOL, RES, ROW, SPLIT, PAIR>(&tmx, &tmw, &tmy, &tmr, &tmx2, &tmw2, p, sm, tmem_base, stage0, base, GridSync{nullptr, 0u});
 
     tc_fence_before_sync();
     __syncthreads();
+    if (PAIR) {   // neither CTA leaves while the other may still read its operands or signal its barriers
+        cluster_arrive();
+        cluster_wait();
+    }
     if (warp == kMmaWarp) {
         if (abort_s) __nanosleep(20000);  // let copies in flight land before the CTA retires
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, p.tmem_cols);
+        if (PAIR) tmem_dealloc_pair(tmem_base, p.tmem_cols);
+        else tmem_dealloc(tmem_base, p.tmem_cols);
         if (lane == 0) DLF_TRACE_POINT(p.status, 7);
     }
+}
+
+template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 1)
+conv_tc_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
+               const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmr,
+               const __grid_constant__ CUtensorMap tmx2, const __grid_constant__ CUtensorMap tmw2, const __grid_constant__ ConvTcParams p) {
+    conv_tc_body<ACT, POOL, RES, ROW, SPLIT, false>(tmx, tmw, tmy, tmr, tmx2, tmw2, p);
+}
+template <int ACT, bool POOL, bool RES, bool ROW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+conv_tc_pair_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
+                    const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmr,
+                    const __grid_constant__ CUtensorMap tmx2, const __grid_constant__ CUtensorMap tmw2, const __grid_constant__ ConvTcParams p) {
+    conv_tc_body<ACT, POOL, RES, ROW, false, true>(tmx, tmw, tmy, tmr, tmx2, tmw2, p);
 }
 
 // ---- several layers in one launch ------------------------------------------------------------------------------------------
@@ -690,7 +754,7 @@ struct SeqParams {
 template <int ACT, bool POOL, bool RES, bool ROW>
 __device__ __noinline__ void conv_seq_layer(const SeqLayer* Y, const ConvTcParams* p, const ConvBars* sm, uint32_t tmem_base, uint8_t* stage0,
                                             uint32_t base, unsigned* sync, unsigned target) {
-    conv_tc_roles<ACT, POOL, RES, ROW, false>(&Y->tmx, &Y->tmw, &Y->tmy, &Y->tmr, &Y->tmx, &Y->tmw, *p, *sm, tmem_base, stage0, base, GridSync{sync, target});
+    conv_tc_roles<ACT, POOL, RES, ROW, false, false>(&Y->tmx, &Y->tmw, &Y->tmy, &Y->tmr, &Y->tmx, &Y->tmw, *p, *sm, tmem_base, stage0, base, GridSync{sync, target});
 }
 
 __global__ void __launch_bounds__(kThreads, 1) conv_seq_kernel(const __grid_constant__ SeqParams sp) {
@@ -836,6 +900,18 @@ template <int ACT>
 KernelFn pick_pool(bool pool, bool res, bool row) {
     return pool ? pick_res<ACT, true>(res, row) : pick_res<ACT, false>(res, row);
 }
+// CTA-pair variants
+template <int ACT>
+KernelFn pick_pair_act(bool pool, bool res, bool row) {
+    if (pool) return res ? conv_tc_pair_kernel<ACT, true, true, false> : conv_tc_pair_kernel<ACT, true, false, false>;
+    if (row) return res ? conv_tc_pair_kernel<ACT, false, true, true> : conv_tc_pair_kernel<ACT, false, false, true>;
+    return res ? conv_tc_pair_kernel<ACT, false, true, false> : conv_tc_pair_kernel<ACT, false, false, false>;
+}
+KernelFn pick_pair(int act, bool pool, bool res, bool row) {
+    if (act == 0) return pick_pair_act<0>(pool, res, row);
+    if (act == 1) return pick_pair_act<1>(pool, res, row);
+    return pick_pair_act<2>(pool, res, row);
+}
 // split-K variants: layers without pooling or residual
 template <int ACT>
 KernelFn pick_split_row(bool row) {
@@ -878,12 +954,12 @@ namespace {
 struct ConvTcLaunch {
     CUtensorMap tmx, tmw, tmy, tmr, tmx2, tmw2;
     ConvTcParams p;
-    int act, pool, res, row, split;
+    int act, pool, res, row, split, pair;
     size_t smem;
     int grid;
 };
 
-int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcLaunch* out) {
+int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool allow_pair, ConvTcLaunch* out) {
     if (!conv_tc_supported(a_in)) return DLF_E_UNSUPPORTED;
     const bool dual = a_in.x2 != nullptr;
     if (dual && !conv_tc_dual_supported(a_in)) return DLF_E_UNSUPPORTED;
@@ -913,6 +989,10 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
     long long m_tiles = 0;
     int bias_bytes = 0;
     int splits = 1;   // split-K shares per tile that configure() lays the channel tiles out for
+    bool pair = false;   // CTA pairs: two pixel tiles per work item, each CTA holds half of the weight slab
+    int bn_force = 0;    // channel-tile width that configure() has to take (0: its choice)
+    auto work_items = [&]() { return (pair ? (m_tiles + 1) / 2 : m_tiles) * p.n_tiles_n; };
+    auto workers = [&]() { return pair ? sm_count / 2 : sm_count; };
     auto set_tile = [&](const Tile& t, int taps_per_stage) {
         tl = t;
         p.TW = tl.tw; p.TH = tl.th; p.TN = tl.tn;
@@ -934,11 +1014,12 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         // never reach into its neighbour's channels.
         long long best_cost = -1;
         for (int bn : {256, 192, 128, 64}) {
-            if (bn > bn_max) continue;
+            if (bn > bn_max || (bn_force && bn != bn_force)) continue;
             const int width = std::min(bn, cout16);
+            if (pair && width % 32) continue;
             const int nt = (cout16 + width - 1) / width;
             if (nt > 1 && width % 64) continue;
-            const long long waves = (m_tiles * nt * splits + sm_count - 1) / sm_count;
+            const long long waves = ((pair ? (m_tiles + 1) / 2 : m_tiles) * nt * splits + workers() - 1) / workers();
             const long long cost = waves * (width + 96);
             if (best_cost < 0 || cost < best_cost) {
                 best_cost = cost;
@@ -950,7 +1031,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         const int out_planes = (a.pool || splits > 1) ? 0 : (p.BN + 63) / 64;   // (split-K tiles are not staged)
         bias_bytes = (p.n_tiles_n * p.BN * 4 + 1023) / 1024 * 1024;
         p.out_buf_bytes = out_planes * kABytes;
-        const int b_bytes = p.tps * p.BN * 128;   // the weight slabs of one 64-channel chunk in a stage
+        const int b_bytes = p.tps * (pair ? p.BN / 2 : p.BN) * 128;   // the weight slabs of one 64-channel chunk in a stage
         const int loads_min = p.tgroups * p.kchunks;
         // Two staging buffers (the stores of one tile drain while the next is written) where the ring keeps
         // three stages, or as many as the tile has loads, beside them; else one.
@@ -1008,6 +1089,16 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         const long long item = std::max(fill, mma) + static_cast<long long>(p.rows) * p.BN * 2 * (a.res ? 2 : 1) * 27 / 10 +
                                (sp > 1 ? static_cast<long long>(p.rows) * p.BN * 8 * 27 / 10 + 600000 : 0) + 40960;
         return rounds * item;
+    };
+    // SM clocks of the current layout: rounds of the grid x cost of an item.  An item takes the slower of its copies (measured:
+    // 57 bytes per clock and SM, whatever the boxes) and its UMMAs (per M = 128, K = 16 instruction N / 2 clocks, at least 72),
+    // plus its output and residual at an SM's share of the HBM rate and a fixed hand-over.
+    auto clocks = [&]() {
+        const double rounds = static_cast<double>((work_items() + workers() - 1) / workers());
+        const double k = static_cast<double>(p.tgroups) * p.kchunks;
+        const double fill = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / 57.0;
+        const double mma = k * p.tps * 4 * std::max(p.BN / 2, 72);
+        return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + (pair ? 800.0 : 0.0);
     };
     // Row mode (3x3, stride 1, pad 1): a tile is TH whole output rows seen with a pitch of Wo + 2, pixel-linear like
     // its input window, so that the three taps of a kernel row read ONE loaded window through descriptors that
@@ -1090,6 +1181,46 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
             bias_bytes = keep_bias;
         }
     }
+    // CTA pairs: either CTA fills half of the weight slab, so an item streams fewer bytes per UMMA; taken where the estimate says
+    // that this outweighs the coarser work items.
+    if (allow_pair && splits == 1 && sm_count >= 2 && m_tiles >= 2) {
+        const ConvTcParams keep = p;
+        const Tile keep_tl = tl;
+        const int keep_bias = bias_bytes;
+        const long long keep_m = m_tiles;
+        double best = clocks();
+        ConvTcParams best_p{};
+        Tile best_tl{};
+        int best_bias = 0;
+        long long best_m = 0;
+        bool found = false;
+        pair = true;
+        for (int mode = 0; mode < 2; mode++) {
+            if (mode == 1) {
+                if (!row_mode) continue;
+                set_tile(tl_row, 3);
+            } else {
+                if (flat) set_tile(Tile{std::min(128, a.Wo), 1, 1}, 1);
+                else set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
+            }
+            for (int bn : {256, 192, 128, 64}) {
+                bn_force = bn;
+                if (!configure(kMaxSmem, 256, 2)) continue;
+                const double c = clocks();
+                if (c < best) {
+                    best = c;
+                    best_p = p; best_tl = tl; best_bias = bias_bytes; best_m = m_tiles;
+                    found = true;
+                }
+            }
+        }
+        bn_force = 0;
+        pair = found;
+        p = found ? best_p : keep;
+        tl = found ? best_tl : keep_tl;
+        bias_bytes = found ? best_bias : keep_bias;
+        m_tiles = found ? best_m : keep_m;
+    }
     // stores in flight: all buffers but one where a buffer also has to take the next tile's residual in time
     p.store_depth = std::max(1, a.res ? p.out_bufs - 1 : p.out_bufs);
     p.splits = splits;
@@ -1098,7 +1229,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         p.counters = static_cast<int*>(a.splitk_ws);
         p.partial = reinterpret_cast<float*>(static_cast<uint8_t*>(a.splitk_ws) + kSplitCounterBytes);
     }
-    const long long n_work = static_cast<long long>(p.tiles_w) * p.tiles_h * p.tiles_n * p.n_tiles_n * splits;
+    const long long n_work = work_items() * splits;
     if (n_work > 0x7fffffffLL) return DLF_E_UNSUPPORTED;
     p.n_work = static_cast<int>(n_work);
     uint32_t cols = 32;
@@ -1110,6 +1241,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
 
     CUtensorMap tmx, tmw, tmy, tmr, tmx2, tmw2;
     const uint64_t taps64 = static_cast<uint64_t>(a.kh) * a.kw;
+    const uint32_t w_rows = static_cast<uint32_t>(pair ? p.BN / 2 : p.BN);
     if (p.grouped) {
         // input seen as (64 channels, W, H, N, C_in / 64): one box carries one 64-channel chunk of a tap's window
         const uint64_t dims[5] = {64, static_cast<uint64_t>(a.W), static_cast<uint64_t>(a.H), static_cast<uint64_t>(a.N),
@@ -1124,7 +1256,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         // weights [cout][tap][cin] seen as (64 channels, cout, tap, C_in / 64)
         const uint64_t wdims[4] = {64, static_cast<uint64_t>(a.Cout), taps64, static_cast<uint64_t>(a.Cin / 64)};
         const uint64_t wstrides[3] = {taps64 * a.Cin * 2, static_cast<uint64_t>(a.Cin) * 2, 128};
-        const uint32_t wbox[4] = {64, static_cast<uint32_t>(p.BN), static_cast<uint32_t>(p.tps), 1};
+        const uint32_t wbox[4] = {64, w_rows, static_cast<uint32_t>(p.tps), 1};
         const uint32_t wes[4] = {1, 1, 1, 1};
         rc = encode_tmap(&tmw, a.w, 4, wdims, wstrides, wbox, wes);
         if (rc) return rc;
@@ -1140,7 +1272,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         if (rc) return rc;
         const uint64_t wdims[3] = {static_cast<uint64_t>(a.Cin), taps64, static_cast<uint64_t>(a.Cout)};
         const uint64_t wstrides[2] = {static_cast<uint64_t>(a.Cin) * 2, taps64 * a.Cin * 2};
-        const uint32_t wbox[3] = {64, 1, static_cast<uint32_t>(p.BN)};
+        const uint32_t wbox[3] = {64, 1, w_rows};
         const uint32_t wes[3] = {1, 1, 1};
         rc = encode_tmap(&tmw, a.w, 3, wdims, wstrides, wbox, wes);
         if (rc) return rc;
@@ -1158,7 +1290,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
         if (rc) return rc;
         const uint64_t wdims[4] = {64, static_cast<uint64_t>(a.Cout), 1, static_cast<uint64_t>(a.Cin2 / 64)};
         const uint64_t wstrides[3] = {static_cast<uint64_t>(a.Cin2) * 2, static_cast<uint64_t>(a.Cin2) * 2, 128};
-        const uint32_t wbox[4] = {64, static_cast<uint32_t>(p.BN), 1, 1};
+        const uint32_t wbox[4] = {64, w_rows, 1, 1};
         const uint32_t wes[4] = {1, 1, 1, 1};
         rc = encode_tmap(&tmw2, a.w2, 4, wdims, wstrides, wbox, wes);
         if (rc) return rc;
@@ -1179,7 +1311,8 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, ConvTcL
             if (rc) return rc;
         }
     }
-    out->grid = std::max(1, std::min(sm_count, p.n_work));
+    out->grid = pair ? 2 * std::max(1, std::min(sm_count / 2, p.n_work)) : std::max(1, std::min(sm_count, p.n_work));
+    out->pair = pair;
     // never two of these CTAs on an SM: each may hold all of tensor memory
     out->smem = std::max<size_t>(static_cast<size_t>(p.bias_off) + bias_bytes + 1024 + (kABytes + 256 - p.a_bytes), 120 * 1024);
 #ifdef DLF_TRACE
@@ -1199,9 +1332,9 @@ int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_
     rc = launch_conv_lat(a, sm_count, status_dev, s);
     if (rc != DLF_E_UNSUPPORTED) return rc;
     ConvTcLaunch L;
-    rc = conv_tc_prepare(a, sm_count, status_dev, &L);
+    rc = conv_tc_prepare(a, sm_count, status_dev, true, &L);
     if (rc) return rc;
-    const KernelFn fn = L.split ? pick_split(L.act, L.row != 0) : pick_kernel(L.act, L.pool != 0, L.res != 0, L.row != 0);
+    const KernelFn fn = L.pair ? pick_pair(L.act, L.pool != 0, L.res != 0, L.row != 0) : L.split ? pick_split(L.act, L.row != 0) : pick_kernel(L.act, L.pool != 0, L.res != 0, L.row != 0);
     cudaError_t e = launch_kernel(fn, L.grid, kThreads, L.smem, s, L.tmx, L.tmw, L.tmy, L.tmr, L.tmx2, L.tmw2, L.p);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
@@ -1223,7 +1356,7 @@ int launch_conv_seq(const ConvArgs* layers, int n_layers, int sm_count, int* sta
         a.splitk_ws = nullptr;   // no split reductions inside a multi-layer launch
         a.splitk_bytes = 0;
         ConvTcLaunch L;
-        rc = conv_tc_prepare(a, sm_count, status_dev, &L);
+        rc = conv_tc_prepare(a, sm_count, status_dev, false, &L);
         if (rc) return rc;
         if (L.split || (L.pool && L.row) || a.x2) return DLF_E_UNSUPPORTED;
         SeqLayer& Y = sp.L[l];
@@ -1251,6 +1384,7 @@ int conv_tc_init() {
                     for (int row = 0; row < (pool ? 1 : 2); row++) {
                         cudaError_t e = cudaFuncSetAttribute(pick_kernel(act, pool != 0, res != 0, row != 0),
                                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+                        if (e == cudaSuccess) e = cudaFuncSetAttribute(pick_pair(act, pool != 0, res != 0, row != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
                         if (e != cudaSuccess) return cuda_fail(e);
                     }
         for (int act = 0; act < 3; act++)
