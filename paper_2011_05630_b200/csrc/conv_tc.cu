@@ -1090,15 +1090,17 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
                                (sp > 1 ? static_cast<long long>(p.rows) * p.BN * 8 * 27 / 10 + 600000 : 0) + 40960;
         return rounds * item;
     };
-    // SM clocks of the current layout: rounds of the grid x cost of an item.  An item takes the slower of its copies (measured:
-    // 57 bytes per clock and SM, whatever the boxes) and its UMMAs (per M = 128, K = 16 instruction N / 2 clocks, at least 72),
-    // plus its output and residual at an SM's share of the HBM rate and a fixed hand-over.
+    // SM clocks of the current layout: rounds of the grid x cost of an item, and the last tile's drain.  An item takes the slower
+    // of its copies (measured: 57 bytes per clock and SM whatever the boxes, 50 where the ring has two stages only) and its UMMAs (per M = 128, K = 16 instruction 72
+    // clocks up to N = 128 - 56 at N = 64 in a pair, whose CTAs read half of B each - and 0.53 N above, and 200 clocks for
+    // the hand-over of a ring stage, 500 where a pair's stage holds one chunk of one tap), plus its output and residual at an SM's share of the HBM rate.
     auto clocks = [&]() {
         const double rounds = static_cast<double>((work_items() + workers() - 1) / workers());
         const double k = static_cast<double>(p.tgroups) * p.kchunks;
-        const double fill = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / 57.0;
-        const double mma = k * p.tps * 4 * std::max(p.BN / 2, 72);
-        return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + (pair ? 800.0 : 0.0);
+        const double fill = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / (p.stages > 2 ? 57.0 : 50.0);
+        const double umma = p.BN > 128 ? p.BN * 0.53 : (pair && p.BN <= 64 ? 56.0 : 72.0);
+        const double mma = k * p.tps * 4 * umma + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 500.0 : 200.0);
+        return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + p.BN * 14.0 + (pair ? 1400.0 : 0.0);
     };
     // Row mode (3x3, stride 1, pad 1): a tile is TH whole output rows seen with a pitch of Wo + 2, pixel-linear like
     // its input window, so that the three taps of a kernel row read ONE loaded window through descriptors that
@@ -1206,6 +1208,11 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
             for (int bn : {256, 192, 128, 64}) {
                 bn_force = bn;
                 if (!configure(kMaxSmem, 256, 2)) continue;
+                // (with one window load per tap and a narrow channel tile little is saved: 128 -> 128 3x3 stride 2 at 28x28, batch
+                // 32, 7.8 us alone, 8.5 us in pairs; 1x1 layers only with four times as many input as output channels: 512 -> 128
+                // at 28x28, batch 32, 10.1 -> 9.3 us, 256 -> 1024 at 14x14 8.5 -> 10.4 us)
+                const bool one = a.kh * a.kw == 1;
+                if (mode == 0 && !a.pool && (one ? dual || a.Cin < 4 * a.Cout : p.BN < 192)) continue;
                 const double c = clocks();
                 if (c < best) {
                     best = c;
