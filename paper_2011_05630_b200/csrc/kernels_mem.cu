@@ -260,31 +260,43 @@ __global__ void __launch_bounds__(256) maxpool_kernel(const __half* x, __half* y
     }
 }
 
-// fp32 sum over (h, w) ascending, times 1/(H*W), one rounding.
-__global__ void __launch_bounds__(128) gavgpool_kernel(const __half* x, __half* y, int N, int HW, int C, long long total) {
-    const int c8n = C / 8;
+// Mean over (h, w): fp32 sums, one rounding.  A block takes 8 channel vectors (128 contiguous bytes of a pixel) of one image
+// and shares the pixels out over 32 groups of threads, whose sums are added in a fixed order; with one thread walking all
+// pixels of its vector the kernel waited for one load after another (2048 channels at 7x7, one image 6.2 us in a network, now
+// 2.4 us).
+constexpr int kAvgVecs = 8, kAvgParts = 32;
+__global__ void __launch_bounds__(kAvgVecs * kAvgParts) gavgpool_kernel(const __half* x, __half* y, int HW, int C, int vec_blocks, int total) {
+    __shared__ float part[kAvgParts][kAvgVecs * 8 + 4];
+    const int v = threadIdx.x % kAvgVecs, q = threadIdx.x / kAvgVecs;
     const float inv = 1.0f / static_cast<float>(HW);
     pdl_launch_dependents();
     pdl_wait();
-    for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<long long>(gridDim.x) * blockDim.x) {
-        const int c8 = static_cast<int>(i % c8n);
-        const int n = static_cast<int>(i / c8n);
+    for (int blk = blockIdx.x; blk < total; blk += gridDim.x) {
+        const int n = blk / vec_blocks, c8 = (blk - n * vec_blocks) * kAvgVecs + v;
         float acc[8];
 #pragma unroll
         for (int j = 0; j < 8; j++) acc[j] = 0.0f;
-        const __half* xp = x + static_cast<long long>(n) * HW * C + c8 * 8;
-        for (int p = 0; p < HW; p++) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(xp + static_cast<long long>(p) * C));
-            const __half* vh = reinterpret_cast<const __half*>(&v);
+        if (c8 * 8 < C) {
+            const __half* xp = x + static_cast<long long>(n) * HW * C + c8 * 8;
+#pragma unroll 4
+            for (int p = q; p < HW; p += kAvgParts) {
+                const uint4 u = __ldg(reinterpret_cast<const uint4*>(xp + static_cast<long long>(p) * C));
+                const __half* vh = reinterpret_cast<const __half*>(&u);
 #pragma unroll
-            for (int j = 0; j < 8; j++) acc[j] += __half2float(vh[j]);
+                for (int j = 0; j < 8; j++) acc[j] += __half2float(vh[j]);
+            }
         }
-        uint4 o;
-        uint32_t* ou = reinterpret_cast<uint32_t*>(&o);
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) ou[j / 2] = pack_half2(acc[j] * inv, acc[j + 1] * inv);
-        *reinterpret_cast<uint4*>(y + static_cast<long long>(n) * C + c8 * 8) = o;
+        for (int j = 0; j < 8; j++) part[q][v * 8 + j] = acc[j];
+        __syncthreads();
+        if (threadIdx.x < kAvgVecs * 8) {   // one thread per channel
+            float sum = 0.0f;
+#pragma unroll 8
+            for (int k = 0; k < kAvgParts; k++) sum += part[k][threadIdx.x];
+            const int c = (blk - n * vec_blocks) * kAvgVecs * 8 + threadIdx.x;
+            if (c < C) y[static_cast<long long>(n) * C + c] = __float2half_rn(sum * inv);
+        }
+        __syncthreads();
     }
 }
 
@@ -409,10 +421,12 @@ int launch_maxpool(const void* x, void* y, int N, int H, int W, int C, int k, in
 
 int launch_gavgpool(const void* x, void* y, int N, int H, int W, int C, int sm_count, cudaStream_t s) {
     if (C % 8) return DLF_E_UNSUPPORTED;
-    const long long total = static_cast<long long>(N) * (C / 8);
+    const int vec_blocks = (C / 8 + kAvgVecs - 1) / kAvgVecs;
+    const long long total = static_cast<long long>(N) * vec_blocks;
     if (total == 0) return DLF_OK;
-    cudaError_t e = launch_kernel(gavgpool_kernel, grid_for((total + 127) / 128, sm_count), 128, 0, s, static_cast<const __half*>(x),
-                                  static_cast<__half*>(y), N, H * W, C, total);
+    if (total > 0x7fffffffLL) return DLF_E_UNSUPPORTED;
+    cudaError_t e = launch_kernel(gavgpool_kernel, grid_for(total, sm_count), kAvgVecs * kAvgParts, 0, s, static_cast<const __half*>(x),
+                                  static_cast<__half*>(y), H * W, C, vec_blocks, static_cast<int>(total));
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
