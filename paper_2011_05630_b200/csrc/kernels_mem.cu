@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -111,113 +112,129 @@ __global__ void __launch_bounds__(128) conv_direct_kernel(ConvArgs a, long long 
 }
 
 // ---- depthwise 3x3 ------------------------------------------------------------------------------------
-// One thread = 8 channels x a strip of kDwStrip output columns of one output row.  The thread's 72
-// weights and 8 biases are converted to fp32 once (the launch makes the total thread count a
-// multiple of C/8, so a thread keeps its channels over the whole grid-stride loop); every input
-// vector of the strip's three rows is loaded once (128 bits), converted once and used by all the
-// outputs it touches.  Lanes run over the channel vectors first, so a warp reads contiguous NHWC
-// runs.  fp32 accumulation in (kh, kw) order, one rounding.
-constexpr int kDwStrip = 4;
-
+// One thread = 4 channels x one output column x a strip of output rows, walked from top to bottom: every input row of three
+// 8-byte vectors is loaded (three rows ahead) and converted once and joins the up to three output rows it touches, so an output
+// costs 9 multiply-adds and 4 to 5 other instructions; loading a strip's whole window at once (the first version: 8 channels
+// x 4 columns of one row) converted every input 4.5 times.  The thread's 36 weights are converted to fp32 once, before the
+// wait for the previous kernel (the launch makes the total thread count a multiple of C/4, so a thread keeps its channels over
+// the whole grid-stride loop).  Lanes run over the channels first, so a warp reads contiguous NHWC runs.  fp32 accumulation
+// from the bias on in (kh, kw) order, one rounding.
 template <int STRIDE>
-__global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total, int strips) {
-    constexpr int kCols = (kDwStrip - 1) * STRIDE + 3;  // input columns one strip reads per row
-    const int c8n = a.Cout / 8;
+__global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total, int strips, int rows_per) {
+    const int c4n = a.Cout / 4;
     const long long tid = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
     const long long nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
     pdl_launch_dependents();
     if (tid >= total) return;
-    const int c0 = static_cast<int>(tid % c8n) * 8;
-    float w[9][8], b[8];
+    const int c0 = static_cast<int>(tid % c4n) * 4;
+    float w[9][4], bias[4];
     {
-        __align__(16) __half wv[72];  // weights of channels c0..c0+7: 72 consecutive halves starting at c0*9
-        const uint4* wp4 = reinterpret_cast<const uint4*>(static_cast<const __half*>(a.w) + static_cast<long long>(c0) * 9);
+        uint2 raw[9];   // weights of channels c0 .. c0 + 3: 36 consecutive halves starting at c0 * 9
+        const uint2* wp = reinterpret_cast<const uint2*>(static_cast<const __half*>(a.w) + static_cast<long long>(c0) * 9);
 #pragma unroll
-        for (int k = 0; k < 9; k++) reinterpret_cast<uint4*>(wv)[k] = __ldg(wp4 + k);
+        for (int k = 0; k < 9; k++) raw[k] = __ldg(wp + k);
+        const __half* wv = reinterpret_cast<const __half*>(raw);
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            b[j] = __ldg(a.bias + c0 + j);
+        for (int j = 0; j < 4; j++) {
+            bias[j] = __ldg(a.bias + c0 + j);
 #pragma unroll
             for (int t = 0; t < 9; t++) w[t][j] = __half2float(wv[j * 9 + t]);
         }
     }
     pdl_wait();   // (the weights above are constants)
     const __half2 lo = __float2half2_rn(a.act >= 1 ? 0.0f : -INFINITY), hi = __float2half2_rn(a.act == 2 ? 6.0f : INFINITY);   // applied to rounded pairs
-    const __half* x = static_cast<const __half*>(a.x);
     const __half* res = static_cast<const __half*>(a.res);
-    __half* y = static_cast<__half*>(a.y);
+    const int in_row = a.W * a.Cin, out_row = a.Wo * a.Cout;
     for (long long i = tid; i < total; i += nthreads) {
-        long long p = i / c8n;
-        const int strip = static_cast<int>(p % strips);
-        p /= strips;
-        const int ho = static_cast<int>(p % a.Ho);
-        const int n = static_cast<int>(p / a.Ho);
-        const int wo0 = strip * kDwStrip;
-        const int wi0 = wo0 * STRIDE - a.pad;
-        float acc[kDwStrip][8];
+        long long q = i / c4n;
+        const int wo = static_cast<int>(q % a.Wo);
+        q /= a.Wo;
+        const int strip = static_cast<int>(q % strips), n = static_cast<int>(q / strips);
+        const int ho0 = strip * rows_per, rows = min(rows_per, a.Ho - ho0);
+        const int wi = wo * STRIDE - a.pad;
+        int hi_ = ho0 * STRIDE - a.pad;   // input row that is fetched next
+        const bool ok0 = wi >= 0 && wi < a.W, ok1 = wi + 1 >= 0 && wi + 1 < a.W, ok2 = wi + 2 >= 0 && wi + 2 < a.W;
+        const __half* src = static_cast<const __half*>(a.x) + (static_cast<long long>(n) * a.H * a.W + wi) * a.Cin + static_cast<long long>(hi_) * in_row + c0;
+        long long off = (static_cast<long long>(n) * a.Ho + ho0) * out_row + static_cast<long long>(wo) * a.Cout + c0;
+        uint2 raw[3][3];   // the next three input rows
+        int left = rows * STRIDE + 3 - STRIDE;   // rows still to fetch
+        auto fetch = [&](int slot) {
+            const bool row_ok = hi_ >= 0 && hi_ < a.H && left > 0;
+            raw[slot][0] = row_ok && ok0 ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
+            raw[slot][1] = row_ok && ok1 ? __ldg(reinterpret_cast<const uint2*>(src + a.Cin)) : make_uint2(0u, 0u);
+            raw[slot][2] = row_ok && ok2 ? __ldg(reinterpret_cast<const uint2*>(src + 2 * a.Cin)) : make_uint2(0u, 0u);
+            left--;
+            hi_++;
+            src += in_row;
+        };
+        float x[3][4];
+        auto next = [&](int slot) {
 #pragma unroll
-        for (int o = 0; o < kDwStrip; o++)
-#pragma unroll
-            for (int j = 0; j < 8; j++) acc[o][j] = 0.0f;
-#pragma unroll
-        for (int r = 0; r < 3; r++) {
-            const int hi_ = ho * STRIDE - a.pad + r;
-            const bool row_ok = hi_ >= 0 && hi_ < a.H;
-            const __half* row = x + ((static_cast<long long>(n) * a.H + min(max(hi_, 0), a.H - 1)) * a.W) * a.Cin + c0;
-            // all loads of the row first, from clamped (always valid) addresses and without branches, so
-            // that they are in flight together; columns outside the image are zeroed afterwards
-            uint4 xv[kCols];
-#pragma unroll
-            for (int j = 0; j < kCols; j++)
-                xv[j] = __ldg(reinterpret_cast<const uint4*>(row + static_cast<long long>(min(max(wi0 + j, 0), a.W - 1)) * a.Cin));
-#pragma unroll
-            for (int j = 0; j < kCols; j++) {
-                const int wi = wi0 + j;
-                // a column outside the image contributes zeros: the vector is cleared with four selects (a multiply
-                // by 0 / 1 per element doubled the load on the FMA pipe, which is what bounds this kernel)
-                if (!(row_ok && wi >= 0 && wi < a.W)) xv[j] = make_uint4(0u, 0u, 0u, 0u);
-                const __half2* xh = reinterpret_cast<const __half2*>(&xv[j]);
-                float xf[8];
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const float2 f = __half22float2(xh[e]);
-                    xf[2 * e] = f.x;
-                    xf[2 * e + 1] = f.y;
-                }
-#pragma unroll
-                for (int o = 0; o < kDwStrip; o++) {
-                    const int s = j - o * STRIDE;  // tap column of output o that reads input column j
-                    if (s >= 0 && s < 3) {
-#pragma unroll
-                        for (int e = 0; e < 8; e++) acc[o][e] = fmaf(xf[e], w[r * 3 + s][e], acc[o][e]);
-                    }
-                }
+            for (int s = 0; s < 3; s++) {
+                const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&raw[slot][s].x)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&raw[slot][s].y));
+                x[s][0] = f0.x; x[s][1] = f0.y; x[s][2] = f1.x; x[s][3] = f1.y;
             }
-        }
+            fetch(slot);
+        };
+        auto add = [&](float (&acc)[4], int r) {
 #pragma unroll
-        for (int o = 0; o < kDwStrip; o++) {
-            const int wo = wo0 + o;
-            if (wo >= a.Wo) break;
-            const long long off = ((static_cast<long long>(n) * a.Ho + ho) * a.Wo + wo) * a.Cout + c0;
-            float v[8];
+            for (int s = 0; s < 3; s++)
 #pragma unroll
-            for (int e = 0; e < 8; e++) v[e] = acc[o][e] + b[e];
+                for (int j = 0; j < 4; j++) acc[j] = fmaf(x[s][j], w[r * 3 + s][j], acc[j]);
+        };
+        auto start = [&](float (&acc)[4]) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) acc[j] = bias[j];
+            add(acc, 0);
+        };
+        auto store = [&](float (&acc)[4]) {
             if (res != nullptr) {
-                const uint4 rv = __ldg(reinterpret_cast<const uint4*>(res + off));
-                const __half2* rh = reinterpret_cast<const __half2*>(&rv);
-#pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const float2 f = __half22float2(rh[e]);
-                    v[2 * e] += f.x;
-                    v[2 * e + 1] += f.y;
-                }
+                const uint2 rv = __ldg(reinterpret_cast<const uint2*>(res + off));
+                const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&rv.x)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&rv.y));
+                acc[0] += f0.x; acc[1] += f0.y; acc[2] += f1.x; acc[3] += f1.y;
             }
-            uint4 outv;
-            uint32_t* ou = reinterpret_cast<uint32_t*>(&outv);
-#pragma unroll
-            for (int e = 0; e < 4; e++)
-                ou[e] = pack_half2_clamp(v[2 * e], v[2 * e + 1], lo, hi);
-            *reinterpret_cast<uint4*>(y + off) = outv;
+            uint2 o;
+            o.x = pack_half2_clamp(acc[0], acc[1], lo, hi);
+            o.y = pack_half2_clamp(acc[2], acc[3], lo, hi);
+            *reinterpret_cast<uint2*>(static_cast<__half*>(a.y) + off) = o;
+            off += out_row;
+        };
+        float u[4], v[4], t[4];
+        fetch(0);
+        fetch(1);
+        fetch(2);
+        if (STRIDE == 1) {
+            // input row j is the last row of output j - 2, the middle one of output j - 1, the first one of output j
+            next(0); start(u);
+            next(1); add(u, 1); start(v);
+            int j = 0;
+#pragma unroll 1
+            while (true) {
+                next(2); add(u, 2); store(u);
+                if (++j == rows) break;
+                add(v, 1); start(t);
+                next(0); add(v, 2); store(v);
+                if (++j == rows) break;
+                add(t, 1); start(u);
+                next(1); add(t, 2); store(t);
+                if (++j == rows) break;
+                add(u, 1); start(v);
+            }
+        } else {
+            next(0); start(u);
+            int j = 0;
+#pragma unroll 1
+            while (true) {
+                next(1); add(u, 1); next(2); add(u, 2); store(u);
+                if (++j == rows) break;
+                start(u);
+                next(0); add(u, 1); next(1); add(u, 2); store(u);
+                if (++j == rows) break;
+                start(u);
+                next(2); add(u, 1); next(0); add(u, 2); store(u);
+                if (++j == rows) break;
+                start(u);
+            }
         }
     }
 }
@@ -385,27 +402,43 @@ int launch_conv_direct(const ConvArgs& a, int sm_count, cudaStream_t s) {
 int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
     if (a.kh != 3 || a.kw != 3 || a.groups != a.Cin || a.Cin != a.Cout || a.Cin % 8 || a.pool) return DLF_E_UNSUPPORTED;
     if (a.stride != 1 && a.stride != 2) return DLF_E_UNSUPPORTED;
-    const int c8n = a.Cout / 8;
-    const int strips = (a.Wo + kDwStrip - 1) / kDwStrip;
-    const long long total = static_cast<long long>(a.N) * a.Ho * strips * c8n;
-    if (total == 0) return DLF_OK;
-    // the total thread count is a multiple of C/8: a thread keeps its channels (and its weights)
-    int step = c8n;
-    for (int d = 2; d <= 128; d *= 2)
-        if (step % 2 == 0) step /= 2;  // blocks needed for (blocks * 128) % c8n == 0: c8n / gcd(c8n, 128)
-    // one resident wave of blocks: a thread converts its 72 weights once and then walks its strips (more blocks than fit
-    // would each pay that prologue again, wave after wave).  A variant with four channels per thread (96 registers,
-    // five blocks per SM instead of three) was measured 20 % slower: the index arithmetic per vector doubles.
+    const int c4n = a.Cout / 4;
     static int occ[2] = {0, 0};
     const int v = a.stride == 1 ? 0 : 1;
     if (occ[v] == 0) {
-        cudaError_t e = v == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[v], dw3x3_kernel<1>, 128, 0)
-                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[v], dw3x3_kernel<2>, 128, 0);
-        if (e != cudaSuccess || occ[v] < 1) occ[v] = 2;
+        int n = 0;
+        cudaError_t e = v == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dw3x3_kernel<1>, 128, 0)
+                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dw3x3_kernel<2>, 128, 0);
+        occ[v] = e != cudaSuccess || n < 1 ? 2 : n;
     }
+    // Rows of a strip: long strips load few rows twice, short ones keep all SMs busy on a small map.  Cost = the slower of the
+    // threads' instructions (about 75 per input row and warp, 2.4 issued per clock and SM) and one thread's walk (a round trip
+    // to L2 and about 120 clocks per row), times the rounds of the grid.
+    const long long columns = static_cast<long long>(a.N) * a.Wo * c4n;
+    int rows_per = 1;
+    double best = -1.0;
+    for (int r = 1; r <= a.Ho; r++) {
+        const int strips = (a.Ho + r - 1) / r;
+        if ((strips - 1) * r >= a.Ho) continue;
+        const double threads = static_cast<double>(columns) * strips, rows_in = r * a.stride + 3 - a.stride;
+        const double rounds = std::ceil(threads / (static_cast<double>(sm_count) * occ[v] * 128));
+        const double cost = std::max(threads / 32 * rows_in * 75.0 / (2.4 * sm_count), rounds * (700.0 + rows_in * 120.0));
+        if (best < 0 || cost < best) {
+            best = cost;
+            rows_per = r;
+        }
+    }
+    const int strips = (a.Ho + rows_per - 1) / rows_per;
+    const long long total = columns * strips;
+    if (total == 0) return DLF_OK;
+    // the total thread count is a multiple of C/4: a thread keeps its channels (and its weights)
+    int step = c4n;
+    for (int d = 2; d <= 128; d *= 2)
+        if (step % 2 == 0) step /= 2;  // blocks needed for (blocks * 128) % c4n == 0: c4n / gcd(c4n, 128)
+    // one resident wave of blocks: a thread converts its weights once and then walks its strips
     long long blocks = std::min<long long>((total + 127) / 128, static_cast<long long>(sm_count) * occ[v]);
     blocks = std::max<long long>(step, blocks / step * step);
-    cudaError_t e = launch_kernel(a.stride == 1 ? dw3x3_kernel<1> : dw3x3_kernel<2>, static_cast<int>(blocks), 128, 0, s, a, total, strips);
+    cudaError_t e = launch_kernel(a.stride == 1 ? dw3x3_kernel<1> : dw3x3_kernel<2>, static_cast<int>(blocks), 128, 0, s, a, total, strips, rows_per);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
