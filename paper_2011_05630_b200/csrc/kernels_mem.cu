@@ -411,9 +411,10 @@ int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
                                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, dw3x3_kernel<2>, 128, 0);
         occ[v] = e != cudaSuccess || n < 1 ? 2 : n;
     }
-    // Rows of a strip: long strips load few rows twice, short ones keep all SMs busy on a small map.  Cost = the slower of the
-    // threads' instructions (about 75 per input row and warp, 2.4 issued per clock and SM) and one thread's walk (a round trip
-    // to L2 and about 120 clocks per row), times the rounds of the grid.
+    // Rows of a strip: long strips load few rows twice, short ones keep all SMs busy on a small map.  A thread's walk costs about
+    // 700 clocks per input row at full occupancy (the latency of its loads; about four rows' worth before the first); the cost
+    // of a strip length is that times the rounds of the grid, a last round that is not full counting a quarter less.  (Against
+    // the longest strip throughout: 96 channels stride 2 at 112x112, batch 64 68 -> 51 us; 24 channels at 51x37, batch 30 6.8 -> 4.3.)
     const long long columns = static_cast<long long>(a.N) * a.Wo * c4n;
     int rows_per = 1;
     double best = -1.0;
@@ -421,8 +422,8 @@ int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
         const int strips = (a.Ho + r - 1) / r;
         if ((strips - 1) * r >= a.Ho) continue;
         const double threads = static_cast<double>(columns) * strips, rows_in = r * a.stride + 3 - a.stride;
-        const double rounds = std::ceil(threads / (static_cast<double>(sm_count) * occ[v] * 128));
-        const double cost = std::max(threads / 32 * rows_in * 75.0 / (2.4 * sm_count), rounds * (700.0 + rows_in * 120.0));
+        const double rounds = threads / (static_cast<double>(sm_count) * occ[v] * 128);
+        const double cost = (0.75 * std::ceil(rounds) + 0.25 * rounds) * (rows_in + 4.0);
         if (best < 0 || cost < best) {
             best = cost;
             rows_per = r;
