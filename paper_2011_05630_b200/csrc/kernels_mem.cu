@@ -113,9 +113,9 @@ __global__ void __launch_bounds__(128) conv_direct_kernel(ConvArgs a, long long 
 
 // ---- depthwise 3x3 ------------------------------------------------------------------------------------
 // One thread = 4 channels x one output column x a strip of output rows, walked from top to bottom: every input row of three
-// 8-byte vectors is loaded (three rows ahead) and converted once and joins the up to three output rows it touches, so an output
-// costs 9 multiply-adds and 4 to 5 other instructions; loading a strip's whole window at once (the first version: 8 channels
-// x 4 columns of one row) converted every input 4.5 times.  The thread's 36 weights are converted to fp32 once, before the
+// 8-byte vectors is loaded (three rows ahead) once and joins the up to three output rows it touches through multiply-adds that
+// take fp16 factors, so an output costs nine of them and 2 to 3 other instructions; loading a strip's whole window at once (the first version: 8 channels
+// x 4 columns of one row) converted every input 4.5 times.  The thread's 36 weights are fetched once, before the
 // wait for the previous kernel (the launch makes the total thread count a multiple of C/4, so a thread keeps its channels over
 // the whole grid-stride loop).  Lanes run over the channels first, so a warp reads contiguous NHWC runs.  fp32 accumulation
 // from the bias on in (kh, kw) order, one rounding.
@@ -127,19 +127,20 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
     pdl_launch_dependents();
     if (tid >= total) return;
     const int c0 = static_cast<int>(tid % c4n) * 4;
-    float w[9][4], bias[4];
+    unsigned short w[9][4];   // (fp16)
+    float bias[4];
     {
         uint2 raw[9];   // weights of channels c0 .. c0 + 3: 36 consecutive halves starting at c0 * 9
         const uint2* wp = reinterpret_cast<const uint2*>(static_cast<const __half*>(a.w) + static_cast<long long>(c0) * 9);
 #pragma unroll
         for (int k = 0; k < 9; k++) raw[k] = __ldg(wp + k);
-        const __half* wv = reinterpret_cast<const __half*>(raw);
+        const unsigned short* wv = reinterpret_cast<const unsigned short*>(raw);
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            bias[j] = __ldg(a.bias + c0 + j);
+        for (int t = 0; t < 9; t++)
 #pragma unroll
-            for (int t = 0; t < 9; t++) w[t][j] = __half2float(wv[j * 9 + t]);
-        }
+            for (int j = 0; j < 4; j++) w[t][j] = wv[j * 9 + t];
+#pragma unroll
+        for (int j = 0; j < 4; j++) bias[j] = __ldg(a.bias + c0 + j);
     }
     pdl_wait();   // (the weights above are constants)
     const __half2 lo = __float2half2_rn(a.act >= 1 ? 0.0f : -INFINITY), hi = __float2half2_rn(a.act == 2 ? 6.0f : INFINITY);   // applied to rounded pairs
@@ -167,12 +168,12 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
             hi_++;
             src += in_row;
         };
-        float x[3][4];
+        unsigned short x[3][4];
         auto next = [&](int slot) {
 #pragma unroll
             for (int s = 0; s < 3; s++) {
-                const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&raw[slot][s].x)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&raw[slot][s].y));
-                x[s][0] = f0.x; x[s][1] = f0.y; x[s][2] = f1.x; x[s][3] = f1.y;
+                unpack_h2(raw[slot][s].x, x[s][0], x[s][1]);
+                unpack_h2(raw[slot][s].y, x[s][2], x[s][3]);
             }
             fetch(slot);
         };
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
 #pragma unroll
             for (int s = 0; s < 3; s++)
 #pragma unroll
-                for (int j = 0; j < 4; j++) acc[j] = fmaf(x[s][j], w[r * 3 + s][j], acc[j]);
+                for (int j = 0; j < 4; j++) acc[j] = fma_f32_f16(x[s][j], w[r * 3 + s][j], acc[j]);
         };
         auto start = [&](float (&acc)[4]) {
 #pragma unroll
@@ -436,7 +437,7 @@ int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
     int step = c4n;
     for (int d = 2; d <= 128; d *= 2)
         if (step % 2 == 0) step /= 2;  // blocks needed for (blocks * 128) % c4n == 0: c4n / gcd(c4n, 128)
-    // one resident wave of blocks: a thread converts its weights once and then walks its strips
+    // one resident wave of blocks: a thread fetches its weights once and then walks its strips
     long long blocks = std::min<long long>((total + 127) / 128, static_cast<long long>(sm_count) * occ[v]);
     blocks = std::max<long long>(step, blocks / step * step);
     cudaError_t e = launch_kernel(a.stride == 1 ? dw3x3_kernel<1> : dw3x3_kernel<2>, static_cast<int>(blocks), 128, 0, s, a, total, strips, rows_per);

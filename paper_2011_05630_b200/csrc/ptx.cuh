@@ -397,6 +397,16 @@ __device__ __forceinline__ void tmem_ld32_wait(uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) : : "memory");
 }
 
+// acc + x * w with fp16 factors (bit patterns): exact product, one fp32 rounding, no conversions.  (Both factors in registers
+// of their own: packed pairs unpacked at every use were measured a fifth slower in the depthwise kernel.)
+__device__ __forceinline__ float fma_f32_f16(unsigned short x, unsigned short w, float acc) {
+    asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc) : "h"(x), "h"(w));
+    return acc;
+}
+__device__ __forceinline__ void unpack_h2(uint32_t v, unsigned short& lo, unsigned short& hi) {
+    asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(v));
+}
+
 template <int ACT>
 __device__ __forceinline__ float act_t(float v) {
     if (ACT >= 1) v = fmaxf(v, 0.0f);
