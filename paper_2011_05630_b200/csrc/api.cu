@@ -494,10 +494,11 @@ static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTi
 }
 
 // The estimate for an inverted-residual block: the fused kernel's own cost model (the tiler's SM clocks, plus one kernel
-// boundary) against one kernel per layer, each at its bytes at 2.5 TB/s - what the depthwise and the narrow pointwise kernels
-// reach on this chip - plus 5 us of fixed cost; the block must win by a tenth.  It replaces the fixed limit on the hidden
-// width of the first version: wide blocks on small maps (many 64-channel steps, few tiles to spread over the SMs) lose, the
-// same blocks at a large batch win.
+// boundary) against one kernel per layer.  Inside a network a layer's own kernel takes 3.1 us plus its bytes at 3.6 TB/s (the
+// depthwise one) or 3.2 TB/s (the pointwise ones) - fitted to MobileNetV2's blocks at 1 to 128 images, each timed both ways:
+// blocks on maps of 14x14 and more win from a few images on (24 -> 144 -> 24 channels at 56x56: 62 us against 95 at 64
+// images, 10 against 10 at one), wide ones on small maps (many 64-channel steps, few tiles to spread over the SMs) lose
+// (160 -> 960 -> 160 at 7x7: 25 against 20 at 64 images), and without an expansion layer only the smallest batches win.
 static bool mbconv_pays(const dlf_net* net, int first, int last, int sms) {
     const MbconvTiling t = mbconv_tiling(mbconv_args(net, first, last, nullptr, nullptr), sms);
     if (!t.ok) return false;
@@ -506,9 +507,9 @@ static bool mbconv_pays(const dlf_net* net, int first, int last, int sms) {
         const Layer& l = net->layers[i];
         const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
                              (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
-        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / 2.5e6) + 5.0;
+        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + 3.1;
     }
-    return t.cost / 1.9e3 + 5.5 < 0.9 * single_us;
+    return t.cost / 1.9e3 + 1.0 < single_us;
 }
 
 static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix, int s_max) {
