@@ -77,6 +77,7 @@ struct ChainLayerP {
     int n_chunks, chunk_n;     // channel chunks of chunk_n (the last one may be smaller)
     int slot, per_pass, bgroups;  // TMEM columns per block, blocks per pass, passes per channel chunk
     int tg, kg, w_rank4;       // taps and K chunks per weight box; 4-d weight view (cin % 64 == 0)
+    int n_boxes;               // resident weights: boxes of the layer
     int w_off;                 // resident weights: byte offset of this layer's slabs, ordered [chunk][K chunk][tap][row]
     int col0, half_cols;       // TMEM region of this layer: first column, columns of one half
     int in_dense, out_dense;   // rows are tile pixels (ty*tw + tx) instead of frame positions: of the layer itself / of what it writes
@@ -91,6 +92,7 @@ struct ChainParams {
     int n_layers;
     int N, H, W;
     int th, tw, halo, pitch, rows;  // frame geometry
+    uint32_t pitch_magic, tw_magic; // ceil(2^20 / pitch), ceil(2^20 / tw): rows (fewer than 4096) are divided by multiplying
     int tiles_h, tiles_w, n_tiles;
     int in_planes, in_group, in_slots, in_ring, in_slot_bytes, in_off;
     int act_off[2], act_plane_bytes[2];
@@ -119,11 +121,11 @@ struct RowPos {
 __device__ __forceinline__ RowPos row_pos(const ChainParams& p, bool dense, int q, int gy0, int gx0) {
     RowPos r;
     if (dense) {
-        r.ty = q / p.tw;
+        r.ty = static_cast<int>((static_cast<uint32_t>(q) * p.tw_magic) >> 20);
         r.tx = q - r.ty * p.tw;
         r.in_tile = q < p.th * p.tw;
     } else {
-        const int fy = q / p.pitch, fx = q - fy * p.pitch;
+        const int fy = static_cast<int>((static_cast<uint32_t>(q) * p.pitch_magic) >> 20), fx = q - fy * p.pitch;
         r.ty = fy - p.halo;
         r.tx = fx - p.halo;
         r.in_tile = r.ty >= 0 && r.ty < p.th && r.tx >= 0 && r.tx < p.tw;
@@ -136,6 +138,15 @@ __device__ __forceinline__ RowPos row_pos(const ChainParams& p, bool dense, int 
 // Row of tile pixel (ty, tx) in the last layer's row layout.
 __device__ __forceinline__ int out_row(const ChainParams& p, int ty, int tx) {
     return p.out_dense ? ty * p.tw + tx : (ty + p.halo) * p.pitch + p.halo + tx;
+}
+
+// Tile t of the group: tile column and row, image.
+struct TilePos {
+    int x, y, n;
+};
+__device__ __forceinline__ TilePos tile_pos(const ChainParams& p, int t) {
+    const int r = t / p.tiles_w, n = r / p.tiles_h;
+    return TilePos{t - r * p.tiles_w, r - n * p.tiles_h, n};
 }
 
 struct EpiCtx {
@@ -178,18 +189,26 @@ __device__ __forceinline__ uint4* tile_ptr(uint8_t* buf, int plane_bytes, int ro
                                     (((g8 & 7) ^ (row & 7)) << 4));
 }
 
-// Drains one pass of an inner layer into the next layer's operand tile (zero outside the image).
-__device__ __forceinline__ void epi_inner(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx) {
+// Where this thread's row of block b of a pass goes; worked out before the accumulator is waited for.
+struct InnerRow {
+    int wrow;             // row of the next layer's operand tile
+    bool live, in_img;
+};
+__device__ __forceinline__ InnerRow inner_row(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx, int b) {
+    const int q = L.qs + (cx.b0 + b) * 128 + cx.row;
+    const RowPos r = row_pos(p, L.in_dense != 0, q, cx.gy0, cx.gx0);
+    InnerRow ir{q, q < L.qs + L.range, r.in_img};
+    if (L.out_dense && !L.in_dense) {   // the group's last 3x3 layer: keep the tile's own pixels, densely
+        ir.live = ir.live && r.in_tile;
+        ir.wrow = r.ty * p.tw + r.tx;
+    }
+    return ir;
+}
+
+// Drains one pass of an inner layer into the next layer's operand tile (zero outside the image); `ir`: block 0's row.
+__device__ __forceinline__ void epi_inner(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx, InnerRow ir) {
 #pragma unroll 1
     for (int b = 0; b < cx.nblk; b++) {
-        const int q = L.qs + (cx.b0 + b) * 128 + cx.row;
-        const RowPos r = row_pos(p, L.in_dense != 0, q, cx.gy0, cx.gx0);
-        bool live = q < L.qs + L.range;
-        int wrow = q;
-        if (L.out_dense && !L.in_dense) {   // the group's last 3x3 layer: keep the tile's own pixels, densely
-            live = live && r.in_tile;
-            wrow = r.ty * p.tw + r.tx;
-        }
         const uint32_t taddr = cx.tmem_lane + cx.tmem_col + b * L.slot;
 #pragma unroll 1
         for (int cc = cx.half * 32; cc < cx.ncols; cc += 64) {
@@ -198,32 +217,42 @@ __device__ __forceinline__ void epi_inner(const ChainParams& p, const ChainLayer
             const int nc = min(32, cx.ncols - cc);
             if (nc == 32) tmem_ld32(taddr + cc, v);
             else tmem_ld16(taddr + cc, v);
-            if (!live) continue;
+            if (!ir.live) continue;
 #pragma unroll
             for (int g = 0; g < 4; g++) {
                 if (g * 8 >= nc) break;
                 const int co = cx.ch0 + cc + g * 8;  // first of 8 channels
                 // channels past cout (padding up to 16) carry zero weights and zero bias: act(0) = 0,
                 // so the next layer's K padding stays zero
-                const uint4 val = r.in_img ? finish8(v + g * 8, cx.bl + co, cx) : make_uint4(0u, 0u, 0u, 0u);
-                *tile_ptr(cx.obuf, cx.oplane, wrow, co >> 3) = val;
+                const uint4 val = ir.in_img ? finish8(v + g * 8, cx.bl + co, cx) : make_uint4(0u, 0u, 0u, 0u);
+                *tile_ptr(cx.obuf, cx.oplane, ir.wrow, co >> 3) = val;
             }
         }
+        if (b + 1 < cx.nblk) ir = inner_row(p, L, cx, b + 1);
     }
 }
 
-// Drains one pass of the group's last layer.  MODE OUT_DIRECT: 16-byte global stores (residual by global loads);
+struct LastRow {
+    int srow;             // row of the staging tile
+    bool live, in_out;    // drained at all / a pixel of the output tile inside the image
+    long long gpix;       // that pixel
+};
+template <int MODE>
+__device__ __forceinline__ LastRow last_row(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx, int b) {
+    const int q = L.qs + (cx.b0 + b) * 128 + cx.row;
+    const RowPos r = row_pos(p, L.in_dense != 0, q, cx.gy0, cx.gx0);
+    const bool in_out = r.in_tile && r.in_img;
+    return LastRow{q - p.stg_base8, q < L.qs + L.range && (MODE == OUT_POOL || in_out), in_out,
+                   MODE == OUT_STAGE ? 0ll : (static_cast<long long>(cx.n) * p.H + r.gy) * p.W + r.gx};
+}
+
+// Drains one pass of the group's last layer (`lr`: block 0's row).  MODE OUT_DIRECT: 16-byte global stores (residual by global loads);
 // OUT_STAGE: staging tile (the residual, if any, already lies there); OUT_POOL: staging tile of the whole frame.
 template <int MODE>
-__device__ __forceinline__ void epi_last(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx) {
+__device__ __forceinline__ void epi_last(const ChainParams& p, const ChainLayerP& L, const EpiCtx& cx, LastRow lr) {
     const bool has_res = p.res != nullptr;
 #pragma unroll 1
     for (int b = 0; b < cx.nblk; b++) {
-        const int q = L.qs + (cx.b0 + b) * 128 + cx.row;
-        const RowPos r = row_pos(p, L.in_dense != 0, q, cx.gy0, cx.gx0);
-        const bool live = q < L.qs + L.range && (MODE == OUT_POOL || (r.in_tile && r.in_img));
-        const long long gpix = (static_cast<long long>(cx.n) * p.H + r.gy) * p.W + r.gx;
-        const int srow = q - p.stg_base8;
         const uint32_t taddr = cx.tmem_lane + cx.tmem_col + b * L.slot;
 #pragma unroll 1
         for (int cc = cx.half * 32; cc < cx.ncols; cc += 64) {
@@ -232,61 +261,69 @@ __device__ __forceinline__ void epi_last(const ChainParams& p, const ChainLayerP
             const int nc = min(32, cx.ncols - cc);
             if (nc == 32) tmem_ld32(taddr + cc, v);
             else tmem_ld16(taddr + cc, v);
-            if (!live) continue;
+            if (!lr.live) continue;
 #pragma unroll
             for (int g = 0; g < 4; g++) {
                 if (g * 8 >= nc) break;
                 const int co = cx.ch0 + cc + g * 8;
                 if (MODE == OUT_STAGE) {
-                    uint4* sp = tile_ptr(cx.obuf, cx.oplane, srow, (cc >> 3) + g);
+                    uint4* sp = tile_ptr(cx.obuf, cx.oplane, lr.srow, (cc >> 3) + g);
                     *sp = has_res ? finish8_res(v + g * 8, cx.bl + co, *sp, cx) : finish8(v + g * 8, cx.bl + co, cx);
                 } else {
                     uint4 val;
-                    if (has_res && co < L.cout && r.in_tile && r.in_img)
-                        val = finish8_res(v + g * 8, cx.bl + co, __ldg(reinterpret_cast<const uint4*>(p.res + gpix * L.cout + co)), cx);
+                    if (has_res && co < L.cout && lr.in_out)
+                        val = finish8_res(v + g * 8, cx.bl + co, __ldg(reinterpret_cast<const uint4*>(p.res + lr.gpix * L.cout + co)), cx);
                     else
                         val = finish8(v + g * 8, cx.bl + co, cx);
-                    if (MODE == OUT_POOL) *tile_ptr(cx.obuf, cx.oplane, srow, co >> 3) = val;
-                    else if (co < L.cout) *reinterpret_cast<uint4*>(p.out + gpix * L.cout + co) = val;
+                    if (MODE == OUT_POOL) *tile_ptr(cx.obuf, cx.oplane, lr.srow, co >> 3) = val;
+                    else if (co < L.cout) *reinterpret_cast<uint4*>(p.out + lr.gpix * L.cout + co) = val;
                 }
             }
         }
+        if (b + 1 < cx.nblk) lr = last_row<MODE>(p, L, cx, b + 1);
     }
 }
 
+// The UMMAs of one kernel row (1x1: of the only tap) and 64-channel chunk, for every block of a pass: up to four K = 16 steps
+// per tap.  Called by one elected lane.  Statements of a single UMMA cost this lane about 200 clocks each, UMMAs that share a
+// statement 66 and less (see umma_f16_row3): taps with fewer than four steps join the row's statement.  Measured as one kernel:
+// two 16 -> 16 3x3 layers on a 32x32 image 8.7 -> 7.2 us, eight 32 -> 32 ones on 16 images of 60x60 412 -> 328.
+template <int K, int KS>
+__device__ __forceinline__ void issue_row(uint32_t d, uint32_t slot_cols, int nblk, uint32_t a, uint32_t b, uint32_t w_tap16, uint32_t idesc, uint32_t acc) {
+#pragma unroll 1
+    for (int blk = 0; blk < nblk; blk++, a += (128 * 128) >> 4, d += slot_cols) {
+        if (K == 3 && KS == 4) {
+#pragma unroll
+            for (uint32_t sx = 0; sx < 3; sx++) umma_f16_x4(d, a + sx * 8u, b + sx * w_tap16, idesc, acc | sx);
+        } else if (K == 3) {
+            umma_f16_row3<KS>(d, a, b, w_tap16, idesc, acc);
+        } else {
+            umma_f16_steps<KS>(d, a, b, idesc, acc);
+        }
+    }
+}
+template <int K>
+__device__ __forceinline__ void issue_row_ks(int ks, uint32_t d, uint32_t slot_cols, int nblk, uint32_t a, uint32_t b, uint32_t w_tap16, uint32_t idesc, uint32_t acc) {
+    if (ks == 4) issue_row<K, 4>(d, slot_cols, nblk, a, b, w_tap16, idesc, acc);
+    else if (ks == 3) issue_row<K, 3>(d, slot_cols, nblk, a, b, w_tap16, idesc, acc);
+    else if (ks == 2) issue_row<K, 2>(d, slot_cols, nblk, a, b, w_tap16, idesc, acc);
+    else issue_row<K, 1>(d, slot_cols, nblk, a, b, w_tap16, idesc, acc);
+}
+
 // The UMMAs of one pass whose operands are all in shared memory already (resident weights; an operand tile of the group,
-// or a resident input frame): for every 64-channel chunk, every tap, every block of the pass, four K = 16 steps.  The
-// issuing warp is bound by its own instruction stream (measured: about 4 cycles per instruction, and a pass of 36 UMMAs
-// cost it 3000 instructions in the general loop below), so this path is kept to a few instructions per UMMA: 32-bit
-// descriptor words, the tap loop unrolled at compile time, nothing but adds inside.
+// or a resident input frame): for every 64-channel chunk, every kernel row, every block of the pass, the row's taps of up to
+// four K = 16 steps.  Called by one elected lane.
 //   a16 / b16: low descriptor words of tap (0, 0), chunk 0, block 0 / of the first weight slab
 template <int K>
 __device__ __forceinline__ void issue_pass_resident(uint32_t d0, uint32_t slot_cols, int nblk, uint32_t a16, uint32_t a_chunk16, uint32_t b16,
                                                     uint32_t w_tap16, uint32_t idesc, int kchunks, int ksteps_last, int pitch) {
 #pragma unroll 1
     for (int kc = 0; kc < kchunks; kc++, a16 += a_chunk16) {
-        const bool whole = kc + 1 < kchunks || ksteps_last == 4;
-#pragma unroll
-        for (int r = 0; r < K; r++) {
-#pragma unroll
-            for (int sx = 0; sx < K; sx++) {
-                uint32_t a = a16 + static_cast<uint32_t>((r * pitch + sx) * 8), d = d0;
-                const uint32_t acc = (kc | r | sx) != 0;
+        const int ks = kc + 1 < kchunks ? 4 : ksteps_last;
+        uint32_t a = a16;
 #pragma unroll 1
-                for (int blk = 0; blk < nblk; blk++, a += (128 * 128) >> 4, d += slot_cols) {
-                    if (elect_one()) {
-                        if (whole) {
-                            umma_f16_x4(d, a, b16, idesc, acc);
-                        } else {
-                            umma_f16_lo(d, a, kDescHiSw128, b16, idesc, acc);
-                            if (ksteps_last > 1) umma_f16_lo(d, a + 2, kDescHiSw128, b16 + 2, idesc, 1);
-                            if (ksteps_last > 2) umma_f16_lo(d, a + 4, kDescHiSw128, b16 + 4, idesc, 1);
-                        }
-                    }
-                }
-                b16 += w_tap16;
-            }
-        }
+        for (int r = 0; r < K; r++, a += static_cast<uint32_t>(pitch * 8), b16 += w_tap16 * K)
+            issue_row_ks<K>(ks, d0, slot_cols, nblk, a, b16, w_tap16, idesc, (kc | r) != 0);
     }
 }
 
@@ -308,42 +345,42 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int* abort_flag = &abort_s;
     const int nl = p.n_layers;
+    // Set-up, spread over the warps (a kernel of one short tile lives for 5 us; one thread initialising all barriers took 0.7 of
+    // them, a warp copying the table word by word 0.4): warp 0 initialises the barriers, two or three per lane, warp 1
+    // prefetches the tensor maps, and the table's words are dealt out warp by warp (lanes that read different words of the
+    // parameter block are served one after the other).
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.L[0]);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&Ls[0]);
         const int words = nl * static_cast<int>(sizeof(ChainLayerP) / 4);
 #pragma unroll 1
-        for (int i = threadIdx.x; i < words; i += kThreads) dst[i] = src[i];
+        for (int i = lane * (kThreads / 32) + warp; i < words; i += kThreads) dst[i] = src[i];
     }
     const ChainLayerP& LL = Ls[nl - 1];
 
-    if (threadIdx.x == 0) {
-        DLF_TRACE_POINT(p.status, 24);
-        abort_s = 0;
-#pragma unroll 1
-        for (int i = 0; i < p.stages; i++) {
-            mbar_init(&wfull_bar[i], 1);
-            mbar_init(&wempty_bar[i], 1);
+    if (warp == 0) {
+        if (lane == 0) {
+            DLF_TRACE_POINT(p.status, 24);
+            abort_s = 0;
         }
-#pragma unroll 1
-        for (int i = 0; i < p.in_slots; i++) {
-            mbar_init(&in_full_bar[i], 1);
-            mbar_init(&in_empty_bar[i], 1);
+        if (lane < kMaxStages) {
+            mbar_init(&wfull_bar[lane], 1);
+            mbar_init(&wempty_bar[lane], 1);
+        } else if (lane < kMaxStages + kMaxInSlots) {
+            mbar_init(&in_full_bar[lane - kMaxStages], 1);
+            mbar_init(&in_empty_bar[lane - kMaxStages], 1);
+        } else if (lane < kMaxStages + kMaxInSlots + 4) {
+            mbar_init(&acc_full_bar[lane & 3], 1);
+            mbar_init(&acc_empty_bar[lane & 3], kEpiWarps);
+        } else if (lane < kMaxStages + kMaxInSlots + 6) {
+            mbar_init(&stg_full_bar[lane & 1], kEpiWarps);
+            mbar_init(&stg_free_bar[lane & 1], 1);
+        } else if (lane == 31) {
+            mbar_init(&act_ready_bar, kEpiWarps);
         }
-#pragma unroll 1
-        for (int i = 0; i < 4; i++) {
-            mbar_init(&acc_full_bar[i], 1);
-            mbar_init(&acc_empty_bar[i], kEpiWarps);
-        }
-        mbar_init(&act_ready_bar, kEpiWarps);
-#pragma unroll 1
-        for (int i = 0; i < kMaxChain; i++) mbar_init(&wres_bar[i], kWeightWarps);
-#pragma unroll 1
-        for (int i = 0; i < 2; i++) {
-            mbar_init(&stg_full_bar[i], kEpiWarps);
-            mbar_init(&stg_free_bar[i], 1);
-        }
+        if (lane < kMaxChain) mbar_init(&wres_bar[lane], kWeightWarps);
         fence_barrier_init();
+    } else if (warp == 1 && lane == 0) {
         tma_prefetch_desc(&p.tmx);
         if (OUT_MODE == OUT_STAGE) {
             tma_prefetch_desc(&p.tmy);
@@ -354,6 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         tmem_alloc(&tmem_base_s, 512);
         tmem_relinquish();
     }
+    const TilePos tile0 = tile_pos(p, blockIdx.x);   // this CTA's first tile (divided out while the set-up runs)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -365,6 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     // address a compile-time-uniform value (an address loaded from shared memory is a per-thread value to the compiler
     // and costs a move into a uniform register at every UMMA).  Checked once; a surprise is reported, not ignored.
     constexpr uint32_t tmem_base = 0;
+    static_assert(kMaxStages + kMaxInSlots + 6 <= 31 && kMaxChain <= 32, "warp 0 initialises the barriers");
     if (threadIdx.x == 0 && tmem_base_s != 0u) {
         abort_s = 1;
         atomicCAS(p.status, 0, 0xb00 | (blockIdx.x << 12));
@@ -381,9 +420,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
             int rd = 0;           // round within the slots
             uint32_t ph = 0;      // phase of the slots' barriers
             bool ok = true;
+            TilePos tp = tile0;
 #pragma unroll 1
-            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
-                const int txi = t % p.tiles_w, tyi = (t / p.tiles_w) % p.tiles_h, n = t / (p.tiles_w * p.tiles_h);
+            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x, tp = tile_pos(p, t)) {
                 int plane = lane;
 #pragma unroll 1
                 for (int rr = 0; rr < rounds_per_tile; rr++) {
@@ -392,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                     if (!ok) break;
                     mbar_expect_tx(&in_full_bar[slot], plane_bytes);
                     tma_load_4d(sbase + p.in_off + static_cast<size_t>(slot) * p.in_slot_bytes, &p.tmx, &in_full_bar[slot], plane * 64,
-                                txi * p.tw - p.halo, tyi * p.th - p.halo, n);
+                                tp.x * p.tw - p.halo, tp.y * p.th - p.halo, tp.n);
                     plane += p.in_group;
                     if (plane >= p.in_planes) plane = lane;
                     if (++rd == ring_rounds) { rd = 0; ph ^= 1u; }
@@ -409,11 +448,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                 const ChainLayerP& L = Ls[l];
                 const int taps = L.k * L.k, tg = L.tg, kg = L.kg, kchunks = L.kchunks, rank4 = L.w_rank4;
                 const uint32_t bytes = static_cast<uint32_t>(tg * kg * L.chunk_n) * 128u;
-                const int n_boxes = L.n_chunks * (taps / tg) * (kchunks / kg);
+                const int n_boxes = L.n_boxes;
                 mbar_expect_tx(&wres_bar[l], static_cast<uint32_t>((n_boxes - role + kWeightWarps - 1) / kWeightWarps) * bytes);
                 // Every CTA wants the same slabs at the same moment: each starts its round at another box, so that the
                 // requests of the 148 CTAs spread over the L2 slices instead of queueing on the same lines.
-                const int first = (static_cast<int>(blockIdx.x) * kWeightWarps) % n_boxes;
+                const int first = ((static_cast<int>(blockIdx.x) & 31) * n_boxes) >> 5;
                 int turn = 0, box = 0;
 #pragma unroll 1
                 for (int c = 0; c < L.n_chunks; c++)
@@ -494,12 +533,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
             for (int l = 0; l < nl && ok; l++) {
                 const ChainLayerP& L = Ls[l];
                 const int region = (l == nl - 1) ? 1 : 0;
-                if (l > 0) {  // group A has written all of the previous layer's tile
-                    ok = mbar_wait_warp<true>(&act_ready_bar, act_ph, abort_flag, p.status, 0x400 | (blockIdx.x << 12));
-                    if (!ok) break;
-                    act_ph ^= 1u;
-                    DLF_TRACE_ACC(tacc, 1, tmark);
-                }
                 const uint32_t abuf = l == 0 ? 0u : base + p.act_off[(l - 1) & 1];
                 const uint32_t aplane_bytes = l == 0 ? 0u : static_cast<uint32_t>(p.act_plane_bytes[(l - 1) & 1]);
                 const int k = L.k, pad = L.pad, taps = k * k, tg = L.tg, kg = L.kg, kchunks = L.kchunks, ksteps_last = L.ksteps_last;
@@ -507,6 +540,12 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                 const uint32_t slot_cols = L.slot, col0 = L.col0, half_cols = L.half_cols, qs = L.qs;
                 const uint32_t w_tap16 = static_cast<uint32_t>(L.chunk_n) * 8u;  // one tap's [chunk_n][64] slab, 16-byte units
                 const bool w_res = stages == 0;
+                if (l > 0) {  // group A has written all of the previous layer's tile (waited for with the layer's parameters in registers)
+                    ok = mbar_wait_warp<true>(&act_ready_bar, act_ph, abort_flag, p.status, 0x400 | (blockIdx.x << 12));
+                    if (!ok) break;
+                    act_ph ^= 1u;
+                    DLF_TRACE_ACC(tacc, 1, tmark);
+                }
                 if (w_res) {   // this layer's resident weights have landed (true at once from the second tile on)
                     ok = mbar_wait_warp<true>(&wres_bar[l], 0u, abort_flag, p.status, 0x600 | (blockIdx.x << 12));
                     if (!ok) break;
@@ -544,8 +583,11 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                             const uint32_t a_chunk16 = (l == 0 ? in_slot_bytes : aplane_bytes) >> 4;
                             const uint32_t a16 = umma_desc_lo(a_base + row0) - static_cast<uint32_t>(pad * (pitch + 1) * 8);
                             const uint32_t b16 = umma_desc_lo(w_res0) + static_cast<uint32_t>(c * kchunks * taps) * w_tap16;
-                            if (k == 3) issue_pass_resident<3>(d_tmem0, slot_cols, nblk, a16, a_chunk16, b16, w_tap16, idesc, kchunks, ksteps_last, pitch);
-                            else issue_pass_resident<1>(d_tmem0, slot_cols, nblk, a16, a_chunk16, b16, w_tap16, idesc, kchunks, ksteps_last, pitch);
+                            if (elect_one()) {
+                                if (k == 3) issue_pass_resident<3>(d_tmem0, slot_cols, nblk, a16, a_chunk16, b16, w_tap16, idesc, kchunks, ksteps_last, pitch);
+                                else issue_pass_resident<1>(d_tmem0, slot_cols, nblk, a16, a_chunk16, b16, w_tap16, idesc, kchunks, ksteps_last, pitch);
+                            }
+                            __syncwarp();
                             DLF_TRACE_ACC(tacc, 4, tmark);
                             if (elect_one()) umma_commit(&acc_full_bar[region * 2 + half]);
                             __syncwarp();
@@ -561,19 +603,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                                 ok = mbar_wait_warp<true>(&in_full_bar[in_slot], in_ph, abort_flag, p.status, 0x300 | (blockIdx.x << 12));
                                 if (!ok) break;
                                 uint32_t a = umma_desc_lo(in_base + static_cast<uint32_t>(in_slot) * in_slot_bytes + row0), d = d_tmem0;
-                                const bool whole = kc + 1 < kchunks || ksteps_last == 4;
-#pragma unroll 1
-                                for (int blk = 0; blk < nblk; blk++, a += (128 * 128) >> 4, d += slot_cols) {
-                                    if (elect_one()) {
-                                        if (whole) {
-                                            umma_f16_x4(d, a, b16, idesc, kc != 0);
-                                        } else {
-                                            umma_f16_lo(d, a, kDescHiSw128, b16, idesc, kc != 0);
-                                            if (ksteps_last > 1) umma_f16_lo(d, a + 2, kDescHiSw128, b16 + 2, idesc, 1);
-                                            if (ksteps_last > 2) umma_f16_lo(d, a + 4, kDescHiSw128, b16 + 4, idesc, 1);
-                                        }
-                                    }
-                                }
+                                if (elect_one()) issue_row_ks<1>(kc + 1 < kchunks ? 4 : ksteps_last, d, slot_cols, nblk, a, b16, 0u, idesc, kc != 0);
+                                __syncwarp();
                                 if (elect_one()) umma_commit(&in_empty_bar[in_slot]);   // the plane is free once these have read it
                                 if (++in_j == in_group) { in_j = 0; if (++in_rd == ring_rounds) { in_rd = 0; in_ph ^= 1u; } }
                             }
@@ -610,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
 #pragma unroll 1
                                     for (int g = 0; g < g_end && ok; g++) {
                                         const int kc = g0 + g;
-                                        const bool whole = kc + 1 < kchunks || ksteps_last == 4;
+                                        const int ks = kc + 1 < kchunks ? 4 : ksteps_last;
                                         uint32_t a_kc;
                                         int in_slot = 0;
                                         if (a_ring) {
@@ -621,28 +652,19 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                                         } else {
                                             a_kc = a16 + static_cast<uint32_t>(kc) * a_chunk16;
                                         }
-                                        uint32_t shift16 = static_cast<uint32_t>((r0 * pitch + sx0) * 8);
-                                        int sx = sx0;
-                                        uint32_t acc = (r0 | sx0 | kc) != 0;
+                                        const uint32_t a = a_kc + static_cast<uint32_t>((r0 * pitch + sx0) * 8), acc = (r0 | sx0 | kc) != 0;
+                                        if (elect_one()) {
+                                            if (k == 3 && tg >= 3) {   // whole kernel rows (boxes of 3 or 9 taps)
 #pragma unroll 1
-                                        for (int tt = 0; tt < tg; tt++, b16 += w_tap16) {
-                                            uint32_t a = a_kc + shift16, d = d_tmem0;
-#pragma unroll 1
-                                            for (int blk = 0; blk < nblk; blk++, a += (128 * 128) >> 4, d += slot_cols) {
-                                                if (elect_one()) {
-                                                    if (whole) {
-                                                        umma_f16_x4(d, a, b16, idesc, acc);
-                                                    } else {
-                                                        umma_f16_lo(d, a, kDescHiSw128, b16, idesc, acc);
-                                                        if (ksteps_last > 1) umma_f16_lo(d, a + 2, kDescHiSw128, b16 + 2, idesc, 1);
-                                                        if (ksteps_last > 2) umma_f16_lo(d, a + 4, kDescHiSw128, b16 + 4, idesc, 1);
-                                                    }
-                                                }
+                                                for (int tt = 0; tt < tg; tt += 3)
+                                                    issue_row_ks<3>(ks, d_tmem0, slot_cols, nblk, a + static_cast<uint32_t>(tt / 3 * pitch * 8),
+                                                                    b16 + tt * w_tap16, w_tap16, idesc, acc | (tt != 0));
+                                            } else {                   // one tap
+                                                issue_row_ks<1>(ks, d_tmem0, slot_cols, nblk, a, b16, 0u, idesc, acc);
                                             }
-                                            acc = 1;
-                                            shift16 += 8;
-                                            if (++sx == k) { sx = 0; shift16 += static_cast<uint32_t>((pitch - k) * 8); }
                                         }
+                                        __syncwarp();
+                                        b16 += tg * w_tap16;
                                         if (a_ring) {   // the plane is free once these have read it
                                             if (elect_one()) umma_commit(&in_empty_bar[in_slot]);
                                             if (++in_j == in_group) { in_j = 0; if (++in_rd == ring_rounds) { in_rd = 0; in_ph ^= 1u; } }
@@ -695,10 +717,10 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         DLF_TRACE_DECL(aacc, amark);  // cycles of CTA 0's first group-A thread: 0 accumulator wait, 1 drain, 2 fences and arrivals
 #pragma unroll 1
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
-            const int txi = t % p.tiles_w, tyi = (t / p.tiles_w) % p.tiles_h;
-            cx.gy0 = tyi * p.th;
-            cx.gx0 = txi * p.tw;
-            cx.n = t / (p.tiles_w * p.tiles_h);
+            const TilePos tp = t == static_cast<int>(blockIdx.x) ? tile0 : tile_pos(p, t);
+            cx.gy0 = tp.y * p.th;
+            cx.gx0 = tp.x * p.tw;
+            cx.n = tp.n;
 #pragma unroll 1
             for (int l = 0; l < nl - 1 && ok; l++) {
                 const ChainLayerP& L = Ls[l];
@@ -714,14 +736,15 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
 #pragma unroll 1
                     for (int b0 = 0; b0 < L.nb && ok; b0 += L.per_pass, pass_i++) {
                         const uint32_t half = pass_i & 1u;
+                        cx.b0 = b0;
+                        cx.nblk = min(L.per_pass, L.nb - b0);
+                        cx.tmem_col = L.col0 + half * L.half_cols;
+                        const InnerRow ir = inner_row(p, L, cx, 0);
                         ok = mbar_wait<true>(&acc_full_bar[half], (pass_i >> 1) & 1u, abort_flag, p.status, 0x700 | (blockIdx.x << 12));
                         if (!ok) break;
                         DLF_TRACE_ACC(aacc, 0, amark);
                         tc_fence_after_sync();
-                        cx.b0 = b0;
-                        cx.nblk = min(L.per_pass, L.nb - b0);
-                        cx.tmem_col = L.col0 + half * L.half_cols;
-                        epi_inner(p, L, cx);
+                        epi_inner(p, L, cx, ir);
                         DLF_TRACE_ACC(aacc, 1, amark);
                         fence_proxy_async_smem();  // UMMA reads these rows through the async proxy
                         tc_fence_before_sync();
@@ -754,7 +777,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         DLF_TRACE_DECL(eacc, emark);  // cycles of CTA 0's first group-B thread: 0 staging wait, 1 accumulator wait, 2 drain, 3 pooled copy-out
 #pragma unroll 1
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
-            const int txi = t % p.tiles_w, tyi = (t / p.tiles_w) % p.tiles_h, n = t / (p.tiles_w * p.tiles_h);
+            const TilePos tp = t == static_cast<int>(blockIdx.x) ? tile0 : tile_pos(p, t);
+            const int txi = tp.x, tyi = tp.y, n = tp.n;
             cx.gy0 = tyi * p.th;
             cx.gx0 = txi * p.tw;
             cx.n = n;
@@ -778,14 +802,15 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
 #pragma unroll 1
                 for (int b0 = 0; b0 < LL.nb && ok; b0 += LL.per_pass, pass_i++) {
                     const uint32_t half = pass_i & 1u;
+                    cx.b0 = b0;
+                    cx.nblk = min(LL.per_pass, LL.nb - b0);
+                    cx.tmem_col = LL.col0 + half * LL.half_cols;
+                    const LastRow lr = last_row<OUT_MODE>(p, LL, cx, 0);
                     ok = mbar_wait(&acc_full_bar[2 + half], (pass_i >> 1) & 1u, abort_flag, p.status, 0x900 | (blockIdx.x << 12));
                     if (!ok) break;
                     DLF_TRACE_ACC(eacc, 1, emark);
                     tc_fence_after_sync();
-                    cx.b0 = b0;
-                    cx.nblk = min(LL.per_pass, LL.nb - b0);
-                    cx.tmem_col = LL.col0 + half * LL.half_cols;
-                    epi_last<OUT_MODE>(p, LL, cx);
+                    epi_last<OUT_MODE>(p, LL, cx, lr);
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty_bar[2 + half]);
@@ -842,60 +867,60 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
             const bool has_res = p.res != nullptr;
             const int n_chunks = LL.n_chunks;
             // boxes of chunk c of tile t: planes x (1 box for a dense tile | one per tile row inside the image)
-            auto boxes_of = [&](int t, int c, int* rows_in) {
-                const int tyi = (t / p.tiles_w) % p.tiles_h;
+            auto boxes_of = [&](const TilePos& tp, int c, int* rows_in) {
                 const int planes = (chunk_cols(LL, c) + 63) >> 6;
-                *rows_in = p.out_dense ? 1 : min(p.th, p.H - tyi * p.th);
+                *rows_in = p.out_dense ? 1 : min(p.th, p.H - tp.y * p.th);
                 return planes * *rows_in;
             };
-            auto box_args = [&](int t, int c, int it, int rows_in, uint32_t sb, uint8_t** smem, int* c0, int* c1, int* c2, int* c3) {
-                const int txi = t % p.tiles_w, tyi = (t / p.tiles_w) % p.tiles_h, n = t / (p.tiles_w * p.tiles_h);
-                const int pl = it / rows_in, ty = it - pl * rows_in;
+            auto box_args = [&](const TilePos& tp, int c, int it, int rows_in, uint32_t sb, uint8_t** smem, int* c0, int* c1, int* c2, int* c3) {
+                const int pl = it < rows_in ? 0 : it / rows_in, ty = it - pl * rows_in;
                 const int srow = p.out_dense ? 0 : out_row(p, ty, 0) - p.stg_base8;
                 *smem = sbase + p.stg_off + sb * p.stg_buf_bytes + static_cast<size_t>(pl) * p.stg_plane_bytes + static_cast<size_t>(srow) * 128;
                 *c0 = c * LL.chunk_n + pl * 64;
-                *c1 = txi * p.tw;
-                *c2 = tyi * p.th + ty;
-                *c3 = n;
+                *c1 = tp.x * p.tw;
+                *c2 = tp.y * p.th + ty;
+                *c3 = tp.n;
             };
             auto fetch_residual = [&](uint32_t u) {   // the u-th (tile, chunk) of this CTA
                 const int t = blockIdx.x + static_cast<int>(u / n_chunks) * gridDim.x, c = static_cast<int>(u % n_chunks);
                 if (t >= p.n_tiles) return;
                 const uint32_t sb = u % p.stg_bufs;
+                const TilePos tp = tile_pos(p, t);
                 int rows_in;
-                const int boxes = boxes_of(t, c, &rows_in);
+                const int boxes = boxes_of(tp, c, &rows_in);
                 if (lane == 0) mbar_expect_tx(&stg_free_bar[sb], static_cast<uint32_t>(boxes) * p.tw * p.out_box_rows * 128u);
                 __syncwarp();
 #pragma unroll 1
                 for (int it = lane; it < boxes; it += 32) {
                     uint8_t* sm;
                     int c0, c1, c2, c3;
-                    box_args(t, c, it, rows_in, sb, &sm, &c0, &c1, &c2, &c3);
+                    box_args(tp, c, it, rows_in, sb, &sm, &c0, &c1, &c2, &c3);
                     tma_load_4d(sm, &p.tmr, &stg_free_bar[sb], c0, c1, c2, c3);
                 }
             };
             if (has_res)
 #pragma unroll 1
                 for (int u = 0; u < p.stg_bufs; u++) fetch_residual(u);
-            uint32_t u = 0;
+            uint32_t u = 0, sb = 0, ph = 0;   // staged chunk, its buffer and the buffer's phase
             bool ok = true;
+            TilePos tp = tile0;
 #pragma unroll 1
-            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
+            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x, tp = tile_pos(p, t)) {
 #pragma unroll 1
                 for (int c = 0; c < n_chunks && ok; c++, u++) {
-                    const uint32_t sb = u % p.stg_bufs, ph = (u / p.stg_bufs) & 1u;
+                    int rows_in;
+                    const int boxes = boxes_of(tp, c, &rows_in);
+                    bool mine = lane < boxes;
+                    uint8_t* sm;
+                    int c0, c1, c2, c3;
+                    box_args(tp, c, lane, rows_in, sb, &sm, &c0, &c1, &c2, &c3);   // (worked out before the wait)
                     ok = mbar_wait_warp(&stg_full_bar[sb], ph, abort_flag, p.status, 0xa00 | (blockIdx.x << 12));
                     if (!ok) break;
-                    int rows_in;
-                    const int boxes = boxes_of(t, c, &rows_in);
-                    bool mine = false;
+                    if (mine) tma_store_4d(&p.tmy, sm, c0, c1, c2, c3);
 #pragma unroll 1
-                    for (int it = lane; it < boxes; it += 32) {
-                        uint8_t* sm;
-                        int c0, c1, c2, c3;
-                        box_args(t, c, it, rows_in, sb, &sm, &c0, &c1, &c2, &c3);
+                    for (int it = lane + 32; it < boxes; it += 32) {
+                        box_args(tp, c, it, rows_in, sb, &sm, &c0, &c1, &c2, &c3);
                         tma_store_4d(&p.tmy, sm, c0, c1, c2, c3);
-                        mine = true;
                     }
                     if (mine) {
                         tma_store_commit();
@@ -904,6 +929,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                     __syncwarp();
                     if (has_res) fetch_residual(u + p.stg_bufs);
                     else if (lane == 0) mbar_arrive(&stg_free_bar[sb]);
+                    if (++sb == static_cast<uint32_t>(p.stg_bufs)) { sb = 0; ph ^= 1u; }
                 }
             }
             tma_store_wait_all();
@@ -1237,6 +1263,7 @@ int launch_chain_tc(const ChainArgs& a, const ChainTiling& t, int sm_count, int*
     p.n_layers = nl;
     p.N = a.N; p.H = a.H; p.W = a.W;
     p.th = t.th; p.tw = t.tw; p.halo = y.halo; p.pitch = y.pitch; p.rows = y.rows;
+    p.pitch_magic = ((1u << 20) + p.pitch - 1) / p.pitch; p.tw_magic = ((1u << 20) + p.tw - 1) / p.tw;
     p.tiles_h = t.tiles_h; p.tiles_w = t.tiles_w; p.n_tiles = t.n_tiles;
     p.in_planes = y.in_planes; p.in_group = t.in_group; p.in_slots = t.in_slots; p.in_ring = t.in_ring;
     p.in_slot_bytes = y.in_slot_bytes; p.in_off = y.in_off;
@@ -1260,6 +1287,7 @@ int launch_chain_tc(const ChainArgs& a, const ChainTiling& t, int sm_count, int*
         L.bias_off = boff;
         boff += g.n_pad;
         L.bias = a.bias[l];
+        L.n_boxes = g.n_chunks * (L.k * L.k / g.wb.tg) * (planes_of(L.cin) / g.wb.kg);
         L.tg = g.wb.tg; L.kg = g.wb.kg; L.w_rank4 = g.wb.rank4; L.w_off = g.w_off;
         const uint64_t taps = static_cast<uint64_t>(a.k[l]) * a.k[l];
         const uint32_t box_n = static_cast<uint32_t>(std::min(g.chunk_n, g.n_pad));
