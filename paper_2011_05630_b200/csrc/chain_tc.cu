@@ -330,9 +330,19 @@ __device__ __forceinline__ void issue_pass_resident(uint32_t d0, uint32_t slot_c
 template <int OUT_MODE>
 __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_constant__ ChainParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t wfull_bar[kMaxStages], wempty_bar[kMaxStages], in_full_bar[kMaxInSlots], in_empty_bar[kMaxInSlots];
-    __shared__ uint64_t acc_full_bar[4], acc_empty_bar[4];  // [region * 2 + half]; region 0 = inner layers, 1 = last layer
-    __shared__ uint64_t act_ready_bar, stg_full_bar[2], stg_free_bar[2], wres_bar[kMaxChain];
+    // the barriers in one array, so that a thread each initialises them: arrival count 1, kEpiWarps, kWeightWarps in this order
+    constexpr int kBars1 = 2 * kMaxStages + 2 * kMaxInSlots + 6, kBarsEpi = 7, kBars = kBars1 + kBarsEpi + kMaxChain;
+    __shared__ uint64_t bars[kBars];
+    uint64_t* const wfull_bar = bars;
+    uint64_t* const wempty_bar = wfull_bar + kMaxStages;
+    uint64_t* const in_full_bar = wempty_bar + kMaxStages;
+    uint64_t* const in_empty_bar = in_full_bar + kMaxInSlots;
+    uint64_t* const acc_full_bar = in_empty_bar + kMaxInSlots;   // [region * 2 + half]; region 0 = inner layers, 1 = last layer
+    uint64_t* const stg_free_bar = acc_full_bar + 4;
+    uint64_t* const acc_empty_bar = bars + kBars1;
+    uint64_t* const stg_full_bar = acc_empty_bar + 4;
+    uint64_t& act_ready_bar = stg_full_bar[2];
+    uint64_t* const wres_bar = bars + kBars1 + kBarsEpi;
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
     // The layers' parameters, copied out of the kernel's parameter block: every role walks the layers of every tile, and
@@ -346,9 +356,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     volatile int* abort_flag = &abort_s;
     const int nl = p.n_layers;
     // Set-up, spread over the warps (a kernel of one short tile lives for 5 us; one thread initialising all barriers took 0.7 of
-    // them, a warp copying the table word by word 0.4): warp 0 initialises the barriers, two or three per lane, warp 1
-    // prefetches the tensor maps, and the table's words are dealt out warp by warp (lanes that read different words of the
-    // parameter block are served one after the other).
+    // them, a warp copying the table word by word 0.4): a thread per barrier, and the table's words are dealt out warp by warp
+    // (lanes that read different words of the parameter block are served one after the other).
     {
         const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.L[0]);
         uint32_t* dst = reinterpret_cast<uint32_t*>(&Ls[0]);
@@ -358,29 +367,15 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     }
     const ChainLayerP& LL = Ls[nl - 1];
 
-    if (warp == 0) {
-        if (lane == 0) {
+    if (threadIdx.x < kBars) {
+        if (threadIdx.x == 0) {
             DLF_TRACE_POINT(p.status, 24);
             abort_s = 0;
         }
-        if (lane < kMaxStages) {
-            mbar_init(&wfull_bar[lane], 1);
-            mbar_init(&wempty_bar[lane], 1);
-        } else if (lane < kMaxStages + kMaxInSlots) {
-            mbar_init(&in_full_bar[lane - kMaxStages], 1);
-            mbar_init(&in_empty_bar[lane - kMaxStages], 1);
-        } else if (lane < kMaxStages + kMaxInSlots + 4) {
-            mbar_init(&acc_full_bar[lane & 3], 1);
-            mbar_init(&acc_empty_bar[lane & 3], kEpiWarps);
-        } else if (lane < kMaxStages + kMaxInSlots + 6) {
-            mbar_init(&stg_full_bar[lane & 1], kEpiWarps);
-            mbar_init(&stg_free_bar[lane & 1], 1);
-        } else if (lane == 31) {
-            mbar_init(&act_ready_bar, kEpiWarps);
-        }
-        if (lane < kMaxChain) mbar_init(&wres_bar[lane], kWeightWarps);
+        const int i = threadIdx.x;
+        mbar_init(&bars[i], i < kBars1 ? 1 : (i < kBars1 + kBarsEpi ? kEpiWarps : kWeightWarps));
         fence_barrier_init();
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == kStoreWarp && lane == 0) {
         tma_prefetch_desc(&p.tmx);
         if (OUT_MODE == OUT_STAGE) {
             tma_prefetch_desc(&p.tmy);
@@ -391,7 +386,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         tmem_alloc(&tmem_base_s, 512);
         tmem_relinquish();
     }
-    const TilePos tile0 = tile_pos(p, blockIdx.x);   // this CTA's first tile (divided out while the set-up runs)
+    TilePos tile0{};   // this CTA's first tile; the input producer's first copy waits for it
+    if (warp == kInputWarp) tile0 = tile_pos(p, blockIdx.x);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -403,7 +399,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
     // address a compile-time-uniform value (an address loaded from shared memory is a per-thread value to the compiler
     // and costs a move into a uniform register at every UMMA).  Checked once; a surprise is reported, not ignored.
     constexpr uint32_t tmem_base = 0;
-    static_assert(kMaxStages + kMaxInSlots + 6 <= 31 && kMaxChain <= 32, "warp 0 initialises the barriers");
     if (threadIdx.x == 0 && tmem_base_s != 0u) {
         abort_s = 1;
         atomicCAS(p.status, 0, 0xb00 | (blockIdx.x << 12));
@@ -717,7 +712,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         DLF_TRACE_DECL(aacc, amark);  // cycles of CTA 0's first group-A thread: 0 accumulator wait, 1 drain, 2 fences and arrivals
 #pragma unroll 1
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
-            const TilePos tp = t == static_cast<int>(blockIdx.x) ? tile0 : tile_pos(p, t);
+            const TilePos tp = tile_pos(p, t);
             cx.gy0 = tp.y * p.th;
             cx.gx0 = tp.x * p.tw;
             cx.n = tp.n;
@@ -777,7 +772,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         DLF_TRACE_DECL(eacc, emark);  // cycles of CTA 0's first group-B thread: 0 staging wait, 1 accumulator wait, 2 drain, 3 pooled copy-out
 #pragma unroll 1
         for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
-            const TilePos tp = t == static_cast<int>(blockIdx.x) ? tile0 : tile_pos(p, t);
+            const TilePos tp = tile_pos(p, t);
             const int txi = tp.x, tyi = tp.y, n = tp.n;
             cx.gy0 = tyi * p.th;
             cx.gx0 = txi * p.tw;
@@ -903,9 +898,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                 for (int u = 0; u < p.stg_bufs; u++) fetch_residual(u);
             uint32_t u = 0, sb = 0, ph = 0;   // staged chunk, its buffer and the buffer's phase
             bool ok = true;
-            TilePos tp = tile0;
 #pragma unroll 1
-            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x, tp = tile_pos(p, t)) {
+            for (int t = blockIdx.x; t < p.n_tiles && ok; t += gridDim.x) {
+                const TilePos tp = tile_pos(p, t);
 #pragma unroll 1
                 for (int c = 0; c < n_chunks && ok; c++, u++) {
                     int rows_in;
