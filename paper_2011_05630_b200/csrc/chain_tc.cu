@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         // Ring positions and phases are kept as counters: a division by a run-time value costs this single warp about a
         // hundred cycles, and the loop around a weight box issues as few as four instructions.
         const uint64_t desc0 = umma_desc_sw128(0);
-        uint32_t pass_ctr[2] = {0, 0}, act_ph = 0, w_ph = 0, in_ph = 0;
+        uint32_t pass_inner = 0, pass_last = 0, act_ph = 0, w_ph = 0, in_ph = 0;   // (an array of the two would live in memory)
         int w_st = 0, in_rd = 0, in_j = 0;   // weight stage; input round within the slots and (streamed planes) plane within the round
         const int in_group = p.in_group, in_ring = p.in_ring, pitch = p.pitch, stages = p.stages;
         const uint32_t in_base = base + p.in_off, in_slot_bytes = p.in_slot_bytes;
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
 #pragma unroll 1
             for (int l = 0; l < nl && ok; l++) {
                 const ChainLayerP& L = Ls[l];
-                const int region = (l == nl - 1) ? 1 : 0;
+                const uint32_t region = (l == nl - 1) ? 1u : 0u;
                 const uint32_t abuf = l == 0 ? 0u : base + p.act_off[(l - 1) & 1];
                 const uint32_t aplane_bytes = l == 0 ? 0u : static_cast<uint32_t>(p.act_plane_bytes[(l - 1) & 1]);
                 const int k = L.k, pad = L.pad, taps = k * k, tg = L.tg, kg = L.kg, kchunks = L.kchunks, ksteps_last = L.ksteps_last;
@@ -555,7 +555,9 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
 #pragma unroll 1
                     for (int b0 = 0; b0 < nb && ok; b0 += per_pass) {
                         const int nblk = min(per_pass, nb - b0);
-                        const uint32_t pc = pass_ctr[region]++;
+                        const uint32_t pc = region ? pass_last : pass_inner;
+                        pass_last += region;
+                        pass_inner += 1u - region;
                         const uint32_t half = pc & 1u;
                         ok = mbar_wait_warp<true>(&acc_empty_bar[region * 2 + half], ((pc >> 1) & 1u) ^ 1u, abort_flag, p.status,
                                             0x500 | (blockIdx.x << 12));
