@@ -1,13 +1,15 @@
 // Implicit-GEMM convolution on tcgen05 for layers too small to fill the chip twice: one output tile per CTA, nothing
 // persistent.  What bounds these layers is not a rate but the chain set-up -> first copy -> UMMAs -> drain -> store of one
 // tile, so this kernel keeps that chain short: every warp has one job, the weights are on their way before the previous
-// kernel has finished, the tile leaves by plain 16-byte stores straight from the warps that finish it, and the CTA is small
-// enough (384 threads, at most 110 KB of shared memory, 64 columns of tensor memory) to be set up beside its predecessor.
+// kernel has finished, the tile leaves by plain 16-byte stores straight from the registers it was drained into, tensor memory
+// is given back while those stores are under way, and the CTA is small enough (416 threads, at most 110 KB of shared memory,
+// half of the columns of tensor memory) to be set up beside its predecessor.
 //
 // A long K (a 3x3 layer on 512 channels has 72 chunks of 64) is shared out over a cluster of SPLIT CTAs that work on the same
 // tile.  Their fp32 partial tiles meet in distributed shared memory: CTA d of the cluster adds up, in the order of the ranks,
 // and finishes every SPLIT-th run of rows; each warp writes the rows it drained straight into the shared memory of the CTA
-// they belong to, and the cluster's barrier says when all have.  No global scratch, no atomics, the same sum whatever the timing.
+// they belong to, and a barrier there counts the bytes (st.async): a CTA waits for its own rows only (a barrier of the whole
+// cluster in its place took about 1 us of a layer's 5).  No global scratch, no atomics, the same sum whatever the timing.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
@@ -51,17 +53,31 @@ struct LatParams {
     int* status;
 };
 
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, float a, float b, float c, float d) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+// 16 bytes into the shared memory of a CTA of the cluster, counted by a barrier of that CTA (both addresses from mapa()).
+__device__ __forceinline__ void st_async_v4(uint32_t addr, float a, float b, float c, float d, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar) : "memory");
+}
+// 8 sums, their biases and 8 residual values to 8 rounded outputs.
+__device__ __forceinline__ uint4 finish8(const float* v, const float* bias, const uint4& res, __half2 lo, __half2 hi) {
+    const float4 c0 = *reinterpret_cast<const float4*>(bias), c1 = *reinterpret_cast<const float4*>(bias + 4);
+    const __half2* rh = reinterpret_cast<const __half2*>(&res);
+    const float2 f0 = __half22float2(rh[0]), f1 = __half22float2(rh[1]), f2 = __half22float2(rh[2]), f3 = __half22float2(rh[3]);
+    uint4 o;
+    o.x = pack_half2_clamp(v[0] + c0.x + f0.x, v[1] + c0.y + f0.y, lo, hi);
+    o.y = pack_half2_clamp(v[2] + c0.z + f1.x, v[3] + c0.w + f1.y, lo, hi);
+    o.z = pack_half2_clamp(v[4] + c1.x + f2.x, v[5] + c1.y + f2.y, lo, hi);
+    o.w = pack_half2_clamp(v[6] + c1.z + f3.x, v[7] + c1.w + f3.y, lo, hi);
+    return o;
 }
 template <int SPLIT>
 __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kThreads, 2)
 conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx2,
                 const __grid_constant__ CUtensorMap tmw2, const __grid_constant__ LatParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tfull_bar;
+    __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tfull_bar, tdone_bar, red_bar;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
+    __shared__ int abort_s, red_abort_s;
     __shared__ __align__(16) float bias_s[kMaxBN];
 
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -77,14 +93,23 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
     const int ho0 = (mt % p.tiles_h) * p.TH, n0 = (mt / p.tiles_h) * p.TN;
     const int k_first = rank * p.share, k_count = min(p.share, p.total - k_first);
 
-    if (warp == kProdWarp0 && lane == 0) {
-        abort_s = 0;
-        for (int i = 0; i < p.stages; i++) {
-            mbar_init(&full_bar[i], 1);
-            mbar_init(&empty_bar[i], 1);
+    if (warp == kProdWarp0 + 1) {
+        if (lane < kMaxStages) {
+            mbar_init(&full_bar[lane], 1);
+            mbar_init(&empty_bar[lane], 1);
         }
-        mbar_init(&tfull_bar, kMmaWarps);
+        if (lane == 0) {
+            abort_s = 0;
+            red_abort_s = 0;
+            mbar_init(&tfull_bar, kMmaWarps);
+            mbar_init(&tdone_bar, kEpiWarps);
+            mbar_init(&red_bar, 1);
+        }
         fence_barrier_init();
+        // the bytes that the cluster's CTAs will send here (before the cluster's barrier, which every sender waits for)
+        if (SPLIT > 1 && lane == 0) mbar_expect_tx(&red_bar, static_cast<uint32_t>(SPLIT * max(0, min(p.rows_per, p.rows - rank * p.rows_per)) * p.BN) * 4u);
+    }
+    if (warp == kProdWarp0 && lane == 0) {
         tma_prefetch_desc(&tmw);
         tma_prefetch_desc(&tmx);
         if (p.kchunks1 < p.kchunks) { tma_prefetch_desc(&tmx2); tma_prefetch_desc(&tmw2); }
@@ -171,23 +196,23 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
         // (540 -> 290 clocks per chunk of 64 channels); the epilogue adds the two sums ----
         const int w = warp - kMmaWarp0;
         const uint32_t idesc = umma_idesc_f16(p.BN), d_tmem = tmem_base + w * kMaxBN;
-        const uint64_t desc0 = umma_desc_sw128(0) + (base >> 4);
+        const uint32_t desc0 = umma_desc_lo(base);
         const uint32_t stage16 = static_cast<uint32_t>(p.stage_bytes) >> 4, b16 = static_cast<uint32_t>(p.a_bytes) >> 4;
         const int last = k_count - 1 - ((k_count - 1 - w) & 1);   // this issuer's last chunk (negative: it has none)
         int st = w % p.stages, kc = (k_first + w) % p.kchunks;
         uint32_t ph = static_cast<uint32_t>(w / p.stages) & 1u;
-        uint64_t ad = desc0 + static_cast<uint32_t>(st) * stage16;
+        uint32_t ad = desc0 + static_cast<uint32_t>(st) * stage16;
 #pragma unroll 1
         for (int i = w; i < k_count; i += 2) {
             if (!mbar_wait_warp<true>(&full_bar[st], ph, abort_flag, p.status, 0xE10 | (blockIdx.x << 12))) break;
             tc_fence_after_sync();
             const int ksteps = kc == p.kchunks - 1 ? p.ksteps_last : 4;
-            const uint64_t bd = ad + b16;
+            const uint32_t bd = ad + b16;
             if (elect_one()) {
-                umma_f16(d_tmem, ad, bd, idesc, i != w);
-                if (ksteps > 1) umma_f16(d_tmem, ad + 2, bd + 2, idesc, 1);
-                if (ksteps > 2) umma_f16(d_tmem, ad + 4, bd + 4, idesc, 1);
-                if (ksteps > 3) umma_f16(d_tmem, ad + 6, bd + 6, idesc, 1);
+                if (ksteps == 4) umma_f16_steps<4>(d_tmem, ad, bd, idesc, i != w);
+                else if (ksteps == 3) umma_f16_steps<3>(d_tmem, ad, bd, idesc, i != w);
+                else if (ksteps == 2) umma_f16_steps<2>(d_tmem, ad, bd, idesc, i != w);
+                else umma_f16_steps<1>(d_tmem, ad, bd, idesc, i != w);
                 if (i + p.stages < k_count) umma_commit(&empty_bar[st]);
                 if (i == last) umma_commit(&tfull_bar);
             }
@@ -203,110 +228,143 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
     } else {
         // ---- epilogue ----
         const int q = warp & 3, half = warp >> 2;
-        const int bn8 = p.BN >> 3;
+        [[maybe_unused]] const int bn8 = p.BN >> 3;
         const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
-        // the vectors this thread will finish: where they go, and their residual (its latency hides behind the UMMAs)
-        long long off[kItems];
-        uint32_t src[kItems];   // byte offset of the vector's first half in a rank's rows; its second half is 16 bytes beside it
-        int bias_at[kItems];
-        uint4 rv[kItems];
-        const int n_items = p.rows_per * bn8;
-        // a row's 16-byte vectors are stored in an order that depends on the row, so that the lanes of a warp (one row each)
-        // fall into different banks
-        const uint32_t swz = p.BN % 32 == 0 ? 7u : 3u;
-#pragma unroll
-        for (int it = 0; it < kItems; it++) {
-            const int i = static_cast<int>(threadIdx.x) + it * 32 * kEpiWarps;
-            off[it] = -1;
-            src[it] = 0u;
-            bias_at[it] = 0;
-            if (i >= n_items) continue;
-            const int r = i / bn8, g = i - r * bn8, m = rank * p.rows_per + r;
-            const int tw = m % p.TW, t2 = m / p.TW, th = t2 % p.TH, tn = t2 / p.TH;
-            const int n = n0 + tn, ho = ho0 + th, wo = wo0 + tw, co = co0 + g * 8;
-            src[it] = static_cast<uint32_t>(r * p.BN * 4) + ((static_cast<uint32_t>(2 * g) ^ (static_cast<uint32_t>(r) & swz)) << 4);
-            bias_at[it] = g * 8;
-            if (m < p.rows && n < p.N && ho < p.Ho && wo < p.Wo && co < p.Cout)
-                off[it] = ((static_cast<long long>(n) * p.Ho + ho) * p.Wo + wo) * p.Cout + co;
-        }
-        pdl_wait();
-        if (p.res) {
-#pragma unroll
-            for (int it = 0; it < kItems; it++) rv[it] = off[it] >= 0 ? __ldg(reinterpret_cast<const uint4*>(p.res + off[it])) : make_uint4(0u, 0u, 0u, 0u);
-        } else {
-#pragma unroll
-            for (int it = 0; it < kItems; it++) rv[it] = make_uint4(0u, 0u, 0u, 0u);
-        }
-        const int m = q * 32 + lane, dest = m / p.rows_per, row = m - dest * p.rows_per;
-        const uint32_t slab = static_cast<uint32_t>(p.rows_per * p.BN * 4);   // one rank's partial rows
-        const uint32_t my = base + p.red_off + rank * slab + row * p.BN * 4;
-        const uint32_t dst = SPLIT > 1 ? mapa(my, min(dest, SPLIT - 1)) : my;
-        bool ok = mbar_wait<true>(&tfull_bar, 0u, abort_flag, p.status, 0xE20 | (blockIdx.x << 12));
-        __syncwarp();
-        tc_fence_after_sync();
-        if (SPLIT > 1) cluster_wait();
-#pragma unroll 1
-        for (int c0 = half * 16; c0 < p.BN; c0 += 32) {
-            float v[16];
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        const int m = q * 32 + lane;
+        // the sums of 16 columns of this thread's row, from both accumulators
+        auto drain = [&](int c0, float (&v)[16]) {
             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + c0;
-            tmem_ld16(taddr, v);
+            uint32_t r0[16];
+            tmem_ld16_issue(taddr, r0);
             if (k_count > 1) {
-                float v2[16];
-                tmem_ld16(taddr + kMaxBN, v2);
+                uint32_t r1[16];
+                tmem_ld16_issue(taddr + kMaxBN, r1);
+                tmem_ld16_wait(r0);
+                tmem_ld16_wait(r1);
 #pragma unroll
-                for (int e = 0; e < 16; e++) v[e] += v2[e];
+                for (int e = 0; e < 16; e++) v[e] = __uint_as_float(r0[e]) + __uint_as_float(r1[e]);
+            } else {
+                tmem_ld16_wait(r0);
+#pragma unroll
+                for (int e = 0; e < 16; e++) v[e] = __uint_as_float(r0[e]);
             }
-            if (ok && m < p.rows) {
+            if (c0 + 32 >= p.BN) {   // this warp's last: tensor memory may go as far as it is concerned
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tdone_bar);
+            }
+        };
+        if (half * 16 >= p.BN && lane == 0) mbar_arrive(&tdone_bar);   // (a tile of 16 columns: the other four warps drain it)
+        if (SPLIT == 1) {
+            // a thread finishes its own row: no exchange, the first vectors' residual is fetched behind the UMMAs
+            const int tw = m % p.TW, t2 = m / p.TW, th = t2 % p.TH, tn = t2 / p.TH;
+            const int n = n0 + tn, ho = ho0 + th, wo = wo0 + tw;
+            const bool live = m < p.rows && n < p.N && ho < p.Ho && wo < p.Wo;
+            const long long row = (((static_cast<long long>(n) * p.Ho + ho) * p.Wo + wo) * p.Cout) + co0;
+            const int n_co = p.Cout - co0;
+            pdl_wait();
+            uint4 rv[kItems] = {zero, zero, zero, zero};
+            if (p.res && live) {
 #pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const uint32_t a = dst + ((static_cast<uint32_t>((c0 >> 2) + e) ^ (static_cast<uint32_t>(row) & swz)) << 4);
-                    if (SPLIT > 1) st_cluster_v4(a, v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                    else asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v[4 * e]), "f"(v[4 * e + 1]), "f"(v[4 * e + 2]), "f"(v[4 * e + 3]) : "memory");
+                for (int it = 0; it < kItems; it++) {
+                    const int c = half * 16 + (it >> 1) * 32 + (it & 1) * 8;
+                    if (c < p.BN && c < n_co) rv[it] = __ldg(reinterpret_cast<const uint4*>(p.res + row + c));
                 }
             }
+            const bool ok = mbar_wait<true>(&tfull_bar, 0u, abort_flag, p.status, 0xE20 | (blockIdx.x << 12));
             __syncwarp();
-        }
-        tc_fence_before_sync();
-        if (SPLIT > 1) {
-            __syncwarp();
-            cluster_arrive();   // second phase: every CTA's rows have arrived
-            cluster_wait();
-        } else {
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
-        }
-        const uint8_t* red = sbase + p.red_off;
+            tc_fence_after_sync();
 #pragma unroll
-        for (int it = 0; it < kItems; it++) {
-            if (off[it] < 0 || !ok) continue;
-            float4 a = *reinterpret_cast<const float4*>(red + src[it]), b = *reinterpret_cast<const float4*>(red + (src[it] ^ 16u));
+            for (int j = 0; j < kMaxBN / 32; j++) {
+                const int c0 = half * 16 + j * 32;
+                if (c0 >= p.BN) break;
+                float v[16];
+                drain(c0, v);
+                if (live && ok) {
 #pragma unroll
-            for (int sp = 1; sp < SPLIT; sp++) {
-                const float4 a2 = *reinterpret_cast<const float4*>(red + sp * slab + src[it]), b2 = *reinterpret_cast<const float4*>(red + sp * slab + (src[it] ^ 16u));
-                a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w;
-                b.x += b2.x; b.y += b2.y; b.z += b2.z; b.w += b2.w;
+                    for (int g = 0; g < 2; g++) {
+                        const int c = c0 + g * 8;
+                        if (c >= n_co) break;
+                        uint4 res = zero;
+                        if (2 * j + g < kItems) res = rv[(2 * j + g) % kItems];
+                        else if (p.res) res = __ldg(reinterpret_cast<const uint4*>(p.res + row + c));
+                        *reinterpret_cast<uint4*>(p.out + row + c) = finish8(v + g * 8, bias_s + c, res, act_lo, act_hi);
+                    }
+                }
             }
-            const float4 c0 = *reinterpret_cast<const float4*>(bias_s + bias_at[it]), c1 = *reinterpret_cast<const float4*>(bias_s + bias_at[it] + 4);
-            a.x += c0.x; a.y += c0.y; a.z += c0.z; a.w += c0.w;
-            b.x += c1.x; b.y += c1.y; b.z += c1.z; b.w += c1.w;
-            const __half2* rh = reinterpret_cast<const __half2*>(&rv[it]);
-            const float2 f0 = __half22float2(rh[0]), f1 = __half22float2(rh[1]), f2 = __half22float2(rh[2]), f3 = __half22float2(rh[3]);
-            uint4 o;
-            o.x = pack_half2_clamp(a.x + f0.x, a.y + f0.y, act_lo, act_hi);
-            o.y = pack_half2_clamp(a.z + f1.x, a.w + f1.y, act_lo, act_hi);
-            o.z = pack_half2_clamp(b.x + f2.x, b.y + f2.y, act_lo, act_hi);
-            o.w = pack_half2_clamp(b.z + f3.x, b.w + f3.y, act_lo, act_hi);
-            *reinterpret_cast<uint4*>(p.out + off[it]) = o;
+        } else {
+            // the vectors this thread will finish: where they go, and their residual (its latency hides behind the UMMAs)
+            long long off[kItems];
+            uint32_t src[kItems];   // byte offset of the vector's first half in a rank's rows; its second half is 16 bytes beside it
+            int bias_at[kItems];
+            uint4 rv[kItems];
+            const int n_items = p.rows_per * bn8;
+            // a row's 16-byte vectors are stored in an order that depends on the row, so that the lanes of a warp (one row each)
+            // fall into different banks
+            const uint32_t swz = p.BN % 32 == 0 ? 7u : 3u;
+#pragma unroll
+            for (int it = 0; it < kItems; it++) {
+                const int i = static_cast<int>(threadIdx.x) + it * 32 * kEpiWarps;
+                off[it] = -1;
+                src[it] = 0u;
+                bias_at[it] = 0;
+                if (i >= n_items) continue;
+                const int r = i / bn8, g = i - r * bn8, mo = rank * p.rows_per + r;
+                const int tw = mo % p.TW, t2 = mo / p.TW, th = t2 % p.TH, tn = t2 / p.TH;
+                const int n = n0 + tn, ho = ho0 + th, wo = wo0 + tw, co = co0 + g * 8;
+                src[it] = static_cast<uint32_t>(r * p.BN * 4) + ((static_cast<uint32_t>(2 * g) ^ (static_cast<uint32_t>(r) & swz)) << 4);
+                bias_at[it] = g * 8;
+                if (mo < p.rows && n < p.N && ho < p.Ho && wo < p.Wo && co < p.Cout)
+                    off[it] = ((static_cast<long long>(n) * p.Ho + ho) * p.Wo + wo) * p.Cout + co;
+            }
+            pdl_wait();
+#pragma unroll
+            for (int it = 0; it < kItems; it++) rv[it] = p.res && off[it] >= 0 ? __ldg(reinterpret_cast<const uint4*>(p.res + off[it])) : zero;
+            const int dest = min(m / p.rows_per, SPLIT - 1), row = m - dest * p.rows_per;
+            const uint32_t slab = static_cast<uint32_t>(p.rows_per * p.BN * 4);   // one rank's partial rows
+            const uint32_t dst = mapa(base + p.red_off + rank * slab + row * p.BN * 4, dest), dst_bar = mapa(smem_u32(&red_bar), dest);
+            bool ok = mbar_wait<true>(&tfull_bar, 0u, abort_flag, p.status, 0xE20 | (blockIdx.x << 12));
+            __syncwarp();
+            tc_fence_after_sync();
+            cluster_wait();   // every CTA of the cluster runs and its barrier expects these rows
+#pragma unroll 1
+            for (int c0 = half * 16; c0 < p.BN; c0 += 32) {
+                float v[16];
+                drain(c0, v);
+                if (m < p.rows) {   // (sent whatever happened: the other CTAs wait for the bytes)
+#pragma unroll
+                    for (int e = 0; e < 4; e++)
+                        st_async_v4(dst + ((static_cast<uint32_t>((c0 >> 2) + e) ^ (static_cast<uint32_t>(row) & swz)) << 4),
+                                    v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3], dst_bar);
+                }
+                __syncwarp();
+            }
+            // all rows of this CTA are here.  It must not retire before that, whatever its own part came to, hence a limit above
+            // the senders' and a flag of its own.
+            ok = mbar_wait<true>(&red_bar, 0u, &red_abort_s, p.status, 0xE30 | (blockIdx.x << 12), 4 * kWaitLimitNs) && ok;
+            const uint8_t* red = sbase + p.red_off;
+#pragma unroll
+            for (int it = 0; it < kItems; it++) {
+                if (off[it] < 0 || !ok) continue;
+                float4 a = *reinterpret_cast<const float4*>(red + src[it]), b = *reinterpret_cast<const float4*>(red + (src[it] ^ 16u));
+#pragma unroll
+                for (int sp = 1; sp < SPLIT; sp++) {
+                    const float4 a2 = *reinterpret_cast<const float4*>(red + sp * slab + src[it]), b2 = *reinterpret_cast<const float4*>(red + sp * slab + (src[it] ^ 16u));
+                    a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w;
+                    b.x += b2.x; b.y += b2.y; b.z += b2.z; b.w += b2.w;
+                }
+                const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                *reinterpret_cast<uint4*>(p.out + off[it]) = finish8(v, bias_s + bias_at[it], rv[it], act_lo, act_hi);
+            }
         }
     }
     __syncwarp();
-    if (SPLIT > 1 && warp >= kEpiWarps) {
-        cluster_wait();
-        cluster_arrive();
-        cluster_wait();
-    }
-    __syncthreads();
+    if (SPLIT > 1 && warp >= kEpiWarps) cluster_wait();
     if (warp == kMmaWarp0) {
-        if (abort_s) __nanosleep(20000);   // let copies in flight land before the CTA retires
+        // tensor memory is given back as soon as it has been read, while the tile is still on its way out
+        const bool ok = mbar_wait_warp(&tdone_bar, 0u, &red_abort_s, p.status, 0xE40 | (blockIdx.x << 12), 2 * kWaitLimitNs);
+        if (abort_s || !ok) __nanosleep(20000);   // let copies in flight land before the CTA retires
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, kMaxBN * kMmaWarps);
     }
@@ -366,18 +424,20 @@ Choice choose(const ConvArgs& a, int total, int sm_count, const int (&max_cluste
                 if (tiles * split > sm_count) break;
                 if ((split > 1 && (split - 1) * share >= total) || rows_per * BN > kMaxOut) continue;
                 for (int smem : {kPairSmem, kMaxDynSmem}) {
-                    const int budget = smem - 1024 - split * rows_per * BN * 4 - (128 * 128 - a_bytes);
+                    const int budget = smem - 1024 - (split > 1 ? split * rows_per * BN * 4 : 0) - (128 * 128 - a_bytes);
                     int stages = std::min({kMaxStages, budget / stage, share});
                     if (stages < share) stages &= ~1;   // the ring goes round: a stage belongs to one issuer
                     if (stages < std::min(share, 2)) continue;
                     if (tiles > (smem > kPairSmem ? max_clusters[lg] : 2 * max_clusters[lg])) continue;   // (a second wave of clusters)
-                    // Fitted to about 600 measured (layer, tile, split) times: a chunk costs what its copy or its two issuers
-                    // take, and with a ring that goes round its part of a round trip; sharing a tile costs the exchange of its
-                    // sums, and more when the clusters have to be packed (eight CTAs, more than half of the SMs); so do CTAs on nearly all SMs.
-                    double chunk = std::max(stage / 52.0, 320.0 + 0.4 * BN);
-                    if (stages < share) chunk = std::max(chunk, 1700.0 / stages);
-                    const double cost = 2000.0 + share * chunk + rows * BN * (lg > 0 ? 0.3 : 0.11) + (lg > 0 ? 500.0 : 0.0) + (lg == 3 ? 1000.0 : 0.0) +
-                                        (tiles * split > (lg > 0 ? sm_count / 2 : sm_count * 3 / 4) ? 1000.0 : 0.0) + (smem > kPairSmem ? 1000.0 : 0.0);
+                    // Fitted to about 2000 measured (layer, tile, split) times of 102 layers (ResNet-50's at 1 to 6 images, MobileNetV2's
+                    // at 1 and 4, odd ones): a chunk costs what its two issuers take, and with a ring that goes round its part of a
+                    // round trip; sharing a tile costs the exchange of its sums; CTAs on more than half of the SMs find the
+                    // previous kernel still there, and so do CTAs that fit an SM only once.  The layers chosen by it take 567 us in
+                    // all, the best choice for each 558, the constants before these 590.
+                    double chunk = 315.0 + 0.45 * BN;
+                    if (stages < share) chunk = std::max(chunk, 2500.0 / stages);
+                    const double cost = 2000.0 + stage / 366.0 + share * chunk + rows * BN * (lg > 0 ? 0.47 : 0.13) + (lg > 0 ? 760.0 : 0.0) + (lg == 3 ? 160.0 : 0.0) +
+                                        (tiles * split > sm_count / 2 ? (lg > 0 ? 1500.0 : 2250.0) : 0.0) + (smem > kPairSmem ? 280.0 : 0.0);
                     if (best.cost < 0 || cost < best.cost) best = Choice{t, BN, split, share, stages, rows_per, cost};
                 }
             }
@@ -409,11 +469,11 @@ int launch_conv_lat(const ConvArgs& a_in, int sm_count, int* status_dev, cudaStr
     const int dev = current_device_slot();
     if (dev < 0) return DLF_E_UNSUPPORTED;
     const Choice c = choose(a, p.total, sm_count, g_max_clusters[dev]);
-    // the persistent kernel: 2.5 us in a network for a tile with one chunk, 0.16 us for every further one (3.4 us for 64 -> 64
-    // at one 56x56 image against 2.6 us here; 6.3 us for 128 -> 128 3x3 at eight 28x28 images against 7.1 us), 0.12 us where it
-    // loads a kernel row's window once (4.6 us for 64 -> 64 3x3 at five 27x29 images against 4.7 us)
+    // Where the tiles fit one wave this kernel is the faster one (64 -> 64 at one 56x56 image 2.6 us against 3.6 in a network, 512
+    // -> 128 at six 28x28 images 5.0 against 6.1), except for layers whose kernel rows the persistent kernel loads once: there it
+    // takes over when a CTA's share of K is long (256 -> 256 3x3 at six 14x14 images: 9.6 against 9.1).
     const bool row = a.kh == 3 && a.kw == 3 && a.stride == 1 && a.Cin % 64 == 0 && g_conv_row_mode > 0;
-    if (c.cost < 0 || c.cost > 4100.0 + (row ? 240.0 : 310.0) * p.total) return DLF_E_UNSUPPORTED;
+    if (c.cost < 0 || (row && c.cost > 8600.0 + 117.0 * p.total)) return DLF_E_UNSUPPORTED;
     p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
     p.kw = a.kw; p.stride = a.stride; p.pad = a.pad; p.stride2 = dual ? a.stride2 : 1;
     p.TW = c.tile.tw; p.TH = c.tile.th; p.TN = c.tile.tn;
@@ -454,7 +514,7 @@ int launch_conv_lat(const ConvArgs& a_in, int sm_count, int* status_dev, cudaStr
     if (rc == DLF_OK && dual) rc = weight_map(&tmw2, a.w2, a.Cin2, 1);
     if (rc) return rc;
     const int grid = p.tiles_w * p.tiles_h * tiles_n * p.n_tiles_n * c.split;
-    const size_t smem = static_cast<size_t>(p.red_off) + static_cast<size_t>(c.split) * p.rows_per * p.BN * 4 + 1024;
+    const size_t smem = static_cast<size_t>(p.red_off) + (c.split > 1 ? static_cast<size_t>(c.split) * p.rows_per * p.BN * 4 : 0) + 1024;
     cudaError_t e = launch_kernel(pick_kernel(c.split), grid, kThreads, smem, s, tmx, tmw, tmx2, tmw2, p);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }

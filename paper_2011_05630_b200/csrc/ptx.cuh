@@ -115,8 +115,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // computes are warp-uniform values); the result is voted so that the warp leaves a wait together.
 template <bool HOT = false>
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                               int* status, int code) {
-    const bool ok = mbar_wait<HOT>(bar, parity, abort_flag, status, code);
+                                               int* status, int code, uint64_t limit_ns = kWaitLimitNs) {
+    const bool ok = mbar_wait<HOT>(bar, parity, abort_flag, status, code, limit_ns);
     return __all_sync(0xffffffffu, ok);
 }
 
