@@ -333,15 +333,10 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
         // ---- MMA issuer: the whole warp walks the loop (warp-uniform addresses), one elected lane issues ----
         if (PAIR && rank != 0) return;   // the first CTA of the pair issues for both
         const uint32_t idesc = PAIR ? umma_idesc_f16_pair(p.BN) : umma_idesc_f16(p.BN);
-        auto umma = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t accumulate) {
-            if (PAIR) umma_f16_pair(d, a, b, idesc, accumulate);
-            else umma_f16(d, a, b, idesc, accumulate);
-        };
         auto commit = [&](uint64_t* bar) {
             if (PAIR) umma_commit_pair(bar);
             else umma_commit(bar);
         };
-        const uint64_t desc0 = umma_desc_sw128(0);
         const uint32_t b_chunk16 = static_cast<uint32_t>(b_rows) * 8u;  // one 64-channel weight slab, in 16-byte units
         const uint32_t a_chunk16 = static_cast<uint32_t>(p.a_bytes) >> 4;  // one 64-channel slab of the tile's pixels (rows rounded up to 8)
         uint32_t it = 0, j = 0, ring_ph = 0;
@@ -372,32 +367,27 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 DLF_TRACE_ACC(macc, 1, mmark);
                 tc_fence_after_sync();
                 const uint32_t sa = base + st * stage_bytes;
-                const uint64_t a0 = desc0 + (sa >> 4), b0 = a0 + static_cast<uint32_t>(p.kg * p.a_bytes >> 4);
+                const uint32_t a0 = umma_desc_lo(sa), b0 = a0 + static_cast<uint32_t>(p.kg * p.a_bytes >> 4);   // (low descriptor words)
                 const int g_end = min(p.kg, p.kchunks - kq * p.kg);
                 if (elect_one()) {
                     if (!ROW) {
 #pragma unroll 1
                         for (int g = 0; g < g_end; g++) {
-                            const uint64_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g) * b_chunk16;
+                            const uint32_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g) * b_chunk16;
                             const int ksteps = (kq * p.kg + g == p.kchunks - 1) ? p.ksteps_last : 4;
-                            umma(d_tmem, ad, bd, (ki | g) != 0);
-                            if (ksteps > 1) umma(d_tmem, ad + 2, bd + 2, 1);
-                            if (ksteps > 2) umma(d_tmem, ad + 4, bd + 4, 1);
-                            if (ksteps > 3) umma(d_tmem, ad + 6, bd + 6, 1);
+                            if (ksteps == 4) umma_f16_steps<4, PAIR>(d_tmem, ad, bd, idesc, (ki | g) != 0);
+                            else if (ksteps == 3) umma_f16_steps<3, PAIR>(d_tmem, ad, bd, idesc, (ki | g) != 0);
+                            else if (ksteps == 2) umma_f16_steps<2, PAIR>(d_tmem, ad, bd, idesc, (ki | g) != 0);
+                            else umma_f16_steps<1, PAIR>(d_tmem, ad, bd, idesc, (ki | g) != 0);
                         }
                     } else {
                         // row mode (whole 64-channel chunks): the three taps of a kernel row read the same window, one
                         // pixel (one 128-byte row) further each
 #pragma unroll 1
                         for (int g = 0; g < g_end; g++) {
-                            uint64_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g * 3) * b_chunk16;
+                            uint32_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g * 3) * b_chunk16;
 #pragma unroll
-                            for (int sx = 0; sx < 3; sx++, ad += 8, bd += b_chunk16) {
-                                umma(d_tmem, ad, bd, (ki | g | sx) != 0);
-                                umma(d_tmem, ad + 2, bd + 2, 1);
-                                umma(d_tmem, ad + 4, bd + 4, 1);
-                                umma(d_tmem, ad + 6, bd + 6, 1);
-                            }
+                            for (int sx = 0; sx < 3; sx++, ad += 8, bd += b_chunk16) umma_f16_steps<4, PAIR>(d_tmem, ad, bd, idesc, (ki | g | sx) != 0);
                         }
                     }
                     commit(&sm.empty_bar[st]);  // frees the stage once these MMAs have read it
@@ -626,20 +616,20 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
 
 }
 
-// Initialises the barriers for a ring of `stages` stages (thread 0; `again`: they hold valid objects already).
-__device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, int stages, bool again, bool pair = false) {
+// Initialises the barriers of a multi-layer launch (thread 0; `again`: they hold valid objects already).
+__device__ __forceinline__ void conv_tc_init_bars(const ConvBars& sm, bool again) {
     if (again) {
         for (int i = 0; i < 8; i++) { mbar_inval(&sm.full_bar[i]); mbar_inval(&sm.empty_bar[i]); }
         for (int i = 0; i < 2; i++) { mbar_inval(&sm.tfull_bar[i]); mbar_inval(&sm.tempty_bar[i]); }
         for (int i = 0; i < kMaxOutBufs; i++) { mbar_inval(&sm.sfull_bar[i]); mbar_inval(&sm.sfree_bar[i]); }
     }
-    for (int i = 0; i < (again ? 8 : stages); i++) {
+    for (int i = 0; i < 8; i++) {
         mbar_init(&sm.full_bar[i], 2);  // the A and the B producer each arrive with their byte count
         mbar_init(&sm.empty_bar[i], 1);
     }
     for (int i = 0; i < 2; i++) {
         mbar_init(&sm.tfull_bar[i], 1);
-        mbar_init(&sm.tempty_bar[i], pair ? 2 * kEpiWarps : kEpiWarps);
+        mbar_init(&sm.tempty_bar[i], kEpiWarps);
     }
     for (int i = 0; i < kMaxOutBufs; i++) {
         mbar_init(&sm.sfull_bar[i], kEpiWarps);
@@ -652,25 +642,38 @@ template <int ACT, bool POOL, bool RES, bool ROW, bool SPLIT, bool PAIR>
 __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmx, const CUtensorMap& tmw, const CUtensorMap& tmy, const CUtensorMap& tmr,
                                              const CUtensorMap& tmx2, const CUtensorMap& tmw2, const ConvTcParams& p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[8], empty_bar[8], tfull_bar[2], tempty_bar[2];
-    __shared__ uint64_t sfull_bar[kMaxOutBufs], sfree_bar[kMaxOutBufs];  // staging buffer: filled by the epilogue / free again (residual landed)
+    // the barriers in one array, a thread each initialises them (one thread for all: 0.5 us in front of every layer)
+    constexpr int kBars = 16 + 4 + 2 * kMaxOutBufs + 1;
+    __shared__ uint64_t bars[kBars];
+    uint64_t* const tdone_bar = bars + kBars - 1;   // the epilogue has read the last accumulator
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
+    __shared__ int abort_s, tdone_abort_s;
 
     if (threadIdx.x == 0) DLF_TRACE_POINT(p.status, 0);
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* stage0 = smem_raw + (base - smem_u32(smem_raw));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const ConvBars sm{full_bar, empty_bar, tfull_bar, tempty_bar, sfull_bar, sfree_bar, &abort_s};
+    const ConvBars sm{bars, bars + 8, bars + 16, bars + 18, bars + 20, bars + 20 + kMaxOutBufs, &abort_s};
 
-    if (threadIdx.x == 0) {
-        abort_s = 0;
-        conv_tc_init_bars(sm, p.stages, false, PAIR);
-        tma_prefetch_desc(&tmx);
-        tma_prefetch_desc(&tmw);
-        if (!POOL) tma_prefetch_desc(&tmy);
-        if (!POOL && RES) tma_prefetch_desc(&tmr);
-        if (p.kchunks1 < p.kchunks) { tma_prefetch_desc(&tmx2); tma_prefetch_desc(&tmw2); }
+    if (warp == 0) {
+        if (lane == 0) {
+            abort_s = 0;
+            tdone_abort_s = 0;
+        }
+        if (lane < kBars) {
+            int count = 1;                                           // empty, tfull, sfree
+            if (lane < 8) count = 2;                                 // full: the A and the B producer each arrive with their byte count
+            else if (lane >= 18 && lane < 20) count = PAIR ? 2 * kEpiWarps : kEpiWarps;   // tempty
+            else if ((lane >= 20 && lane < 20 + kMaxOutBufs) || lane == kBars - 1) count = kEpiWarps;   // sfull, tdone
+            mbar_init(&bars[lane], count);
+        }
+        fence_barrier_init();
+    } else if (warp == kStoreWarp) {
+        if (lane == 0) tma_prefetch_desc(&tmx);
+        if (lane == 1) tma_prefetch_desc(&tmw);
+        if (lane == 2 && !POOL) tma_prefetch_desc(&tmy);
+        if (lane == 3 && !POOL && RES) tma_prefetch_desc(&tmr);
+        if (lane == 4 && p.kchunks1 < p.kchunks) { tma_prefetch_desc(&tmx2); tma_prefetch_desc(&tmw2); }
     }
     if (warp == kMmaWarp) {
         if (PAIR) {
@@ -697,17 +700,31 @@ __device__ __forceinline__ void conv_tc_body(const CUtensorMap& tmx, const CUten
 
     conv_tc_roles<ACT, POOL, RES, ROW, SPLIT, PAIR>(&tmx, &tmw, &tmy, &tmr, &tmx2, &tmw2, p, sm, tmem_base, stage0, base, GridSync{nullptr, 0u});
 
+    if (!PAIR) {
+        // Every warp leaves on its own; tensor memory is given back as soon as it has been read, while the last tile is still on
+        // its way out (what a layer spends behind its last store delays the next one).
+        if (warp < kEpiWarps) {
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tdone_bar);
+        } else if (warp == kMmaWarp) {
+            const bool ok = mbar_wait_warp(tdone_bar, 0u, &tdone_abort_s, p.status, 0x800 | (blockIdx.x << 12), 4 * kWaitLimitNs);
+            if (abort_s || !ok) __nanosleep(20000);  // let copies in flight land before the CTA retires
+            tc_fence_after_sync();
+            tmem_dealloc(tmem_base, p.tmem_cols);
+            if (lane == 0) DLF_TRACE_POINT(p.status, 7);
+        }
+        return;
+    }
     tc_fence_before_sync();
     __syncthreads();
-    if (PAIR) {   // neither CTA leaves while the other may still read its operands or signal its barriers
-        cluster_arrive();
-        cluster_wait();
-    }
+    // neither CTA leaves while the other may still read its operands or signal its barriers
+    cluster_arrive();
+    cluster_wait();
     if (warp == kMmaWarp) {
-        if (abort_s) __nanosleep(20000);  // let copies in flight land before the CTA retires
+        if (abort_s) __nanosleep(20000);
         tc_fence_after_sync();
-        if (PAIR) tmem_dealloc_pair(tmem_base, p.tmem_cols);
-        else tmem_dealloc(tmem_base, p.tmem_cols);
+        tmem_dealloc_pair(tmem_base, p.tmem_cols);
         if (lane == 0) DLF_TRACE_POINT(p.status, 7);
     }
 }
@@ -774,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_seq_kernel(const __grid_cons
 
     if (threadIdx.x == 0) {
         abort_s = 0;
-        conv_tc_init_bars(sm, 8, false);
+        conv_tc_init_bars(sm, false);
     }
     if (warp == kMmaWarp) {
         tmem_alloc(&tmem_base_s, 512);
@@ -792,7 +809,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_seq_kernel(const __grid_cons
         for (int i = threadIdx.x; i < static_cast<int>(sizeof(ConvTcParams) / 4); i += kThreads)
             reinterpret_cast<int*>(&p_s)[i] = reinterpret_cast<const int*>(&Y.p)[i];
         if (threadIdx.x == 0) {   // fresh barriers for this layer's ring (every role is past the previous layer: see the barrier below)
-            if (l > 0) conv_tc_init_bars(sm, 8, true);
+            if (l > 0) conv_tc_init_bars(sm, true);
             tma_prefetch_desc(&Y.tmx);
             tma_prefetch_desc(&Y.tmw);
         }

@@ -331,37 +331,40 @@ __device__ __forceinline__ void umma_f16_x4(uint32_t d_tmem, uint32_t a_lo, uint
 // = 8 units further per tap, B one slab of `w_tap16` units), in a single statement each: statements of their own cost the
 // issuing thread about 200 clocks per UMMA in a loop over taps, members of one statement 66 (two 16 -> 16 3x3 layers on one
 // 32x32 image: 9.2 -> 7.5 us as one kernel).
-#define DLF_UMMA_STEP(AO, KO)                                                                                                        \
+#define DLF_UMMA_STEP(CG, AO, KO)                                                                                                    \
     "add.u32 ta, %1, " #AO ";\n\tadd.u32 tb, tc, " #KO ";\n\tmov.b64 da, {ta, %5};\n\tmov.b64 db, {tb, %5};\n\t"                     \
-    "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t"
-#define DLF_UMMA_FIRST                                                                                                               \
+    "tcgen05.mma.cta_group::" #CG ".kind::f16 [%0], da, db, %3, p;\n\t"
+#define DLF_UMMA_FIRST(CG)                                                                                                           \
     "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t.reg .b32 ta, tb, tc;\n\tsetp.ne.b32 p, %4, 0;\n\tmov.b32 tc, %2;\n\t"              \
-    DLF_UMMA_STEP(0, 0) "setp.eq.b32 p, %3, %3;\n\t"
+    DLF_UMMA_STEP(CG, 0, 0) "setp.eq.b32 p, %3, %3;\n\t"
 #define DLF_UMMA_NEXT_TAP "add.u32 tc, tc, %6;\n\t"
 #define DLF_UMMA_OPS                                                                                                                 \
     "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHiSw128), "r"(w_tap16) : "memory"
 template <int KS>
 __device__ __forceinline__ void umma_f16_row3(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t w_tap16, uint32_t idesc, uint32_t accumulate) {
     if (KS == 1)
-        asm volatile(DLF_UMMA_FIRST DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(8, 0) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(16, 0) DLF_UMMA_OPS);
+        asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(1, 8, 0) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(1, 16, 0) DLF_UMMA_OPS);
     if (KS == 2)
-        asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(8, 0) DLF_UMMA_STEP(10, 2) DLF_UMMA_NEXT_TAP
-                     DLF_UMMA_STEP(16, 0) DLF_UMMA_STEP(18, 2) DLF_UMMA_OPS);
+        asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 2, 2) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(1, 8, 0) DLF_UMMA_STEP(1, 10, 2) DLF_UMMA_NEXT_TAP
+                     DLF_UMMA_STEP(1, 16, 0) DLF_UMMA_STEP(1, 18, 2) DLF_UMMA_OPS);
     if (KS == 3)
-        asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_STEP(4, 4) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(8, 0) DLF_UMMA_STEP(10, 2)
-                     DLF_UMMA_STEP(12, 4) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(16, 0) DLF_UMMA_STEP(18, 2) DLF_UMMA_STEP(20, 4) DLF_UMMA_OPS);
-    if (KS == 4)
-        asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_STEP(4, 4) DLF_UMMA_STEP(6, 6) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(8, 0)
-                     DLF_UMMA_STEP(10, 2) DLF_UMMA_STEP(12, 4) DLF_UMMA_STEP(14, 6) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(16, 0)
-                     DLF_UMMA_STEP(18, 2) DLF_UMMA_STEP(20, 4) DLF_UMMA_STEP(22, 6) DLF_UMMA_OPS);
+        asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 2, 2) DLF_UMMA_STEP(1, 4, 4) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(1, 8, 0) DLF_UMMA_STEP(1, 10, 2)
+                     DLF_UMMA_STEP(1, 12, 4) DLF_UMMA_NEXT_TAP DLF_UMMA_STEP(1, 16, 0) DLF_UMMA_STEP(1, 18, 2) DLF_UMMA_STEP(1, 20, 4) DLF_UMMA_OPS);
 }
-template <int KS>
+template <int KS, bool PAIR = false>
 __device__ __forceinline__ void umma_f16_steps(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
     const uint32_t w_tap16 = 0u;
-    if (KS == 1) asm volatile(DLF_UMMA_FIRST DLF_UMMA_OPS);
-    if (KS == 2) asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_OPS);
-    if (KS == 3) asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_STEP(4, 4) DLF_UMMA_OPS);
-    if (KS == 4) asm volatile(DLF_UMMA_FIRST DLF_UMMA_STEP(2, 2) DLF_UMMA_STEP(4, 4) DLF_UMMA_STEP(6, 6) DLF_UMMA_OPS);
+    if (!PAIR) {
+        if (KS == 1) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_OPS);
+        if (KS == 2) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 2, 2) DLF_UMMA_OPS);
+        if (KS == 3) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 2, 2) DLF_UMMA_STEP(1, 4, 4) DLF_UMMA_OPS);
+        if (KS == 4) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 2, 2) DLF_UMMA_STEP(1, 4, 4) DLF_UMMA_STEP(1, 6, 6) DLF_UMMA_OPS);
+    } else {   // of a CTA pair
+        if (KS == 1) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_OPS);
+        if (KS == 2) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_STEP(2, 2, 2) DLF_UMMA_OPS);
+        if (KS == 3) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_STEP(2, 2, 2) DLF_UMMA_STEP(2, 4, 4) DLF_UMMA_OPS);
+        if (KS == 4) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_STEP(2, 2, 2) DLF_UMMA_STEP(2, 4, 4) DLF_UMMA_STEP(2, 6, 6) DLF_UMMA_OPS);
+    }
 }
 #undef DLF_UMMA_STEP
 #undef DLF_UMMA_FIRST
