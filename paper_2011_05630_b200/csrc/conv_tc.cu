@@ -487,10 +487,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                                 uint4 o;
                                 uint32_t* ou = reinterpret_cast<uint32_t*>(&o);
 #pragma unroll
-                                for (int e = 0; e < 4; e++) {
-                                    const __half2 hv = act_h2<ACT>(__floats2half2_rn(a[2 * e], a[2 * e + 1]));
-                                    ou[e] = *reinterpret_cast<const uint32_t*>(&hv);
-                                }
+                                for (int e = 0; e < 4; e++) ou[e] = round_act<ACT>(a[2 * e], a[2 * e + 1]);
                                 if (co < p.Cout) *reinterpret_cast<uint4*>(p.out + pix * p.Cout + co) = o;
                             }
                         }
@@ -539,43 +536,37 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 for (int g = 0; g < 4; g++) {
                     if (g * 8 >= nc) break;
                     const int co = c.co0 + cc + g * 8;  // first of 8 channels
-                    float a[8];
-                    const float4 b0 = *reinterpret_cast<const float4*>(bias_s + co);
-                    const float4 b1 = *reinterpret_cast<const float4*>(bias_s + co + 4);
-                    a[0] = __uint_as_float(r[g * 8 + 0]) + b0.x; a[1] = __uint_as_float(r[g * 8 + 1]) + b0.y; a[2] = __uint_as_float(r[g * 8 + 2]) + b0.z; a[3] = __uint_as_float(r[g * 8 + 3]) + b0.w;
-                    a[4] = __uint_as_float(r[g * 8 + 4]) + b1.x; a[5] = __uint_as_float(r[g * 8 + 5]) + b1.y; a[6] = __uint_as_float(r[g * 8 + 6]) + b1.z; a[7] = __uint_as_float(r[g * 8 + 7]) + b1.w;
+                    float2 a[4];
+                    const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bias_s + co), b1 = *reinterpret_cast<const ulonglong2*>(bias_s + co + 4);   // pairs
+                    a[0] = add_f2(r[g * 8 + 0], r[g * 8 + 1], b0.x);
+                    a[1] = add_f2(r[g * 8 + 2], r[g * 8 + 3], b0.y);
+                    a[2] = add_f2(r[g * 8 + 4], r[g * 8 + 5], b1.x);
+                    a[3] = add_f2(r[g * 8 + 6], r[g * 8 + 7], b1.y);
                     const int g8 = (cc >> 3) + g;
                     uint4* sptr = reinterpret_cast<uint4*>(sout + (g8 >> 3) * kABytes + m * 128 + (((g8 & 7) ^ (m & 7)) << 4));
-                    if (RES && !POOL) {   // the residual tile was loaded into the staging buffer (zero outside the tensor)
-                        const uint4 rv = *sptr;
-                        const __half2* rh = reinterpret_cast<const __half2*>(&rv);
+                    if (RES) {   // the residual tile was loaded into the staging buffer (zero outside the tensor); pooled: see res_load
+                        const uint4 rv = !POOL ? *sptr : (((rok >> g) & 1u) ? rcur[g] : make_uint4(0u, 0u, 0u, 0u));
+                        const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
+                        const unsigned short one = 0x3C00u;   // (residual x 1.0 + sum: no conversion)
 #pragma unroll
                         for (int e = 0; e < 4; e++) {
-                            const float2 f = __half22float2(rh[e]);
-                            a[2 * e] += f.x;
-                            a[2 * e + 1] += f.y;
-                        }
-                    }
-                    if (RES && POOL) {
-                        const bool okg = (rok >> g) & 1u;
-                        const __half2* rh = reinterpret_cast<const __half2*>(&rcur[g]);
-#pragma unroll
-                        for (int e = 0; e < 4; e++) {
-                            const float2 f = __half22float2(rh[e]);
-                            a[2 * e] += okg ? f.x : 0.0f;
-                            a[2 * e + 1] += okg ? f.y : 0.0f;
+                            unsigned short lo, hi;
+                            unpack_h2(rw[e], lo, hi);
+                            a[e].x = fma_f32_f16(lo, one, a[e].x);
+                            a[e].y = fma_f32_f16(hi, one, a[e].y);
                         }
                     }
                     uint4 o;
                     uint32_t* ou = reinterpret_cast<uint32_t*>(&o);
 #pragma unroll
                     for (int e = 0; e < 4; e++) {
-                        __half2 hv = act_h2<ACT>(__floats2half2_rn(a[2 * e], a[2 * e + 1]));   // (clamped after the rounding: same bits)
+                        ou[e] = round_act<ACT>(a[e].x, a[e].y);   // (the activation after the rounding: same bits)
                         if (POOL) {  // rounded first, then the max over the 2x2 window held by this warp
+                            __half2 hv = *reinterpret_cast<__half2*>(&ou[e]);
                             hv = __hmax2(hv, __shfl_xor_sync(0xffffffffu, hv, 1));
                             hv = __hmax2(hv, __shfl_xor_sync(0xffffffffu, hv, p.TW));
+                            ou[e] = *reinterpret_cast<uint32_t*>(&hv);
                         }
-                        ou[e] = *reinterpret_cast<uint32_t*>(&hv);
                     }
                     if (POOL) {
                         if (writer && co < p.Cout) *reinterpret_cast<uint4*>(p.out + opix * p.Cout + co) = o;

@@ -74,22 +74,10 @@ struct MbParams {
     int* status;
 };
 
-// Two fp32 additions in one instruction (both operands register pairs).
-__device__ __forceinline__ float2 add_f2(uint32_t a0, uint32_t a1, uint64_t b) {
-    uint64_t r;
-    float2 f;
-    asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tadd.rn.f32x2 %0, t, %3;\n\t}" : "=l"(r) : "r"(a0), "r"(a1), "l"(b));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(r));
-    return f;
-}
-// A pair rounded to fp16 with its activation: ReLU6 through the conversion's own ReLU, anything else as a clamp to [lo, hi].
+// A pair rounded to fp16 with its activation: ReLU6, or a clamp to [lo, hi].
 template <bool RELU6>
-__device__ __forceinline__ uint32_t round_act(float a, float b, __half2 lo, __half2 hi) {
-    if (!RELU6) return pack_half2_clamp(a, b, lo, hi);
-    uint32_t r;
-    asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    const __half2 h = __hmin2(*reinterpret_cast<const __half2*>(&r), __float2half2_rn(6.0f));
-    return *reinterpret_cast<const uint32_t*>(&h);
+__device__ __forceinline__ uint32_t round_clamp(float a, float b, __half2 lo, __half2 hi) {
+    return RELU6 ? round_act<2>(a, b) : pack_half2_clamp(a, b, lo, hi);
 }
 
 // RELU6: both the expansion's and the depthwise layer's activation
@@ -380,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) mbconv_tc_kernel(const __grid_con
 #pragma unroll
                                     for (int e = 0; e < 4; e++) {
                                         const float2 f = add_f2(r[g * 8 + 2 * e], r[g * 8 + 2 * e + 1], bb[g * 4 + e]);
-                                        val[e] = round_act<RELU6>(f.x, f.y, lo1, hi1);
+                                        val[e] = round_clamp<RELU6>(f.x, f.y, lo1, hi1);
                                     }
                                     if (!((all_in >> b) & 1u) && !((in_img >> b) & 1u)) val[0] = val[1] = val[2] = val[3] = 0u;   // the depthwise layer's padding
                                     *reinterpret_cast<uint4*>(dst + g * 16) = make_uint4(val[0], val[1], val[2], val[3]);
@@ -482,7 +470,7 @@ __global__ void __launch_bounds__(kThreads, 1) mbconv_tc_kernel(const __grid_con
                     };
                     auto store = [&](const float (&acc)[4]) {
                         *reinterpret_cast<uint2*>(hd + o * 128 + (((cl >> 1) ^ (o & 7)) << 4)) =
-                            make_uint2(round_act<RELU6>(acc[0], acc[1], lo2, hi2), round_act<RELU6>(acc[2], acc[3], lo2, hi2));
+                            make_uint2(round_clamp<RELU6>(acc[0], acc[1], lo2, hi2), round_clamp<RELU6>(acc[2], acc[3], lo2, hi2));
                         o += p.tw;
                     };
                     float u[4], v[4], n[4];

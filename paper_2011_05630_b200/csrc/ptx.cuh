@@ -488,12 +488,25 @@ __device__ __forceinline__ uint32_t pack_half2_clamp(float a, float b, __half2 l
     const __half2 h = __hmin2(__hmax2(__floats2half2_rn(a, b), lo), hi);
     return *reinterpret_cast<const uint32_t*>(&h);
 }
-// The activation of a rounded pair: none, ReLU, ReLU6.
+// Epilogue arithmetic in few instructions (it bounds the memory-bound layers): two fp32 additions at once, and a pair rounded
+// to fp16 with its activation (none, ReLU, ReLU6), ReLU being part of the conversion.
+__device__ __forceinline__ float2 add_f2(uint32_t a0, uint32_t a1, uint64_t b) {
+    uint64_t r;
+    float2 f;
+    asm("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tadd.rn.f32x2 %0, t, %3;\n\t}" : "=l"(r) : "r"(a0), "r"(a1), "l"(b));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(r));
+    return f;
+}
 template <int ACT>
-__device__ __forceinline__ __half2 act_h2(__half2 h) {
-    if (ACT >= 1) h = __hmax2(h, __float2half2_rn(0.0f));
-    if (ACT == 2) h = __hmin2(h, __float2half2_rn(6.0f));
-    return h;
+__device__ __forceinline__ uint32_t round_act(float a, float b) {
+    uint32_t r;
+    if (ACT == 0) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    else asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+    if (ACT == 2) {
+        const __half2 h = __hmin2(*reinterpret_cast<const __half2*>(&r), __float2half2_rn(6.0f));
+        r = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    return r;
 }
 
 }  // namespace dlf

@@ -100,7 +100,7 @@ __device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint64_t ad, uint64_
     }
 }
 
-template <int CIN>
+template <int CIN, int ACT>
 __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_constant__ CUtensorMap tmy, const StemParams p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t wfull_bar, pfull_bar[2], pempty_bar[2], tfull_bar[kGroups], tempty_bar[kGroups];
@@ -304,7 +304,6 @@ __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_const
         const int q = warp & 3;
         const int m = q * 32 + lane;
         const bool issuer = (threadIdx.x & 127) == 0;
-        const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
         uint8_t* sout = sbase + p.stage_off + grp * kStage;
         uint32_t seq = 0, ph = 0;
         auto group_sync = [&]() {
@@ -340,13 +339,10 @@ __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_const
                     }
 #pragma unroll
                     for (int g = 0; g < 4; g++) {
-                        const float4 b0 = *reinterpret_cast<const float4*>(bias_s + cc + g * 8), b1 = *reinterpret_cast<const float4*>(bias_s + cc + g * 8 + 4);
-                        uint4 out;
-                        // (the activation as a clamp of the rounded pair: rounding is monotone and the bounds are fp16 values)
-                        out.x = pack_half2_clamp(__uint_as_float(r[g * 8 + 0]) + b0.x, __uint_as_float(r[g * 8 + 1]) + b0.y, act_lo, act_hi);
-                        out.y = pack_half2_clamp(__uint_as_float(r[g * 8 + 2]) + b0.z, __uint_as_float(r[g * 8 + 3]) + b0.w, act_lo, act_hi);
-                        out.z = pack_half2_clamp(__uint_as_float(r[g * 8 + 4]) + b1.x, __uint_as_float(r[g * 8 + 5]) + b1.y, act_lo, act_hi);
-                        out.w = pack_half2_clamp(__uint_as_float(r[g * 8 + 6]) + b1.z, __uint_as_float(r[g * 8 + 7]) + b1.w, act_lo, act_hi);
+                        const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bias_s + cc + g * 8), b1 = *reinterpret_cast<const ulonglong2*>(bias_s + cc + g * 8 + 4);
+                        const float2 v0 = add_f2(r[g * 8 + 0], r[g * 8 + 1], b0.x), v1 = add_f2(r[g * 8 + 2], r[g * 8 + 3], b0.y);
+                        const float2 v2 = add_f2(r[g * 8 + 4], r[g * 8 + 5], b1.x), v3 = add_f2(r[g * 8 + 6], r[g * 8 + 7], b1.y);
+                        const uint4 out = make_uint4(round_act<ACT>(v0.x, v0.y), round_act<ACT>(v1.x, v1.y), round_act<ACT>(v2.x, v2.y), round_act<ACT>(v3.x, v3.y));
                         const int g8 = (cc >> 3) + g;
                         *reinterpret_cast<uint4*>(sout + m * 128 + (((g8 & 7) ^ (m & 7)) << 4)) = out;
                     }
@@ -436,13 +432,17 @@ bool input_ok(const ConvArgs& a) {
 }
 
 typedef void (*KernelFn)(const CUtensorMap, const StemParams);
-KernelFn pick_kernel(int cin) {
+template <int ACT>
+KernelFn pick_kernel_act(int cin) {
     switch (cin) {
-        case 1: return stem_tc_kernel<1>;
-        case 2: return stem_tc_kernel<2>;
-        case 3: return stem_tc_kernel<3>;
-        default: return stem_tc_kernel<4>;
+        case 1: return stem_tc_kernel<1, ACT>;
+        case 2: return stem_tc_kernel<2, ACT>;
+        case 3: return stem_tc_kernel<3, ACT>;
+        default: return stem_tc_kernel<4, ACT>;
     }
+}
+KernelFn pick_kernel(int cin, int act) {
+    return act == DLF_ACT_RELU6 ? pick_kernel_act<2>(cin) : (act == DLF_ACT_RELU ? pick_kernel_act<1>(cin) : pick_kernel_act<0>(cin));
 }
 
 }  // namespace
@@ -458,8 +458,8 @@ int stem_tc_init() {
     const int dev = current_device_slot();
     if (dev < 0) return DLF_E_UNSUPPORTED;
     if (!attr_set[dev]) {
-        for (int cin = 1; cin <= 4; cin++) {
-            cudaError_t e = cudaFuncSetAttribute(pick_kernel(cin), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+        for (int v = 0; v < 12; v++) {
+            cudaError_t e = cudaFuncSetAttribute(pick_kernel(1 + v / 3, v % 3), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         attr_set[dev] = true;
@@ -509,7 +509,7 @@ int launch_stem_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_
     }
     const int grid = std::max(1, std::min(sm_count, p.n_work));
     const size_t smem = std::max<size_t>(l.smem, 120 * 1024);   // (one CTA of a persistent grid per SM)
-    cudaError_t e = launch_kernel(pick_kernel(a.Cin), grid, kThreads, smem, s, tmy, p);
+    cudaError_t e = launch_kernel(pick_kernel(a.Cin, a.act), grid, kThreads, smem, s, tmy, p);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
