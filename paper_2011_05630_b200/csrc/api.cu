@@ -469,28 +469,48 @@ static bool make_group(const dlf_net* net, int first, int last, int sms, Group* 
 // ---- what the tuner may propose as one group --------------------------------------------------------------------
 // Algorithm 1 grows a block while the layers can run as one kernel AND that kernel is expected to pay (Sec. IV-B: fusing
 // helps layers with few operations and hurts heavy ones).  For a dense chain the estimate is the fused kernel's own cost
-// model (the tiler's SM clocks at 1.9 GHz, plus one kernel boundary) against one kernel per layer: the slower of a layer's
-// operations at 600 TFLOP/s and its bytes at 5.5 TB/s (what the single-layer kernel reaches on this chip) plus 7 us of
-// fixed cost per kernel (measured: no single-layer kernel takes less inside a network); the group must win by 15 %
-// (estimate and measurement differ by up to a quarter either way; groups that merely break even lose inside a network).
+// model (the tiler's SM clocks at 1.9 GHz: measured 0.85 to 1.3 times as long) against one kernel per layer: 2.4 us (3x3: 3.1)
+// plus the slowest of the latency of its 64-channel chunks, its rounds of 128-pixel tiles (twice as long where a pixel's
+// channels are no multiple of 32 bytes), its operations at 600 TFLOP/s and its bytes at 5.5 TB/s.  Fitted to 90 random chains
+// of 2 to 8 layers timed both ways: 16 -> 16 3x3 at 5 images of 35x32 9.3 us fused against 12.3 for three layers, 24 -> 24 at
+// 10 of 81x79 66 against 113 for four, 64 -> 64 1x1 at 5 of 41x38 7.3 against 6.4 for two.
 // A chain may not swallow the expansion layer of an inverted-residual block (the layer a depthwise convolution reads):
 // that block fuses better as a whole.  Inverted-residual blocks follow the measured rule on the hidden width.  Groups
 // handed over through L2 are proposed only when the option asks for them (measured: a device-wide barrier per layer is no
 // cheaper than a kernel boundary).  `prefix`: the layers may also be the beginning of a pattern that can still grow.
-// The estimate for a dense chain handed over in shared memory: true if the fused kernel is expected to beat one kernel per
-// layer on `sms` SMs (see above).  `tiling` receives the fused kernel's tiling.
-static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling) {
+// A layer of a dense chain as a kernel of its own inside a network (see above).
+static double single_layer_us(const Layer& l, int sms) {
+    const double chunks = static_cast<double>(l.d.kh * l.d.kw * ((l.d.cin + 63) / 64));
+    const double rounds = static_cast<double>(l.in[0] * l.in[1] * l.in[2]) / (128.0 * sms) * ((l.d.cout + 255) / 256);
+    const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
+                         (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
+    return 2.4 + (l.d.kh == 3 ? 0.7 : 0.0) +
+           std::max({0.1 * chunks, rounds * (0.75 + 0.3 * chunks) * (l.d.cin % 16 ? 2.0 : 1.0), static_cast<double>(l.flops) / 600e6, bytes / 5.5e6});
+}
+// The chain first..last as one kernel; negative if it cannot run as one.
+static double chain_us(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling) {
     const ChainTiling t = chain_tc_tiling(chain_args(net, first, last, nullptr, nullptr), sms, net->dev_sms > 0 ? net->dev_sms : sms);
     if (tiling) *tiling = t;
-    if (!t.ok) return false;
-    double single_us = 0.0;
-    for (int i = first; i <= last; i++) {
-        const Layer& l = net->layers[i];
-        const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
-                             (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
-        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / 5.5e6) + 7.0;
+    return t.ok ? 1.1 * t.cost / 1.9e3 + 0.3 : -1.0;
+}
+// True if the fused kernel is expected to beat one kernel per layer on `sms` SMs.  `tiling` receives the fused kernel's tiling.
+static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling) {
+    const double fused = chain_us(net, first, last, sms, tiling);
+    double single = 0.0;
+    for (int i = first; i <= last; i++) single += single_layer_us(net->layers[i], sms);
+    return fused >= 0.0 && fused < 0.97 * single;
+}
+// True if a block that has reached layer last - 1 should go on: some longer chain from `first` beats the block so far and
+// single layers behind it (two 1x1 layers may not pay where three do; the longest chain that pays is rarely the best one).
+static bool chain_grows(const dlf_net* net, int first, int last, int sms) {
+    double rest = last - 1 == first ? single_layer_us(net->layers[first], sms) : chain_us(net, first, last - 1, sms, nullptr);
+    if (rest < 0.0) return false;
+    for (int e = last; e < static_cast<int>(net->layers.size()) && span_is_chain(net, first, e); e++) {
+        rest += single_layer_us(net->layers[e], sms);
+        const double fused = chain_us(net, first, e, sms, nullptr);
+        if (fused >= 0.0 && fused < 0.97 * rest) return true;
     }
-    return t.cost / 1.9e3 + 5.5 < 0.85 * single_us;
+    return false;
 }
 
 // The estimate for an inverted-residual block: the fused kernel's own cost model (the tiler's SM clocks, plus one kernel
@@ -528,7 +548,7 @@ static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix,
     const int n = static_cast<int>(net->layers.size());
     for (int i = first; i <= last; i++)
         if (i + 1 < n && net->layers[i + 1].d.op == DLF_DWCONV && net->layers[i + 1].d.src == i) return false;
-    return chain_pays(net, first, last, s_max, nullptr);
+    return prefix ? chain_grows(net, first, last, s_max) : chain_pays(net, first, last, s_max, nullptr);
 }
 
 static int launch_group(dlf_net* net, const Group& g, const void* in_dev, void* final_out, cudaStream_t s) {
