@@ -184,9 +184,11 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
 // arrival is made of bounded waits.)
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// Arrives on a barrier of any CTA of the cluster (an address from mapa()).
+// Arrives on a barrier of any CTA of the cluster (an address from mapa()).  The arrival publishes nothing but itself: what it
+// stands for is an accumulator that has been read (tcgen05.wait::ld), and a release at cluster scope would wait for every store
+// to shared memory before it (1100 clocks per tile of a CTA pair's epilogue).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 // Loads of a CTA pair: into this CTA's shared memory, completing on a barrier of either CTA (an address from mapa()).
 __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2) {
