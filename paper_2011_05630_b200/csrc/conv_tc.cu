@@ -27,6 +27,9 @@
 // start 0, 1 and 2 pixels into it; the window crosses L2 -> shared memory three times per chunk instead of nine.
 // Chosen where it cuts the bytes a CTA streams by a fifth or more (measured: 64 -> 128 at 112x112 34 -> 23 us,
 // 512 -> 512 at 14x14 23 -> 17 us, the ResNet-50 3x3 layers 8 % faster; neutral where the weight slabs dominate).
+// Column mode (3x3, stride 1, whole 64-channel chunks; also pooled): the same with the taps of a kernel column, which read the
+// window whole tile rows further: see set_tile_col.  128 -> 128 at 112x112 with a 2x2 pool, batch 8 30.2 -> 23.1 us, 512 -> 512
+// at 14x14 with a pool 19.4 -> 13.3, 64 -> 64 at 224x224 with a pool (in the fused-group kernel before) 47.9 -> 39.9.
 // The epilogue is specialised at compile time on (activation, pool, residual): it is the part of
 // the kernel that bounds memory-bound layers, and runtime branches there cost more than the math.
 #include <cuda.h>
@@ -61,7 +64,8 @@ struct ConvTcParams {
     int BN, n_tiles_n, acc_stride;
     int kchunks, ksteps_last;
     int a_bytes;               // one 64-channel slab of the tile's pixels in a ring stage: rows rounded up to 8, x 128 bytes
-    int tps, tgroups;          // taps per ring stage (3 = a whole kernel row, see the row mode) and tap groups per K-chunk group
+    int tps, tgroups;          // taps per ring stage (3 = a whole kernel row or column, see the row and column modes) and tap groups per K-chunk group
+    int a_rows, col, tap_rows; // pixels of a stage's window; 1: column mode; rows of the window from one tap of the stage to the next
     int kg, kgroups, grouped;  // K chunks per ring stage; stages per tap; 1 = 5-d / 4-d maps (cin % 64 == 0)
     int stages;
     int store_depth;              // TMA stores of finished tiles in flight (1 .. out_bufs)
@@ -247,12 +251,12 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 if (!grid_wait(gs, lane, abort_flag, p.status)) return;   // the input may be a layer of this launch
             }
             const uint32_t parity = role & 1;
-            const uint32_t my_bytes = static_cast<uint32_t>(p.kg) * (is_b ? static_cast<uint32_t>(kTps * b_rows) : static_cast<uint32_t>(p.rows)) * 128u;
+            const uint32_t my_bytes = static_cast<uint32_t>(p.kg) * (is_b ? static_cast<uint32_t>(kTps * b_rows) : static_cast<uint32_t>(p.a_rows)) * 128u;
             uint32_t it = 0;
             bool ok = true;
             DLF_TRACE_DECL(pacc, pmark);  // cycles of CTA 0's producers: 0 wait for a free stage, 1 issue
-            // One ring stage: K-chunk group kq of tap group tg (row mode: tap group tg = kernel row tg, its window
-            // loaded once at the row's first tap).  False once a wait has given up.
+            // One ring stage: K-chunk group kq of tap group tg (row and column modes: kernel row or column r = tg, its window
+            // loaded once).  False once a wait has given up.
             // (ring position and phase are kept as counters: no division on the way to a copy)
             int ring_st = 0;
             uint32_t ring_ph = 0;
@@ -272,17 +276,18 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 __syncwarp();
                 if (lane < p.kg) {   // a chunk past C_in / 64 lies outside the tensor map and arrives as zeros
                     const int kc = kq * p.kg + lane;
-                    const bool second = kc >= p.kchunks1;   // (1x1 layers with whole 64-channel chunks only: see conv_tc_dual_supported)
+                    const bool second = !ROW && kc >= p.kchunks1;   // (1x1 layers with whole 64-channel chunks only: see conv_tc_dual_supported)
                     if constexpr (PAIR) {
                         const uint32_t bar = mapa(smem_u32(&sm.full_bar[st]), 0);
                         if (is_b) {
                             uint8_t* dst = sa + p.kg * p.a_bytes + lane * kTps * b_rows * 128;
                             const int co = c.co0 + rank * b_rows;
                             if (second) tma_load_4d_pair(dst, tmw2_p, bar, 0, co, 0, kc - p.kchunks1);
+                            else if (ROW) tma_load_5d_pair(dst, tmw_p, bar, 0, co, 0, r, kc);
                             else if (p.grouped) tma_load_4d_pair(dst, tmw_p, bar, 0, co, tap, kc);
                             else tma_load_3d_pair(dst, tmw_p, bar, kc * 64, tap, co);
                         } else {
-                            const int wi = c.wo0 * p.stride - p.pad + s, hi = c.ho0 * p.stride - p.pad + r;
+                            const int wi = c.wo0 * p.stride - p.pad + (ROW ? (p.col ? r : 0) : s), hi = c.ho0 * p.stride - p.pad + (ROW && p.col ? 0 : r);
                             uint8_t* dst = sa + lane * p.a_bytes;
                             if (second) tma_load_5d_pair(dst, tmx2_p, bar, 0, c.wo0 * p.stride2, c.ho0 * p.stride2, c.n0, kc - p.kchunks1);
                             else if (p.grouped) tma_load_5d_pair(dst, tmx_p, bar, 0, wi, hi, c.n0, kc);
@@ -291,10 +296,11 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                     } else if (is_b) {
                         uint8_t* dst = sa + p.kg * p.a_bytes + lane * kTps * p.BN * 128;
                         if (second) tma_load_4d(dst, tmw2_p, &sm.full_bar[st], 0, c.co0, 0, kc - p.kchunks1);
+                        else if (ROW) tma_load_5d(dst, tmw_p, &sm.full_bar[st], 0, c.co0, 0, r, kc);
                         else if (p.grouped) tma_load_4d(dst, tmw_p, &sm.full_bar[st], 0, c.co0, tap, kc);
                         else tma_load_3d(dst, tmw_p, &sm.full_bar[st], kc * 64, tap, c.co0);
                     } else {
-                        const int wi = c.wo0 * p.stride - p.pad + s, hi = c.ho0 * p.stride - p.pad + r;
+                        const int wi = c.wo0 * p.stride - p.pad + (ROW ? (p.col ? r : 0) : s), hi = c.ho0 * p.stride - p.pad + (ROW && p.col ? 0 : r);
                         uint8_t* dst = sa + lane * p.a_bytes;
                         if (second) tma_load_5d(dst, tmx2_p, &sm.full_bar[st], 0, c.wo0 * p.stride2, c.ho0 * p.stride2, c.n0, kc - p.kchunks1);
                         else if (p.grouped) tma_load_5d(dst, tmx_p, &sm.full_bar[st], 0, wi, hi, c.n0, kc);
@@ -338,6 +344,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
             else umma_commit(bar);
         };
         const uint32_t b_chunk16 = static_cast<uint32_t>(b_rows) * 8u;  // one 64-channel weight slab, in 16-byte units
+        const uint32_t tap16 = static_cast<uint32_t>(p.tap_rows) * 8u;
         const uint32_t a_chunk16 = static_cast<uint32_t>(p.a_bytes) >> 4;  // one 64-channel slab of the tile's pixels (rows rounded up to 8)
         uint32_t it = 0, j = 0, ring_ph = 0;
         int ring_st = 0;   // ring position and phase as counters: no division in the issue loop
@@ -381,13 +388,13 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                             else umma_f16_steps<1, PAIR>(d_tmem, ad, bd, idesc, (ki | g) != 0);
                         }
                     } else {
-                        // row mode (whole 64-channel chunks): the three taps of a kernel row read the same window, one
-                        // pixel (one 128-byte row) further each
+                        // row and column modes (whole 64-channel chunks): the three taps of a kernel row (column) read the same
+                        // window, one pixel = 128 bytes (one row of the tile) further each
 #pragma unroll 1
                         for (int g = 0; g < g_end; g++) {
                             uint32_t ad = a0 + static_cast<uint32_t>(g) * a_chunk16, bd = b0 + static_cast<uint32_t>(g * 3) * b_chunk16;
 #pragma unroll
-                            for (int sx = 0; sx < 3; sx++, ad += 8, bd += b_chunk16) umma_f16_steps<4, PAIR>(d_tmem, ad, bd, idesc, (ki | g | sx) != 0);
+                            for (int sx = 0; sx < 3; sx++, ad += tap16, bd += b_chunk16) umma_f16_steps<4, PAIR>(d_tmem, ad, bd, idesc, (ki | g | sx) != 0);
                         }
                     }
                     commit(&sm.empty_bar[st]);  // frees the stage once these MMAs have read it
@@ -897,8 +904,7 @@ typedef void (*KernelFn)(const CUtensorMap, const CUtensorMap, const CUtensorMap
 
 template <int ACT, bool POOL, bool RES>
 KernelFn pick_row(bool row) {
-    if constexpr (POOL) return conv_tc_kernel<ACT, POOL, RES, false, false>;   // the row mode has no pooled epilogue
-    else return row ? conv_tc_kernel<ACT, POOL, RES, true, false> : conv_tc_kernel<ACT, POOL, RES, false, false>;
+    return row ? conv_tc_kernel<ACT, POOL, RES, true, false> : conv_tc_kernel<ACT, POOL, RES, false, false>;
 }
 template <int ACT, bool POOL>
 KernelFn pick_res(bool res, bool row) {
@@ -911,6 +917,7 @@ KernelFn pick_pool(bool pool, bool res, bool row) {
 // CTA-pair variants
 template <int ACT>
 KernelFn pick_pair_act(bool pool, bool res, bool row) {
+    if (pool && row) return res ? conv_tc_pair_kernel<ACT, true, true, true> : conv_tc_pair_kernel<ACT, true, false, true>;
     if (pool) return res ? conv_tc_pair_kernel<ACT, true, true, false> : conv_tc_pair_kernel<ACT, true, false, false>;
     if (row) return res ? conv_tc_pair_kernel<ACT, false, true, true> : conv_tc_pair_kernel<ACT, false, false, true>;
     return res ? conv_tc_pair_kernel<ACT, false, true, false> : conv_tc_pair_kernel<ACT, false, false, false>;
@@ -1005,6 +1012,9 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         tl = t;
         p.TW = tl.tw; p.TH = tl.th; p.TN = tl.tn;
         p.rows = tl.tw * tl.th * tl.tn;
+        p.col = 0;
+        p.a_rows = p.rows;
+        p.tap_rows = 1;
         p.a_bytes = (p.rows + 7) / 8 * 8 * 128;
         p.tiles_w = (a.Wo + tl.tw - 1) / tl.tw;
         p.tiles_h = (a.Ho + tl.th - 1) / tl.th;
@@ -1048,7 +1058,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
             // the UMMA always reads 128 rows of a slab (two more in the row mode): behind a shorter one it reads on
             // into whatever follows (those accumulator rows are never stored), which must still be this CTA's
             // shared memory
-            const int fixed = p.out_bufs * p.out_buf_bytes + bias_bytes + 1024 + (kABytes + 256 - p.a_bytes);
+            const int fixed = p.out_bufs * p.out_buf_bytes + bias_bytes + 1024 + std::max(0, kABytes + 256 - p.a_bytes);
             // K chunks per ring stage: every stage costs the issuing threads a fixed handshake (barrier wait,
             // TMA issue, commit), so a stage carries as many 64-channel chunks as leave room for >= 2 stages
             p.kg = 1;
@@ -1107,8 +1117,22 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         const double k = static_cast<double>(p.tgroups) * p.kchunks;
         const double fill = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / (p.stages > 2 ? 57.0 : 50.0);
         const double umma = p.BN > 128 ? p.BN * 0.53 : (pair && p.BN <= 64 ? 56.0 : 72.0);
-        const double mma = k * p.tps * 4 * umma + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 500.0 : 200.0);
+        double mma = k * p.tps * 4 * umma + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 500.0 : 200.0);
+        // column mode: bound by shared memory itself, 128 bytes per clock for the UMMAs' operands (4 KB of pixels and 32 bytes per
+        // row of B that this CTA holds), the copies that arrive and the staged output
+        const double b_rows = pair ? p.BN / 2 : p.BN;
+        if (p.col) mma = k * (p.tps * 4 * std::max(p.BN * 0.53, 32.0 + b_rows / 4) + (p.a_bytes + p.tps * b_rows * 128) / 128) + p.rows * p.BN / 32.0 + p.tgroups * p.kgroups * 100.0;
         return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + p.BN * 14.0 + (pair ? 1400.0 : 0.0);
+    };
+    // Column mode (3x3, stride 1, pad 1, whole 64-channel chunks): a tile is TW x TH pixels with TW a multiple of 8, and a stage's
+    // window its TH + 2 rows at one kernel column's offset: the three taps of the column read it 0, 1 and 2 tile rows further, on
+    // whole swizzle atoms, where the row mode's windows start one pixel apart and the tensor core reads every atom twice.
+    auto set_tile_col = [&](int tw, int th) {
+        set_tile(Tile{tw, th, 1}, 3);
+        p.col = 1;
+        p.a_rows = tw * (th + 2);
+        p.tap_rows = tw;
+        p.a_bytes = p.a_rows * 128;
     };
     // Row mode (3x3, stride 1, pad 1): a tile is TH whole output rows seen with a pitch of Wo + 2, pixel-linear like
     // its input window, so that the three taps of a kernel row read ONE loaded window through descriptors that
@@ -1236,6 +1260,44 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         bias_bytes = found ? best_bias : keep_bias;
         m_tiles = found ? best_m : keep_m;
     }
+    if (g_conv_row_mode > 0 && allow_pair && splits == 1 && a.kh == 3 && a.kw == 3 && a.stride == 1 && a.pad == 1 && p.grouped && a.W == a.Wo && a.H == a.Ho) {
+        const ConvTcParams keep = p;
+        const Tile keep_tl = tl;
+        const int keep_bias = bias_bytes;
+        const long long keep_m = m_tiles;
+        const bool keep_pair = pair;
+        double best = clocks();
+        ConvTcParams best_p{};
+        Tile best_tl{};
+        int best_bias = 0;
+        long long best_m = 0;
+        bool found = false, best_pair = false;
+        for (int tw = 8; tw <= 64 && tw < a.Wo + 8; tw += 8) {
+            if (a.pool && tw != 8 && tw != 16) continue;   // (2x2 windows are reduced by warp shuffles)
+            const int th_max = a.pool ? 128 / tw : std::min(a.Ho, 128 / tw), rows_h = (a.Ho + th_max - 1) / th_max;
+            set_tile_col(tw, a.pool ? th_max : (a.Ho + rows_h - 1) / rows_h);
+            for (int pr = 0; pr < 2; pr++) {
+                pair = pr != 0;
+                if (pair && (sm_count < 2 || m_tiles < 2)) continue;
+                for (int bn : {256, 192, 128, 64}) {
+                    bn_force = bn;
+                    if (!configure(kMaxSmem, 256, 2)) continue;
+                    const double c = clocks();
+                    if (c < best) {
+                        best = c;
+                        best_p = p; best_tl = tl; best_bias = bias_bytes; best_m = m_tiles; best_pair = pair;
+                        found = true;
+                    }
+                }
+            }
+        }
+        bn_force = 0;
+        pair = found ? best_pair : keep_pair;
+        p = found ? best_p : keep;
+        tl = found ? best_tl : keep_tl;
+        bias_bytes = found ? best_bias : keep_bias;
+        m_tiles = found ? best_m : keep_m;
+    }
     // stores in flight: all buffers but one where a buffer also has to take the next tile's residual in time
     p.store_depth = std::max(1, a.res ? p.out_bufs - 1 : p.out_bufs);
     p.splits = splits;
@@ -1263,17 +1325,26 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
                                   static_cast<uint64_t>(a.Cin / 64)};
         const uint64_t strides[4] = {static_cast<uint64_t>(a.Cin) * 2, static_cast<uint64_t>(a.W) * a.Cin * 2,
                                      static_cast<uint64_t>(a.H) * a.W * a.Cin * 2, 128};
-        const uint32_t box[5] = {64, static_cast<uint32_t>(tl.tw * a.stride), static_cast<uint32_t>(tl.th * a.stride),
+        const uint32_t box[5] = {64, static_cast<uint32_t>(tl.tw * a.stride), static_cast<uint32_t>((tl.th + (p.col ? 2 : 0)) * a.stride),
                                  static_cast<uint32_t>(tl.tn), 1};
         const uint32_t es[5] = {1, static_cast<uint32_t>(a.stride), static_cast<uint32_t>(a.stride), 1, 1};
         int rc = encode_tmap(&tmx, a.x, 5, dims, strides, box, es);
         if (rc) return rc;
         // weights [cout][tap][cin] seen as (64 channels, cout, tap, C_in / 64)
-        const uint64_t wdims[4] = {64, static_cast<uint64_t>(a.Cout), taps64, static_cast<uint64_t>(a.Cin / 64)};
-        const uint64_t wstrides[3] = {taps64 * a.Cin * 2, static_cast<uint64_t>(a.Cin) * 2, 128};
-        const uint32_t wbox[4] = {64, w_rows, static_cast<uint32_t>(p.tps), 1};
-        const uint32_t wes[4] = {1, 1, 1, 1};
-        rc = encode_tmap(&tmw, a.w, 4, wdims, wstrides, wbox, wes);
+        if (p.tps == 3) {   // ... the taps as (within the kernel row or column, kernel row or column)
+            const uint64_t row = static_cast<uint64_t>(a.Cin) * 6, px = static_cast<uint64_t>(a.Cin) * 2;
+            const uint64_t wdims[5] = {64, static_cast<uint64_t>(a.Cout), 3, 3, static_cast<uint64_t>(a.Cin / 64)};
+            const uint64_t wstrides[4] = {taps64 * a.Cin * 2, p.col ? row : px, p.col ? px : row, 128};
+            const uint32_t wbox[5] = {64, w_rows, 3, 1, 1};
+            const uint32_t wes[5] = {1, 1, 1, 1, 1};
+            rc = encode_tmap(&tmw, a.w, 5, wdims, wstrides, wbox, wes);
+        } else {
+            const uint64_t wdims[4] = {64, static_cast<uint64_t>(a.Cout), taps64, static_cast<uint64_t>(a.Cin / 64)};
+            const uint64_t wstrides[3] = {taps64 * a.Cin * 2, static_cast<uint64_t>(a.Cin) * 2, 128};
+            const uint32_t wbox[4] = {64, w_rows, static_cast<uint32_t>(p.tps), 1};
+            const uint32_t wes[4] = {1, 1, 1, 1};
+            rc = encode_tmap(&tmw, a.w, 4, wdims, wstrides, wbox, wes);
+        }
         if (rc) return rc;
     } else {
         const uint64_t dims[4] = {static_cast<uint64_t>(a.Cin), static_cast<uint64_t>(a.W), static_cast<uint64_t>(a.H),
@@ -1329,7 +1400,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
     out->grid = pair ? 2 * std::max(1, std::min(sm_count / 2, p.n_work)) : std::max(1, std::min(sm_count, p.n_work));
     out->pair = pair;
     // never two of these CTAs on an SM: each may hold all of tensor memory
-    out->smem = std::max<size_t>(static_cast<size_t>(p.bias_off) + bias_bytes + 1024 + (kABytes + 256 - p.a_bytes), 120 * 1024);
+    out->smem = std::max<size_t>(static_cast<size_t>(p.bias_off) + bias_bytes + 1024 + std::max(0, kABytes + 256 - p.a_bytes), 120 * 1024);
 #ifdef DLF_TRACE
     fprintf(stderr, "conv_tc: tile %dx%dx%d rows %d BN %d x %d splits %d kgs %d kg %d kgroups %d stages %d out_bufs %d work %d grid %d\n", tl.tn, tl.th, tl.tw,
             p.rows, p.BN, p.n_tiles_n, p.splits, p.kgs, p.kg, p.kgroups, p.stages, p.out_bufs, p.n_work, out->grid);
@@ -1396,7 +1467,7 @@ int conv_tc_init() {
         for (int act = 0; act < 3; act++)
             for (int pool = 0; pool < 2; pool++)
                 for (int res = 0; res < 2; res++)
-                    for (int row = 0; row < (pool ? 1 : 2); row++) {
+                    for (int row = 0; row < 2; row++) {
                         cudaError_t e = cudaFuncSetAttribute(pick_kernel(act, pool != 0, res != 0, row != 0),
                                                              cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
                         if (e == cudaSuccess) e = cudaFuncSetAttribute(pick_pair(act, pool != 0, res != 0, row != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
