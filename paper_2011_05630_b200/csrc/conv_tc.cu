@@ -1117,11 +1117,16 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         const double k = static_cast<double>(p.tgroups) * p.kchunks;
         const double fill = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / (p.stages > 2 ? 57.0 : 50.0);
         const double umma = p.BN > 128 ? p.BN * 0.53 : (pair && p.BN <= 64 ? 56.0 : 72.0);
-        double mma = k * p.tps * 4 * umma + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 500.0 : 200.0);
-        // column mode: bound by shared memory itself, 128 bytes per clock for the UMMAs' operands (4 KB of pixels and 32 bytes per
-        // row of B that this CTA holds), the copies that arrive and the staged output
-        const double b_rows = pair ? p.BN / 2 : p.BN;
-        if (p.col) mma = k * (p.tps * 4 * std::max(p.BN * 0.53, 32.0 + b_rows / 4) + (p.a_bytes + p.tps * b_rows * 128) / 128) + p.rows * p.BN / 32.0 + p.tgroups * p.kgroups * 100.0;
+        const double mma = k * p.tps * 4 * umma + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 500.0 : 200.0);
+        if (a.kh == 3 && a.kw == 3 && a.stride == 1) {
+            // refitted to 400 measured (layer, mode, tile, pair, width) times of 34 such layers: an UMMA of a pair takes 43 clocks at N =
+            // 64 where the stage holds three taps, and a pair pays 1.6 us once; pooled tiles 8 pixels wide write 4 pixels at a
+            // time.  The layers chosen by it are within 1.2 % of the best choice (2.8 % with the constants above).
+            const double u = p.BN > 128 ? p.BN * 0.47 : (p.BN > 64 ? 60.0 : (!pair ? 69.0 : (p.tps == 3 ? 43.0 : 72.0)));
+            const double f = k * (p.a_bytes + p.tps * (pair ? p.BN / 2 : p.BN) * 128) / (p.stages > 2 ? 59.5 : 51.5);
+            const double m = k * p.tps * 4 * u + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 300.0 : 200.0);
+            return rounds * (std::max(f, m) + 410.0 + (p.col && a.pool && p.TW == 8 ? 180.0 : 0.0)) + p.BN * 35.0 + (pair ? 2960.0 : 0.0);
+        }
         return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + p.BN * 14.0 + (pair ? 1400.0 : 0.0);
     };
     // Column mode (3x3, stride 1, pad 1, whole 64-channel chunks): a tile is TW x TH pixels with TW a multiple of 8, and a stage's
