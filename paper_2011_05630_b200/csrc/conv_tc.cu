@@ -1127,7 +1127,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
             const double m = k * p.tps * 4 * u + p.tgroups * p.kgroups * (pair && p.tps * p.kg == 1 ? 300.0 : 200.0);
             return rounds * (std::max(f, m) + 410.0 + (p.col && a.pool && p.TW == 8 ? 180.0 : 0.0)) + p.BN * 35.0 + (pair ? 2960.0 : 0.0);
         }
-        return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 22.0 + 600.0) + p.BN * 14.0 + (pair ? 1400.0 : 0.0);
+        return rounds * (std::max(fill, mma) + p.rows * p.BN * 2 * (a.res ? 2 : 1) / 31.0 + 600.0) + p.BN * 14.0 + (pair ? 2600.0 : 0.0);
     };
     // Column mode (3x3, stride 1, pad 1, whole 64-channel chunks): a tile is TW x TH pixels with TW a multiple of 8, and a stage's
     // window its TH + 2 rows at one kernel column's offset: the three taps of the column read it 0, 1 and 2 tile rows further, on
@@ -1220,88 +1220,48 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
             bias_bytes = keep_bias;
         }
     }
-    // CTA pairs: either CTA fills half of the weight slab, so an item streams fewer bytes per UMMA; taken where the estimate says
-    // that this outweighs the coarser work items.
-    if (allow_pair && splits == 1 && sm_count >= 2 && m_tiles >= 2) {
-        const ConvTcParams keep = p;
-        const Tile keep_tl = tl;
-        const int keep_bias = bias_bytes;
-        const long long keep_m = m_tiles;
+    // CTA pairs (either CTA fills half of the weight slab, so an item streams fewer bytes per UMMA), the image-shaped tile with every
+    // channel width, and the column mode: whatever the estimate says is fastest.  (A second source was measured without pairs
+    // only.)  512 -> 512 1x1 at eight 60x60 images 21.5 -> 19.4 us against the width alone, 128 -> 128 3x3 stride 2 at 28x28, batch 32 16.4 ->
+    // 13.8, 128 -> 512 1x1 there 11.8 -> 10.7.
+    if (allow_pair && splits == 1) {
+        struct Layout { ConvTcParams p; Tile tl; int bias_bytes; long long m_tiles; bool pair; };
+        Layout best_l{p, tl, bias_bytes, m_tiles, pair};
         double best = clocks();
-        ConvTcParams best_p{};
-        Tile best_tl{};
-        int best_bias = 0;
-        long long best_m = 0;
-        bool found = false;
-        pair = true;
-        for (int mode = 0; mode < 2; mode++) {
-            if (mode == 1) {
-                if (!row_mode) continue;
-                set_tile(tl_row, 3);
-            } else {
-                if (flat) set_tile(Tile{std::min(128, a.Wo), 1, 1}, 1);
-                else set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
-            }
+        auto consider = [&](int pr) {   // the tile that is set, every channel width
+            pair = pr != 0;
+            if (pair && (dual || sm_count < 2 || m_tiles < 2)) return;
             for (int bn : {256, 192, 128, 64}) {
                 bn_force = bn;
                 if (!configure(kMaxSmem, 256, 2)) continue;
-                // (with one window load per tap and a narrow channel tile little is saved: 128 -> 128 3x3 stride 2 at 28x28, batch
-                // 32, 7.8 us alone, 8.5 us in pairs; 1x1 layers only with four times as many input as output channels: 512 -> 128
-                // at 28x28, batch 32, 10.1 -> 9.3 us, 256 -> 1024 at 14x14 8.5 -> 10.4 us)
-                const bool one = a.kh * a.kw == 1;
-                if (mode == 0 && !a.pool && (one ? dual || a.Cin < 4 * a.Cout : p.BN < 192)) continue;
                 const double c = clocks();
                 if (c < best) {
                     best = c;
-                    best_p = p; best_tl = tl; best_bias = bias_bytes; best_m = m_tiles;
-                    found = true;
+                    best_l = Layout{p, tl, bias_bytes, m_tiles, pair};
                 }
             }
-        }
-        bn_force = 0;
-        pair = found;
-        p = found ? best_p : keep;
-        tl = found ? best_tl : keep_tl;
-        bias_bytes = found ? best_bias : keep_bias;
-        m_tiles = found ? best_m : keep_m;
-    }
-    if (g_conv_row_mode > 0 && allow_pair && splits == 1 && a.kh == 3 && a.kw == 3 && a.stride == 1 && a.pad == 1 && p.grouped && a.W == a.Wo && a.H == a.Ho) {
-        const ConvTcParams keep = p;
-        const Tile keep_tl = tl;
-        const int keep_bias = bias_bytes;
-        const long long keep_m = m_tiles;
-        const bool keep_pair = pair;
-        double best = clocks();
-        ConvTcParams best_p{};
-        Tile best_tl{};
-        int best_bias = 0;
-        long long best_m = 0;
-        bool found = false, best_pair = false;
-        for (int tw = 8; tw <= 64 && tw < a.Wo + 8; tw += 8) {
-            if (a.pool && tw != 8 && tw != 16) continue;   // (2x2 windows are reduced by warp shuffles)
-            const int th_max = a.pool ? 128 / tw : std::min(a.Ho, 128 / tw), rows_h = (a.Ho + th_max - 1) / th_max;
-            set_tile_col(tw, a.pool ? th_max : (a.Ho + rows_h - 1) / rows_h);
-            for (int pr = 0; pr < 2; pr++) {
-                pair = pr != 0;
-                if (pair && (sm_count < 2 || m_tiles < 2)) continue;
-                for (int bn : {256, 192, 128, 64}) {
-                    bn_force = bn;
-                    if (!configure(kMaxSmem, 256, 2)) continue;
-                    const double c = clocks();
-                    if (c < best) {
-                        best = c;
-                        best_p = p; best_tl = tl; best_bias = bias_bytes; best_m = m_tiles; best_pair = pair;
-                        found = true;
-                    }
-                }
+        };
+        const bool three = a.kh == 3 && a.kw == 3 && a.stride == 1;
+        for (int pr = 0; pr < 2; pr++) {
+            if (!(three && pr == 0)) {
+                if (flat && pr) set_tile(Tile{std::min(128, a.Wo), 1, 1}, 1);
+                else set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
+                consider(pr);
             }
+            if (row_mode && pr) {
+                set_tile(tl_row, 3);
+                consider(pr);
+            }
+            if (g_conv_row_mode > 0 && three && a.pad == 1 && p.grouped && a.W == a.Wo && a.H == a.Ho)
+                for (int tw = 8; tw <= 64 && tw < a.Wo + 8; tw += 8) {
+                    if (a.pool && tw != 8 && tw != 16) continue;   // (2x2 windows are reduced by warp shuffles)
+                    const int th_max = a.pool ? 128 / tw : std::min(a.Ho, 128 / tw), rows_h = (a.Ho + th_max - 1) / th_max;
+                    set_tile_col(tw, a.pool ? th_max : (a.Ho + rows_h - 1) / rows_h);
+                    consider(pr);
+                }
         }
         bn_force = 0;
-        pair = found ? best_pair : keep_pair;
-        p = found ? best_p : keep;
-        tl = found ? best_tl : keep_tl;
-        bias_bytes = found ? best_bias : keep_bias;
-        m_tiles = found ? best_m : keep_m;
+        p = best_l.p; tl = best_l.tl; bias_bytes = best_l.bias_bytes; m_tiles = best_l.m_tiles; pair = best_l.pair;
     }
     // stores in flight: all buffers but one where a buffer also has to take the next tile's residual in time
     p.store_depth = std::max(1, a.res ? p.out_bufs - 1 : p.out_bufs);
