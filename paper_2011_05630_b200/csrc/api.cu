@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <limits>
 #include <new>
 #include <vector>
@@ -414,7 +415,8 @@ static bool single_kind(const dlf_net* net, int i, Kind* kind) {
     return false;
 }
 
-static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling);
+typedef std::map<std::pair<int, int>, double> SpanTimes;
+static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling, SpanTimes* memo = nullptr);
 
 static bool make_group(const dlf_net* net, int first, int last, int sms, Group* g) {
     g->first = first; g->last = last; g->sms = sms;
@@ -491,31 +493,39 @@ static double single_layer_us(const Layer& l, int sms) {
     const double rounds = static_cast<double>(l.in[0] * l.in[1] * l.in[2]) / (128.0 * sms) * ((l.d.cout + 255) / 256);
     const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
                          (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
+    if (l.d.kh == 1 && l.d.cin <= 64 && l.d.cout <= 64) return 2.0 + bytes / 5e6;   // (streams its bytes: conv_narrow.cu)
     return 2.4 + (l.d.kh == 3 ? 0.7 : 0.0) +
            std::max({0.1 * chunks, rounds * (0.75 + 0.3 * chunks) * (l.d.cin % 16 ? 2.0 : 1.0), static_cast<double>(l.flops) / 600e6, bytes / 5.5e6});
 }
 // The chain first..last as one kernel; negative if it cannot run as one.
-static double chain_us(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling) {
+// (`memo`: the spans of one tuner pass, each asked for several times; tiling a span takes 0.1 ms)
+static double chain_us(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling, SpanTimes* memo = nullptr) {
+    if (memo) {
+        const auto it = memo->find({first, last});
+        if (it != memo->end()) return it->second;
+        return (*memo)[{first, last}] = chain_us(net, first, last, sms, tiling);
+    }
     const ChainTiling t = chain_tc_tiling(chain_args(net, first, last, nullptr, nullptr), sms, net->dev_sms > 0 ? net->dev_sms : sms);
     if (tiling) *tiling = t;
     return t.ok ? 1.1 * t.cost / 1.9e3 + 0.3 : -1.0;
 }
 // True if the fused kernel is expected to beat one kernel per layer on `sms` SMs.  `tiling` receives the fused kernel's tiling.
-static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling) {
-    const double fused = chain_us(net, first, last, sms, tiling);
+static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling, SpanTimes* memo) {
+    const double fused = chain_us(net, first, last, sms, tiling, memo);
     double single = 0.0;
     for (int i = first; i <= last; i++) single += single_layer_us(net->layers[i], sms);
     return fused >= 0.0 && fused < 0.97 * single;
 }
 // True if a block that has reached layer last - 1 should go on: some longer chain from `first` beats the block so far and
 // single layers behind it (two 1x1 layers may not pay where three do; the longest chain that pays is rarely the best one).
-static bool chain_grows(const dlf_net* net, int first, int last, int sms) {
-    double rest = last - 1 == first ? single_layer_us(net->layers[first], sms) : chain_us(net, first, last - 1, sms, nullptr);
+static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTimes* memo) {
+    double rest = last - 1 == first ? single_layer_us(net->layers[first], sms) : chain_us(net, first, last - 1, sms, nullptr, memo);
     if (rest < 0.0) return false;
     for (int e = last; e < static_cast<int>(net->layers.size()) && span_is_chain(net, first, e); e++) {
         rest += single_layer_us(net->layers[e], sms);
-        const double fused = chain_us(net, first, e, sms, nullptr);
+        const double fused = chain_us(net, first, e, sms, nullptr, memo);
         if (fused >= 0.0 && fused < 0.97 * rest) return true;
+        if (fused < 0.0 || fused > 1.4 * rest) break;   // (longer ones only fall further behind)
     }
     return false;
 }
@@ -539,7 +549,7 @@ static bool mbconv_pays(const dlf_net* net, int first, int last, int sms) {
     return t.cost / 1.9e3 + 1.0 < single_us;
 }
 
-static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix, int s_max) {
+static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix, int s_max, SpanTimes* memo = nullptr) {
     if (first == last) return true;
     if (net->opt_no_tc) return false;
     if (span_is_mbconv(net, first, last, prefix)) {
@@ -555,7 +565,7 @@ static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix,
     const int n = static_cast<int>(net->layers.size());
     for (int i = first; i <= last; i++)
         if (i + 1 < n && net->layers[i + 1].d.op == DLF_DWCONV && net->layers[i + 1].d.src == i) return false;
-    return prefix ? chain_grows(net, first, last, s_max) : chain_pays(net, first, last, s_max, nullptr);
+    return prefix ? chain_grows(net, first, last, s_max, memo) : chain_pays(net, first, last, s_max, nullptr, memo);
 }
 
 // Some of the batch's images: every map is one image after another, so a group's part of the batch is the same launch from
@@ -1150,6 +1160,7 @@ int dlf_net_autotune(const dlf_net* net, const dlf_tuner_params* params, int* n_
     const int n = static_cast<int>(net->layers.size());
     double sum_op = 0.0, sum_mp = 0.0;
     int block = 0, start = 0, ng = 0;
+    SpanTimes memo;
     for (int i = 0; i < n; i++) {
         const Layer& l = net->layers[i];
         if (is_param(l)) {
@@ -1159,11 +1170,11 @@ int dlf_net_autotune(const dlf_net* net, const dlf_tuner_params* params, int* n_
         }
         // a block may grow while its layers are, or can still become, a group one kernel runs; it may
         // close only where they already are one (inside an inverted-residual block it keeps growing)
-        bool forced = (i == n - 1) || !tuner_may_fuse(net, start, i + 1, true, s_max);
-        const bool closable = (i == start) || tuner_may_fuse(net, start, i, false, s_max);
+        bool forced = (i == n - 1) || !tuner_may_fuse(net, start, i + 1, true, s_max, &memo);
+        const bool closable = (i == start) || tuner_may_fuse(net, start, i, false, s_max, &memo);
         if (!forced && params->legalise) {
             Group g;
-            if (i + 1 > start && tuner_may_fuse(net, start, i + 1, false, s_max))
+            if (i + 1 > start && tuner_may_fuse(net, start, i + 1, false, s_max, &memo))
                 forced = !make_group(net, start, i + 1, s_max, &g);
         }
         if (block > 0) {

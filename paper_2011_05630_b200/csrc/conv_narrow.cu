@@ -1,0 +1,148 @@
+// Pointwise (1x1, stride 1) convolution with at most 64 input channels: a stream of pixels in, a stream out, with so little
+// arithmetic per byte that memory is the only bound there should be.  The tcgen05 kernels spend 1700 clocks of hand-overs per
+// 128-pixel tile of such a layer (copy, UMMA, tensor memory, staging tile, TMA store), up to five times its bytes' time; here a
+// warp multiplies 16 pixels at a time in registers (mma.m16n8k16) and neither shared nor tensor memory is used.
+//
+// The order of K and of the output channels is free, so both are chosen for wide accesses: in a block of 32 input channels lane
+// c of a quad holds channels 8c .. 8c + 7 of its two pixels - one 16-byte load each, and one 16-byte load per weight row -
+// and the output channels are dealt out so that a lane ends up with 2 NT neighbouring ones of a pixel.  A warp keeps the weights
+// of 32 output channels in registers; the warps of wider layers share their pixels through L1.  Sums in fp32, then bias,
+// residual, activation, one rounding.
+// Measured: 32 -> 16 at 112x112, batch 64 41.0 -> 12.6 us (its bytes 11.9), 16 -> 96 there 99 -> 38, 24 -> 24 at 96x96, batch 16
+// 17.6 -> 4.5, 64 -> 64 at 28x28, batch 8 3.5 -> 3.1.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace dlf {
+
+namespace {
+
+constexpr int kWarps = 8;
+constexpr int kTiles = 2;   // 16-pixel tiles a warp has in flight
+
+__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// KB: blocks of 32 input channels; NT: eights of output channels of a warp (Cout = 8 NT blocks)
+template <int KB, int NT, int ACT>
+__global__ void __launch_bounds__(32 * kWarps) conv_narrow_kernel(const __half* __restrict__ x, const __half* __restrict__ w, const float* __restrict__ bias,
+                                                                   const __half* res, __half* y, int cin, int cout, int blocks, long long pixels) {
+    constexpr int kOwn = 2 * NT;   // neighbouring channels of a pixel that a lane finishes
+    const int warp = threadIdx.x >> 5, block = warp % blocks;   // the warp's block of 8 NT output channels; the warps of a CTA that share pixels
+    const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    pdl_launch_dependents();
+    uint4 wb[KB][NT];
+    float2 b2[NT];
+#pragma unroll
+    for (int t = 0; t < NT; t++) {
+        const int co = block * 8 * NT + (g >> 1) * kOwn + 2 * t + (g & 1);   // column g of the t-th eight
+#pragma unroll
+        for (int kb = 0; kb < KB; kb++) {
+            const int ci = kb * 32 + c * 8;
+            wb[kb][t] = ci < cin ? __ldg(reinterpret_cast<const uint4*>(w + co * cin + ci)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        b2[t] = make_float2(__ldg(bias + block * 8 * NT + c * kOwn + 2 * t), __ldg(bias + block * 8 * NT + c * kOwn + 2 * t + 1));
+    }
+    pdl_wait();
+    const int groups = static_cast<int>(blockDim.x >> 5) / blocks;   // pixel groups of the CTA
+    const long long step = static_cast<long long>(gridDim.x) * groups * 16 * kTiles;
+    for (long long p0 = (static_cast<long long>(blockIdx.x) * groups + warp / blocks) * 16 * kTiles; p0 < pixels; p0 += step) {
+        uint4 a[kTiles][KB][2];
+#pragma unroll
+        for (int m = 0; m < kTiles; m++)
+#pragma unroll
+            for (int h = 0; h < 2; h++)
+#pragma unroll
+                for (int kb = 0; kb < KB; kb++) {
+                    const long long px = p0 + m * 16 + h * 8 + g;
+                    const int ci = kb * 32 + c * 8;
+                    a[m][kb][h] = px < pixels && ci < cin ? __ldg(reinterpret_cast<const uint4*>(x + px * cin + ci)) : make_uint4(0u, 0u, 0u, 0u);
+                }
+#pragma unroll
+        for (int m = 0; m < kTiles; m++) {
+            float d[NT][4];
+#pragma unroll
+            for (int t = 0; t < NT; t++) {
+                d[t][0] = d[t][1] = d[t][2] = d[t][3] = 0.0f;
+#pragma unroll
+                for (int kb = 0; kb < KB; kb++) {
+                    const uint4 lo = a[m][kb][0], hi = a[m][kb][1], b = wb[kb][t];
+                    mma16816(d[t], lo.x, hi.x, lo.y, hi.y, b.x, b.y);
+                    mma16816(d[t], lo.z, hi.z, lo.w, hi.w, b.z, b.w);
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const long long px = p0 + m * 16 + h * 8 + g;
+                if (px >= pixels) continue;
+                const long long at = px * cout + block * 8 * NT + c * kOwn;
+                uint32_t out[NT];
+#pragma unroll
+                for (int t = 0; t < NT; t++) {
+                    float v0 = d[t][2 * h] + b2[t].x, v1 = d[t][2 * h + 1] + b2[t].y;
+                    if (res) {
+                        const float2 r = __half22float2(__ldg(reinterpret_cast<const __half2*>(res + at + 2 * t)));
+                        v0 += r.x;
+                        v1 += r.y;
+                    }
+                    out[t] = round_act<ACT>(v0, v1);
+                }
+                if (NT == 4) {
+                    *reinterpret_cast<uint4*>(y + at) = make_uint4(out[0], out[1 % NT], out[2 % NT], out[3 % NT]);
+                } else if (NT == 2) {
+                    *reinterpret_cast<uint2*>(y + at) = make_uint2(out[0], out[1 % NT]);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < NT; t++) *reinterpret_cast<uint32_t*>(y + at + 2 * t) = out[t];
+                }
+            }
+        }
+    }
+}
+
+typedef void (*KernelFn)(const __half*, const __half*, const float*, const __half*, __half*, int, int, int, long long);
+template <int KB, int NT>
+KernelFn pick_act(int act) {
+    return act == DLF_ACT_RELU6 ? conv_narrow_kernel<KB, NT, 2> : (act == DLF_ACT_RELU ? conv_narrow_kernel<KB, NT, 1> : conv_narrow_kernel<KB, NT, 0>);
+}
+template <int KB>
+KernelFn pick_nt(int nt, int act) {
+    switch (nt) {
+        case 1: return pick_act<KB, 1>(act);
+        case 2: return pick_act<KB, 2>(act);
+        case 3: return pick_act<KB, 3>(act);
+        default: return pick_act<KB, 4>(act);
+    }
+}
+
+}  // namespace
+
+int launch_conv_narrow(const ConvArgs& a, int sm_count, cudaStream_t s) {
+    if (a.kh != 1 || a.kw != 1 || a.stride != 1 || a.pad != 0 || a.groups != 1 || a.pool || a.x2 || a.Cin % 8 || a.Cin > 64) return DLF_E_UNSUPPORTED;
+    if (a.Cout % 8 || (a.Cout > 32 && a.Cout % 32) || a.Cout > 32 * kWarps) return DLF_E_UNSUPPORTED;
+    const long long pixels = static_cast<long long>(a.N) * a.H * a.W;
+    // with two blocks of input channels and three or more of output channels this kernel's multiply-adds outweigh its bytes: it
+    // wins where the hand-overs of the few tiles count (64 -> 256 at eight 28x28 images 3.9 us against 5.1, at twelve 56x56 ones 9.1
+    // against 9.1, at 32 of them 18.9 against 13.8)
+    if (a.Cin > 32 && a.Cout > 64 && pixels * a.Cout > 3000000) return DLF_E_UNSUPPORTED;
+    // (and on few pixels the cluster kernel, whose weights are on their way before the layer before it ends: a network's six such
+    // layers on one 56x56 image take 2.5 us more here)
+    if (a.Cin > 32 && pixels < 5000) return DLF_E_UNSUPPORTED;
+    const int blocks = std::max(1, a.Cout / 32), groups = kWarps / blocks;
+    const long long ctas = (pixels + 16 * kTiles * groups - 1) / (16 * kTiles * groups);
+    const int grid = static_cast<int>(std::min<long long>(ctas, 4ll * sm_count)), nt = std::min(a.Cout / 8, 4);
+    cudaError_t e = launch_kernel(a.Cin <= 32 ? pick_nt<1>(nt, a.act) : pick_nt<2>(nt, a.act), grid, 32 * blocks * groups, 0, s,
+                                  static_cast<const __half*>(a.x), static_cast<const __half*>(a.w), a.bias, static_cast<const __half*>(a.res),
+                                  static_cast<__half*>(a.y), a.Cin, a.Cout, blocks, pixels);
+    return e == cudaSuccess ? DLF_OK : cuda_fail(e);
+}
+
+}  // namespace dlf

@@ -1380,6 +1380,8 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
 int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s) {
     int rc = conv_tc_init();
     if (rc) return rc;
+    rc = launch_conv_narrow(a, sm_count, s);
+    if (rc != DLF_E_UNSUPPORTED) return rc;
     rc = launch_conv_lat(a, sm_count, status_dev, s);
     if (rc != DLF_E_UNSUPPORTED) return rc;
     ConvTcLaunch L;

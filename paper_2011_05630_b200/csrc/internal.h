@@ -147,6 +147,7 @@ bool chain_tc_layer_supported(int cin, int cout, int k);
 int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s);
 // conv_lat.cu: the same layers without pooling where one tile per CTA covers them; DLF_E_UNSUPPORTED: not such a layer.
 int conv_lat_init();
+int launch_conv_narrow(const ConvArgs& a, int sm_count, cudaStream_t s);   // DLF_E_UNSUPPORTED: not a layer of its kind
 int launch_conv_lat(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s);
 // Several layers as one persistent kernel with device-wide barriers between them (conv_tc.cu).
 bool conv_seq_layer_supported(const ConvArgs& a);
