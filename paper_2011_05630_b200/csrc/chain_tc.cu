@@ -515,7 +515,6 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         // ---- UMMA issuer: the whole warp walks the loops (warp-uniform addresses), one elected lane issues ----
         // Ring positions and phases are kept as counters: a division by a run-time value costs this single warp about a
         // hundred cycles, and the loop around a weight box issues as few as four instructions.
-        const uint64_t desc0 = umma_desc_sw128(0);
         uint32_t pass_inner = 0, pass_last = 0, act_ph = 0, w_ph = 0, in_ph = 0;   // (an array of the two would live in memory)
         int w_st = 0, in_rd = 0, in_j = 0;   // weight stage; input round within the slots and (streamed planes) plane within the round
         const int in_group = p.in_group, in_ring = p.in_ring, pitch = p.pitch, stages = p.stages;

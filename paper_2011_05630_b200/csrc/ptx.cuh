@@ -244,16 +244,8 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 // eight rows per 1024-byte swizzle atom, atoms of consecutive row groups 1024 bytes apart.
 // The swizzle is a function of the absolute shared-memory address (bits 7..9 select the XOR of
 // bits 4..6), so a start address on any 128-byte row of a 1024-byte-aligned buffer is valid with
-// base-offset field left at zero.
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);        // start address, 16-byte units
-    d |= static_cast<uint64_t>(1) << 16;                        // leading byte offset (unused here)
-    d |= static_cast<uint64_t>(1024 >> 4) << 32;                // stride byte offset between row groups
-    d |= static_cast<uint64_t>(1) << 46;                        // descriptor version of this architecture
-    d |= static_cast<uint64_t>(2) << 61;                        // 128-byte swizzle
-    return d;
-}
+// base-offset field left at zero.  umma_desc_lo() and kDescHiSw128 below are its two words: start address in 16-byte units and a
+// leading offset of 1 (unused); 1024 bytes between row groups, the descriptor version and the swizzle.
 // Instruction descriptor: fp16 x fp16 -> fp32, both operands K-major, M = 128, given N.
 __host__ __device__ constexpr uint32_t umma_idesc_f16(int n) {
     return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
@@ -262,14 +254,6 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int n) {
 // rows in either CTA; the descriptors' addresses hold in both.
 __host__ __device__ constexpr uint32_t umma_idesc_f16_pair(int n) {
     return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
-}
-__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 // The barrier at this offset in both CTAs of the pair gets one arrival when every UMMA issued so far has completed.
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
@@ -382,8 +366,6 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* m, const void* s
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // Waits until the committed stores have finished READING shared memory (the buffer may be reused).
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// ... all but the newest committed store have finished reading.
-__device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 // ... all but the newest `pending` (0..3) committed stores of this thread have finished reading.
 __device__ __forceinline__ void tma_store_wait_read_n(int pending) {
     if (pending <= 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -466,23 +448,12 @@ __device__ __forceinline__ void unpack_h2(uint32_t v, unsigned short& lo, unsign
     asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(v));
 }
 
-template <int ACT>
-__device__ __forceinline__ float act_t(float v) {
-    if (ACT >= 1) v = fmaxf(v, 0.0f);
-    if (ACT == 2) v = fminf(v, 6.0f);
-    return v;
-}
-
 __device__ __forceinline__ float apply_act(float v, int act) {
     if (act >= 1) v = fmaxf(v, 0.0f);
     if (act == 2) v = fminf(v, 6.0f);
     return v;
 }
 
-__device__ __forceinline__ uint32_t pack_half2(float a, float b) {
-    __half2 h = __floats2half2_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&h);
-}
 // Two values rounded to fp16, then clamped to [lo, hi] as a pair.  Rounding is monotone and the bounds used (0, 6, the
 // infinities) are fp16 values, so clamping after the rounding gives the same bits as clamping before it - at one
 // instruction per bound and PAIR instead of one per bound and value.
