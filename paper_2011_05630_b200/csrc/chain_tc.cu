@@ -723,8 +723,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
                 cx.obuf = sbase + p.act_off[l & 1];
                 cx.oplane = p.act_plane_bytes[l & 1];
                 cx.bl = bias_s + L.bias_off;
-                cx.act_lo = __float2half2_rn(L.act >= 1 ? 0.0f : -INFINITY);
-                cx.act_hi = __float2half2_rn(L.act == 2 ? 6.0f : INFINITY);
+                cx.act_lo = act_lo(L.act);
+                cx.act_hi = act_hi(L.act);
 #pragma unroll 1
                 for (int c = 0; c < L.n_chunks && ok; c++) {
                     cx.ncols = chunk_cols(L, c);
@@ -765,8 +765,8 @@ __global__ void __launch_bounds__(kThreads, 1) chain_tc_kernel(const __grid_cons
         cx.half = wb >> 2;
         cx.tmem_lane = tmem_base + (static_cast<uint32_t>((wb & 3) * 32) << 16);
         cx.bl = bias_s + LL.bias_off;
-        cx.act_lo = __float2half2_rn(LL.act >= 1 ? 0.0f : -INFINITY);
-        cx.act_hi = __float2half2_rn(LL.act == 2 ? 6.0f : INFINITY);
+        cx.act_lo = act_lo(LL.act);
+        cx.act_hi = act_hi(LL.act);
         cx.oplane = p.stg_plane_bytes;
         uint32_t pass_i = 0, use_i = 0;
         bool ok = true;

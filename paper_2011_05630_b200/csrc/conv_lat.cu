@@ -229,7 +229,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
         // ---- epilogue ----
         const int q = warp & 3, half = warp >> 2;
         [[maybe_unused]] const int bn8 = p.BN >> 3;
-        const __half2 act_lo = __float2half2_rn(p.act == DLF_ACT_NONE ? -INFINITY : 0.0f), act_hi = __float2half2_rn(p.act == DLF_ACT_RELU6 ? 6.0f : INFINITY);
+        const __half2 lo = act_lo(p.act), hi = act_hi(p.act);
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
         const int m = q * 32 + lane;
         // the sums of 16 columns of this thread's row, from both accumulators
@@ -289,7 +289,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
                         uint4 res = zero;
                         if (2 * j + g < kItems) res = rv[(2 * j + g) % kItems];
                         else if (p.res) res = __ldg(reinterpret_cast<const uint4*>(p.res + row + c));
-                        *reinterpret_cast<uint4*>(p.out + row + c) = finish8(v + g * 8, bias_s + c, res, act_lo, act_hi);
+                        *reinterpret_cast<uint4*>(p.out + row + c) = finish8(v + g * 8, bias_s + c, res, lo, hi);
                     }
                 }
             }
@@ -355,7 +355,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
                     b.x += b2.x; b.y += b2.y; b.z += b2.z; b.w += b2.w;
                 }
                 const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                *reinterpret_cast<uint4*>(p.out + off[it]) = finish8(v, bias_s + bias_at[it], rv[it], act_lo, act_hi);
+                *reinterpret_cast<uint4*>(p.out + off[it]) = finish8(v, bias_s + bias_at[it], rv[it], lo, hi);
             }
         }
     }

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
         for (int j = 0; j < 4; j++) bias[j] = __ldg(a.bias + c0 + j);
     }
     pdl_wait();   // (the weights above are constants)
-    const __half2 lo = __float2half2_rn(a.act >= 1 ? 0.0f : -INFINITY), hi = __float2half2_rn(a.act == 2 ? 6.0f : INFINITY);   // applied to rounded pairs
+    const __half2 lo = act_lo(a.act), hi = act_hi(a.act);   // applied to rounded pairs
     const __half* res = static_cast<const __half*>(a.res);
     const int in_row = a.W * a.Cin, out_row = a.Wo * a.Cout;
     for (long long i = tid; i < total; i += nthreads) {

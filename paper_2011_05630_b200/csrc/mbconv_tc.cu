@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) mbconv_tc_kernel(const __grid_con
         // A warp takes a lane quarter and every other 16-column slice, keeps the slice's biases in registers and has the next row
         // block's TMEM load in flight while it works on this one.
         const int q = warp & 3, half = (warp >> 2) & 1;
-        const __half2 lo1 = __float2half2_rn(p.act1 >= 1 ? 0.0f : -INFINITY), hi1 = __float2half2_rn(p.act1 == 2 ? 6.0f : INFINITY);
+        const __half2 lo1 = act_lo(p.act1), hi1 = act_hi(p.act1);
         int fyx[kMaxNb];   // frame position of this thread's row in each block, -1: no such row
 #pragma unroll
         for (int b = 0; b < kMaxNb; b++) {
@@ -402,8 +402,8 @@ __global__ void __launch_bounds__(kThreads, 1) mbconv_tc_kernel(const __grid_con
     } else {
         // ---- depthwise layer and epilogue 2 -----------------------------------------------------------------------------------
         const int q = warp & 3, half = (warp >> 2) & 1, gw = warp - kGroupWarps;
-        const __half2 lo2 = __float2half2_rn(p.act2 >= 1 ? 0.0f : -INFINITY), hi2 = __float2half2_rn(p.act2 == 2 ? 6.0f : INFINITY);
-        const __half2 lo3 = __float2half2_rn(p.act3 >= 1 ? 0.0f : -INFINITY), hi3 = __float2half2_rn(p.act3 == 2 ? 6.0f : INFINITY);
+        const __half2 lo2 = act_lo(p.act2), hi2 = act_hi(p.act2);
+        const __half2 lo3 = act_lo(p.act3), hi3 = act_hi(p.act3);
         DLF_TRACE_DECL(wacc, wmark);  // 0 hidden frame wait, 1 Hd wait, 2 depthwise, 3 projection wait, 4 epilogue 2
         auto depthwise = [&](uint32_t c, int hc) -> bool {
             const int jn = min(4, (p.hid - hc * 64) >> 4);

@@ -454,15 +454,19 @@ __device__ __forceinline__ float apply_act(float v, int act) {
     return v;
 }
 
-// Two values rounded to fp16, then clamped to [lo, hi] as a pair.  Rounding is monotone and the bounds used (0, 6, the
-// infinities) are fp16 values, so clamping after the rounding gives the same bits as clamping before it - at one
-// instruction per bound and PAIR instead of one per bound and value.
+// Two values rounded to fp16, then clamped to [lo, hi] as a pair.  Rounding is monotone and the bounds used (0 and 6) are
+// fp16 values, so clamping after the rounding gives the same bits as clamping before it - at one instruction per bound and
+// PAIR instead of one per bound and value.  An open bound is a NaN: min and max then return their other operand, whatever it
+// is.  A NaN stays one without an activation, and is 0 behind ReLU and ReLU6 (max(NaN, 0)), in every kernel (round_act).
+__device__ __forceinline__ __half2 act_lo(int act) { return __float2half2_rn(act >= 1 ? 0.0f : __int_as_float(0x7fffffff)); }
+__device__ __forceinline__ __half2 act_hi(int act) { return __float2half2_rn(act == 2 ? 6.0f : __int_as_float(0x7fffffff)); }
 __device__ __forceinline__ uint32_t pack_half2_clamp(float a, float b, __half2 lo, __half2 hi) {
     const __half2 h = __hmin2(__hmax2(__floats2half2_rn(a, b), lo), hi);
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 // Epilogue arithmetic in few instructions (it bounds the memory-bound layers): two fp32 additions at once, and a pair rounded
-// to fp16 with its activation (none, ReLU, ReLU6), ReLU being part of the conversion.
+// to fp16 with its activation (none, ReLU, ReLU6).  (The conversion's own ReLU would save the max - ResNet-50 b32 590.7 us instead
+// of 594.7, MobileNetV2 b64 543.8 instead of 553.1 - but it keeps a NaN, which ReLU6's min then turns into 6.)
 __device__ __forceinline__ float2 add_f2(uint32_t a0, uint32_t a1, uint64_t b) {
     uint64_t r;
     float2 f;
@@ -472,14 +476,10 @@ __device__ __forceinline__ float2 add_f2(uint32_t a0, uint32_t a1, uint64_t b) {
 }
 template <int ACT>
 __device__ __forceinline__ uint32_t round_act(float a, float b) {
-    uint32_t r;
-    if (ACT == 0) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    else asm("cvt.rn.relu.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
-    if (ACT == 2) {
-        const __half2 h = __hmin2(*reinterpret_cast<const __half2*>(&r), __float2half2_rn(6.0f));
-        r = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    return r;
+    __half2 h = __floats2half2_rn(a, b);
+    if (ACT >= 1) h = __hmax2(h, __float2half2_rn(0.0f));
+    if (ACT == 2) h = __hmin2(h, __float2half2_rn(6.0f));
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 }  // namespace dlf
