@@ -12,7 +12,9 @@
 //   stride 1: unit u = pixels u, u + 1 (each pixel stored twice); kernel columns 4i .. 4i+3 = units x + 4i, x + 4i + 2
 //   stride 2: unit u = pixels 2u, 2u + 1;                         kernel columns 4i .. 4i+3 = units x + 2i, x + 2i + 1
 //   stride 4: even and odd pairs in two planes;                   kernel columns 4i .. 4i+3 = unit x + i of either plane
-// Kernel columns past k_w, the fourth channel and output channels past C_out meet zero weights.
+// Kernel columns past k_w, the fourth channel and output channels past C_out meet zero weights.  The columns past k_w are pixels
+// beside the window all the same, and an infinity or a NaN among them times zero is a NaN in every channel: a row whose first
+// sum is one is worked out again from the window alone (redo_pixel; one comparison per row where there is none).
 //
 // Work item = 1 .. 4 tiles of 8 x 16 output pixels (M = 128) side by side that share one patch.  Eight warps build
 // patches (two buffers), two warps issue the UMMAs of alternate tiles (N = C_out), four groups of four warps each own one
@@ -97,6 +99,26 @@ __device__ __forceinline__ void issue_tile(uint32_t d_tmem, uint64_t ad, uint64_
     for (int r = 0; r < KH; r++, ad += a_row16) {
 #pragma unroll
         for (int i = 0; i < STEPS; i++, bd += b_step16) umma_f16(d_tmem, ad + static_cast<uint32_t>(i) * a_step16, bd, idesc, (r | i) != 0);
+    }
+}
+
+// An output pixel's channels by the definition, into its row of the staging tile.
+template <int CIN, int ACT>
+__device__ __noinline__ void redo_pixel(const __half* x, const __half* w, const float* bias, int H, int W, int kh, int kw, int Cout, int n, int hi0, int wi0, int m, uint8_t* sout) {
+    for (int co = 0; co < Cout; co += 2) {
+        float v[2] = {0.0f, 0.0f};
+        for (int r = 0; r < kh; r++) {
+            if (static_cast<unsigned>(hi0 + r) >= static_cast<unsigned>(H)) continue;
+            for (int s = 0; s < kw; s++) {
+                if (static_cast<unsigned>(wi0 + s) >= static_cast<unsigned>(W)) continue;
+                const __half* px = x + ((static_cast<long long>(n) * H + hi0 + r) * W + wi0 + s) * CIN;
+                for (int j = 0; j < 2; j++) {
+                    const __half* wt = w + (((co + j) * kh + r) * kw + s) * CIN;
+                    for (int c = 0; c < CIN; c++) v[j] = fmaf(__half2float(px[c]), __half2float(wt[c]), v[j]);
+                }
+            }
+        }
+        *reinterpret_cast<uint32_t*>(sout + m * 128 + (((co >> 3) ^ (m & 7)) << 4) + (co & 7) * 2) = round_act<ACT>(v[0] + bias[co], v[1] + bias[co + 1]);
     }
 }
 
@@ -329,9 +351,11 @@ __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_const
                 tmem_ld32_issue(taddr, r);
                 if (issuer) tma_store_wait_read();
                 group_sync();   // the staging tile's last store has read it
+                bool redo = false;
 #pragma unroll 1
                 for (int cc = 0; cc < p.BN; cc += 32) {
                     tmem_ld32_wait(r);
+                    if (cc == 0) redo = isnan(__uint_as_float(r[0]));
                     if (cc + 32 >= p.BN) {
                         tc_fence_before_sync();
                         __syncwarp();
@@ -350,6 +374,11 @@ __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_const
                         __syncwarp();
                         tmem_ld32_issue(taddr + cc + 32, r);
                     }
+                }
+                if (redo) {
+                    const int wo = o.wo0 + k * kTileW + (m & (kTileW - 1)), ho = o.ho0 + m / kTileW;
+                    if (wo < p.Wo && ho < p.Ho)
+                        redo_pixel<CIN, ACT>(p.x, p.w, bias_s, p.H, p.W, p.kh, p.kw, p.Cout, o.n, ho * p.stride - p.pad, wo * p.stride - p.pad, m, sout);
                 }
                 fence_proxy_async_smem();
                 group_sync();

@@ -54,3 +54,18 @@ def test_nan_and_infinity(case, act):
     for i, v in enumerate((np.inf, -np.inf, np.nan)):
         x[n - 1, (2 + 5 * i) % h, (3 + 4 * i) % w, i] = v
     check_nonfinite(layers, params, x, ends, sms, name + " " + act)
+
+
+# kernel widths that leave columns of a K step over: the pixels beside a window are read and must not count
+@pytest.mark.parametrize("cin,cout,k,stride,pad,n,h,w", [
+    (3, 64, 7, 2, 3, 2, 45, 50), (3, 32, 3, 2, 1, 1, 37, 41), (3, 64, 11, 4, 2, 1, 67, 71), (3, 64, 3, 1, 1, 1, 20, 35), (1, 16, 5, 2, 2, 1, 24, 40),
+    (2, 40, 1, 1, 0, 1, 19, 21), (4, 24, 9, 4, 4, 1, 40, 41), (3, 8, 5, 1, 0, 1, 17, 33)])
+def test_stem_keeps_them_in_their_windows(cin, cout, k, stride, pad, n, h, w):
+    for act in ("none", "relu6"):
+        layers = [_conv(cin, cout, k, stride=stride, pad=pad, act=act)]
+        params = synth.layer_params("nonfinite stem", layers)
+        x = synth.network_input("nonfinite stem", n, h, w, cin)
+        for i, v in enumerate((np.inf, -np.inf, np.nan, np.inf)):
+            x[n - 1, (3 + 4 * i) % h, (5 + 7 * i) % w, i % cin] = v
+        x[n - 1, 0, 0, 0], x[0, h - 1, w - 1, cin - 1] = np.inf, np.nan
+        check_nonfinite(layers, params, x, [0], 0, "stem " + ("relu6" if act == "relu6" else ""))
