@@ -120,6 +120,7 @@ struct dlf_net {
     dlf::GraphCache graph, graph_timed;
     // dlf_net_run_host on a large batch: the plan's first groups once per part of the batch, and the rest (see host_head)
     dlf::GraphCache host_part[dlf::kHostParts], host_rest;
+    bool host_whole = false;   // the plan's groups could not be captured for parts of the batch
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t host_event[dlf::kHostParts + 1] = {};
     std::vector<cudaEvent_t> group_events;
@@ -627,7 +628,7 @@ static int launch_group_part(dlf_net* net, const Group& g, const void* in_dev, c
 // more than it hides.  From page-locked memory at 224x224: ResNet-50, 32 images 810 -> 785 us (six groups), MobileNetV2, 64
 // images 960 -> 800 (five).
 static int host_head(const dlf_net* net) {
-    if (!net->opt_graph || net->N < 2 * kHostParts || net->in_bytes < (8u << 20)) return 0;
+    if (!net->opt_graph || net->host_whole || net->N < 2 * kHostParts || net->in_bytes < (8u << 20)) return 0;
     const double copy_us = net->in_bytes / 50e3;
     double sum = 0.0;
     int count = 0;
@@ -704,6 +705,7 @@ static void invalidate_graphs(dlf_net* net) {
     net->graph_timed.drop();
     for (GraphCache& gc : net->host_part) gc.drop();
     net->host_rest.drop();
+    net->host_whole = false;
 }
 
 // Captures the launches of every group of the plan into one executable graph (thread-local
@@ -798,9 +800,16 @@ static int run_graph(dlf_net* net, GraphCache* gc, const void* in_dev, void* out
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
 
-// The input in kHostParts copies on a stream of the net's own, the plan's first `head` groups for a part as soon as it is there,
-// then the other groups for the whole batch.  Leaves the output in its workspace slot.
-static int run_host_parts(dlf_net* net, const void* in_host, int head, cudaStream_t s) {
+// First image of every part, and one past the last part's.  A part starts on a multiple of four bytes, as the first-layer kernel
+// reads its input in words (an odd number of 2-byte elements per image: the parts hold even numbers of images, but for the last).
+static void host_part_bounds(const dlf_net* net, int (&n0)[kHostParts + 1]) {
+    const int unit = net->in_bytes / net->N % 4 ? 2 : 1;
+    for (int i = 0; i < kHostParts; i++) n0[i] = static_cast<int>(static_cast<int64_t>(net->N) * i / kHostParts) / unit * unit;
+    n0[kHostParts] = net->N;
+}
+
+// What run_host_parts() launches; enqueues nothing.
+static int build_host_parts(dlf_net* net, int head) {
     cudaError_t e = cudaSuccess;
     if (!net->copy_stream) e = cudaStreamCreateWithFlags(&net->copy_stream, cudaStreamNonBlocking);
     for (cudaEvent_t& ev : net->host_event)
@@ -808,9 +817,8 @@ static int run_host_parts(dlf_net* net, const void* in_host, int head, cudaStrea
     if (e != cudaSuccess) return cuda_fail(e);
     uint8_t* in_dev = net->ws + net->in_off;
     void* out_dev = net->ws + net->layers.back().off;
-    const size_t image = net->in_bytes / net->N;
     int n0[kHostParts + 1];
-    for (int i = 0; i <= kHostParts; i++) n0[i] = static_cast<int>(static_cast<int64_t>(net->N) * i / kHostParts);
+    host_part_bounds(net, n0);
     for (int i = 0; i <= kHostParts; i++) {
         GraphCache* gc = i < kHostParts ? &net->host_part[i] : &net->host_rest;
         if (gc->exec) continue;
@@ -818,7 +826,17 @@ static int run_host_parts(dlf_net* net, const void* in_host, int head, cudaStrea
         const int rc = i < kHostParts ? build_graph(net, gc, in_dev, out_dev, false, 0, head, &part) : build_graph(net, gc, in_dev, out_dev, false, head);
         if (rc) return rc;
     }
-    e = cudaEventRecord(net->host_event[kHostParts], s);   // what the stream holds so far may still read the workspace or write the host buffer
+    return DLF_OK;
+}
+
+// The input in kHostParts copies on a stream of the net's own, the plan's first groups for a part as soon as it is there, then
+// the other groups for the whole batch.  Leaves the output in its workspace slot.
+static int run_host_parts(dlf_net* net, const void* in_host, cudaStream_t s) {
+    uint8_t* in_dev = net->ws + net->in_off;
+    const size_t image = net->in_bytes / net->N;
+    int n0[kHostParts + 1];
+    host_part_bounds(net, n0);
+    cudaError_t e = cudaEventRecord(net->host_event[kHostParts], s);   // what the stream holds so far may still read the workspace or write the host buffer
     if (e == cudaSuccess) e = cudaStreamWaitEvent(net->copy_stream, net->host_event[kHostParts], 0);
     for (int i = 0; i < kHostParts && e == cudaSuccess; i++) {
         e = cudaMemcpyAsync(in_dev + n0[i] * image, static_cast<const uint8_t*>(in_host) + n0[i] * image, (n0[i + 1] - n0[i]) * image, cudaMemcpyHostToDevice, net->copy_stream);
@@ -830,7 +848,7 @@ static int run_host_parts(dlf_net* net, const void* in_host, int head, cudaStrea
     }
     if (e == cudaSuccess) e = cudaGraphLaunch(net->host_rest.exec, s);
     if (e != cudaSuccess) return cuda_fail(e);
-    net->last_out = out_dev;
+    net->last_out = net->ws + net->layers.back().off;
     return DLF_OK;
 }
 
@@ -1261,9 +1279,14 @@ int dlf_net_run_host(dlf_net* net, const void* in_f16_host, void* out_f16_host, 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const Layer& z = net->layers.back();
     cudaError_t e = cudaSuccess;
-    const int head = host_head(net);
+    int head = host_head(net);
+    if (head > 0 && build_host_parts(net, head) != DLF_OK) {   // (a part is refused where the whole batch may not be)
+        invalidate_graphs(net);
+        net->host_whole = true;
+        head = 0;
+    }
     if (head > 0) {
-        rc = run_host_parts(net, in_f16_host, head, s);
+        rc = run_host_parts(net, in_f16_host, s);
         if (rc) return rc;
     } else {
         e = cudaMemcpyAsync(net->ws + net->in_off, in_f16_host, net->in_bytes, cudaMemcpyHostToDevice, s);

@@ -45,3 +45,28 @@ def test_parts_of_a_batch(layers, n, h, w, c):
             # a part may run through other tiles: sums in another order, single fp16 roundings carried on through the layers
             assert float((y.float() - ref).norm() / ref.norm()) < 2e-3
     s.close()
+
+
+@pytest.mark.parametrize("n,h,w", [(27, 203, 261), (29, 203, 261), (30, 203, 261), (19, 287, 287)])
+def test_parts_of_images_with_an_odd_number_of_elements(n, h, w):
+    """An image of 2 mod 4 bytes: a part may not start on an odd one, whatever the quarters of the batch come to."""
+    layers = nw.resnet18()
+    assert h * w * 3 % 2 == 1 and n * h * w * 3 * 2 >= 8 << 20
+    g = torch.Generator(device="cuda").manual_seed(n)
+    params = []
+    for l in layers:
+        if l["op"] not in ("conv", "fc"):
+            params.append(None)
+            continue
+        shape = (l["cout"], l["kh"], l["kw"], l["cin"]) if l["op"] == "conv" else (l["cout"], l["cin"])
+        params.append(((torch.randn(shape, generator=g, device="cuda") * int(np.prod(shape[1:])) ** -0.5).half().cpu().numpy(),
+                       (torch.randn(l["cout"], generator=g, device="cuda") * 0.1).cpu().numpy()))
+    s = Session(layers, params, n, h, w, 3)
+    s.set_plan(*plans.tuned_plan(s.net, len(layers)))
+    x = (torch.rand((n, h, w, 3), generator=g, device="cuda") * 2 - 1).half()
+    ref = s.run(x).float().cpu()
+    xh, y = x.cpu().pin_memory(), torch.empty(s.out_shape, dtype=torch.float16, pin_memory=True)
+    B.net_run_host(s.net, xh.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    s.close()
+    # single fp16 roundings (see above)
+    assert float((y.float() - ref).norm() / ref.norm()) < 2e-3
