@@ -1247,6 +1247,7 @@ ChainTiling chain_tc_tiling(const ChainArgs& a, int sm_count, int device_sms) {
 
 int launch_chain_tc(const ChainArgs& a, const ChainTiling& t, int sm_count, int* status_dev, cudaStream_t s) {
     if (!t.ok) return DLF_E_PLAN;
+    if (!aligned(16, a.x, a.res, a.y)) return DLF_E_INVALID_ARG;
     {
         int rc = chain_tc_init();
         if (rc) return rc;

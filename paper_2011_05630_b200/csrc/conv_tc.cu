@@ -1378,6 +1378,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
 }  // namespace
 
 int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s) {
+    if (!aligned(16, a.x, a.w, a.res, a.y, a.x2, a.w2) || !aligned(4, a.bias, a.bias2)) return DLF_E_INVALID_ARG;
     int rc = conv_tc_init();
     if (rc) return rc;
     rc = launch_conv_narrow(a, sm_count, s);
@@ -1406,6 +1407,7 @@ int launch_conv_seq(const ConvArgs* layers, int n_layers, int sm_count, int* sta
     size_t smem = 0;
     for (int l = 0; l < n_layers; l++) {
         ConvArgs a = layers[l];
+        if (!aligned(16, a.x, a.w, a.res, a.y)) return DLF_E_INVALID_ARG;
         a.splitk_ws = nullptr;   // no split reductions inside a multi-layer launch
         a.splitk_bytes = 0;
         ConvTcLaunch L;

@@ -70,6 +70,11 @@ struct ChainTiling {
     bool ok;
 };
 
+// True if every pointer is a multiple of `bytes` (null ones are).  Each launch checks the buffers that its kernel reads or
+// writes with vector accesses - a caller's among them - so that a misaligned one is DLF_E_INVALID_ARG and not a device fault.
+template <typename... P>
+inline bool aligned(uintptr_t bytes, P... ptrs) { return (((reinterpret_cast<uintptr_t>(ptrs) & (bytes - 1)) == 0) && ...); }
+
 int cuda_fail(cudaError_t e);  // records the error for dlf_last_cuda_error, returns DLF_E_CUDA
 int cuda_fail_drv(int e);
 

@@ -404,6 +404,7 @@ int launch_conv_direct(const ConvArgs& a, int sm_count, cudaStream_t s) {
 int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
     if (a.kh != 3 || a.kw != 3 || a.groups != a.Cin || a.Cin != a.Cout || a.Cin % 8 || a.pool) return DLF_E_UNSUPPORTED;
     if (a.stride != 1 && a.stride != 2) return DLF_E_UNSUPPORTED;
+    if (!aligned(8, a.x, a.res, a.y)) return DLF_E_INVALID_ARG;
     const int c4n = a.Cout / 4;
     static int occ[2] = {0, 0};
     const int v = a.stride == 1 ? 0 : 1;
@@ -448,6 +449,7 @@ int launch_dw3x3(const ConvArgs& a, int sm_count, cudaStream_t s) {
 int launch_maxpool(const void* x, void* y, int N, int H, int W, int C, int k, int stride, int pad, int Ho, int Wo,
                    int sm_count, cudaStream_t s) {
     if (C % 8) return DLF_E_UNSUPPORTED;
+    if (!aligned(16, x, y)) return DLF_E_INVALID_ARG;
     const long long total = static_cast<long long>(N) * Ho * Wo * (C / 8);
     if (total == 0) return DLF_OK;
     cudaError_t e = launch_kernel(maxpool_kernel, grid_for((total + 255) / 256, sm_count), 256, 0, s, static_cast<const __half*>(x),
@@ -457,6 +459,7 @@ int launch_maxpool(const void* x, void* y, int N, int H, int W, int C, int k, in
 
 int launch_gavgpool(const void* x, void* y, int N, int H, int W, int C, int sm_count, cudaStream_t s) {
     if (C % 8) return DLF_E_UNSUPPORTED;
+    if (!aligned(16, x)) return DLF_E_INVALID_ARG;
     const int vec_blocks = (C / 8 + kAvgVecs - 1) / kAvgVecs;
     const long long total = static_cast<long long>(N) * vec_blocks;
     if (total == 0) return DLF_OK;
@@ -469,6 +472,7 @@ int launch_gavgpool(const void* x, void* y, int N, int H, int W, int C, int sm_c
 int launch_fc(const void* x, const void* w, const float* bias, void* y, int N, int K, int M, int act, int sm_count,
               cudaStream_t s) {
     if (K % 8) return DLF_E_UNSUPPORTED;
+    if (!aligned(16, x)) return DLF_E_INVALID_ARG;
     if (N == 0) return DLF_OK;
     const int o_blocks = (M + kFcFo - 1) / kFcFo, n_blocks = (N + kFcNb - 1) / kFcNb;
     const int grid = grid_for(static_cast<long long>(o_blocks) * n_blocks, sm_count);

@@ -762,6 +762,7 @@ int mbconv_tc_init() {
 
 int launch_mbconv_tc(const MbconvArgs& a, const MbconvTiling& t, int sm_count, int* status_dev, cudaStream_t s) {
     if (!t.ok) return DLF_E_PLAN;
+    if (!aligned(16, a.x, a.res, a.y)) return DLF_E_INVALID_ARG;
     int rc = mbconv_tc_init();
     if (rc) return rc;
     MbLayout L;

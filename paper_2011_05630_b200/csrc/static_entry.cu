@@ -44,6 +44,7 @@ extern "C" int dlf_conv_chain_run_static(const dlf_layer_desc* layers, int n_lay
     using namespace dlf;
     if (!layers || !x_f16_dev || !w_f16_dev || !bias_dev || !y_f16_dev) return DLF_E_INVALID_ARG;
     if (n_layers < 1 || n_layers > kMaxChain || N < 1 || H < 1 || W < 1 || sm_count < 1) return DLF_E_INVALID_ARG;
+    if (!aligned(16, x_f16_dev, y_f16_dev)) return DLF_E_INVALID_ARG;
     // shapes first: nothing is enqueued unless every layer fits
     ConvArgs a[kMaxChain];
     int h = H, w = W;
@@ -54,7 +55,7 @@ extern "C" int dlf_conv_chain_run_static(const dlf_layer_desc* layers, int n_lay
         if (d.cin < 8 || d.cout < 8) return DLF_E_SHAPE;
         if (d.src != i - 1 || (i > 0 && d.cin != layers[i - 1].cout)) return DLF_E_SHAPE;
         if (d.kh < 1 || d.kw < 1 || d.stride < 1 || d.pad < 0 || h + 2 * d.pad < d.kh || w + 2 * d.pad < d.kw) return DLF_E_SHAPE;
-        if (!w_f16_dev[i] || !bias_dev[i]) return DLF_E_INVALID_ARG;
+        if (!w_f16_dev[i] || !bias_dev[i] || !aligned(16, w_f16_dev[i]) || !aligned(4, bias_dev[i])) return DLF_E_INVALID_ARG;
         ConvArgs& c = a[i];
         std::memset(&c, 0, sizeof(c));
         c.N = N; c.H = h; c.W = w; c.Cin = d.cin; c.Cout = d.cout;

@@ -498,7 +498,7 @@ int stem_tc_init() {
 
 int launch_stem_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s) {
     if (!stem_tc_supported(a)) return DLF_E_UNSUPPORTED;
-    if (reinterpret_cast<uintptr_t>(a.x) & 3u) return DLF_E_INVALID_ARG;
+    if (!aligned(4, a.x) || !aligned(16, a.y)) return DLF_E_INVALID_ARG;
     int rc = stem_tc_init();
     if (rc) return rc;
     const Layout l = pick_layout(a, sm_count);

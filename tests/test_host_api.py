@@ -104,6 +104,13 @@ def test_allocation_free_entry_rejects_bad_layers_before_any_launch(layer, statu
     assert B.lib().dlf_conv_chain_run_static(arr, 1, 1, 6, 6, 256, ptrs, ptrs, 256, 1, None) == status
 
 
+@pytest.mark.parametrize("x,w,bias,y", [(264, 256, 256, 256), (256, 264, 256, 256), (256, 256, 258, 256), (256, 256, 256, 258)])
+def test_allocation_free_entry_rejects_misaligned_pointers(x, w, bias, y):
+    import ctypes as C
+    arr = (B.LayerDesc * 1)(B.LayerDesc(B.OPS["conv"], 0, 8, 8, 3, 3, 1, 1, 1, -1, -2, 0))
+    assert B.lib().dlf_conv_chain_run_static(arr, 1, 1, 6, 6, x, (C.c_void_p * 1)(w), (C.c_void_p * 1)(bias), y, 1, None) == B.E_INVALID_ARG
+
+
 # ---- the auto-tuner against the restated Algorithm 1 ----------------------------------------------------
 # Which spans one kernel can run, and which of them are worth proposing, is the library's own rule (four fused kernels
 # and their cost estimates - nothing the paper defines): the test takes it from dlf_net_tuner_may_fuse as an INPUT and
