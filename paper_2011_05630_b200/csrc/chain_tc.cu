@@ -272,7 +272,7 @@ __device__ __forceinline__ void epi_last(const ChainParams& p, const ChainLayerP
                 } else {
                     uint4 val;
                     if (has_res && co < L.cout && lr.in_out)
-                        val = finish8_res(v + g * 8, cx.bl + co, __ldg(reinterpret_cast<const uint4*>(p.res + lr.gpix * L.cout + co)), cx);
+                        val = finish8_res(v + g * 8, cx.bl + co, ld_map(reinterpret_cast<const uint4*>(p.res + lr.gpix * L.cout + co)), cx);
                     else
                         val = finish8(v + g * 8, cx.bl + co, cx);
                     if (MODE == OUT_POOL) *tile_ptr(cx.obuf, cx.oplane, lr.srow, co >> 3) = val;

@@ -269,7 +269,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
 #pragma unroll
                 for (int it = 0; it < kItems; it++) {
                     const int c = half * 16 + (it >> 1) * 32 + (it & 1) * 8;
-                    if (c < p.BN && c < n_co) rv[it] = __ldg(reinterpret_cast<const uint4*>(p.res + row + c));
+                    if (c < p.BN && c < n_co) rv[it] = ld_map(reinterpret_cast<const uint4*>(p.res + row + c));
                 }
             }
             const bool ok = mbar_wait<true>(&tfull_bar, 0u, abort_flag, p.status, 0xE20 | (blockIdx.x << 12));
@@ -288,7 +288,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
                         if (c >= n_co) break;
                         uint4 res = zero;
                         if (2 * j + g < kItems) res = rv[(2 * j + g) % kItems];
-                        else if (p.res) res = __ldg(reinterpret_cast<const uint4*>(p.res + row + c));
+                        else if (p.res) res = ld_map(reinterpret_cast<const uint4*>(p.res + row + c));
                         *reinterpret_cast<uint4*>(p.out + row + c) = finish8(v + g * 8, bias_s + c, res, lo, hi);
                     }
                 }
@@ -320,7 +320,7 @@ conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__
             }
             pdl_wait();
 #pragma unroll
-            for (int it = 0; it < kItems; it++) rv[it] = p.res && off[it] >= 0 ? __ldg(reinterpret_cast<const uint4*>(p.res + off[it])) : zero;
+            for (int it = 0; it < kItems; it++) rv[it] = p.res && off[it] >= 0 ? ld_map(reinterpret_cast<const uint4*>(p.res + off[it])) : zero;
             const int dest = min(m / p.rows_per, SPLIT - 1), row = m - dest * p.rows_per;
             const uint32_t slab = static_cast<uint32_t>(p.rows_per * p.BN * 4);   // one rank's partial rows
             const uint32_t dst = mapa(base + p.red_off + rank * slab + row * p.BN * 4, dest), dst_bar = mapa(smem_u32(&red_bar), dest);

@@ -515,7 +515,7 @@ __device__ __forceinline__ void conv_tc_roles(const CUtensorMap* tmx_p, const CU
                 for (int g = 0; g < 4; g++) {
                     const int co = c.co0 + cc + g * 8;
                     const bool okg = valid && cc + g * 8 < ncols && co < p.Cout;
-                    rv[g] = __ldg(reinterpret_cast<const uint4*>(p.res + (okg ? pix * p.Cout + co : 0)));
+                    rv[g] = ld_map(reinterpret_cast<const uint4*>(p.res + (okg ? pix * p.Cout + co : 0)));
                     okm |= (okg ? 1u : 0u) << g;
                 }
             };

@@ -162,9 +162,9 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
         int left = rows * STRIDE + 3 - STRIDE;   // rows still to fetch
         auto fetch = [&](int slot) {
             const bool row_ok = hi_ >= 0 && hi_ < a.H && left > 0;
-            raw[slot][0] = row_ok && ok0 ? __ldg(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
-            raw[slot][1] = row_ok && ok1 ? __ldg(reinterpret_cast<const uint2*>(src + a.Cin)) : make_uint2(0u, 0u);
-            raw[slot][2] = row_ok && ok2 ? __ldg(reinterpret_cast<const uint2*>(src + 2 * a.Cin)) : make_uint2(0u, 0u);
+            raw[slot][0] = row_ok && ok0 ? ld_map(reinterpret_cast<const uint2*>(src)) : make_uint2(0u, 0u);
+            raw[slot][1] = row_ok && ok1 ? ld_map(reinterpret_cast<const uint2*>(src + a.Cin)) : make_uint2(0u, 0u);
+            raw[slot][2] = row_ok && ok2 ? ld_map(reinterpret_cast<const uint2*>(src + 2 * a.Cin)) : make_uint2(0u, 0u);
             left--;
             hi_++;
             src += in_row;
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(128) dw3x3_kernel(ConvArgs a, long long total,
         };
         auto store = [&](float (&acc)[4]) {
             if (res != nullptr) {
-                const uint2 rv = __ldg(reinterpret_cast<const uint2*>(res + off));
+                const uint2 rv = ld_map(reinterpret_cast<const uint2*>(res + off));
                 const float2 f0 = __half22float2(*reinterpret_cast<const __half2*>(&rv.x)), f1 = __half22float2(*reinterpret_cast<const __half2*>(&rv.y));
                 acc[0] += f0.x; acc[1] += f0.y; acc[2] += f1.x; acc[3] += f1.y;
             }
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256) maxpool_kernel(const __half* x, __half* y
 #pragma unroll 3
             for (int s = 0; s < k; s++) {
                 const int wi = min(max(wo * stride - pad + s, w_lo), w_hi);
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + ((static_cast<long long>(n) * H + hi) * W + wi) * C + c8 * 8));
+                const uint4 v = ld_map(reinterpret_cast<const uint4*>(x + ((static_cast<long long>(n) * H + hi) * W + wi) * C + c8 * 8));
                 const __half2* vh = reinterpret_cast<const __half2*>(&v);
 #pragma unroll
                 for (int j = 0; j < 4; j++) best[j] = __hmax2(best[j], vh[j]);
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(kAvgVecs * kAvgParts) gavgpool_kernel(const __
             const __half* xp = x + static_cast<long long>(n) * HW * C + c8 * 8;
 #pragma unroll 4
             for (int p = q; p < HW; p += kAvgParts) {
-                const uint4 u = __ldg(reinterpret_cast<const uint4*>(xp + static_cast<long long>(p) * C));
+                const uint4 u = ld_map(reinterpret_cast<const uint4*>(xp + static_cast<long long>(p) * C));
                 const __half* vh = reinterpret_cast<const __half*>(&u);
 #pragma unroll
                 for (int j = 0; j < 8; j++) acc[j] += __half2float(vh[j]);
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(256) fc_kernel(const __half* x, const __half* 
 #pragma unroll
             for (int j = 0; j < kFcNb; j++) {
                 const int n = min(n0 + j, N - 1);
-                xv[j] = __ldg(reinterpret_cast<const uint4*>(x + static_cast<long long>(n) * K) + k8);
+                xv[j] = ld_map(reinterpret_cast<const uint4*>(x + static_cast<long long>(n) * K) + k8);
             }
 #pragma unroll
             for (int e = 0; e < 4; e++) {

@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(kThreads, 1) mbconv_tc_kernel(const __grid_con
 #pragma unroll
                         for (int e = 0; e < 8; e++) a[e] = __uint_as_float(v[b][g * 8 + e]) + bb[g * 8 + e];
                         if (has_res) {   // staged: loaded into the staging buffer by TMA, zero outside the tensor
-                            const uint4 rv = staged ? *sp : __ldg(reinterpret_cast<const uint4*>(p.res + gpix * p.Cout + co));
+                            const uint4 rv = staged ? *sp : ld_map(reinterpret_cast<const uint4*>(p.res + gpix * p.Cout + co));
                             const __half2* rh = reinterpret_cast<const __half2*>(&rv);
 #pragma unroll
                             for (int e = 0; e < 4; e++) {

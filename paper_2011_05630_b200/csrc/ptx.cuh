@@ -47,6 +47,11 @@ __device__ __forceinline__ uint64_t global_ns() {
 // and its memory operations are visible.  Both are no-ops for a normal launch.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Maps and residuals are read with ordinary loads: the kernel before this one may still be writing them when this one's CTAs
+// start, while __ldg (and a const __restrict__ argument) promises data that stays as it is for the kernel's whole life, and a
+// load that promises that may be moved above pdl_wait().  __ldg is for weights and biases.
+template <typename T>
+__device__ __forceinline__ T ld_map(const T* p) { return *p; }
 
 // ---- mbarrier ---------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

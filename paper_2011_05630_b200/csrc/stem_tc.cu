@@ -247,14 +247,14 @@ __global__ void __launch_bounds__(kThreads, 1) stem_tc_kernel(const __grid_const
 #pragma unroll
                     for (int u = 0; u < kUnroll; u++)
 #pragma unroll
-                        for (int e = 0; e < kWords; e++) w[u][e] = __ldg(x32 + gw[u] + e);
+                        for (int e = 0; e < kWords; e++) w[u][e] = ld_map(x32 + gw[u] + e);
                 } else {
 #pragma unroll
                     for (int u = 0; u < kUnroll; u++)
 #pragma unroll
                         for (int e = 0; e < kWords; e++) {
                             const int k = max(min(gw[u] + e, p.last_word), 0);
-                            const uint32_t full = __ldg(x32 + min(k, p.last_word - p.tail));
+                            const uint32_t full = ld_map(x32 + min(k, p.last_word - p.tail));
                             w[u][e] = k > p.last_word - p.tail ? tail_word : full;
                         }
                 }
