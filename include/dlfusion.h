@@ -213,6 +213,12 @@ int dlf_net_group_model(const dlf_net* net, int group, int64_t* flops, int64_t* 
  * "conv_direct", "dw3x3", "fc", "maxpool", "gavgpool"); the string is owned by the library. */
 const char* dlf_net_group_kernel(const dlf_net* net, int group);
 
+/* What dlf_net_run launches for group g of the current plan: the kernel's name with its template arguments ("conv_lat_kernel<4>"
+ * is a cluster of four CTAs; a 3x3 layer's ring stages "by rows" or "by columns" of the kernel), CTAs and threads per CTA.
+ * "conv_tc" of dlf_net_group_kernel stands for several kernels, chosen by the layer's size and the SM count: conv_narrow, conv_lat,
+ * conv_tc and conv_tc_pair.  Launches nothing; needs weights and workspace like a run.  Any out-pointer may be NULL. */
+int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes, int* grid, int* block);
+
 /* Options (debugging and ablation); setting one clears the plan, which must be set again.
  *   DLF_OPT_NO_TENSOR_CORE   1: route every dense convolution to the CUDA-core direct kernel
  *                               (multi-layer groups then become illegal).

@@ -77,6 +77,7 @@ def lib():
             "dlf_net_boundary_tensor": (C.c_int, [vp, C.c_int, C.POINTER(vp), i64p]),
             "dlf_net_group_model": (C.c_int, [vp, C.c_int, i64p, i64p, C.POINTER(C.c_double), ip]),
             "dlf_net_group_kernel": (C.c_char_p, [vp, C.c_int]),
+            "dlf_net_group_launch": (C.c_int, [vp, C.c_int, C.c_char_p, C.c_size_t, C.POINTER(C.c_int), C.POINTER(C.c_int)]),
             "dlf_net_set_option": (C.c_int, [vp, C.c_int, C.c_int]),
             "dlf_conv_chain_run_static": (C.c_int, [C.POINTER(LayerDesc), C.c_int, C.c_int, C.c_int, C.c_int, vp,
                                                     C.POINTER(vp), C.POINTER(vp), vp, C.c_int, vp]),
@@ -257,6 +258,13 @@ def net_group_model(net, g):
 
 def net_group_kernel(net, g):
     return lib().dlf_net_group_kernel(net, g).decode()
+
+
+def net_group_launch(net, g):
+    """(kernel with its template arguments, CTAs, threads per CTA) of group g of the current plan."""
+    name, grid, block = C.create_string_buffer(256), C.c_int(), C.c_int()
+    _check(lib().dlf_net_group_launch(net, g, name, len(name), C.byref(grid), C.byref(block)), "dlf_net_group_launch")
+    return name.value.decode(), grid.value, block.value
 
 
 def net_set_option(net, option, value):

@@ -4,13 +4,17 @@
 // auto-tuner (Eq. 5 + Algorithm 1) and the reduced brute-force search (Sec. V).
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <cxxabi.h>
 
 #include <algorithm>
 #include <cmath>
+#include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <limits>
 #include <new>
+#include <string>
 #include <vector>
 
 #include "internal.h"
@@ -20,6 +24,7 @@ namespace dlf {
 static thread_local int g_last_cuda_error = 0;
 int g_use_pdl = 1;
 thread_local const GraphNodeUpdate* g_node_update = nullptr;
+thread_local LaunchRecord* g_launch_record = nullptr;
 int g_conv_row_mode = 1;
 
 int cuda_fail(cudaError_t e) {
@@ -1527,6 +1532,34 @@ int dlf_net_group_model(const dlf_net* net, int group, int64_t* flops, int64_t* 
 const char* dlf_net_group_kernel(const dlf_net* net, int group) {
     if (!net || group < 0 || group >= static_cast<int>(net->plan.size())) return "";
     return kKindName[net->plan[group].kind];
+}
+
+int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes, int* grid, int* block) {
+    if (!net || group < 0 || group >= static_cast<int>(net->plan.size()) || (name && name_bytes == 0)) return DLF_E_INVALID_ARG;
+    int rc = check_ready(net);
+    if (rc) return rc;
+    LaunchRecord rec{nullptr, 0, 0, ""};
+    g_launch_record = &rec;
+    rc = launch_group(net, net->plan[group], net->ws + net->in_off, net->ws + net->layers.back().off, nullptr);
+    g_launch_record = nullptr;
+    if (rc) return rc;
+    if (grid) *grid = rec.grid;
+    if (block) *block = rec.block;
+    if (name) {
+        const char* mangled = nullptr;
+        cudaError_t e = cudaFuncGetName(&mangled, rec.func);
+        if (e != cudaSuccess) return cuda_fail(e);
+        // "void dlf::(anonymous namespace)::kernel<1, 2>(arguments)" -> "kernel<1, 2>"
+        char* full = abi::__cxa_demangle(mangled, nullptr, nullptr, nullptr);
+        std::string text = full ? full : mangled;
+        std::free(full);
+        const size_t args = text.rfind(">(") != std::string::npos ? text.find(">(") + 1 : text.rfind('(');
+        text = text.substr(0, args);
+        const size_t scope = text.substr(0, text.find('<')).rfind("::");
+        if (scope != std::string::npos) text = text.substr(scope + 2);
+        std::snprintf(name, name_bytes, "%s%s", text.c_str(), rec.note);
+    }
+    return DLF_OK;
 }
 
 int dlf_net_set_option(dlf_net* net, int option, int value) {

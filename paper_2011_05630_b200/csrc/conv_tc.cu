@@ -1388,6 +1388,7 @@ int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_
     ConvTcLaunch L;
     rc = conv_tc_prepare(a, sm_count, status_dev, true, &L);
     if (rc) return rc;
+    if (g_launch_record) g_launch_record->note = !L.row ? "" : (L.p.col ? " by columns" : " by rows");
     const KernelFn fn = L.pair ? pick_pair(L.act, L.pool != 0, L.res != 0, L.row != 0) : L.split ? pick_split(L.act, L.row != 0) : pick_kernel(L.act, L.pool != 0, L.res != 0, L.row != 0);
     cudaError_t e = launch_kernel(fn, L.grid, kThreads, L.smem, s, L.tmx, L.tmw, L.tmy, L.tmr, L.tmx2, L.tmw2, L.p);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);

@@ -100,12 +100,27 @@ struct GraphNodeUpdate {
 };
 extern thread_local const GraphNodeUpdate* g_node_update;
 
+// While set (calling thread only), launch_kernel() writes the launch down instead of launching: what runs a group, for
+// dlf_net_group_launch().  `note`: what a kernel's name does not say, from its launch function.
+struct LaunchRecord {
+    const void* func;
+    int grid, block;
+    const char* note;
+};
+extern thread_local LaunchRecord* g_launch_record;
+
 // Launches a kernel, optionally with programmatic dependent launch (the kernel must then call
 // pdl_wait() before it touches anything its predecessor in the stream produces).
 extern int g_use_pdl;
 extern int g_conv_row_mode;  // conv_tc row mode: 0 never, 1 where it cuts the streamed bytes by a fifth, 2 wherever it applies
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_opt(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args&&... args) {
+    if (g_launch_record) {
+        g_launch_record->func = reinterpret_cast<const void*>(kernel);
+        g_launch_record->grid = grid;
+        g_launch_record->block = block;
+        return cudaSuccess;
+    }
     if (g_node_update) {
         std::tuple<KArgs...> vals(static_cast<KArgs>(args)...);
         void* ptrs[sizeof...(KArgs)];

@@ -94,6 +94,10 @@ class Session:
         t.copy_(src)
         return t.cpu().numpy().reshape(shape)
 
+    def launches(self):
+        """(kernel, CTAs, threads per CTA) of every group, as a run launches it."""
+        return [B.net_group_launch(self.net, g) for g in range(self.n_groups)]
+
     def kernels(self):
         return [B.net_group_kernel(self.net, g) for g in range(self.n_groups)]
 

@@ -1,0 +1,77 @@
+"""Which kernel a layer's size and SM count send it to, and what that kernel makes of it: every variant of the single-layer
+convolution kernels is asked for by name, so that an estimate that moves cannot leave one of them untested."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2011_05630_b200 import binding as B
+from tests import gpu_util as G
+from tests.test_gpu_parity import _conv, _mk
+
+ALL = 0   # all SMs
+# (kernel, layer, n, h, w, SMs)
+CASES = [
+    # pointwise layers of at most 64 input channels: one and two blocks of them, partial ones, one to four eights of output channels
+    ("conv_narrow_kernel<1, 1, 0>", _conv(8, 8, 1, act="none"), 1, 1, 1, ALL),
+    ("conv_narrow_kernel<1, 2, 2>", _conv(24, 16, 1, act="relu6"), 3, 17, 13, ALL),
+    ("conv_narrow_kernel<1, 3, 1>", _conv(24, 24, 1, res_src=-1), 5, 31, 29, ALL),
+    ("conv_narrow_kernel<1, 4, 2>", _conv(16, 96, 1, act="relu6"), 4, 56, 57, ALL),
+    ("conv_narrow_kernel<2, 1, 1>", _conv(64, 8, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 2, 0>", _conv(40, 16, 1, act="none"), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 3, 1>", _conv(48, 24, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 4, 1>", _conv(56, 192, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 4, 1>", _conv(64, 64, 1, res_src=-1), 7, 28, 28, ALL),
+    # one tile per CTA, K over clusters of 1 to 8
+    ("conv_lat_kernel<1>", _conv(64, 64, 1), 1, 56, 56, ALL),
+    ("conv_lat_kernel<1>", _conv(64, 64, 3, res_src=-1), 5, 27, 29, ALL),
+    ("conv_lat_kernel<2>", _conv(24, 40, 3), 2, 9, 11, ALL),
+    ("conv_lat_kernel<2>", _conv(2048, 1000, 1, act="none"), 3, 1, 1, 20),
+    ("conv_lat_kernel<4>", _conv(136, 72, 3), 1, 13, 13, ALL),
+    ("conv_lat_kernel<4>", _conv(192, 192, 3, act="relu6", res_src=-1), 1, 14, 14, 40),
+    ("conv_lat_kernel<8>", _conv(512, 512, 3, act="none"), 1, 7, 7, ALL),
+    ("conv_lat_kernel<8>", _conv(96, 16, 5), 1, 5, 7, 20),
+    # persistent, one CTA to a work item
+    ("conv_tc_kernel<1, false, false, false, false>", _conv(72, 64, 1), 1, 20, 23, 2),
+    ("conv_tc_kernel<1, false, true, true, false> by rows", _conv(64, 64, 3, res_src=-1), 1, 20, 23, 2),
+    ("conv_tc_kernel<1, false, false, true, false> by columns", _conv(64, 128, 3), 1, 20, 23, 3),
+    ("conv_tc_kernel<1, true, true, true, false> by columns", _conv(64, 64, 3, pool=2, res_src=-1), 1, 20, 23, 2),
+    ("conv_tc_kernel<1, false, false, true, true> by rows", _conv(1024, 16, 3), 1, 14, 14, 4),    # K shared out between CTAs
+    # ... two: pixel lists, strides, partial last chunks, pooling, odd SM counts (the last SM stays out)
+    ("conv_tc_pair_kernel<1, false, false, false>", _conv(512, 192, 1), 1, 20, 23, 3),
+    ("conv_tc_pair_kernel<1, false, true, false>", _conv(512, 512, 1, res_src=-1), 1, 20, 23, 7),
+    ("conv_tc_pair_kernel<1, true, true, false>", _conv(512, 512, 1, pool=2, res_src=-1), 1, 20, 23, 5),
+    ("conv_tc_pair_kernel<0, false, false, false>", _conv(512, 64, 1, stride=2, pad=0, act="none"), 1, 61, 59, 2),
+    ("conv_tc_pair_kernel<1, false, false, false>", _conv(72, 192, 3), 2, 33, 31, 2),
+    ("conv_tc_pair_kernel<2, true, false, false>", _conv(200, 320, 3, pool=2, act="relu6"), 1, 20, 23, 5),
+    ("conv_tc_pair_kernel<1, false, true, true> by rows", _conv(64, 64, 3, res_src=-1), 1, 61, 59, 5),
+    ("conv_tc_pair_kernel<1, false, false, true> by rows", _conv(64, 192, 3), 1, 20, 23, 2),
+    ("conv_tc_pair_kernel<1, false, false, true> by columns", _conv(64, 128, 3), 2, 33, 31, 7),
+    ("conv_tc_pair_kernel<1, false, true, true> by columns", _conv(64, 64, 3, res_src=-1), 2, 33, 31, 2),
+    ("conv_tc_pair_kernel<1, true, true, true> by columns", _conv(64, 64, 3, pool=2, res_src=-1), 3, 28, 28, 7),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "%s-%d-%d-k%d-S%d" % (c[0].replace("_kernel", "").replace(" ", ""), c[1]["cin"], c[1]["cout"], c[1]["kh"], c[5]))
+def test_variant(case):
+    kernel, layer, n, h, w, sms = case
+    sess, xd, ref = _mk([layer], "variant", n, h, w, layer["cin"])
+    sms = sms or B.device_sm_count()
+    G.check_plan(sess, xd, ref, [0], [sms], kernel)
+    name, grid, _ = sess.launches()[0]
+    sess.close()
+    assert name == kernel
+    if not name.startswith("conv_narrow"):
+        assert grid <= sms
+
+
+def test_the_query_follows_the_plan():
+    layers = [_conv(16, 16, 3), _conv(16, 16, 3, src=0)]
+    sess, _, _ = _mk(layers, "query", 1, 32, 32, 16)
+    sess.set_plan([0, 1], [20, 20])
+    assert [a[0].split("<")[0] for a in sess.launches()] == ["conv_lat_kernel"] * 2
+    sess.set_plan([1], [8])
+    assert sess.launches()[0][0].startswith("chain_tc_kernel") and sess.launches()[0][1] == 8
+    with pytest.raises(B.DlfError):
+        B.net_group_launch(sess.net, 1)
+    sess.close()
