@@ -142,7 +142,7 @@ constexpr size_t kSplitKBytes = kSplitKCounterBytes + (16u << 20);
 
 static bool is_param(const Layer& l) { return l.d.op == DLF_CONV || l.d.op == DLF_DWCONV || l.d.op == DLF_FC; }
 
-static int query_sms(int* out) {
+int query_sms(int* out) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);

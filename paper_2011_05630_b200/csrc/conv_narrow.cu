@@ -22,7 +22,7 @@ namespace dlf {
 
 namespace {
 
-constexpr int kWarps = 8;
+constexpr int kWarps = 8, kWideWarps = 24;   // of a CTA: where the plan gives the layer all SMs / fewer (see launch_conv_narrow)
 constexpr int kTiles = 2;   // 16-pixel tiles a warp has in flight
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -32,8 +32,8 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
 }
 
 // KB: blocks of 32 input channels; NT: eights of output channels of a warp (Cout = 8 NT blocks)
-template <int KB, int NT, int ACT>
-__global__ void __launch_bounds__(32 * kWarps) conv_narrow_kernel(const __half* x, const __half* __restrict__ w, const float* __restrict__ bias,
+template <int KB, int NT, int ACT, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) conv_narrow_kernel(const __half* x, const __half* __restrict__ w, const float* __restrict__ bias,
                                                                    const __half* res, __half* y, int cin, int cout, int blocks, long long pixels) {
     constexpr int kOwn = 2 * NT;   // neighbouring channels of a pixel that a lane finishes
     // The residual is fetched ahead of the sums where there are many of them (64 -> 64 with a residual at seven 28x28 images 3.5 us
@@ -122,17 +122,17 @@ __global__ void __launch_bounds__(32 * kWarps) conv_narrow_kernel(const __half* 
 }
 
 typedef void (*KernelFn)(const __half*, const __half*, const float*, const __half*, __half*, int, int, int, long long);
-template <int KB, int NT>
+template <int KB, int NT, int WARPS>
 KernelFn pick_act(int act) {
-    return act == DLF_ACT_RELU6 ? conv_narrow_kernel<KB, NT, 2> : (act == DLF_ACT_RELU ? conv_narrow_kernel<KB, NT, 1> : conv_narrow_kernel<KB, NT, 0>);
+    return act == DLF_ACT_RELU6 ? conv_narrow_kernel<KB, NT, 2, WARPS> : (act == DLF_ACT_RELU ? conv_narrow_kernel<KB, NT, 1, WARPS> : conv_narrow_kernel<KB, NT, 0, WARPS>);
 }
-template <int KB>
+template <int KB, int WARPS>
 KernelFn pick_nt(int nt, int act) {
     switch (nt) {
-        case 1: return pick_act<KB, 1>(act);
-        case 2: return pick_act<KB, 2>(act);
-        case 3: return pick_act<KB, 3>(act);
-        default: return pick_act<KB, 4>(act);
+        case 1: return pick_act<KB, 1, WARPS>(act);
+        case 2: return pick_act<KB, 2, WARPS>(act);
+        case 3: return pick_act<KB, 3, WARPS>(act);
+        default: return pick_act<KB, 4, WARPS>(act);
     }
 }
 
@@ -149,10 +149,19 @@ int launch_conv_narrow(const ConvArgs& a, int sm_count, cudaStream_t s) {
     // (and on few pixels the cluster kernel, whose weights are on their way before the layer before it ends: a network's six such
     // layers on one 56x56 image take 2.5 us more here)
     if (a.Cin > 32 && pixels < 5000) return DLF_E_UNSUPPORTED;
-    const int blocks = std::max(1, a.Cout / 32), groups = kWarps / blocks;
+    int sms = 0;
+    const int rc = query_sms(&sms);
+    if (rc) return rc;
+    // Four CTAs per SM spread over all SMs that are free, so a plan that gives the layer fewer gets one large CTA for each of them.
+    // With two blocks of input channels too few warps fit into one: the tcgen05 kernels are as fast there (64 -> 64 with a residual
+    // at 33 images of 56x56 on 74 SMs 13.8 us against 16.3, 64 -> 256 with one at three 6.1 against 7.1).
+    const bool wide = sm_count < sms;
+    if (wide && a.Cin > 32) return DLF_E_UNSUPPORTED;
+    const int ctas_sm = wide ? 1 : 4, blocks = std::max(1, a.Cout / 32), groups = (wide ? kWideWarps : kWarps) / blocks;
     const long long ctas = (pixels + 16 * kTiles * groups - 1) / (16 * kTiles * groups);
-    const int grid = static_cast<int>(std::min<long long>(ctas, 4ll * sm_count)), nt = std::min(a.Cout / 8, 4);
-    cudaError_t e = launch_kernel(a.Cin <= 32 ? pick_nt<1>(nt, a.act) : pick_nt<2>(nt, a.act), grid, 32 * blocks * groups, 0, s,
+    const int grid = static_cast<int>(std::min<long long>(ctas, static_cast<long long>(ctas_sm) * sm_count)), nt = std::min(a.Cout / 8, 4);
+    const KernelFn fn = a.Cin > 32 ? pick_nt<2, kWarps>(nt, a.act) : (wide ? pick_nt<1, kWideWarps>(nt, a.act) : pick_nt<1, kWarps>(nt, a.act));
+    cudaError_t e = launch_kernel(fn, grid, 32 * blocks * groups, 0, s,
                                   static_cast<const __half*>(a.x), static_cast<const __half*>(a.w), a.bias, static_cast<const __half*>(a.res),
                                   static_cast<__half*>(a.y), a.Cin, a.Cout, blocks, pixels);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);

@@ -77,6 +77,7 @@ inline bool aligned(uintptr_t bytes, P... ptrs) { return (((reinterpret_cast<uin
 
 int cuda_fail(cudaError_t e);  // records the error for dlf_last_cuda_error, returns DLF_E_CUDA
 int cuda_fail_drv(int e);
+int query_sms(int* out);       // SMs of the current device
 
 // A kernel's shared-memory attribute belongs to a device, not to the process: the *_init functions keep one
 // "done" flag per device, indexed by the current device.  -1: no current device or beyond the table.

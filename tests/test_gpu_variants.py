@@ -13,15 +13,15 @@ ALL = 0   # all SMs
 # (kernel, layer, n, h, w, SMs)
 CASES = [
     # pointwise layers of at most 64 input channels: one and two blocks of them, partial ones, one to four eights of output channels
-    ("conv_narrow_kernel<1, 1, 0>", _conv(8, 8, 1, act="none"), 1, 1, 1, ALL),
-    ("conv_narrow_kernel<1, 2, 2>", _conv(24, 16, 1, act="relu6"), 3, 17, 13, ALL),
-    ("conv_narrow_kernel<1, 3, 1>", _conv(24, 24, 1, res_src=-1), 5, 31, 29, ALL),
-    ("conv_narrow_kernel<1, 4, 2>", _conv(16, 96, 1, act="relu6"), 4, 56, 57, ALL),
-    ("conv_narrow_kernel<2, 1, 1>", _conv(64, 8, 1), 2, 61, 59, ALL),
-    ("conv_narrow_kernel<2, 2, 0>", _conv(40, 16, 1, act="none"), 2, 61, 59, ALL),
-    ("conv_narrow_kernel<2, 3, 1>", _conv(48, 24, 1), 2, 61, 59, ALL),
-    ("conv_narrow_kernel<2, 4, 1>", _conv(56, 192, 1), 2, 61, 59, ALL),
-    ("conv_narrow_kernel<2, 4, 1>", _conv(64, 64, 1, res_src=-1), 7, 28, 28, ALL),
+    ("conv_narrow_kernel<1, 1, 0, 8>", _conv(8, 8, 1, act="none"), 1, 1, 1, ALL),
+    ("conv_narrow_kernel<1, 2, 2, 8>", _conv(24, 16, 1, act="relu6"), 3, 17, 13, ALL),
+    ("conv_narrow_kernel<1, 3, 1, 8>", _conv(24, 24, 1, res_src=-1), 5, 31, 29, ALL),
+    ("conv_narrow_kernel<1, 4, 2, 8>", _conv(16, 96, 1, act="relu6"), 4, 56, 57, ALL),
+    ("conv_narrow_kernel<2, 1, 1, 8>", _conv(64, 8, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 2, 0, 8>", _conv(40, 16, 1, act="none"), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 3, 1, 8>", _conv(48, 24, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 4, 1, 8>", _conv(56, 192, 1), 2, 61, 59, ALL),
+    ("conv_narrow_kernel<2, 4, 1, 8>", _conv(64, 64, 1, res_src=-1), 7, 28, 28, ALL),
     # one tile per CTA, K over clusters of 1 to 8
     ("conv_lat_kernel<1>", _conv(64, 64, 1), 1, 56, 56, ALL),
     ("conv_lat_kernel<1>", _conv(64, 64, 3, res_src=-1), 5, 27, 29, ALL),
@@ -63,6 +63,18 @@ def test_variant(case):
     assert name == kernel
     if not name.startswith("conv_narrow"):
         assert grid <= sms
+
+
+@pytest.mark.parametrize("cin,cout,act,res", [(8, 8, "none", False), (24, 16, "relu6", False), (24, 24, "relu", True), (32, 32, "relu", False),
+                                               (16, 96, "relu6", False), (32, 256, "none", False), (64, 64, "relu", True)])
+def test_narrow_layers_keep_to_the_sm_count(cin, cout, act, res):
+    """One CTA on each of the SMs that the plan names, whatever is free beside them."""
+    sess, xd, ref = _mk([_conv(cin, cout, 1, act=act, res_src=-1 if res else -2)], "knob", 2, 61, 59, cin)
+    for sms in (B.device_sm_count() - 1, 37, 2, 1):
+        G.check_plan(sess, xd, ref, [0], [sms], "narrow S=%d" % sms)
+        name, grid, _ = sess.launches()[0]
+        assert grid <= sms and name.startswith("conv_narrow") == (cin <= 32), (name, grid)
+    sess.close()
 
 
 def test_the_query_follows_the_plan():
