@@ -835,7 +835,8 @@ static int build_host_parts(dlf_net* net, int head) {
 }
 
 // The input in kHostParts copies on a stream of the net's own, the plan's first groups for a part as soon as it is there, then
-// the other groups for the whole batch.  Leaves the output in its workspace slot.
+// the other groups for the whole batch.  Leaves the output in its workspace slot.  Each part's groups are launched ahead of the
+// next copy: one from pageable memory holds this thread until it is almost done.
 static int run_host_parts(dlf_net* net, const void* in_host, cudaStream_t s) {
     uint8_t* in_dev = net->ws + net->in_off;
     const size_t image = net->in_bytes / net->N;
@@ -846,13 +847,14 @@ static int run_host_parts(dlf_net* net, const void* in_host, cudaStream_t s) {
     for (int i = 0; i < kHostParts && e == cudaSuccess; i++) {
         e = cudaMemcpyAsync(in_dev + n0[i] * image, static_cast<const uint8_t*>(in_host) + n0[i] * image, (n0[i + 1] - n0[i]) * image, cudaMemcpyHostToDevice, net->copy_stream);
         if (e == cudaSuccess) e = cudaEventRecord(net->host_event[i], net->copy_stream);
-    }
-    for (int i = 0; i < kHostParts && e == cudaSuccess; i++) {
-        e = cudaStreamWaitEvent(s, net->host_event[i], 0);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, net->host_event[i], 0);
         if (e == cudaSuccess) e = cudaGraphLaunch(net->host_part[i].exec, s);
     }
     if (e == cudaSuccess) e = cudaGraphLaunch(net->host_rest.exec, s);
-    if (e != cudaSuccess) return cuda_fail(e);
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(net->copy_stream);   // the caller's buffer is no longer read
+        return cuda_fail(e);
+    }
     net->last_out = net->ws + net->layers.back().off;
     return DLF_OK;
 }

@@ -70,3 +70,24 @@ def test_parts_of_images_with_an_odd_number_of_elements(n, h, w):
     s.close()
     # single fp16 roundings (see above)
     assert float((y.float() - ref).norm() / ref.norm()) < 2e-3
+
+
+def test_parts_from_pageable_memory():
+    """Buffers that are not page-locked, overwritten as soon as the call is back."""
+    layers = _chain()
+    g = torch.Generator().manual_seed(7)
+    params = [((torch.randn((l["cout"], l["kh"], l["kw"], l["cin"]), generator=g) * (l["kh"] * l["kw"] * l["cin"]) ** -0.5).half().numpy(),
+               (torch.randn(l["cout"], generator=g) * 0.1).numpy()) for l in layers]
+    s = Session(layers, params, 20, 128, 120, 16)
+    s.set_plan(*plans.tuned_plan(s.net, len(layers)))
+    x = (torch.rand((20, 128, 120, 16), generator=g) * 2 - 1).half()
+    y = torch.empty(s.out_shape, dtype=torch.float16)
+    for _ in range(3):
+        xh = x.clone()
+        y.fill_(float("nan"))
+        B.net_run_host(s.net, xh.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        xh.fill_(float("nan"))
+        ref = s.run(x.cuda()).float().cpu()
+        assert float((y.float() - ref).norm() / ref.norm()) < 2e-3   # (see above)
+        x = -x
+    s.close()
