@@ -237,10 +237,11 @@ int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes,
  *   DLF_OPT_PDL              1 (default): the tensor-core kernels are launched with programmatic
  *                               dependent launch, so that a kernel's set-up overlaps the tail of
  *                               its predecessor; 0: plain stream order.  Process-wide.
- *   DLF_OPT_CONV_ROW_MODE    1 (default): a single 3x3 stride-1 convolution whose C_in is a multiple of 64 and
- *                               whose image is at most 126 pixels wide loads a kernel row's input window once for
- *                               its three taps where that cuts the bytes a CTA streams by a fifth; 0: never (one
- *                               window load per tap); 2: wherever it applies.  Process-wide; does not clear the plan. */
+ *   DLF_OPT_CONV_ROW_MODE    1 (default): a single 3x3 stride-1 convolution whose C_in is a multiple of 64 may load
+ *                               the input window of a kernel row (images of at most 126 pixels per row, no pool) or of a
+ *                               kernel column once for its three taps, where the estimate of the launch says that this
+ *                               is the fastest; 0: never (one window load per tap); 2: by rows wherever it applies.
+ *                               Process-wide; does not clear the plan. */
 enum { DLF_OPT_NO_TENSOR_CORE = 1, /* 2 is unused */ DLF_OPT_SINGLE_AS_CHAIN = 3, DLF_OPT_CUDA_GRAPH = 4, DLF_OPT_PDL = 5,
        DLF_OPT_CONV_ROW_MODE = 6, DLF_OPT_GROUP_KERNEL = 7 };
 int dlf_net_set_option(dlf_net* net, int option, int value);

@@ -473,6 +473,7 @@ int launch_conv_lat(const ConvArgs& a_in, int sm_count, int* status_dev, cudaStr
     // -> 128 at six 28x28 images 5.0 against 6.1), except for layers whose kernel rows the persistent kernel loads once: there it
     // takes over when a CTA's share of K is long (256 -> 256 3x3 at six 14x14 images: 9.6 against 9.1).
     const bool row = a.kh == 3 && a.kw == 3 && a.stride == 1 && a.Cin % 64 == 0 && g_conv_row_mode > 0;
+    if (g_conv_row_mode > 1 && conv_tc_row_mode(a)) return DLF_E_UNSUPPORTED;   // (asked for)
     if (c.cost < 0 || (row && c.cost > 8600.0 + 117.0 * p.total)) return DLF_E_UNSUPPORTED;
     p.N = a.N; p.Ho = a.Ho; p.Wo = a.Wo; p.Cout = a.Cout;
     p.kw = a.kw; p.stride = a.stride; p.pad = a.pad; p.stride2 = dual ? a.stride2 : 1;

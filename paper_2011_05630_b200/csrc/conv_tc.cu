@@ -954,6 +954,11 @@ bool conv_tc_supported(const ConvArgs& a) {
     return true;
 }
 
+// Row mode (conv_tc_prepare): 3x3, stride 1, pad 1, whole 64-channel chunks, at most 126 pixels in an image's row.
+bool conv_tc_row_mode(const ConvArgs& a) {
+    return g_conv_row_mode > 0 && a.kh == 3 && a.kw == 3 && a.stride == 1 && a.pad == 1 && !a.pool && a.Cin % 64 == 0 && a.Wo + 2 <= 128;
+}
+
 // The second source joins a 1x1 stride-1 layer chunk by chunk of 64 channels; both channel counts are whole chunks.
 bool conv_tc_dual_supported(const ConvArgs& a) {
     if (!conv_tc_supported(a)) return false;
@@ -1149,7 +1154,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
     Tile tl_row{};
     int bias_row = 0;
     double cost_row = 0.0;
-    if (g_conv_row_mode > 0 && a.kh == 3 && a.kw == 3 && a.stride == 1 && a.pad == 1 && !a.pool && p.grouped && a.Wo + 2 <= 128 && a.W == a.Wo && a.H == a.Ho) {
+    if (conv_tc_row_mode(a)) {
         const int th_row = std::min(a.Ho, 128 / (a.Wo + 2));
         // several whole images per tile where they fit (an image's rows stay together, so the shifted reads of its
         // valid pixels never reach the next image)
@@ -1224,6 +1229,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
     // channel width, and the column mode: whatever the estimate says is fastest.  (A second source was measured without pairs
     // only.)  512 -> 512 1x1 at eight 60x60 images 21.5 -> 19.4 us against the width alone, 128 -> 128 3x3 stride 2 at 28x28, batch 32 16.4 ->
     // 13.8, 128 -> 512 1x1 there 11.8 -> 10.7.
+    const bool row_only = row_mode && g_conv_row_mode > 1;   // (asked for: only pairs are left to choose)
     if (allow_pair && splits == 1) {
         struct Layout { ConvTcParams p; Tile tl; int bias_bytes; long long m_tiles; bool pair; };
         Layout best_l{p, tl, bias_bytes, m_tiles, pair};
@@ -1243,7 +1249,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         };
         const bool three = a.kh == 3 && a.kw == 3 && a.stride == 1;
         for (int pr = 0; pr < 2; pr++) {
-            if (!(three && pr == 0)) {
+            if (!(three && pr == 0) && !row_only) {
                 if (flat && pr) set_tile(Tile{std::min(128, a.Wo), 1, 1}, 1);
                 else set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
                 consider(pr);
@@ -1252,7 +1258,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
                 set_tile(tl_row, 3);
                 consider(pr);
             }
-            if (g_conv_row_mode > 0 && three && a.pad == 1 && p.grouped && a.W == a.Wo && a.H == a.Ho)
+            if (g_conv_row_mode > 0 && !row_only && three && a.pad == 1 && p.grouped)
                 for (int tw = 8; tw <= 64 && tw < a.Wo + 8; tw += 8) {
                     if (a.pool && tw != 8 && tw != 16) continue;   // (2x2 windows are reduced by warp shuffles)
                     const int th_max = a.pool ? 128 / tw : std::min(a.Ho, 128 / tw), rows_h = (a.Ho + th_max - 1) / th_max;

@@ -164,6 +164,7 @@ int launch_stall(int* status_dev, unsigned long long limit_ns, cudaStream_t s);
 
 // conv_tc.cu
 bool conv_tc_supported(const ConvArgs& a);
+bool conv_tc_row_mode(const ConvArgs& a);
 bool chain_tc_layer_supported(int cin, int cout, int k);
 int launch_conv_tc(const ConvArgs& a, int sm_count, int* status_dev, cudaStream_t s);
 // conv_lat.cu: the same layers without pooling where one tile per CTA covers them; DLF_E_UNSUPPORTED: not such a layer.

@@ -7,6 +7,7 @@ pytestmark = pytest.mark.gpu
 
 from paper_2011_05630_b200 import binding as B
 from tests import gpu_util as G
+from tests import test_gpu_parity as TP
 from tests.test_gpu_parity import _conv, _mk
 
 ALL = 0   # all SMs
@@ -86,4 +87,41 @@ def test_the_query_follows_the_plan():
     assert sess.launches()[0][0].startswith("chain_tc_kernel") and sess.launches()[0][1] == 8
     with pytest.raises(B.DlfError):
         B.net_group_launch(sess.net, 1)
+    sess.close()
+
+
+def test_row_mode_option():
+    """2: by rows wherever that applies, pairs or not; 0: neither by rows nor by columns."""
+    for n, h, w, layer in TP.ROW_MODE:
+        sess, xd, ref = _mk([layer], "rowmode", n, h, w, layer["cin"])
+        try:
+            for mode in (2, 0):
+                B.net_set_option(sess.net, B.OPT_CONV_ROW_MODE, mode)
+                for sms in (B.device_sm_count(), 5):
+                    G.check_plan(sess, xd, ref, [0], [sms], "row mode %d S=%d" % (mode, sms))
+                    name = sess.launches()[0][0]
+                    assert name.endswith(" by rows") == (mode == 2 and w <= 126), (mode, w, name)
+                    assert mode == 2 or "columns" not in name, (mode, w, name)
+        finally:
+            B.net_set_option(sess.net, B.OPT_CONV_ROW_MODE, 1)
+        sess.close()
+
+
+def test_split_reduction_over_a_pixel_list():
+    """A fully connected layer of many images and a long K on few SMs: the variant of the persistent kernel that shares K out."""
+    n, k, m = 200, 25088, 1000
+    layers = [dict(_conv(k, m, 1), op="fc")]
+    g = torch.Generator(device="cuda").manual_seed(1)
+    w = (torch.randn((m, k), generator=g, device="cuda") * k ** -0.5).half()
+    b = torch.randn((m,), generator=g, device="cuda") * 0.1
+    x = (torch.rand((n, 1, 1, k), generator=g, device="cuda") * 2 - 1).half()
+    sess = TP.Session(layers, [(w.cpu().numpy(), b.cpu().numpy())], n, 1, 1, k)
+    sess.set_plan([0], [20])
+    assert sess.launches()[0][0] == "conv_tc_kernel<1, false, false, false, true>"
+    ref = (x.reshape(n, k).double() @ w.double().T + b.double()).clamp(min=0)
+    for _ in range(2):   # (the arrival counters are back at zero after a launch)
+        got = sess.run(x).reshape(n, m).double()
+        # one rounding to fp16, and 25088 fp32 additions to partial sums below 8: 25088 * 8 * 2^-24 / 2 = 0.006 at the very worst,
+        # its square root's share (1e-4) as a rule
+        assert bool(((got - ref).abs() <= 2 ** -11 * ref + 1e-3).all())
     sess.close()
