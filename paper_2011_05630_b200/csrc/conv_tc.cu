@@ -884,18 +884,23 @@ Tile pick_tile(int N, int Ho, int Wo, int pool) {
         return best;
     }
     int best_rows = 0;
-    for (int tn = 1; tn <= std::min(N, 128); tn++)
-        for (int th = 1; th <= std::min(Ho, 128 / tn); th++) {
-            const int tw_max = std::min(Wo, 128 / (tn * th));
-            const int tw = (Wo + (Wo + tw_max - 1) / tw_max - 1) / ((Wo + tw_max - 1) / tw_max);  // as many tiles per row, evenly wide
+    // (of the heights that make the same number of tile rows the least is never worse, and so for the images)
+    for (int tn = 1, parts_n = 0; tn <= std::min(N, 128); tn++) {
+        if ((N + tn - 1) / tn == parts_n) continue;
+        parts_n = (N + tn - 1) / tn;
+        for (int th = 1, parts_h = 0; th <= std::min(Ho, 128 / tn); th++) {
+            if ((Ho + th - 1) / th == parts_h) continue;
+            parts_h = (Ho + th - 1) / th;
+            const int tw_max = std::min(Wo, 128 / (tn * th)), cols = (Wo + tw_max - 1) / tw_max, tw = (Wo + cols - 1) / cols;  // as many tiles per row, evenly wide
             const int rows = tn * th * tw;
-            const long long tiles = static_cast<long long>((Wo + tw - 1) / tw) * ((Ho + th - 1) / th) * ((N + tn - 1) / tn);
+            const long long tiles = static_cast<long long>((Wo + tw - 1) / tw) * parts_h * parts_n;
             if (best_tiles < 0 || tiles < best_tiles || (tiles == best_tiles && (rows < best_rows || (rows == best_rows && tw > best.tw)))) {
                 best_tiles = tiles;
                 best_rows = rows;
                 best = Tile{tw, th, tn};
             }
         }
+    }
     return best;
 }
 
@@ -1005,7 +1010,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         p.stride2 = a.stride2;
     }
     p.grouped = (a.Cin % 64 == 0) ? 1 : 0;
-    Tile tl{};
+    Tile tl{}, tl_image{};
     long long m_tiles = 0;
     int bias_bytes = 0;
     int splits = 1;   // split-K shares per tile that configure() lays the channel tiles out for
@@ -1195,7 +1200,8 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         splits = best_s;
         set_tile(Tile{best_r, 1, 1}, 1);
     } else {
-        set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
+        tl_image = pick_tile(a.N, a.Ho, a.Wo, a.pool);
+        set_tile(tl_image, 1);
     }
     if (!configure(kMaxSmem, 256, 1)) return DLF_E_UNSUPPORTED;
     if (row_mode && (g_conv_row_mode > 1 || cost_row < 0.8 * stream_cost())) {
@@ -1251,7 +1257,7 @@ int conv_tc_prepare(const ConvArgs& a_in, int sm_count, int* status_dev, bool al
         for (int pr = 0; pr < 2; pr++) {
             if (!(three && pr == 0) && !row_only) {
                 if (flat && pr) set_tile(Tile{std::min(128, a.Wo), 1, 1}, 1);
-                else set_tile(pick_tile(a.N, a.Ho, a.Wo, a.pool), 1);
+                else set_tile(flat ? pick_tile(a.N, a.Ho, a.Wo, a.pool) : tl_image, 1);
                 consider(pr);
             }
             if (row_mode && pr) {
