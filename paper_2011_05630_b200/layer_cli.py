@@ -56,7 +56,7 @@ def main():
     sess.set_plan([len(layers) - 1], [B.device_sm_count()])
     for _ in range(a.reps):
         sess.run(xd)
-    print("ran", sess.kernels(), "x", a.reps)
+    print("ran", sess.launches(), "x", a.reps)
 
 
 if __name__ == "__main__":
