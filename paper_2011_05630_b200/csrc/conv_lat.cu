@@ -43,7 +43,7 @@ struct LatParams {
     int TN;
     int kchunks, kchunks1, ksteps_last;     // 64-channel chunks per tap (both sources), of the first source; UMMAs of the last one
     int total, share;                       // (tap, chunk) pairs of K, and how many a CTA of the cluster takes
-    int stride2, grouped;
+    int stride2;
     int stages, a_bytes, stage_bytes, red_off;
     int rows_per, act;
     const float* bias;

@@ -142,10 +142,12 @@ int launch_conv_narrow(const ConvArgs& a, int sm_count, cudaStream_t s) {
     if (a.kh != 1 || a.kw != 1 || a.stride != 1 || a.pad != 0 || a.groups != 1 || a.pool || a.x2 || a.Cin % 8 || a.Cin > 64) return DLF_E_UNSUPPORTED;
     if (a.Cout % 8 || (a.Cout > 32 && a.Cout % 32) || a.Cout > 32 * kWarps) return DLF_E_UNSUPPORTED;
     const long long pixels = static_cast<long long>(a.N) * a.H * a.W;
-    // with two blocks of input channels and three or more of output channels this kernel's multiply-adds outweigh its bytes: it
-    // wins where the hand-overs of the few tiles count (64 -> 256 at eight 28x28 images 3.9 us against 5.1, at twelve 56x56 ones 9.1
-    // against 9.1, at 32 of them 18.9 against 13.8)
-    if (a.Cin > 32 && a.Cout > 64 && pixels * a.Cout > 3000000) return DLF_E_UNSUPPORTED;
+    // With two blocks of input channels this kernel's multiply-adds outweigh its bytes once there is enough work to hide the tcgen05
+    // kernel's hand-overs: 64 -> 256 at 9000 / 12500 / 16000 / 37632 pixels 3.2 / 4.6 / 5.3 / 8.6 us against 4.5 / 5.6 / 5.2 / 8.0 there,
+    // with a residual 4.2 / 6.2 / 7.3 / 12.1 against 4.9 / 5.9 / 5.9 / 8.8.  Up to 64 output channels it stays ahead at any size (64 -> 64 at
+    // 100000 pixels 7.1 against 8.3), but for a residual beside a whole 64-channel chunk (37632 / 50000 / 100000 pixels 4.2 / 6.1 / 9.9
+    // against 5.3 / 6.1 / 9.0; 40 -> 64 9.3 against 14.3).  The line in the tens of thousands of pixels is where one round of the grid ends.
+    if (a.Cin > 32 && (a.Cout > 64 || (a.Cout == 64 && a.Cin == 64 && a.res)) && pixels * a.Cout > 3000000) return DLF_E_UNSUPPORTED;
     // (and on few pixels the cluster kernel, whose weights are on their way before the layer before it ends: a network's six such
     // layers on one 56x56 image take 2.5 us more here)
     if (a.Cin > 32 && pixels < 5000) return DLF_E_UNSUPPORTED;

@@ -38,6 +38,8 @@ CASES = [
     ("conv_tc_kernel<1, false, false, true, false> by columns", _conv(64, 128, 3), 1, 20, 23, 3),
     ("conv_tc_kernel<1, true, true, true, false> by columns", _conv(64, 64, 3, pool=2, res_src=-1), 1, 20, 23, 2),
     ("conv_tc_kernel<1, false, false, true, true> by rows", _conv(1024, 16, 3), 1, 14, 14, 4),    # K shared out between CTAs
+    ("conv_tc_kernel<1, false, true, false, false>", _conv(64, 64, 1, res_src=-1), 16, 56, 56, ALL),   # (without a residual: conv_narrow)
+    ("conv_narrow_kernel<2, 4, 1, 8>", _conv(64, 64, 1), 16, 56, 56, ALL),
     # ... two: pixel lists, strides, partial last chunks, pooling, odd SM counts (the last SM stays out)
     ("conv_tc_pair_kernel<1, false, false, false>", _conv(512, 192, 1), 1, 20, 23, 3),
     ("conv_tc_pair_kernel<1, false, true, false>", _conv(512, 512, 1, res_src=-1), 1, 20, 23, 7),
