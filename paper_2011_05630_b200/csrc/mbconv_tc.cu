@@ -7,9 +7,9 @@
 //   2. epilogue 1 (warps 0-7): bias, activation, fp16 rounding, zero outside the image (the depthwise layer's
 //      padding) -> hidden frame H in shared memory, rows of 64 channels 144 bytes apart (a row per lane on the way in, a row
 //      per half warp on the way out: neither conflicts, and no address needs a swizzle);
-//   3. depthwise 3x3 (warps 8-15, fp32): a thread keeps four channels' weights in registers and walks down a column of the
-//      tile; every input value is loaded and converted once per column it is used in and joins the three output rows it
-//      touches (packed fp32 multiply-adds); bias, activation, rounding -> dense tile Hd, the next operand;
+//   3. depthwise 3x3 (warps 8-15, fp32 sums): a thread keeps four channels' fp16 weights in registers and walks down a column
+//      of the tile; every input value is loaded once per column it is used in and joins the three output rows it touches
+//      (multiply-adds with fp16 factors); bias, activation, rounding -> dense tile Hd, the next operand;
 //   4. projection (tensor core): D2[tile rows x C_out] += Hd * W2[:, chunk]^T, accumulated in tensor memory across the chunks
 //      (fp32, the same sum as the unchunked layer);
 // then epilogue 2 (warps 8-15, behind the next tile's first depthwise chunk): bias, residual, activation, fp16 rounding.
