@@ -490,7 +490,7 @@ static bool make_group(const dlf_net* net, int first, int last, int sms, Group* 
 // of 2 to 8 layers timed both ways: 16 -> 16 3x3 at 5 images of 35x32 9.3 us fused against 12.3 for three layers, 24 -> 24 at
 // 10 of 81x79 66 against 113 for four, 64 -> 64 1x1 at 5 of 41x38 7.3 against 6.4 for two.
 // A chain may not swallow the expansion layer of an inverted-residual block (the layer a depthwise convolution reads):
-// that block fuses better as a whole.  Inverted-residual blocks follow the measured rule on the hidden width.  Groups
+// that block fuses better as a whole.  Inverted-residual blocks have an estimate of their own (mbconv_pays).  Groups
 // handed over through L2 are proposed only when the option asks for them (measured: a device-wide barrier per layer is no
 // cheaper than a kernel boundary).  `prefix`: the layers may also be the beginning of a pattern that can still grow.
 // A layer of a dense chain as a kernel of its own inside a network (see above).
@@ -1555,8 +1555,9 @@ int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes,
         char* full = abi::__cxa_demangle(mangled, nullptr, nullptr, nullptr);
         std::string text = full ? full : mangled;
         std::free(full);
-        const size_t args = text.rfind(">(") != std::string::npos ? text.find(">(") + 1 : text.rfind('(');
-        text = text.substr(0, args);
+        const std::string anon = "(anonymous namespace)::";
+        for (size_t at = text.find(anon); at != std::string::npos; at = text.find(anon)) text.erase(at, anon.size());
+        text = text.substr(0, text.find('('));
         const size_t scope = text.substr(0, text.find('<')).rfind("::");
         if (scope != std::string::npos) text = text.substr(scope + 2);
         std::snprintf(name, name_bytes, "%s%s", text.c_str(), rec.note);

@@ -92,6 +92,21 @@ def test_the_query_follows_the_plan():
     sess.close()
 
 
+@pytest.mark.parametrize("kernel,layers,ends", [
+    ("conv_seq_kernel", [_conv(128, 128, 3, stride=2), _conv(128, 64, 1, src=0)], [1]),
+    ("dw3x3_kernel<2>", [_conv(16, 16, 3, stride=2, groups=16, op="dwconv")], [0]),
+    ("maxpool_kernel", [dict(_conv(16, 16, 3, stride=2, act="none"), op="maxpool")], [0]),
+    ("gavgpool_kernel", [dict(_conv(16, 16, 1, act="none"), op="gavgpool")], [0]),
+    ("conv_direct_kernel", [_conv(6, 16, 3)], [0]),
+    ("mbconv_tc_kernel<1, true>", [_conv(16, 96, 1, act="relu6"), _conv(96, 96, 3, groups=96, op="dwconv", act="relu6", src=0), _conv(96, 16, 1, src=1, act="none")], [2]),
+], ids=lambda v: v if isinstance(v, str) else None)
+def test_names_of_the_other_kernels(kernel, layers, ends):
+    sess, xd, ref = _mk(layers, "names", 1, 20, 20, layers[0]["cin"])
+    G.check_plan(sess, xd, ref, ends, [B.device_sm_count()] * len(ends), kernel)
+    assert [a[0] for a in sess.launches()] == [kernel]
+    sess.close()
+
+
 def test_row_mode_option():
     """2: by rows wherever that applies, pairs or not; 0: neither by rows nor by columns."""
     for n, h, w, layer in TP.ROW_MODE:
