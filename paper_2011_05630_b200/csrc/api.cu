@@ -536,13 +536,19 @@ static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTi
     return false;
 }
 
-// The estimate for an inverted-residual block: the fused kernel's own cost model (the tiler's SM clocks, plus one kernel
-// boundary) against one kernel per layer.  Inside a network a layer's own kernel takes 3.1 us plus its bytes at 3.6 TB/s (the
-// depthwise one) or 3.2 TB/s (the pointwise ones) - fitted to MobileNetV2's blocks at 1 to 128 images, each timed both ways:
-// blocks on maps of 14x14 and more win from a few images on (24 -> 144 -> 24 channels at 56x56: 62 us against 95 at 64
-// images, 10 against 10 at one), wide ones on small maps (many 64-channel steps, few tiles to spread over the SMs) lose
-// (160 -> 960 -> 160 at 7x7: 25 against 20 at 64 images), and without an expansion layer only the smallest batches win.
-static bool mbconv_pays(const dlf_net* net, int first, int last, int sms) {
+// The estimate for an inverted-residual block: the fused kernel's own (the tiler's SM clocks; the persistent kernel's leaves out
+// 1.8 us of launch, fill and drain, the other one's is about 0.6 low on the smallest blocks) against one kernel per layer.  Inside a network a layer's own kernel takes 2.9 us plus its bytes at
+// 3.6 TB/s (the depthwise one) or 3.2 TB/s (the pointwise ones) - fitted to MobileNetV2's blocks at 1 to 128 images, each timed
+// both ways: on few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.6 us against 8.7), from a few
+// images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
+// small maps lose at many images (160 -> 960 -> 160 at 7x7: 27 us against 20 at 64), and so does a block without an expansion layer.
+// (`memo`: 1 or 0 for the blocks of one tuner pass, each asked for several times)
+static bool mbconv_pays(const dlf_net* net, int first, int last, int sms, SpanTimes* memo = nullptr) {
+    if (memo) {
+        const auto it = memo->find({first, last});
+        if (it != memo->end()) return it->second > 0.0;
+        return ((*memo)[{first, last}] = mbconv_pays(net, first, last, sms) ? 1.0 : 0.0) > 0.0;
+    }
     const MbconvTiling t = mbconv_tiling(mbconv_args(net, first, last, nullptr, nullptr), sms);
     if (!t.ok) return false;
     double single_us = 0.0;
@@ -550,9 +556,9 @@ static bool mbconv_pays(const dlf_net* net, int first, int last, int sms) {
         const Layer& l = net->layers[i];
         const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
                              (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
-        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + 3.1;
+        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + 2.9;
     }
-    return t.cost / 1.9e3 + 1.0 < single_us;
+    return t.cost / 1.9e3 + (t.split > 0 ? 0.6 : 1.8) < single_us;
 }
 
 static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix, int s_max, SpanTimes* memo = nullptr) {
@@ -561,7 +567,7 @@ static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix,
     if (span_is_mbconv(net, first, last, prefix)) {
         // (the layers may be the beginning of the block: the estimate is made for the whole of it)
         const int full_last = first + (net->layers[first].d.op == DLF_CONV ? 2 : 1);
-        return full_last < static_cast<int>(net->layers.size()) && span_is_mbconv(net, first, full_last, false) && mbconv_pays(net, first, full_last, s_max);
+        return full_last < static_cast<int>(net->layers.size()) && span_is_mbconv(net, first, full_last, false) && mbconv_pays(net, first, full_last, s_max, memo);
     }
     if (net->opt_group_kernel == 2 && span_is_seq(net, first, last)) return true;
     // a projection and the expansion layer it is added to are one product with a longer K: never slower than the two kernels
@@ -702,6 +708,7 @@ int kernels_init() {
     int rc = conv_tc_init();
     if (rc == DLF_OK) rc = chain_tc_init();
     if (rc == DLF_OK) rc = mbconv_tc_init();
+    if (rc == DLF_OK) rc = mbconv_lat_init();
     return rc ? rc : stem_tc_init();
 }
 

@@ -53,23 +53,6 @@ struct LatParams {
     int* status;
 };
 
-// 16 bytes into the shared memory of a CTA of the cluster, counted by a barrier of that CTA (both addresses from mapa()).
-__device__ __forceinline__ void st_async_v4(uint32_t addr, float a, float b, float c, float d, uint32_t bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar) : "memory");
-}
-// 8 sums, their biases and 8 residual values to 8 rounded outputs.
-__device__ __forceinline__ uint4 finish8(const float* v, const float* bias, const uint4& res, __half2 lo, __half2 hi) {
-    const float4 c0 = *reinterpret_cast<const float4*>(bias), c1 = *reinterpret_cast<const float4*>(bias + 4);
-    const __half2* rh = reinterpret_cast<const __half2*>(&res);
-    const float2 f0 = __half22float2(rh[0]), f1 = __half22float2(rh[1]), f2 = __half22float2(rh[2]), f3 = __half22float2(rh[3]);
-    uint4 o;
-    o.x = pack_half2_clamp(v[0] + c0.x + f0.x, v[1] + c0.y + f0.y, lo, hi);
-    o.y = pack_half2_clamp(v[2] + c0.z + f1.x, v[3] + c0.w + f1.y, lo, hi);
-    o.z = pack_half2_clamp(v[4] + c1.x + f2.x, v[5] + c1.y + f2.y, lo, hi);
-    o.w = pack_half2_clamp(v[6] + c1.z + f3.x, v[7] + c1.w + f3.y, lo, hi);
-    return o;
-}
 template <int SPLIT>
 __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kThreads, 2)
 conv_lat_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx2,

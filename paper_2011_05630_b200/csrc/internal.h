@@ -194,6 +194,8 @@ struct MbconvArgs {
 struct MbconvTiling {
     int th, tw, fh, fw, nb1, nb2, tiles_h, tiles_w, n_tiles, stages, stage_bytes;
     int out_planes;  // 64-channel planes of the output staging buffer, 0 = none (direct stores)
+    int bh, units, job_units, parts, split;   // mbconv_lat.cu (split > 0): output rows of a unit (8 columns wide), units of a tile and of one accumulator,
+                                              // warps of a unit, CTAs of a tile
     size_t smem_bytes;
     double redundancy;
     double cost;     // the tiler's time estimate (SM clocks)
@@ -203,6 +205,10 @@ bool mbconv_supported(const MbconvArgs& a);
 MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count);
 int mbconv_tc_init();
 int launch_mbconv_tc(const MbconvArgs& a, const MbconvTiling& t, int sm_count, int* status_dev, cudaStream_t s);
+// mbconv_lat.cu: the same block where one tile per CTA or cluster covers it
+MbconvTiling mbconv_lat_tiling(const MbconvArgs& a, int sm_count);
+int mbconv_lat_init();
+int launch_mbconv_lat(const MbconvArgs& a, const MbconvTiling& t, int sm_count, int* status_dev, cudaStream_t s);
 
 // chain_tc.cu
 ChainTiling chain_tc_tiling(const ChainArgs& a, int sm_count, int device_sms);

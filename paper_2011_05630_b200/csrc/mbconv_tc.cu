@@ -702,7 +702,7 @@ bool mbconv_supported(const MbconvArgs& a) {
 
 // Output tile of the fused block from the SM count: candidates whose buffers and accumulators fit,
 // least (waves x per-tile work) in SM clocks.
-MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
+static MbconvTiling persistent_tiling(const MbconvArgs& a, int sm_count) {
     MbconvTiling best{};
     best.ok = false;
     if (!mbconv_supported(a) || sm_count < 1) return best;
@@ -748,6 +748,14 @@ MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
     return best;
 }
 
+// The kernel of mbconv_lat.cu where its tiles fit the chip at once and its estimate is the lower one.  (That one includes the launch; this
+// kernel's own leaves out about 1.7 us of it.  64 -> 384 -> 64 at 14x14: 12.8 -> 6.6 us at one image, 18.5 -> 13.3 at 64;
+// 160 -> 960 -> 160 at 7x7: 23.1 -> 7.2 at one.  24 -> 144 -> 24 at 56x56, eight images: 15.4 here, one wave of tiles is none there.)
+MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
+    const MbconvTiling t = persistent_tiling(a, sm_count), l = mbconv_lat_tiling(a, sm_count);
+    return l.ok && (!t.ok || l.cost < 0.97 * (t.cost + 3200.0)) ? l : t;
+}
+
 int mbconv_tc_init() {
     static bool attr_set[kMaxDevices] = {};
     const int dev = current_device_slot();
@@ -764,6 +772,7 @@ int mbconv_tc_init() {
 
 int launch_mbconv_tc(const MbconvArgs& a, const MbconvTiling& t, int sm_count, int* status_dev, cudaStream_t s) {
     if (!t.ok) return DLF_E_PLAN;
+    if (t.split > 0) return launch_mbconv_lat(a, t, sm_count, status_dev, s);
     if (!aligned(16, a.x, a.res, a.y)) return DLF_E_INVALID_ARG;
     int rc = mbconv_tc_init();
     if (rc) return rc;

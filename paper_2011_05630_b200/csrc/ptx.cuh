@@ -287,6 +287,11 @@ __device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64
 // start-address field of the lower word changes from one MMA to the next.
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+// An operand that lies along M instead (rows of 64 consecutive M values of ONE k, eight k to a 1024-byte swizzle atom, atoms of
+// further k right behind, further 64 values of M `lbo` bytes away): its low descriptor word, and the instruction descriptor's
+// bit that says so of operand A.
+constexpr uint32_t kIdescAmn = 1u << 15;
+__device__ __forceinline__ uint32_t umma_desc_mn_lo(uint32_t saddr, int lbo) { return ((saddr & 0x3FFFFu) >> 4) | (static_cast<uint32_t>(lbo >> 4) << 16); }
 __device__ __forceinline__ void umma_f16_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t idesc,
                                             uint32_t accumulate) {
     asm volatile(
@@ -356,6 +361,15 @@ __device__ __forceinline__ void umma_f16_steps(uint32_t d_tmem, uint32_t a_lo, u
         if (KS == 3) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_STEP(2, 2, 2) DLF_UMMA_STEP(2, 4, 4) DLF_UMMA_OPS);
         if (KS == 4) asm volatile(DLF_UMMA_FIRST(2) DLF_UMMA_STEP(2, 2, 2) DLF_UMMA_STEP(2, 4, 4) DLF_UMMA_STEP(2, 6, 6) DLF_UMMA_OPS);
     }
+}
+// ... with operand A along M: 16 k are two 1024-byte atoms, 128 units a step.
+template <int KS>
+__device__ __forceinline__ void umma_f16_mn_steps(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    const uint32_t w_tap16 = 0u;
+    if (KS == 1) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_OPS);
+    if (KS == 2) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 128, 2) DLF_UMMA_OPS);
+    if (KS == 3) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 128, 2) DLF_UMMA_STEP(1, 256, 4) DLF_UMMA_OPS);
+    if (KS == 4) asm volatile(DLF_UMMA_FIRST(1) DLF_UMMA_STEP(1, 128, 2) DLF_UMMA_STEP(1, 256, 4) DLF_UMMA_STEP(1, 384, 6) DLF_UMMA_OPS);
 }
 #undef DLF_UMMA_STEP
 #undef DLF_UMMA_FIRST
@@ -485,6 +499,24 @@ __device__ __forceinline__ uint32_t round_act(float a, float b) {
     if (ACT >= 1) h = __hmax2(h, __float2half2_rn(0.0f));
     if (ACT == 2) h = __hmin2(h, __float2half2_rn(6.0f));
     return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// 16 bytes into the shared memory of a CTA of the cluster, counted by a barrier of that CTA (both addresses from mapa()).
+__device__ __forceinline__ void st_async_v4(uint32_t addr, float a, float b, float c, float d, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar) : "memory");
+}
+// 8 sums, their biases and 8 residual values to 8 rounded outputs.
+__device__ __forceinline__ uint4 finish8(const float* v, const float* bias, const uint4& res, __half2 lo, __half2 hi) {
+    const float4 c0 = *reinterpret_cast<const float4*>(bias), c1 = *reinterpret_cast<const float4*>(bias + 4);
+    const __half2* rh = reinterpret_cast<const __half2*>(&res);
+    const float2 f0 = __half22float2(rh[0]), f1 = __half22float2(rh[1]), f2 = __half22float2(rh[2]), f3 = __half22float2(rh[3]);
+    uint4 o;
+    o.x = pack_half2_clamp(v[0] + c0.x + f0.x, v[1] + c0.y + f0.y, lo, hi);
+    o.y = pack_half2_clamp(v[2] + c0.z + f1.x, v[3] + c0.w + f1.y, lo, hi);
+    o.z = pack_half2_clamp(v[4] + c1.x + f2.x, v[5] + c1.y + f2.y, lo, hi);
+    o.w = pack_half2_clamp(v[6] + c1.z + f3.x, v[7] + c1.w + f3.y, lo, hi);
+    return o;
 }
 
 }  // namespace dlf

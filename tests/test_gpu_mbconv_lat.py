@@ -1,0 +1,43 @@
+"""Inverted-residual blocks on few images (one tile per CTA or cluster): every cluster size, hidden widths that leave the last chunk or
+its last 32-channel group part empty, windows over every edge of the image, several units to an accumulator, units past the
+last one, one and four input planes, outputs wider than one product, SM counts that leave no room for clusters."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2011_05630_b200 import binding as B
+from tests import gpu_util as G
+from tests.test_gpu_parity import _conv, _mk
+
+# (n, h, w, cin, hidden, cout, stride, SMs (0: all), CTAs of a cluster, activation)
+CASES = [
+    (1, 7, 7, 160, 960, 160, 1, 0, 8, "relu6"),      # residual
+    (1, 14, 14, 64, 384, 64, 1, 0, 4, "relu6"),      # chunks of 96 channels, residual
+    (2, 9, 11, 40, 240, 64, 1, 0, 2, "relu6"),       # last group of half the width
+    (5, 20, 29, 72, 528, 136, 1, 0, 2, "relu6"),     # several chunks per CTA, two units to an accumulator
+    (1, 28, 28, 32, 192, 32, 1, 0, 1, "relu6"),      # last chunk of two groups
+    (3, 30, 29, 24, 144, 24, 1, 0, 1, "relu6"),      # last chunk of half a group
+    (40, 14, 14, 64, 384, 64, 1, 0, 1, "relu6"),     # four units to an accumulator, of two images
+    (1, 15, 17, 24, 144, 32, 2, 0, 2, "relu"),
+    (1, 7, 7, 160, 960, 320, 1, 0, 8, "relu6"),      # projection issued as two halves
+    (3, 13, 9, 96, 160, 448, 1, 0, 1, "none"),       # the widest output
+    (1, 1, 1, 8, 128, 8, 1, 0, 1, "relu6"),          # one pixel
+    (1, 3, 2, 256, 1024, 16, 2, 0, 8, "relu6"),      # four input planes
+    (2, 16, 16, 16, 128, 16, 1, 7, 1, "relu6"),
+    (1, 8, 8, 16, 128, 16, 1, 1, 1, "relu"),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "n%d_%dx%d_%d_%d_%d_s%d_sm%d" % c[:8])
+def test_block(case):
+    n, h, w, cin, hid, cout, stride, sms, split, act = case
+    layers = [_conv(cin, hid, 1, act=act), _conv(hid, hid, 3, stride=stride, act=act, groups=hid, op="dwconv", src=0),
+              _conv(hid, cout, 1, act="none", src=1, res_src=-1 if stride == 1 and cin == cout else -2)]
+    sess, xd, ref = _mk(layers, "mbl", n, h, w, cin)
+    G.check_plan(sess, xd, ref, [2], [sms or B.device_sm_count()], "block")
+    assert sess.launches()[0][0] == "mbconv_lat_kernel<%d, %s, %d>" % (stride, "true" if act == "relu6" else "false", split)
+    assert sess.launches()[0][1] <= (sms or B.device_sm_count())
+    first = sess.run(xd).clone()
+    assert bool((sess.run(xd) == first).all())   # the same sum whatever the timing
+    sess.close()
