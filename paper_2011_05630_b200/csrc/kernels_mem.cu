@@ -320,67 +320,82 @@ __global__ void __launch_bounds__(kAvgVecs * kAvgParts) gavgpool_kernel(const __
 }
 
 // ---- fully connected --------------------------------------------------------------------------------------
-// A block owns 8 output features and streams their weight rows once per batch tile of 8 images;
-// threads stride over K in 128-bit pieces, accumulate 8x8 partial sums in fp32, then reduce.
+// A block owns 8 output features and streams their weight rows once per batch tile of NB images; threads stride over K in 128-bit
+// pieces, accumulate 8 x NB partial sums in fp32, then reduce.  Bound by latencies: the first weights are on their way before the wait
+// for the previous kernel, the next ones while the present ones are worked on, and one image pays for one (64 sums of eight images
+// were 320 shuffles a thread whatever the batch).  2048 -> 1000 at one image 5.1 -> 3.0 us, at two 4.5 -> 3.0.
 constexpr int kFcFo = 8;
-constexpr int kFcNb = 8;
 
+template <int NB>
 __global__ void __launch_bounds__(256) fc_kernel(const __half* x, const __half* w, const float* bias, __half* y, int N,
                                                  int K, int M, int act, int o_blocks, int n_blocks) {
-    __shared__ float red[8][kFcFo * kFcNb];
+    __shared__ float red[8][kFcFo * NB];
     const int k8n = K / 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4 wv[kFcFo];
+    auto load_w = [&](int blk, int k8) {
+        const int o0 = (blk % o_blocks) * kFcFo;
+#pragma unroll
+        for (int i = 0; i < kFcFo; i++) {
+            const int o = min(o0 + i, M - 1);
+            wv[i] = __ldcs(reinterpret_cast<const uint4*>(w + static_cast<long long>(o) * K) + k8);
+        }
+    };
     pdl_launch_dependents();
+    if (static_cast<int>(threadIdx.x) < k8n && static_cast<int>(blockIdx.x) < o_blocks * n_blocks) load_w(blockIdx.x, threadIdx.x);   // (constants)
     pdl_wait();
     for (int blk = blockIdx.x; blk < o_blocks * n_blocks; blk += gridDim.x) {
-        const int o0 = (blk % o_blocks) * kFcFo, n0 = (blk / o_blocks) * kFcNb;
-        float acc[kFcFo][kFcNb];
+        const int o0 = (blk % o_blocks) * kFcFo, n0 = (blk / o_blocks) * NB;
+        float acc[kFcFo][NB];
 #pragma unroll
         for (int i = 0; i < kFcFo; i++)
 #pragma unroll
-            for (int j = 0; j < kFcNb; j++) acc[i][j] = 0.0f;
+            for (int j = 0; j < NB; j++) acc[i][j] = 0.0f;
         for (int k8 = threadIdx.x; k8 < k8n; k8 += blockDim.x) {
-            uint4 wv[kFcFo], xv[kFcNb];
+            uint4 xv[NB], wc[kFcFo];
+            auto next_w = [&]() {
+                if (k8 + static_cast<int>(blockDim.x) < k8n) load_w(blk, k8 + blockDim.x);
+                else if (blk + static_cast<int>(gridDim.x) < o_blocks * n_blocks) load_w(blk + gridDim.x, threadIdx.x);
+            };
 #pragma unroll
-            for (int i = 0; i < kFcFo; i++) {
-                const int o = min(o0 + i, M - 1);
-                wv[i] = __ldcs(reinterpret_cast<const uint4*>(w + static_cast<long long>(o) * K) + k8);
-            }
-#pragma unroll
-            for (int j = 0; j < kFcNb; j++) {
+            for (int j = 0; j < NB; j++) {
                 const int n = min(n0 + j, N - 1);
                 xv[j] = ld_map(reinterpret_cast<const uint4*>(x + static_cast<long long>(n) * K) + k8);
             }
 #pragma unroll
-            for (int e = 0; e < 4; e++) {
-                float2 xf[kFcNb];
+            for (int i = 0; i < kFcFo; i++) wc[i] = wv[i];
+            if (NB <= 2) next_w();   // (more images leave no registers for it)
 #pragma unroll
-                for (int j = 0; j < kFcNb; j++) xf[j] = __half22float2(reinterpret_cast<const __half2*>(&xv[j])[e]);
+            for (int e = 0; e < 4; e++) {
+                float2 xf[NB];
+#pragma unroll
+                for (int j = 0; j < NB; j++) xf[j] = __half22float2(reinterpret_cast<const __half2*>(&xv[j])[e]);
 #pragma unroll
                 for (int i = 0; i < kFcFo; i++) {
-                    const float2 wf = __half22float2(reinterpret_cast<const __half2*>(&wv[i])[e]);
+                    const float2 wf = __half22float2(reinterpret_cast<const __half2*>(&wc[i])[e]);
 #pragma unroll
-                    for (int j = 0; j < kFcNb; j++) {
+                    for (int j = 0; j < NB; j++) {
                         acc[i][j] = fmaf(wf.x, xf[j].x, acc[i][j]);
                         acc[i][j] = fmaf(wf.y, xf[j].y, acc[i][j]);
                     }
                 }
             }
+            if (NB > 2) next_w();
         }
 #pragma unroll
         for (int i = 0; i < kFcFo; i++)
 #pragma unroll
-            for (int j = 0; j < kFcNb; j++) {
+            for (int j = 0; j < NB; j++) {
                 float v = acc[i][j];
 #pragma unroll
                 for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-                if (lane == 0) red[warp][i * kFcNb + j] = v;
+                if (lane == 0) red[warp][i * NB + j] = v;
             }
         __syncthreads();
-        if (threadIdx.x < kFcFo * kFcNb) {
+        if (threadIdx.x < kFcFo * NB) {
             float v = 0.0f;
             for (int wq = 0; wq < 8; wq++) v += red[wq][threadIdx.x];
-            const int o = o0 + threadIdx.x / kFcNb, n = n0 + threadIdx.x % kFcNb;
+            const int o = o0 + threadIdx.x / NB, n = n0 + threadIdx.x % NB;
             if (o < M && n < N) y[static_cast<long long>(n) * M + o] = __float2half_rn(apply_act(v + bias[o], act));
         }
         __syncthreads();
@@ -474,9 +489,11 @@ int launch_fc(const void* x, const void* w, const float* bias, void* y, int N, i
     if (K % 8) return DLF_E_UNSUPPORTED;
     if (!aligned(16, x)) return DLF_E_INVALID_ARG;
     if (N == 0) return DLF_OK;
-    const int o_blocks = (M + kFcFo - 1) / kFcFo, n_blocks = (N + kFcNb - 1) / kFcNb;
+    const int nb = N == 1 ? 1 : (N <= 2 ? 2 : (N <= 4 ? 4 : 8));
+    const int o_blocks = (M + kFcFo - 1) / kFcFo, n_blocks = (N + nb - 1) / nb;
     const int grid = grid_for(static_cast<long long>(o_blocks) * n_blocks, sm_count);
-    cudaError_t e = launch_kernel(fc_kernel, grid, 256, 0, s, static_cast<const __half*>(x), static_cast<const __half*>(w), bias,
+    auto* const kernel = nb == 1 ? fc_kernel<1> : (nb == 2 ? fc_kernel<2> : (nb == 4 ? fc_kernel<4> : fc_kernel<8>));
+    cudaError_t e = launch_kernel(kernel, grid, 256, 0, s, static_cast<const __half*>(x), static_cast<const __half*>(w), bias,
                                   static_cast<__half*>(y), N, K, M, act, o_blocks, n_blocks);
     return e == cudaSuccess ? DLF_OK : cuda_fail(e);
 }
