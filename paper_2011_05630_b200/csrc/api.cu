@@ -569,7 +569,10 @@ static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix,
         const int full_last = first + (net->layers[first].d.op == DLF_CONV ? 2 : 1);
         return full_last < static_cast<int>(net->layers.size()) && span_is_mbconv(net, first, full_last, false) && mbconv_pays(net, first, full_last, s_max, memo);
     }
-    if (net->opt_group_kernel == 2 && span_is_seq(net, first, last)) return true;
+    if (net->opt_group_kernel == 2 && span_is_seq(net, first, last)) {   // (not into a block that fuses better as a whole)
+        const int end = last + 2;
+        return end >= static_cast<int>(net->layers.size()) || !span_is_mbconv(net, last, end, false) || !mbconv_pays(net, last, end, s_max, memo);
+    }
     // a projection and the expansion layer it is added to are one product with a longer K: never slower than the two kernels
     if (span_is_projadd(net, first, last)) return true;
     if (!span_is_chain(net, first, last)) return false;

@@ -753,7 +753,7 @@ static MbconvTiling persistent_tiling(const MbconvArgs& a, int sm_count) {
 // 160 -> 960 -> 160 at 7x7: 23.1 -> 7.2 at one.  24 -> 144 -> 24 at 56x56, eight images: 15.4 here, one wave of tiles is none there.)
 MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
     const MbconvTiling t = persistent_tiling(a, sm_count), l = mbconv_lat_tiling(a, sm_count);
-    return l.ok && (!t.ok || l.cost < 0.97 * (t.cost + 3200.0)) ? l : t;
+    return t.ok && l.ok && l.cost < 0.97 * (t.cost + 3200.0) ? l : t;   // (what this kernel cannot hold is no group: plans stay as legal as they were)
 }
 
 int mbconv_tc_init() {

@@ -20,6 +20,7 @@ CASES = [
     (3, 30, 29, 24, 144, 24, 1, 0, 1, "relu6"),      # last chunk of half a group
     (40, 14, 14, 64, 384, 64, 1, 0, 1, "relu6"),     # four units to an accumulator, of two images
     (1, 15, 17, 24, 144, 32, 2, 0, 2, "relu"),
+    (1, 57, 50, 16, 96, 24, 2, 0, 1, "relu6"),       # a chunk of three groups
     (1, 7, 7, 160, 960, 320, 1, 0, 8, "relu6"),      # projection issued as two halves
     (3, 13, 9, 96, 160, 448, 1, 0, 1, "none"),       # the widest output
     (1, 1, 1, 8, 128, 8, 1, 0, 1, "relu6"),          # one pixel
