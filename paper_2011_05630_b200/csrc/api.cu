@@ -638,9 +638,9 @@ static int launch_group_part(dlf_net* net, const Group& g, const void* in_dev, c
 }
 // How many of the plan's first groups dlf_net_run_host works off part by part while the rest of the input is still on its way
 // (0: the input is copied as a whole).  Only a batch whose copy takes long enough (8 MB are 150 us), and groups whose own time,
-// about half of the copy's, hides behind it: a part's launches are less efficient than the whole batch's, so a longer head costs
+// about three fifths of the copy's by the estimates, hides behind it: a part's launches are less efficient than the whole batch's, so a longer head costs
 // more than it hides.  From page-locked memory at 224x224: ResNet-50, 32 images 810 -> 785 us (six groups), MobileNetV2, 64
-// images 960 -> 800 (five).
+// images 960 -> 800 (five), 762 with the next block (three quarters of the copy: 764, ResNet-18, 32 images 428 -> 445).
 static int host_head(const dlf_net* net) {
     if (!net->opt_graph || net->host_whole || net->N < 2 * kHostParts || net->in_bytes < (8u << 20)) return 0;
     const double copy_us = net->in_bytes / 50e3;
@@ -654,7 +654,7 @@ static int host_head(const dlf_net* net) {
         bytes += static_cast<double>(net->layers[g.last].bytes) * (net->layers[g.last].d.res_src != -2 ? 2 : 1);
         for (int i = g.first; i <= g.last; i++) flops += static_cast<double>(net->layers[i].flops);
         sum += g.kind == K_MBCONV ? g.mb_tiling.cost / 1.9e3 : (g.kind == K_CHAIN_TC ? g.tiling.cost / 1.9e3 : 2.0 + std::max(bytes / 3.5e6, flops / 500e6));
-        if (sum > 0.55 * copy_us) break;
+        if (sum > 0.6 * copy_us) break;
         count++;
     }
     return count;
