@@ -322,8 +322,9 @@ __global__ void __launch_bounds__(kAvgVecs * kAvgParts) gavgpool_kernel(const __
 // ---- fully connected --------------------------------------------------------------------------------------
 // A block owns 8 output features and streams their weight rows once per batch tile of NB images; threads stride over K in 128-bit
 // pieces, accumulate 8 x NB partial sums in fp32, then reduce.  Bound by latencies: the first weights are on their way before the wait
-// for the previous kernel, the next ones while the present ones are worked on, and one image pays for one (64 sums of eight images
-// were 320 shuffles a thread whatever the batch).  2048 -> 1000 at one image 5.1 -> 3.0 us, at two 4.5 -> 3.0.
+// for the previous kernel, the next ones while the present ones are worked on, one image pays for one (64 sums of eight images
+// were 320 shuffles a thread whatever the batch), and a warp's sums are exchanged in halves.  2048 -> 1000 at one image 5.15 -> 3.1 us,
+// at six 5.15 -> 4.1; 4096 -> 1000 at eight 6.7 -> 5.7.
 constexpr int kFcFo = 8;
 
 template <int NB>
@@ -382,15 +383,29 @@ __global__ void __launch_bounds__(256) fc_kernel(const __half* x, const __half* 
             }
             if (NB > 2) next_w();
         }
+        // A warp's sums: at every step of the exchange a lane keeps half of its values and sends the other half (64 values in 62 shuffles, the
+        // same tree as a sum of each by itself in 320); in the end lane l holds values `at`, at + 1, ...
+        float v[kFcFo * NB];
 #pragma unroll
-        for (int i = 0; i < kFcFo; i++)
+        for (int i = 0; i < kFcFo * NB; i++) v[i] = acc[i / NB][i % NB];
+        int at = 0;
+        constexpr int kLeft = kFcFo * NB > 32 ? kFcFo * NB / 32 : 1;   // values of a lane in the end
 #pragma unroll
-            for (int j = 0; j < NB; j++) {
-                float v = acc[i][j];
+        for (int d = 16, n = kFcFo * NB / 2; d > 0; d >>= 1, n >>= 1) {
+            if (n > 0) {
+                const bool up = (lane & d) != 0;
 #pragma unroll
-                for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-                if (lane == 0) red[warp][i * NB + j] = v;
+                for (int i = 0; i < n; i++) {
+                    const float send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+                }
+                at += up ? n : 0;
+            } else {
+                v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);   // (fewer values than lanes: the last steps add what is there)
             }
+        }
+#pragma unroll
+        for (int i = 0; i < kLeft; i++) red[warp][at + i] = v[i];   // (lanes that hold the same value write the same)
         __syncthreads();
         if (threadIdx.x < kFcFo * NB) {
             float v = 0.0f;
