@@ -1,13 +1,15 @@
 """Inverted-residual blocks on few images (one tile per CTA or cluster): every cluster size, hidden widths that leave the last chunk or
 its last 32-channel group part empty, windows over every edge of the image, several units to an accumulator, units past the
-last one, one and four input planes, outputs wider than one product, SM counts that leave no room for clusters."""
+last one, one and four input planes, outputs wider than one product, SM counts that leave no room for clusters; infinities and NaN."""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from paper_2011_05630_b200 import binding as B
+from paper_2011_05630_b200 import binding as B, synth
 from tests import gpu_util as G
+from tests.test_gpu_nonfinite import check_nonfinite
 from tests.test_gpu_parity import _conv, _mk
 
 # (n, h, w, cin, hidden, cout, stride, SMs (0: all), CTAs of a cluster, activation)
@@ -42,3 +44,14 @@ def test_block(case):
     first = sess.run(xd).clone()
     assert bool((sess.run(xd) == first).all())   # the same sum whatever the timing
     sess.close()
+
+
+@pytest.mark.parametrize("act", ["none", "relu", "relu6"])
+@pytest.mark.parametrize("stride", [1, 2])
+def test_nan_and_infinity(stride, act):
+    layers = [_conv(16, 128, 1, act=act), _conv(128, 128, 3, stride=stride, act=act, groups=128, op="dwconv", src=0), _conv(128, 24, 1, act=act, src=1)]
+    params = synth.layer_params("mbl nonfinite", layers)
+    x = synth.network_input("mbl nonfinite", 1, 21, 19, 16)
+    for i, v in enumerate((np.inf, -np.inf, np.nan)):
+        x[0, (2 + 8 * i) % 21, (3 + 6 * i) % 19, i] = v
+    check_nonfinite(layers, params, x, [2], 0, "mbconv_lat " + act)
