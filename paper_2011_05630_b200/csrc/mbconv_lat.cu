@@ -140,9 +140,12 @@ __device__ __forceinline__ void depthwise_task(const LatBlockParams& p, const Dw
     unsigned short x[NX];
     uint32_t raw[NX];
     int iy = t.y0, left = in_rows;
+    // A row is used once it has landed (wait()); the one behind it is on its way while it is worked on, but over no branch and from no trip
+    // of a loop to the next: until the wait its registers hold nothing that may be copied.
+    auto wait = [&]() { ld_row_wait<NX>(raw); };
     ld_row_issue<NX>(src, raw);
+    wait();
     auto next = [&]() {
-        ld_row_wait<NX>(raw);
         const uint32_t row_in = static_cast<unsigned>(iy) < static_cast<unsigned>(p.H) ? 0xffffffffu : 0u;
         uint32_t h[NP];
 #pragma unroll
@@ -161,8 +164,8 @@ __device__ __forceinline__ void depthwise_task(const LatBlockParams& p, const Dw
             x[2 * i] = a;
             if (2 * i + 1 < NX) x[(2 * i + 1) % NX] = b;
         }
-        src += NX;
-        if (--left > 0) ld_row_issue<NX>(src, raw);   // the next row, in flight while this one is worked on
+        if (--left > 0) src += NX;   // (behind the last row that one once more: a load in one branch alone would have to be merged with what `raw` holds in the other)
+        ld_row_issue<NX>(src, raw);
         iy++;
     };
     auto add = [&](float (&acc)[kUnitW], int r) {
@@ -177,6 +180,7 @@ __device__ __forceinline__ void depthwise_task(const LatBlockParams& p, const Dw
         add(acc, 0);
     };
     int v = t.v0;
+    const uint32_t live = t.live;
     auto store = [&](const float (&acc)[kUnitW]) {
         uint4 o;
         o.x = round_clamp<RELU6>(acc[0], acc[1], lo2, hi2);
@@ -184,7 +188,8 @@ __device__ __forceinline__ void depthwise_task(const LatBlockParams& p, const Dw
         o.z = round_clamp<RELU6>(acc[4], acc[5], lo2, hi2);
         o.w = round_clamp<RELU6>(acc[6], acc[7], lo2, hi2);
         const uint32_t at = t.dst + ((v & 8) ? t.lbo : 0u) + (((static_cast<uint32_t>(v) & 7u) ^ t.k7) << 4);
-        if (t.live) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w) : "memory");
+        asm volatile("{\n .reg .pred live;\n setp.ne.u32 live, %5, 0;\n @live st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n}"
+                     ::"r"(at), "r"(o.x), "r"(o.y), "r"(o.z), "r"(o.w), "r"(live) : "memory");
         v++;
     };
     const int rows = t.rows;
@@ -192,27 +197,27 @@ __device__ __forceinline__ void depthwise_task(const LatBlockParams& p, const Dw
     if (STRIDE == 1) {
         // input row j is the last row of output j - 2, the middle one of output j - 1, the first one of output j
         float c[kUnitW];
-        next(); start(a);
-        next(); add(a, 1); start(b);
+        next(); start(a); wait();
+        next(); add(a, 1); start(b); wait();
         int j = 0;
 #pragma unroll 1
         while (true) {
-            next(); add(a, 2); store(a);
+            next(); add(a, 2); store(a); wait();
             if (++j == rows) break;
             add(b, 1); start(c);
-            next(); add(b, 2); store(b);
+            next(); add(b, 2); store(b); wait();
             if (++j == rows) break;
             add(c, 1); start(a);
-            next(); add(c, 2); store(c);
+            next(); add(c, 2); store(c); wait();
             if (++j == rows) break;
             add(a, 1); start(b);
         }
     } else {
-        next(); start(a);
+        next(); start(a); wait();
 #pragma unroll 1
         for (int j = 0;;) {
-            next(); add(a, 1);
-            next(); add(a, 2); store(a);
+            next(); add(a, 1); wait();
+            next(); add(a, 2); store(a); wait();
             if (++j == rows) break;
             start(a);
         }
@@ -364,11 +369,10 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kThreads, 1) mbc
                 uint32_t v[16];
                 tmem_ld16_issue(taddr + c0, v);
                 tmem_ld16_wait(v);
-                if (at < 0 || !ok) continue;
 #pragma unroll
                 for (int g = 0; g < 2; g++) {
                     const int co = c0 + g * 8;
-                    if (co >= p.Cout) break;
+                    if (at < 0 || !ok || co >= p.Cout) break;
                     uint4 rv = make_uint4(0u, 0u, 0u, 0u);
                     if (p.res) rv = ld_map(reinterpret_cast<const uint4*>(p.res + at + co));
                     float a[8];
@@ -376,6 +380,7 @@ __global__ void __cluster_dims__(SPLIT, 1, 1) __launch_bounds__(kThreads, 1) mbc
                     for (int e = 0; e < 8; e++) a[e] = __uint_as_float(v[g * 8 + e]);
                     *reinterpret_cast<uint4*>(p.out + at + co) = finish8(a, b2s + co, rv, lo3, hi3);
                 }
+                __syncwarp();   // (the next load is the whole warp's)
             }
         } else {
             const uint32_t swz = p.n2_pad % 32 == 0 ? 7u : 3u;   // (a row's 16-byte vectors in an order that depends on the row: other banks)
