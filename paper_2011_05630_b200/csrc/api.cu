@@ -536,8 +536,8 @@ static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTi
     return false;
 }
 
-// The estimate for an inverted-residual block: the fused kernel's own (the tiler's SM clocks; the persistent kernel's leaves out
-// 1.8 us of launch, fill and drain, the other one's is about 0.6 low on the smallest blocks) against one kernel per layer.  Inside a network a layer's own kernel takes 2.9 us plus its bytes at
+// The estimate for an inverted-residual block: the fused kernel's own, launch included, against one kernel per layer.  Inside a network a
+// layer's own kernel takes 2.9 us plus its bytes at
 // 3.6 TB/s (the depthwise one) or 3.2 TB/s (the pointwise ones) - fitted to MobileNetV2's blocks at 1 to 128 images, each timed
 // both ways: on few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.6 us against 8.7), from a few
 // images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
@@ -558,7 +558,7 @@ static bool mbconv_pays(const dlf_net* net, int first, int last, int sms, SpanTi
                              (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
         single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + 2.9;
     }
-    return t.cost / 1.9e3 + (t.split > 0 ? 0.6 : 1.8) < single_us;
+    return t.us < single_us;
 }
 
 static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix, int s_max, SpanTimes* memo = nullptr) {
@@ -653,7 +653,7 @@ static int host_head(const dlf_net* net) {
         double bytes = static_cast<double>(net->layers[g.first].in[0] * net->layers[g.first].in[1] * net->layers[g.first].in[2] * net->layers[g.first].in[3] * 2), flops = 0.0;
         bytes += static_cast<double>(net->layers[g.last].bytes) * (net->layers[g.last].d.res_src != -2 ? 2 : 1);
         for (int i = g.first; i <= g.last; i++) flops += static_cast<double>(net->layers[i].flops);
-        sum += g.kind == K_MBCONV ? g.mb_tiling.cost / 1.9e3 : (g.kind == K_CHAIN_TC ? g.tiling.cost / 1.9e3 : 2.0 + std::max(bytes / 3.5e6, flops / 500e6));
+        sum += g.kind == K_MBCONV ? g.mb_tiling.us : (g.kind == K_CHAIN_TC ? g.tiling.cost / 1.9e3 : 2.0 + std::max(bytes / 3.5e6, flops / 500e6));
         if (sum > 0.6 * copy_us) break;
         count++;
     }

@@ -196,9 +196,10 @@ struct MbconvTiling {
     int out_planes;  // 64-channel planes of the output staging buffer, 0 = none (direct stores)
     int bh, units, job_units, parts, split;   // mbconv_lat.cu (split > 0): output rows of a unit (8 columns wide), units of a tile and of one accumulator,
                                               // warps of a unit, CTAs of a tile
+    bool narrow;     // mbconv_lat.cu: several chunks of 64 or fewer hidden channels per CTA, half of the depthwise warps without work
     size_t smem_bytes;
     double redundancy;
-    double cost;     // the tiler's time estimate (SM clocks)
+    double us;       // estimated time among other kernels, launch included
     bool ok;
 };
 bool mbconv_supported(const MbconvArgs& a);

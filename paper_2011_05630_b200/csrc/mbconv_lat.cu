@@ -639,11 +639,11 @@ bool lat_layout(const MbconvArgs& a, int bh, int U, int UG, int parts, int split
     return false;
 }
 
-// SM clocks of the block, launch included: least squares over 6000 measured choices of nine MobileNetV2 blocks at 1 to 64 images (6 %
-// rms; the choices made by it take 535 us in all over 46 cases, the best ones 526).  A round is what a lane quarter's four warps do
-// side by side, a job what one accumulator takes to be issued and handed over; a cluster's exchange of sums takes 1.5 us, less the
-// smaller a CTA's share of them.
-double lat_cost(const MbconvArgs& a, const LatLayout& L, int bh, int U, int UG, int parts, int split, int sm_count) {
+// What one choice of units and clusters takes against another one of the same block, in SM clocks: least squares over 6000 measured choices
+// of nine MobileNetV2 blocks at 1 to 64 images (the choices made by it take 535 us in all over 46 cases, the best ones 526).  A round is
+// what a lane quarter's four warps do side by side, a job what one accumulator takes to be issued and handed over; a cluster's exchange of
+// sums takes 1.5 us, less the smaller a CTA's share of them.
+double lat_rank(const MbconvArgs& a, const LatLayout& L, int bh, int U, int UG, int parts, int split, int sm_count) {
     const int tasks = U * parts, rounds = L.per_cta * ((tasks + 3) / 4), jobs = L.per_cta * (U / UG), side = std::min(4, tasks);
     const double in_rows = (L.part_rows - 1) * a.stride + 3;
     const double load = (0.4 * L.per_cta * L.cg * 32 * (L.n2 * 2 + L.kin * 128) + 3.7 * U * L.kin * L.xplane) / 57.0;
@@ -651,15 +651,30 @@ double lat_cost(const MbconvArgs& a, const LatLayout& L, int bh, int U, int UG, 
            80.0 * L.n2 * U * bh / 16.0 + (L.n_tiles * split > sm_count / 2 ? 1650.0 : 0.0) + (split > 1 ? 3465.0 - 598.0 * (split == 2 ? 1 : split == 4 ? 2 : 3) : 0.0);
 }
 
+// The time of the choice that was made, among other kernels and launch included: least squares over 12300 measured choices for 3900 blocks
+// (8 to 256 channels in, to 320 out, 16 to 1024 hidden, maps of 4x4 to 130x112, 1 to 64 images, 16 to 148 SMs; 6.3 % rms, at most 26 % too low,
+// where lat_rank is 10 % and 74).  What those nine blocks do not show: chunks that wait for each other because there is room for one
+// accumulator or one Hd buffer only, and the expansion's own time, which goes with its columns and input planes.
+double lat_us(const MbconvArgs& a, const LatLayout& L, int bh, int U, int UG, int parts, int split, int sm_count) {
+    const int tasks = U * parts, rounds = L.per_cta * ((tasks + 3) / 4), jobs = L.per_cta * (U / UG), side = std::min(4, tasks);
+    const double in_rows = (L.part_rows - 1) * a.stride + 3;
+    const double load = (0.6 * L.per_cta * L.cg * 32 * (L.n2 * 2 + L.kin * 128) + 0.7 * U * L.kin * L.xplane) / 57.0;
+    double clocks = 8730.0 + rounds * in_rows * (114.0 + 97.0 * side) + 448.0 * jobs + 73.0 * std::max(0, tasks - 4) * L.per_cta + load + 1.8 * L.per_cta * L.kin * U * L.npx +
+                  41.0 * L.n2 * U * bh / 16.0 + (L.n_tiles * split > sm_count / 2 ? 1076.0 : 0.0) + (split > 1 ? 1266.0 + 197.0 * (split == 2 ? 1 : split == 4 ? 2 : 3) : 0.0);
+    if (L.per_cta > 1) clocks += (L.hdbufs == 1 ? 962.0 * L.per_cta : 0.0) + (L.slots == 1 ? 593.0 * jobs : 0.0);
+    return clocks / 1.9e3;
+}
+
 }  // namespace
 
-// Units and clusters of the block, least estimated time; not `ok` where the block is none of this kernel's: no expansion layer, more
+// Units and clusters of the block, the least of lat_rank; not `ok` where the block is none of this kernel's: no expansion layer, more
 // tiles than fit the chip at once, or fewer than 128 hidden channels at stride 1, where lane quarters would stand idle (at stride 2 the
 // persistent kernel's walk over four times the outputs' inputs costs more than that: 16 -> 96 -> 24 at 112x112, one image 9.2 -> 7.2 us,
 // three 10.7 -> 8.2).
 MbconvTiling mbconv_lat_tiling(const MbconvArgs& a, int sm_count) {
     MbconvTiling best{};
     best.ok = false;
+    double best_rank = 0.0;
     if (!a.has_expand || (a.hid < 128 && a.stride == 1) || !mbconv_supported(a) || sm_count < 1) return best;
     const int Ho = (a.H + 2 - 3) / a.stride + 1, Wo = (a.W + 2 - 3) / a.stride + 1;
     const long long unit_cols = static_cast<long long>(a.N) * ((Wo + kUnitW - 1) / kUnitW);
@@ -673,11 +688,13 @@ MbconvTiling mbconv_lat_tiling(const MbconvArgs& a, int sm_count) {
                     for (int split = 1; split <= 8; split *= 2) {
                         LatLayout L;
                         if (!lat_layout(a, bh, U, UG, parts, split, sm_count, &L)) continue;
-                        const double cost = lat_cost(a, L, bh, U, UG, parts, split, sm_count);
-                        if (best.ok && cost >= best.cost) continue;
+                        const double rank = lat_rank(a, L, bh, U, UG, parts, split, sm_count);
+                        if (best.ok && rank >= best_rank) continue;
+                        best_rank = rank;
                         best.bh = bh; best.units = U; best.job_units = UG; best.parts = parts; best.split = split; best.n_tiles = L.n_tiles;
                         best.smem_bytes = L.smem;
-                        best.cost = cost;
+                        best.narrow = L.cg <= 2 && L.per_cta > 1;
+                        best.us = lat_us(a, L, bh, U, UG, parts, split, sm_count);
                         best.redundancy = static_cast<double>(L.fpx) / (std::min(bh, Ho) * a.stride * std::min(kUnitW, Wo) * a.stride);
                         best.ok = true;
                     }

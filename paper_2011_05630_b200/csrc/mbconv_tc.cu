@@ -740,7 +740,7 @@ static MbconvTiling persistent_tiling(const MbconvArgs& a, int sm_count) {
                 best.stages = L.stages; best.stage_bytes = L.stage_bytes;
                 best.smem_bytes = L.smem;
                 best.out_planes = L.so_planes;
-                best.cost = cost;
+                best.us = (cost + 3200.0) / 1.9e3;   // (launch, fill and drain)
                 best.redundancy = static_cast<double>(L.FR) / (std::min(th, Ho) * a.stride * std::min(tw, Wo) * a.stride);
                 best.ok = true;
             }
@@ -748,12 +748,14 @@ static MbconvTiling persistent_tiling(const MbconvArgs& a, int sm_count) {
     return best;
 }
 
-// The kernel of mbconv_lat.cu where its tiles fit the chip at once and its estimate is the lower one.  (That one includes the launch; this
-// kernel's own leaves out about 1.7 us of it.  64 -> 384 -> 64 at 14x14: 12.8 -> 6.6 us at one image, 18.5 -> 13.3 at 64;
-// 160 -> 960 -> 160 at 7x7: 23.1 -> 7.2 at one.  24 -> 144 -> 24 at 56x56, eight images: 15.4 here, one wave of tiles is none there.)
+// The kernel of mbconv_lat.cu where its tiles fit the chip at once and its estimate is clearly the lower one: both are within 6 to 9 % as a
+// rule, and further apart where that kernel works on narrow chunks.  Over 2350 blocks that both can run, each timed: 0.690 of the persistent
+// kernel's time, against 0.688 with the better of the two each time; slower than it by more than 5 % in five, 12 % at the most.
+// 64 -> 384 -> 64 at 14x14: 12.8 -> 6.5 us at one image; 24 -> 144 -> 24 at 56x56, eight images: 15.4 here, one wave of tiles is none there;
+// 128 -> 768 -> 104, stride 2 at 41x37, 27 images: 46 here, 75 there.
 MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
     const MbconvTiling t = persistent_tiling(a, sm_count), l = mbconv_lat_tiling(a, sm_count);
-    return t.ok && l.ok && l.cost < 0.97 * (t.cost + 3200.0) ? l : t;   // (what this kernel cannot hold is no group: plans stay as legal as they were)
+    return t.ok && l.ok && l.us < (l.narrow ? 0.8 : 0.93) * t.us ? l : t;   // (what this kernel cannot hold is no group: plans stay as legal as they were)
 }
 
 int mbconv_tc_init() {
