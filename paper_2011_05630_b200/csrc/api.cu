@@ -537,9 +537,10 @@ static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTi
 }
 
 // The estimate for an inverted-residual block: the fused kernel's own, launch included, against one kernel per layer.  Inside a network a
-// layer's own kernel takes 2.9 us plus its bytes at
-// 3.6 TB/s (the depthwise one) or 3.2 TB/s (the pointwise ones) - fitted to MobileNetV2's blocks at 1 to 128 images, each timed
-// both ways: on few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.6 us against 8.7), from a few
+// layer's own kernel takes 3.3 us (a pointwise one of at most 64 channels on either side 2.8) plus its bytes at 3.6 TB/s (the depthwise
+// one) or 3.2 TB/s (the pointwise ones): the best of the constants over 3400 random blocks, each timed both ways among nine others of
+// its kind; what is proposed takes 2.3 % longer than the better of the two in the geometric mean, the former 2.9 us a layer 3.1 %.
+// On few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.6 us against 8.7), from a few
 // images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
 // small maps lose at many images (160 -> 960 -> 160 at 7x7: 27 us against 20 at 64), and so does a block without an expansion layer.
 // (`memo`: 1 or 0 for the blocks of one tuner pass, each asked for several times)
@@ -556,7 +557,8 @@ static bool mbconv_pays(const dlf_net* net, int first, int last, int sms, SpanTi
         const Layer& l = net->layers[i];
         const double bytes = static_cast<double>(l.in[0] * l.in[1] * l.in[2] * l.in[3] * 2) + static_cast<double>(l.bytes) + static_cast<double>(l.w_elems * 2) +
                              (l.d.res_src != -2 ? static_cast<double>(l.bytes) : 0.0);
-        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + 2.9;
+        const bool narrow = l.d.op == DLF_CONV && l.d.cin <= 64 && l.d.cout <= 64;
+        single_us += std::max(static_cast<double>(l.flops) / 600e6, bytes / (l.d.op == DLF_DWCONV ? 3.6e6 : 3.2e6)) + (narrow ? 2.8 : 3.3);
     }
     return t.us < single_us;
 }
