@@ -503,6 +503,7 @@ static double single_layer_us(const Layer& l, int sms) {
     return 2.4 + (l.d.kh == 3 ? 0.7 : 0.0) +
            std::max({0.1 * chunks, rounds * (0.75 + 0.3 * chunks) * (l.d.cin % 16 ? 2.0 : 1.0), static_cast<double>(l.flops) / 600e6, bytes / 5.5e6});
 }
+static double tiling_us(const ChainTiling& t) { return 1.1 * t.cost / 1.9e3 + 0.3; }
 // The chain first..last as one kernel; negative if it cannot run as one.
 // (`memo`: the spans of one tuner pass, each asked for several times; tiling a span takes 0.1 ms)
 static double chain_us(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling, SpanTimes* memo = nullptr) {
@@ -513,7 +514,7 @@ static double chain_us(const dlf_net* net, int first, int last, int sms, ChainTi
     }
     const ChainTiling t = chain_tc_tiling(chain_args(net, first, last, nullptr, nullptr), sms, net->dev_sms > 0 ? net->dev_sms : sms);
     if (tiling) *tiling = t;
-    return t.ok ? 1.1 * t.cost / 1.9e3 + 0.3 : -1.0;
+    return t.ok ? tiling_us(t) : -1.0;
 }
 // True if the fused kernel is expected to beat one kernel per layer on `sms` SMs.  `tiling` receives the fused kernel's tiling.
 static bool chain_pays(const dlf_net* net, int first, int last, int sms, ChainTiling* tiling, SpanTimes* memo) {
@@ -640,9 +641,12 @@ static int launch_group_part(dlf_net* net, const Group& g, const void* in_dev, c
 }
 // How many of the plan's first groups dlf_net_run_host works off part by part while the rest of the input is still on its way
 // (0: the input is copied as a whole).  Only a batch whose copy takes long enough (8 MB are 150 us), and groups whose own time,
-// about three fifths of the copy's by the estimates, hides behind it: a part's launches are less efficient than the whole batch's, so a longer head costs
-// more than it hides.  From page-locked memory at 224x224: ResNet-50, 32 images 810 -> 785 us (six groups), MobileNetV2, 64
-// images 960 -> 800 (five), 762 with the next block (three quarters of the copy: 764, ResNet-18, 32 images 428 -> 445).
+// about 0.64 of the copy's by the estimates, hides behind it: a part's launches are less efficient than the whole batch's, so a longer head
+// costs more than it hides; and none whose part has neither 32 pixels nor two tiles of 32 pixels by 64 channels for each SM: its four
+// launches then take almost four times the whole one's.  A layer by itself is taken to cost 3.3 us beside its bytes, as in mbconv_pays, and to
+// reach 400 TFLOP/s.  From page-locked memory, some of 31 batches that were tried: MobileNetV2, 64 images 748 us (five groups; 800 with four,
+// 740 with six), 48 images 616 (five; 653 with four); AlexNet, 28 images 302 (two convolutions; 348 with all five); ResNet-18, 28 images
+// 399 (405 with one group more).  0.45 to 0.72, 0 to 128 pixels and 400 to 500 TFLOP/s were tried (at 0.72 ResNet-18 is 4 % slower).
 static int host_head(const dlf_net* net) {
     if (!net->opt_graph || net->host_whole || net->N < 2 * kHostParts || net->in_bytes < (8u << 20)) return 0;
     const double copy_us = net->in_bytes / 50e3;
@@ -655,8 +659,10 @@ static int host_head(const dlf_net* net) {
         double bytes = static_cast<double>(net->layers[g.first].in[0] * net->layers[g.first].in[1] * net->layers[g.first].in[2] * net->layers[g.first].in[3] * 2), flops = 0.0;
         bytes += static_cast<double>(net->layers[g.last].bytes) * (net->layers[g.last].d.res_src != -2 ? 2 : 1);
         for (int i = g.first; i <= g.last; i++) flops += static_cast<double>(net->layers[i].flops);
-        sum += g.kind == K_MBCONV ? g.mb_tiling.us : (g.kind == K_CHAIN_TC ? g.tiling.cost / 1.9e3 : 2.0 + std::max(bytes / 3.5e6, flops / 500e6));
-        if (sum > 0.6 * copy_us) break;
+        const double pixels = net->N / kHostParts * static_cast<double>(net->layers[g.last].ho_pre) * net->layers[g.last].wo_pre;
+        if (pixels < 32.0 * net->dev_sms && pixels * net->layers[g.last].d.cout < 2.0 * 32 * 64 * net->dev_sms) break;
+        sum += g.kind == K_MBCONV ? g.mb_tiling.us : (g.kind == K_CHAIN_TC ? tiling_us(g.tiling) : 3.3 + std::max(bytes / 3.5e6, flops / 400e6));
+        if (sum > 0.64 * copy_us) break;
         count++;
     }
     return count;
