@@ -234,7 +234,7 @@ int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes,
  *                               group of the plan (captured on the first run and whenever the
  *                               input / output pointers, weights, workspace or plan change);
  *                               0: launch the kernels one by one.  Does not clear the plan.
- *   DLF_OPT_PDL              1 (default): the kernels (conv_seq excepted) are launched with programmatic
+ *   DLF_OPT_PDL              1 (default): the kernels (conv_seq and a run's first one excepted) are launched with programmatic
  *                               dependent launch, so that a kernel's set-up overlaps the tail of
  *                               its predecessor; 0: plain stream order.  Process-wide.
  *   DLF_OPT_CONV_ROW_MODE    1 (default): a single 3x3 stride-1 convolution whose C_in is a multiple of 64 may load

@@ -23,6 +23,7 @@ namespace dlf {
 
 static thread_local int g_last_cuda_error = 0;
 int g_use_pdl = 1;
+thread_local bool g_stream_order = false;
 thread_local const GraphNodeUpdate* g_node_update = nullptr;
 thread_local LaunchRecord* g_launch_record = nullptr;
 int g_conv_row_mode = 1;
@@ -1260,7 +1261,9 @@ int dlf_net_run(dlf_net* net, const void* in_f16_dev, void* out_f16_dev, void* s
         if (rc) return rc;
     } else {
         for (const Group& g : net->plan) {
+            g_stream_order = &g == &net->plan[0];
             rc = launch_group(net, g, in_f16_dev, out_f16_dev, s);
+            g_stream_order = false;
             if (rc) return rc;
         }
     }

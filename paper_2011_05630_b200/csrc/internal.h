@@ -111,8 +111,10 @@ struct LaunchRecord {
 extern thread_local LaunchRecord* g_launch_record;
 
 // Launches a kernel, optionally with programmatic dependent launch (the kernel must then call
-// pdl_wait() before it touches anything its predecessor in the stream produces).
+// pdl_wait() before it touches anything its predecessor in the stream produces; weights and biases, which it may read ahead of
+// that, are produced before the run: a run's first kernel is launched in plain stream order, g_stream_order, calling thread only).
 extern int g_use_pdl;
+extern thread_local bool g_stream_order;
 extern int g_conv_row_mode;  // conv_tc row mode: 0 never, 1 where it cuts the streamed bytes by a fifth, 2 wherever it applies
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_opt(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s, bool pdl, Args&&... args) {
@@ -143,7 +145,7 @@ inline cudaError_t launch_kernel_opt(void (*kernel)(KArgs...), int grid, int blo
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = pdl && !g_stream_order ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
