@@ -1,6 +1,7 @@
 """Inverted-residual blocks as one kernel: the depthwise walk's columns, strips and lanes (hidden chunks of 64, 48, 32 and 16
 channels), both strides, maps smaller than a tile, ragged tiles, many tiles per CTA, one SM, blocks without an expansion layer,
-wide outputs (issued as two halves, direct stores)."""
+wide outputs (issued as two halves, direct stores).  `test_block` takes the kernel that the sizes send a block to ("mbconv_tc" is the
+group's kind: the persistent kernel, or on few images the one by clusters), `test_persistent_kernel` asks for the former by name."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -37,4 +38,33 @@ def test_block(case):
     for s in (B.device_sm_count(), 7, 1):
         G.check_plan(sess, xd, ref, [last], [s], "block S=%d" % s)
         assert sess.kernels() == ["mbconv_tc"]
+    sess.close()
+
+
+# (n, h, w, cin, hidden, cout, stride, activation): sizes at which the persistent kernel is the faster one on all SMs
+PERSISTENT = [
+    (33, 21, 19, 24, 144, 24, 1, "relu6"),      # last chunk of 16 channels, residual
+    (60, 21, 19, 16, 80, 40, 2, "relu"),        # the same, stride 2
+    (60, 21, 19, 32, 160, 32, 2, "relu6"),      # last chunk of 32
+    (60, 21, 19, 40, 240, 40, 1, "relu6"),      # last chunk of 48, residual
+    (17, 21, 19, 24, 48, 16, 2, "none"),        # that one alone
+    (33, 21, 19, 64, 192, 64, 1, "none"),       # whole chunks, residual
+    (17, 21, 19, 72, 208, 136, 1, "relu"),      # two input planes
+    (9, 21, 19, 160, 320, 160, 1, "relu6"),     # three, residual
+    (9, 21, 19, 200, 400, 24, 2, "none"),       # four
+    (5, 21, 19, 136, 272, 320, 1, "relu6"),     # projection issued as two halves
+    (9, 21, 19, 136, 272, 320, 2, "relu6"),
+]
+
+
+@pytest.mark.parametrize("case", PERSISTENT, ids=lambda c: "n%d_%dx%d_%d_%d_%d_s%d" % c[:7])
+def test_persistent_kernel(case):
+    n, h, w, cin, hid, cout, stride, act = case
+    layers = [_conv(cin, hid, 1, act=act), _conv(hid, hid, 3, stride=stride, act=act, groups=hid, op="dwconv", src=0),
+              _conv(hid, cout, 1, act="none", src=1, res_src=-1 if stride == 1 and cin == cout else -2)]
+    sess, xd, ref = _mk(layers, "mb", n, h, w, cin)
+    for s in (B.device_sm_count(), 37):
+        G.check_plan(sess, xd, ref, [2], [s], "block S=%d" % s)
+        name, grid, _ = sess.launches()[0]
+        assert name == "mbconv_tc_kernel<%d, %s>" % (stride, "true" if act == "relu6" else "false") and 2 < grid <= s, (name, grid)
     sess.close()

@@ -1,6 +1,7 @@
-"""Inverted-residual blocks on few images (one tile per CTA or cluster): every cluster size, hidden widths that leave the last chunk or
-its last 32-channel group part empty, windows over every edge of the image, several units to an accumulator, units past the
-last one, one and four input planes, outputs wider than one product, SM counts that leave no room for clusters; infinities and NaN."""
+"""Inverted-residual blocks on few images (one tile per CTA or cluster): every cluster size at both strides, hidden widths that leave the
+last chunk or its last 32-channel group part empty, chunks of 64, 96 and 128 channels, one buffer of each and several, windows over every
+edge of the image, a unit's rows by one, two and four warps, several units to an accumulator and several accumulators, units past the
+last one, one to four input planes, outputs wider than one product, SM counts that leave no room for clusters; infinities and NaN."""
 import numpy as np
 import pytest
 
@@ -29,6 +30,20 @@ CASES = [
     (1, 3, 2, 256, 1024, 16, 2, 0, 8, "relu6"),      # four input planes
     (2, 16, 16, 16, 128, 16, 1, 7, 1, "relu6"),
     (1, 8, 8, 16, 128, 16, 1, 1, 1, "relu"),
+    (29, 6, 5, 16, 176, 144, 1, 20, 1, "relu6"),     # three units, an accumulator each, the last tile short of two
+    (21, 27, 9, 16, 336, 24, 2, 20, 1, "relu6"),     # eight units, two to an accumulator, the last tile short of five
+    (1, 6, 38, 8, 320, 32, 1, 20, 4, "none"),        # a cluster with four units to an accumulator, units past the last
+    (7, 9, 5, 160, 304, 96, 2, 0, 4, "relu6"),       # the same at stride 2, three input planes
+    (3, 7, 20, 16, 496, 56, 2, 20, 4, "relu"),       # a cluster with three accumulators
+    (4, 14, 14, 96, 576, 160, 2, 0, 4, "relu6"),     # two chunks per CTA of a cluster
+    (1, 4, 9, 160, 592, 16, 2, 0, 8, "relu"),        # ... of 64 channels
+    (1, 13, 13, 256, 544, 256, 1, 20, 4, "relu6"),   # three chunks of 64 per CTA, one buffer of each, residual
+    (4, 10, 37, 160, 144, 352, 2, 60, 1, "relu6"),   # the same without a cluster, projection issued as two halves
+    (3, 6, 5, 136, 192, 136, 1, 60, 1, "relu6"),     # two chunks of 128 channels through one buffer
+    (1, 15, 4, 96, 352, 24, 2, 20, 4, "relu6"),      # chunks of 96 channels, rows by two warps
+    (19, 13, 12, 8, 304, 8, 2, 20, 1, "relu6"),      # rows by four warps, one accumulator
+    (4, 112, 112, 16, 96, 24, 2, 0, 1, "relu6"),     # two units, an accumulator each, rows by two warps
+    (7, 7, 7, 160, 960, 160, 1, 0, 8, "none"),
 ]
 
 

@@ -173,6 +173,27 @@ def test_the_tuner_proposes_the_blocks_that_are_faster_as_one_kernel(n, h, w, ci
     B.net_destroy(net)
 
 
+def test_with_the_hand_over_through_l2_a_run_of_layers_ends_ahead_of_a_block_that_pays():
+    layers = nw.mobilenet_v2()
+    heads = [i for i in range(3, len(layers) - 2) if layers[i + 1]["op"] == "dwconv" and layers[i]["op"] == "conv"]
+    seen = set()
+    for batch in (1, 64):
+        net = B.net_create(layers, batch, 224, 224, 3)
+        B.net_set_option(net, B.OPT_GROUP_KERNEL, 2)
+        for i in heads:   # the projection of the block before and this block's expansion: a run of two dense convolutions
+            pays = B.net_tuner_may_fuse(net, i, i + 2, False, 148)
+            assert B.net_tuner_may_fuse(net, i - 1, i, False, 148) == (not pays), (batch, i)
+            seen.add(pays)
+        B.net_set_option(net, B.OPT_GROUP_KERNEL, 0)
+        assert not any(B.net_tuner_may_fuse(net, i - 1, i, False, 148) for i in heads)   # (not proposed without the option)
+        B.net_destroy(net)
+    assert seen == {True, False}
+    net = B.net_create(nw.resnet50(), 1, 224, 224, 3)
+    B.net_set_option(net, B.OPT_GROUP_KERNEL, 2)
+    assert all(B.net_tuner_may_fuse(net, a, a + 3, False, 148) for a in (2, 6, 10))
+    B.net_destroy(net)
+
+
 # ---- the search's dynamic programme against exhaustive enumeration --------------------------------------------------
 def test_bruteforce_table_on_the_hand_worked_example():
     # the table of tests/test_oracle_model.py: three layers, core counts {1, 2}
