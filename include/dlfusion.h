@@ -9,7 +9,11 @@
  * (Sec. III-B: the output of a fused layer is produced on chip and reused at once); a
  * group's last layer is written to HBM.  All plans compute the same values: activations
  * are fp16, arithmetic is fp32, and every layer's result is rounded to fp16 once
- * (round-to-nearest-even) whether or not it leaves the chip.
+ * (round-to-nearest-even) whether or not it leaves the chip.  The order of a sum's additions
+ * belongs to the kernel and its tiling, which follow the group's size, N and the SM count: the
+ * same image in another batch, under another plan or in a part of a batch (dlf_net_run_host)
+ * may differ by single roundings (a network's output by up to 5e-4 of its 2-norm).  The same
+ * call on the same net gives the same bits.
  *
  * Conventions
  *   - Every call returns an int status: DLF_OK or a negative DLF_E_* code.  Nothing throws,
@@ -216,7 +220,7 @@ const char* dlf_net_group_kernel(const dlf_net* net, int group);
 /* What dlf_net_run launches for group g of the current plan: the kernel's name with its template arguments ("conv_lat_kernel<4>"
  * is a cluster of four CTAs; a 3x3 layer's ring stages "by rows" or "by columns" of the kernel), CTAs and threads per CTA.
  * "conv_tc" of dlf_net_group_kernel stands for several kernels, chosen by the layer's size and the SM count: conv_narrow, conv_lat,
- * conv_tc and conv_tc_pair.  Launches nothing; needs weights and workspace like a run.  Any out-pointer may be NULL. */
+ * conv_tc and conv_tc_pair; "mbconv_tc" for two: mbconv_tc and, where a block's tiles fit the SMs at once, mbconv_lat.  Launches nothing; needs weights and workspace like a run.  Any out-pointer may be NULL. */
 int dlf_net_group_launch(dlf_net* net, int group, char* name, size_t name_bytes, int* grid, int* block);
 
 /* Options (debugging and ablation); setting one clears the plan, which must be set again.

@@ -542,9 +542,10 @@ static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTi
 // layer's own kernel takes 3.3 us (a pointwise one of at most 64 channels on either side 2.8) plus its bytes at 3.6 TB/s (the depthwise
 // one) or 3.2 TB/s (the pointwise ones): the best of the constants over 3400 random blocks, each timed both ways among nine others of
 // its kind; what is proposed takes 2.3 % longer than the better of the two in the geometric mean, the former 2.9 us a layer 3.1 %.
-// On few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.6 us against 8.7), from a few
-// images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
-// small maps lose at many images (160 -> 960 -> 160 at 7x7: 27 us against 20 at 64), and so does a block without an expansion layer.
+// On few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.5 us against 10.4 by three kernels back to back),
+// from a few images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
+// small maps lose at many images (160 -> 960 -> 160 at 7x7: 23 us against 22 at 64), and so does a block without an expansion layer
+// (32 -> 16 at 112x112, 64 images: 86 against 46).
 // (`memo`: 1 or 0 for the blocks of one tuner pass, each asked for several times)
 static bool mbconv_pays(const dlf_net* net, int first, int last, int sms, SpanTimes* memo = nullptr) {
     if (memo) {
@@ -573,7 +574,9 @@ static bool tuner_may_fuse(const dlf_net* net, int first, int last, bool prefix,
         const int full_last = first + (net->layers[first].d.op == DLF_CONV ? 2 : 1);
         return full_last < static_cast<int>(net->layers.size()) && span_is_mbconv(net, first, full_last, false) && mbconv_pays(net, first, full_last, s_max, memo);
     }
-    if (net->opt_group_kernel == 2 && span_is_seq(net, first, last)) {   // (not into a block that fuses better as a whole)
+    // Not into a block that fuses better as a whole: with everything fused that can be, MobileNetV2 takes 0.56 ms in 25 groups at 64 images
+    // and 0.12 in 22 at one; 1.04 and 0.41 in 37 where a projection and the next block's expansion are one of them.
+    if (net->opt_group_kernel == 2 && span_is_seq(net, first, last)) {
         const int end = last + 2;
         return end >= static_cast<int>(net->layers.size()) || !span_is_mbconv(net, last, end, false) || !mbconv_pays(net, last, end, s_max, memo);
     }

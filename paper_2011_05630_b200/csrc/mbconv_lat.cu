@@ -17,9 +17,9 @@
 // that finishes them (st.async, counted by that CTA's barrier; conv_lat.cu), which adds them up in the order of the ranks, then bias,
 // residual, activation, rounding.  Every intermediate is rounded to fp16 where the layer-by-layer execution rounds it.
 //
-// 64 -> 384 -> 64 channels at 14x14: 12.8 -> 6.5 us at one image (three kernels 8.7), 18.7 -> 13.2 at 64; 96 -> 576 -> 96 there at 64
-// 24.7 -> 19.4; 160 -> 960 -> 160 at 7x7, one image: 23.1 -> 7.0 (three kernels 8.9); 32 -> 192 -> 32 at 28x28, one image 9.8 -> 6.5,
-// eight 10.8 -> 8.2; MobileNetV2 b1 166.4 -> 121.7 us, b64 556 -> 519.
+// Against mbconv_tc.cu's kernel: 64 -> 384 -> 64 channels at 14x14 12.7 -> 6.5 us at one image (three kernels 10.4), 18.4 -> 12.8 at 64;
+// 96 -> 576 -> 96 there at 64 24.7 -> 18.8; 160 -> 960 -> 160 at 7x7, one image 23.0 -> 7.1 (three kernels 11.1); 32 -> 192 -> 32 at 28x28,
+// one image 10.1 -> 6.6, eight 10.8 -> 8.1; MobileNetV2 b1 166 -> 113 us, b64 554 -> 513.
 // Measured bounds: a row of eight outputs takes a scheduler about 205 clocks (72 multiply-adds with fp16 factors, 2 clocks each; rounding,
 // clamps and unpacking, half rate, on the other pipe); a control warp's step between two chunks 500-1000.
 // With many tiles per CTA the kernel of mbconv_tc.cu is the faster one (24 -> 144 -> 24 at 56x56, 64 images 64.8 us against 68 of a
@@ -669,8 +669,8 @@ double lat_us(const MbconvArgs& a, const LatLayout& L, int bh, int U, int UG, in
 
 // Units and clusters of the block, the least of lat_rank; not `ok` where the block is none of this kernel's: no expansion layer, more
 // tiles than fit the chip at once, or fewer than 128 hidden channels at stride 1, where lane quarters would stand idle (at stride 2 the
-// persistent kernel's walk over four times the outputs' inputs costs more than that: 16 -> 96 -> 24 at 112x112, one image 9.2 -> 7.2 us,
-// three 10.7 -> 8.2).
+// persistent kernel's walk over four times the outputs' inputs costs more than that: 16 -> 96 -> 24 at 112x112, one image 9.1 -> 7.1 us,
+// three 10.2 -> 8.5).
 MbconvTiling mbconv_lat_tiling(const MbconvArgs& a, int sm_count) {
     MbconvTiling best{};
     best.ok = false;

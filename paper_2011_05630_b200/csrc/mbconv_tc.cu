@@ -751,7 +751,7 @@ static MbconvTiling persistent_tiling(const MbconvArgs& a, int sm_count) {
 // The kernel of mbconv_lat.cu where its tiles fit the chip at once and its estimate is clearly the lower one: both are within 6 to 9 % as a
 // rule, and further apart where that kernel works on narrow chunks.  Over 2350 blocks that both can run, each timed: 0.690 of the persistent
 // kernel's time, against 0.688 with the better of the two each time; slower than it by more than 5 % in five, 12 % at the most.
-// 64 -> 384 -> 64 at 14x14: 12.8 -> 6.5 us at one image; 24 -> 144 -> 24 at 56x56, eight images: 15.4 here, one wave of tiles is none there;
+// 64 -> 384 -> 64 at 14x14: 12.7 -> 6.5 us at one image; 24 -> 144 -> 24 at 56x56, eight images: 15.3 here, one wave of tiles is none there;
 // 128 -> 768 -> 104, stride 2 at 41x37, 27 images: 46 here, 75 there.
 MbconvTiling mbconv_tiling(const MbconvArgs& a, int sm_count) {
     const MbconvTiling t = persistent_tiling(a, sm_count), l = mbconv_lat_tiling(a, sm_count);
