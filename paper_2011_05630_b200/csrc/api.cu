@@ -541,7 +541,7 @@ static bool chain_grows(const dlf_net* net, int first, int last, int sms, SpanTi
 // The estimate for an inverted-residual block: the fused kernel's own, launch included, against one kernel per layer.  Inside a network a
 // layer's own kernel takes 3.3 us (a pointwise one of at most 64 channels on either side 2.8) plus its bytes at 3.6 TB/s (the depthwise
 // one) or 3.2 TB/s (the pointwise ones): the best of the constants over 3400 random blocks, each timed both ways among nine others of
-// its kind; what is proposed takes 2.3 % longer than the better of the two in the geometric mean, the former 2.9 us a layer 3.1 %.
+// its kind; what is proposed takes 2.4 % longer than the better of the two in the geometric mean, with 2.9 us a layer 3.1 %.
 // On few images the clusters of mbconv_lat.cu win (14x14, 64 -> 384 -> 64 at one image 6.5 us against 10.4 by three kernels back to back),
 // from a few images on maps of 14x14 and more the persistent kernel (24 -> 144 -> 24 at 56x56: 65 us against 96 at 64 images); wide blocks on
 // small maps lose at many images (160 -> 960 -> 160 at 7x7: 23 us against 22 at 64), and so does a block without an expansion layer
